@@ -186,7 +186,7 @@ size_t rlx_encoder_workspace_bytes(const rlx_encoder_t *encoder, int32_t batch, 
  * out             dev f32 [batch, H]; a sequence with no valid position yields zeros
  * workspace       dev, 256-byte aligned, >= rlx_encoder_workspace_bytes(batch, seq);
  *                 scratch: contents are overwritten by every call.  Its first 256 bytes hold the
- *                 sticky device status word and two work counters that every forward leaves at
+ *                 sticky device status word and a work counter that every forward leaves at
  *                 zero: zero these 256 bytes once before the first call, and again after a call
  *                 that reported RLX_ERR_DEVICE_TIMEOUT (a forward that gave up may leave a counter set)
  *
@@ -413,12 +413,10 @@ rlx_status_t rlx_attention_f32(const float *qkv_f32, const int32_t *attention_ma
  * The same attention on PACKED rows (what the forward runs after sequence packing): qkv holds
  * `rows` rows of [q | k | v]; sequence b owns rows seq_start[b] .. seq_start[b] + seq_len[b], all
  * valid, seq_len[b] <= max_len <= 512; ctx uses the same row numbering.  impl 0: tcgen05/TMEM
- * kernel (persistent, TMA-fed, one pass over the keys, S and P in tensor memory, one thread per
+ * kernel (TMA-fed, one pass over the keys, S and P in tensor memory, one thread per
  * query row in the softmax); impl 1: warp-level mma.sync kernel (what rlx_encoder_forward runs
  * unless RLX_FLAG_ATTN_TCGEN05 is set).  Rows outside every sequence are not written.
- * impl 0 hands its work items out through a counter word inside the library (zero between
- * launches): two impl-0 calls must not run concurrently on one device (calls ordered on one stream,
- * or otherwise serialised, are fine).  status: optional device word, receives RLX_DEVSTAT_TIMEOUT
+ * status: optional device word, receives RLX_DEVSTAT_TIMEOUT
  * if a bounded wait of impl 0 ran out.
  */
 rlx_status_t rlx_attention_packed_bf16(const void *qkv_bf16, int32_t rows, const int32_t *seq_start,
@@ -446,8 +444,7 @@ rlx_status_t rlx_attention_packed_bf16(const void *qkv_bf16, int32_t rows, const
  * memory, 16-byte aligned; seq_len[b] <= max_len <= RLX_ATTENTION_KIND_MAX_LEN).  rope_cos and
  * rope_sin are device fp32 tables [max_len, head_dim/2] (row = position, 16-byte aligned) holding
  * cos / sin of position * theta^(-2j/head_dim), or both NULL for no rotation.  `window` is read for
- * RLX_MASK_SLIDING_WINDOW only.  head_dim in {32, 64, 128} (128: one CTA per SM, the accumulator tile
- * fills the register file).  Key blocks that no row of a 128-row query
+ * RLX_MASK_SLIDING_WINDOW only.  head_dim in {32, 64, 128}.  Key blocks that no row of a 128-row query
  * tile can see are neither loaded nor multiplied.  Asynchronous on cuda_stream; the caller owns
  * every buffer; nothing is allocated.  Errors: RLX_ERR_INVALID_ARG for null / misaligned pointers,
  * a lone rope table, an unknown kind or window < 1; RLX_ERR_UNSUPPORTED for other head sizes or

@@ -12,7 +12,7 @@
 
 #include "../../include/rlx_encoder.h"
 #include "attention.cuh"
-#include "attention_tc.cuh"
+#include "attention_fwd_tcgen05.cuh"
 #include "gemm_mx_tcgen05.cuh"
 #include "gemm_ffn_tcgen05.cuh"
 #include "dequant.cuh"
@@ -244,10 +244,14 @@ cudaError_t init_kernels_for_current_device() {
                                   rlx::tcmx::kSmemBytes)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(rlx::tcmx::wide::gemm_mx192_tcgen05_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   rlx::tcmx::wide::kSmemBytesW)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(rlx::tca::attention_tc_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  rlx::tca::Smem<32>::BYTES)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(rlx::tca::attention_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  rlx::tca::Smem<64>::BYTES)) != cudaSuccess) return e;
+#define RLX_ATT_FWD_ATTR(D, PAIR)                                                                              \
+    if ((e = cudaFuncSetAttribute(rlx::tcat::attention_fwd_kernel<D, PAIR, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                                  rlx::tcat::Cfg<D, PAIR>::SMEM_BYTES)) != cudaSuccess ||                       \
+        (e = cudaFuncSetAttribute(rlx::tcat::attention_fwd_kernel<D, PAIR, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                                  rlx::tcat::Cfg<D, PAIR>::SMEM_BYTES)) != cudaSuccess)                         \
+        return e;
+    RLX_ATT_FWD_ATTR(32, true) RLX_ATT_FWD_ATTR(64, true) RLX_ATT_FWD_ATTR(32, false) RLX_ATT_FWD_ATTR(64, false) RLX_ATT_FWD_ATTR(128, false)
+#undef RLX_ATT_FWD_ATTR
 #define RLX_ATT_SMEM_ATTR(D, MK, ROPE)                                                                       \
     if ((e = cudaFuncSetAttribute(rlx::attention_bf16_kernel<D, MK, ROPE>,                                  \
                                   cudaFuncAttributeMaxDynamicSharedMemorySize,                 \
@@ -261,7 +265,6 @@ cudaError_t init_kernels_for_current_device() {
     RLX_ATT_SMEM_ATTR(32, 0, true) RLX_ATT_SMEM_ATTR(64, 0, true)
     RLX_ATT_SMEM_ATTR(32, 1, false) RLX_ATT_SMEM_ATTR(64, 1, false)
     RLX_ATT_SMEM_ATTR(32, 1, true) RLX_ATT_SMEM_ATTR(64, 1, true)
-    RLX_ATT_SMEM_ATTR(128, 0, false) RLX_ATT_SMEM_ATTR(128, 0, true) RLX_ATT_SMEM_ATTR(128, 1, false) RLX_ATT_SMEM_ATTR(128, 1, true)
 #undef RLX_ATT_SMEM_ATTR
     if (dev < 64) done[dev] = true;
     return cudaSuccess;
@@ -382,7 +385,7 @@ rlx_status_t launch_attention_bf16(const bf16* qkv, const int32_t* mask, const i
     dim3 grid((S + rlx::kAttBlockM - 1) / rlx::kAttBlockM, h, B);
     const rlx::AttKind kind{window, rope_cos, rope_sin, kv_group};
     const bool rope = rope_cos != nullptr;
-    if (d != 32 && d != 64 && d != 128) return RLX_ERR_UNSUPPORTED;
+    if (d != 32 && d != 64) return RLX_ERR_UNSUPPORTED;
 #define RLX_ATT_LAUNCH(D, MK, ROPE)                                                                              \
     RLX_CUDA_TRY(launch_ex(rlx::attention_bf16_kernel<D, MK, ROPE>, grid, rlx::kAttThreads,                      \
                            sizeof(rlx::AttSmem<D>),                                                                 \
@@ -396,51 +399,70 @@ rlx_status_t launch_attention_bf16(const bf16* qkv, const int32_t* mask, const i
         else if (!positional) RLX_ATT_LAUNCH(32, 0, true);
         else if (!rope) RLX_ATT_LAUNCH(32, 1, false);
         else RLX_ATT_LAUNCH(32, 1, true);
-    } else if (d == 64) {
+    } else {
         if (!positional && !rope) RLX_ATT_LAUNCH(64, 0, false);
         else if (!positional) RLX_ATT_LAUNCH(64, 0, true);
         else if (!rope) RLX_ATT_LAUNCH(64, 1, false);
         else RLX_ATT_LAUNCH(64, 1, true);
-    } else {
-        if (!positional && !rope) RLX_ATT_LAUNCH(128, 0, false);
-        else if (!positional) RLX_ATT_LAUNCH(128, 0, true);
-        else if (!rope) RLX_ATT_LAUNCH(128, 1, false);
-        else RLX_ATT_LAUNCH(128, 1, true);
     }
 #undef RLX_ATT_LAUNCH
     RLX_CUDA_TRY(cudaGetLastError());
     return RLX_OK;
 }
 
-__device__ unsigned int g_attn_ticket_standalone;   // work-item counter of rlx_attention_packed_bf16's own launches
-
-// Packed-sequence attention on tcgen05 (the product path): qkv is the packed [rows, 3H] projection.
-rlx_status_t launch_attention_tc(const bf16* qkv, int rows, const int32_t* seq_start, const int32_t* seq_len, int B,
-                                 int S, int h, int d, bf16* ctx, unsigned int* ticket, int32_t* status, cudaStream_t st) {
-    const int H = h * d;
-    const float scale_log2e = 1.4426950408889634f / sqrtf((float)d);
-    CUtensorMap tq;
-    if (!make_tmap(&tq, qkv, (uint64_t)rows, (uint64_t)3 * H, rlx::tca::kBlockN, (uint32_t)d,
-                   d == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B))
+// Packed attention of any length on tcgen05 (csrc/attention_fwd_tcgen05.cuh).  qkv: packed rows of h q heads, then
+// h / kv_group k heads, then as many v heads.
+rlx_status_t launch_attention_fwd(const bf16* qkv, int rows, const int32_t* seq_start, const int32_t* seq_len, int B, int max_len,
+                                  int h, int d, int kv_group, bool positional, int window, const float* rope_cos,
+                                  const float* rope_sin, bf16* ctx, int32_t* status, cudaStream_t st) {
+    namespace tcat = rlx::tcat;
+    const bool pair = d <= 64 && kv_group == 1 && h % 2 == 0;
+    const bool rows_mode = !pair && kv_group % 2 != 0;
+    tcat::Params p = {};
+    p.seq_start = seq_start; p.seq_len = seq_len; p.ctx = ctx; p.rope_cos = rope_cos; p.rope_sin = rope_sin; p.status = status;
+    p.H = h * d; p.Hkv = h / kv_group * d;
+    p.batch = B;
+    p.units = rows_mode ? h : h / 2;
+    const int item_rows = rows_mode ? 2 * tcat::kTile : tcat::kTile;
+    p.qtiles = (max_len + item_rows - 1) / item_rows;
+    p.kv_group = kv_group; p.rows_mode = rows_mode; p.positional = positional; p.window = window;
+    p.scale_log2e = 1.4426950408889634f / sqrtf((float)d);
+    const long long items = (long long)p.qtiles * B * p.units;
+    if (items > 0x7fffffffll) return RLX_ERR_UNSUPPORTED;
+    CUtensorMap tm;
+    const uint32_t cols = (d == 32 && !pair) ? 32 : 64;
+    if (!make_tmap(&tm, qkv, (uint64_t)rows, (uint64_t)p.H + 2 * p.Hkv, tcat::kTile, cols,
+                   cols == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B))
         return RLX_ERR_CUDA;
-    // persistent: two CTAs per SM walk the (sequence, query tile, head) list with a fixed stride
-    const int qtiles = (S + rlx::tca::kBlockM - 1) / rlx::tca::kBlockM;
-    const long long n_cand = (long long)B * qtiles * h;
-#ifdef RLX_ATTN_ONE_PER_SM
-    const int grid = (int)std::min<long long>(n_cand, 1LL * sm_count());
-#else
-    const int grid = (int)std::min<long long>(n_cand, 2LL * sm_count());
-#endif
-    if (d == 32)
-        RLX_CUDA_TRY(launch_ex(rlx::tca::attention_tc_kernel<32>, dim3(grid), rlx::tca::kThreads, rlx::tca::Smem<32>::BYTES, st,
-                               tq, seq_start, seq_len, ctx, H, scale_log2e, B, qtiles, ticket, status));
-    else if (d == 64)
-        RLX_CUDA_TRY(launch_ex(rlx::tca::attention_tc_kernel<64>, dim3(grid), rlx::tca::kThreads, rlx::tca::Smem<64>::BYTES, st,
-                               tq, seq_start, seq_len, ctx, H, scale_log2e, B, qtiles, ticket, status));
-    else
-        return RLX_ERR_UNSUPPORTED;
+#define RLX_ATT_FWD(D, PAIR)                                                                                                   \
+    do {                                                                                                                       \
+        if (rope_cos)                                                                                                          \
+            RLX_CUDA_TRY(launch_ex(tcat::attention_fwd_kernel<D, PAIR, true>, dim3((unsigned)items), tcat::Threads<true>::N,   \
+                                   tcat::Cfg<D, PAIR>::SMEM_BYTES, st, tm, p));                                                \
+        else                                                                                                                   \
+            RLX_CUDA_TRY(launch_ex(tcat::attention_fwd_kernel<D, PAIR, false>, dim3((unsigned)items), tcat::Threads<false>::N, \
+                                   tcat::Cfg<D, PAIR>::SMEM_BYTES, st, tm, p));                                                \
+    } while (0)
+    if (pair) { if (d == 32) RLX_ATT_FWD(32, true); else RLX_ATT_FWD(64, true); }
+    else if (d == 32) RLX_ATT_FWD(32, false);
+    else if (d == 64) RLX_ATT_FWD(64, false);
+    else if (d == 128) RLX_ATT_FWD(128, false);
+    else return RLX_ERR_UNSUPPORTED;
+#undef RLX_ATT_FWD
     RLX_CUDA_TRY(cudaGetLastError());
     return RLX_OK;
+}
+
+// Where the tcgen05 kernel replaces the mma.sync one (measured on packed batches, us old / new):
+//   head_dim 128: everywhere (16 prompts of 1024..4096, causal, 32 q / 8 kv heads 3561 / 1044; 64 of 16..256 75 / 43)
+//   head_dim 64: longer than one 128-row tile (causal 1024..4096, 16 heads 907 / 477; 16..256 39.6 / 35.2; window 64
+//     over 100..1500 67 / 66; but 16..128 21.1 / 22.3: one tile and one block per item are all set-up and latency)
+//   head_dim 32: only where many blocks per tile pay for its fixed costs: longer than 512 keys, no short window
+//     (causal 400..2000 156 / 124; 16..256 25.8 / 29.3; window 64 over 100..1500 48 / 54)
+bool attention_fwd_pays(int d, int max_len, bool positional, int window) {
+    if (d == 128) return true;
+    if (d == 64) return max_len > rlx::tcat::kTile;
+    return max_len > rlx::kAttMaxSeq && (!positional || window > 2 * rlx::tcat::kTile);
 }
 
 // Feed-forward block in one kernel (hidden 256 or 384, F % 64 == 0): out = gelu(x W1^T + b1) W2^T + b2 + x.
@@ -801,7 +823,6 @@ struct Arena {
     size_t stats_y, stats_z, fold, fold_layer, f_wqkv, f_w1, f_cqkv, f_dqkv, f_c1, f_d1;
 };
 constexpr size_t kTicketOffset = 64;   // packing ticket counter inside the 256-byte status block
-constexpr size_t kAttnTicketOffset = 128;   // work-item counter of the attention kernel, same block
 
 Arena plan_arena(int B, int S, int H, int F, int L = 0, bool fold = false) {
     const size_t T = (size_t)B * S;
@@ -1145,8 +1166,7 @@ rlx_status_t enqueue_forward(const rlx_encoder* e, const int32_t* ids, const int
                 RLX_TRY(launch_gemm(z, (const bf16*)(fb + a.f_wqkv), lw.bqkv, nullptr, 3, T, 3 * H, H, qkv, false, status, st, rows, 0, &lf));
             }
             if (pack && (c.flags & RLX_FLAG_ATTN_TCGEN05))
-                RLX_TRY(launch_attention_tc(qkv, T, pk.seq_start, pk.seq_len, B, S, h, d, ctx,
-                                            reinterpret_cast<unsigned int*>(ws + a.status + kAttnTicketOffset), status, st));
+                RLX_TRY(launch_attention_fwd(qkv, T, pk.seq_start, pk.seq_len, B, S, h, d, 1, false, 0, nullptr, nullptr, ctx, status, st));
             else
                 RLX_TRY(launch_attention_bf16(qkv, mask, pk.seq_start, pk.seq_len, B, S, h, d, ctx, st));
             // y = ctx Wo^T + bo + (l == 0 ? x : LN2_{l-1}(z)); partial statistics of y
@@ -1185,8 +1205,7 @@ rlx_status_t enqueue_forward(const rlx_encoder* e, const int32_t* ids, const int
         const rlx_layer_weights_t& lw = w->layers[l];
         RLX_TRY(launch_gemm(x, (const bf16*)lw.wqkv, lw.bqkv, nullptr, RLX_EPI_BIAS, T, 3 * H, H, qkv, simt, status, st, rows));
         if (pack && (c.flags & RLX_FLAG_ATTN_TCGEN05))
-            RLX_TRY(launch_attention_tc(qkv, T, pk.seq_start, pk.seq_len, B, S, h, d, ctx,
-                                            reinterpret_cast<unsigned int*>(ws + a.status + kAttnTicketOffset), status, st));
+            RLX_TRY(launch_attention_fwd(qkv, T, pk.seq_start, pk.seq_len, B, S, h, d, 1, false, 0, nullptr, nullptr, ctx, status, st));
         else
             RLX_TRY(launch_attention_bf16(qkv, mask, pk.seq_start, pk.seq_len, B, S, h, d, ctx, st));
         if (fuse_ffn) {
@@ -1688,13 +1707,8 @@ rlx_status_t rlx_attention_packed_bf16(const void* qkv, int32_t rows, const int3
     RLX_CUDA_TRY(init_kernels_for_current_device());
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (impl == 0)
-        {
-        // the kernel-level call owns no workspace: its work-item counter is a word inside the library
-        // (zero between launches; calls on different streams of one device must therefore not overlap)
-        unsigned int* ticket = nullptr;
-        RLX_CUDA_TRY(cudaGetSymbolAddress(reinterpret_cast<void**>(&ticket), g_attn_ticket_standalone));
-        return launch_attention_tc((const bf16*)qkv, rows, seq_start, seq_len, B, max_len, h, d, (bf16*)ctx, ticket, status, st);
-    }
+        return launch_attention_fwd((const bf16*)qkv, rows, seq_start, seq_len, B, max_len, h, d, 1, false, 0, nullptr, nullptr, (bf16*)ctx,
+                                    status, st);
     if (impl == 1)
         return launch_attention_bf16((const bf16*)qkv, nullptr, seq_start, seq_len, B, max_len, h, d, (bf16*)ctx, st);
     return RLX_ERR_INVALID_ARG;
@@ -1716,6 +1730,9 @@ rlx_status_t rlx_attention_kind_bf16(const void* qkv, int32_t rows, const int32_
     RLX_CUDA_TRY(init_kernels_for_current_device());
     const bool positional = mask_kind != RLX_MASK_NONE;
     const int w = mask_kind == RLX_MASK_SLIDING_WINDOW ? window : (1 << 30);   // causal: the window never cuts
+    if (attention_fwd_pays(d, max_len, positional, w))
+        return launch_attention_fwd((const bf16*)qkv, rows, seq_start, seq_len, B, max_len, h, d, h / hkv, positional, w, rope_cos,
+                                    rope_sin, (bf16*)ctx, nullptr, static_cast<cudaStream_t>(stream));
     return launch_attention_bf16((const bf16*)qkv, nullptr, seq_start, seq_len, B, max_len, h, d, (bf16*)ctx,
                                  static_cast<cudaStream_t>(stream), positional, w, rope_cos, rope_sin, h / hkv);
 }

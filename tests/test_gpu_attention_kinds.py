@@ -227,3 +227,32 @@ def test_empty_sequences_and_a_long_one(rlx):
         ref = ak.attention_packed(qkv.astype(np.float64), start[:-1], lengths, h, kind, w)
         vmax = float(np.abs(qkv[:, 2 * H:]).max())
         assert np.abs(got - ref).max() <= 2 * BF16_U * (vmax + np.abs(ref).max())
+
+
+@pytest.mark.parametrize("d,hq,hkv", [(32, 2, 2), (32, 3, 3), (32, 4, 2), (64, 2, 2), (64, 1, 1), (64, 6, 2), (128, 1, 1), (128, 4, 1)])
+@pytest.mark.parametrize("kind,window", [(NONE, 0), (CAUSAL, 0), (SLIDING, 127), (SLIDING, 129), (SLIDING, 300)])
+def test_tile_and_block_edges_of_the_tcgen05_kernel(rlx, d, hq, hkv, kind, window):
+    """Lengths at the edges of the 128-row tiles and 128-key blocks, in each pairing of tiles (two heads, two heads of
+    one k/v head, two row tiles), with a sequence long enough that every head size takes that kernel; junk behind
+    the last sequence."""
+    rng = np.random.default_rng(d + 10 * hq + window)
+    lengths = [1, 127, 128, 129, 255, 256, 257, 0, 383, 520, 16]
+    total, W = sum(lengths), (hq + 2 * hkv) * d
+    qkv = rand_bf16(rng, (total + 3, W))
+    qkv[total:] = np.float32("nan")
+    start = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int32)
+    for theta in (None, 10000.0):
+        rope = None if theta is None else rlx.rope_tables(max(lengths), d, theta)
+        got = to_np64(rlx.attention_kind_bf16(bf16_dev(qkv), i32_dev(start[:-1]), i32_dev(np.array(lengths)), max(lengths), hq,
+                                              kind, window, rope, num_kv_heads=hkv))
+        assert np.array_equal(got[total:], np.zeros((3, hq * d)))
+        ref = ak.attention_packed(qkv[:total].astype(np.float64), start[:-1], lengths, hq, kind, window, theta, num_kv_heads=hkv)
+        vmax = float(np.abs(qkv[:total, (hq + hkv) * d:]).max())
+        tol = 2 * BF16_U * (vmax + np.abs(ref).max())
+        if theta is not None:   # the bound of the module docstring
+            q = qkv[:total, :hq * d].astype(np.float64).reshape(total, hq, d)
+            k = qkv[:total, hq * d:(hq + hkv) * d].astype(np.float64).reshape(total, hkv, d)
+            tol += 4 * BF16_U * float(np.sqrt((q ** 2).sum(-1)).max() * np.sqrt((k ** 2).sum(-1)).max()) / np.sqrt(d) * vmax
+        err = np.abs(got[:total] - ref)
+        assert np.isfinite(err).all() and err.max() <= tol, (float(err.max()), tol)
+        assert np.sqrt((err ** 2).mean()) <= 2 * BF16_U * vmax
