@@ -7,22 +7,26 @@
 //                columns are neighbours in memory, so one tile brings q, k or v of both)
 //   otherwise    the same rows of two query heads of one K / V head (grouped-query layouts), or two consecutive
 //                row tiles of one head (everything else: "rows mode")
-// Items are numbered with the last row tiles first (under the causal mask these are the long ones), one CTA of the
-// grid per item; a CTA that has finished takes over the next one that has not been launched yet
-// (clusterlaunchcontrol), so tensor memory and barriers are set up once per SM, the loads of the next item run
-// behind the current one, and no counter in global memory is needed: calls on several streams do not meet.
+// The CTAs (one per SM) walk the items that exist with a fixed stride, last row tiles first (under the causal mask these
+// are the long ones): a warp scans the sequence lengths 32 at a time, so tiles past a sequence's end cost nothing and
+// no counter in global memory is needed (calls on several streams do not meet).
 //
-//   warps 0..3, 4..7  softmax of tile 0 / tile 1, one thread per query row (no shuffles): 128 scores of a block
-//                     from tensor memory to registers, block maximum, exponentials, P (bf16) back over the
-//                     scores; at the end of an item O / row sum -> global
-//   warp 8            items and TMA: Q tiles, then K and V blocks through one ring
-//   warp 9            MMA issue:  S_t = Q_t K^T, O_t += P_t V (P read from tensor memory, V MN-major);
-//                     in the order PV_0(j) S_0(j+1) PV_1(j) S_1(j+1), across item boundaries too
+//   warps 0..3, 4..7  softmax of tile 0 / tile 1, one thread per query row (no shuffles): the scores of a block from
+//                     tensor memory to registers, block maximum, exponentials, P (bf16) back over the scores; at the
+//                     end of an item O / row sum -> global
+//   warp 8            TMA: Q tiles, K and V blocks through a ring each
+//   warp 9            MMA issue.  Score jobs q = 2 * block + tile go round NSB score buffers: PV(q), then S(q + NSB)
+//                     into the buffer that P(q) has left, across item boundaries too (P is read from tensor memory,
+//                     V is MN-major).  This warp is the pace-maker: between two instructions the tensor pipe waits for
+//                     its scalar code, so stage numbers, phases and descriptors are carried, never divided out (3900 ->
+//                     see below cycles per pair of blocks at head_dim 64)
+//   warp 10           items
 //   warps 12..15      (rotary form only) rotate the Q tiles and K blocks in shared memory before they are used
 //
 // The reference maximum of a row stays the one of its first block unless a later block exceeds it by more than 2^8
-// (then P <= 256 is still exact in range); only then is the row of O rescaled in tensor memory.  S_t(j+1) is issued
-// behind PV_t(j) by the same thread, so a warp that has seen S_t(j+1) may read and write O_t.
+// (then P <= 256 is still exact in range); only then does the warp wait for PV_t(j-1) and rescale its rows of O in
+// tensor memory.  Parity waits that skip completions are safe because the tensor pipe completes in issue order: a
+// group that has seen S(q) knows that everything issued before it, PV(q - NSB) included, is complete.
 // All mbarrier waits are bounded.
 #pragma once
 #include <cuda.h>
@@ -35,8 +39,8 @@ namespace tcat {
 
 using namespace rlx::tc;
 
-constexpr int kTile = 128;       // query rows per tile and keys per block
-constexpr int kItemRing = 4;
+constexpr int kTile = 128;     // query rows per tile
+constexpr int kItemRing = 2;
 constexpr float kRescaleAbove = 8.f;   // exp2 units
 
 __host__ __device__ constexpr uint32_t idesc_attn(int m, int n, int b_mn) {
@@ -77,47 +81,31 @@ __device__ __forceinline__ float ex2f(float x) {
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-// Work stealing: ask for a CTA of this grid that has not been launched; the answer (16 bytes) lands in shared memory.
-__device__ __forceinline__ void steal_request(uint32_t smem_answer, uint32_t bar) {
-    asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];"
-                 ::"r"(smem_answer), "r"(bar) : "memory");
-}
-__device__ __forceinline__ int steal_answer(uint32_t smem_answer) {   // block index taken over, or -1
-    uint32_t ok, x = 0;
-    asm volatile(
-        "{\n"
-        ".reg .pred p;\n"
-        ".reg .b128 h;\n"
-        "ld.shared.b128 h, [%2];\n"
-        "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, h;\n"
-        "selp.u32 %0, 1, 0, p;\n"
-        "mov.u32 %1, 0;\n"
-        "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %1, h;\n"
-        "}\n"
-        : "=r"(ok), "=r"(x) : "r"(smem_answer) : "memory");
-    return ok ? (int)x : -1;
-}
-
 template <int D, bool PAIR>
 struct Cfg {
+    static constexpr int KB = 128;                            // keys per block
+    static constexpr int NSB = D == 128 ? 2 : 3;              // score buffers (the accumulators take 2 * D columns)
     static constexpr int W = PAIR ? 2 * D : D;                // columns of a q / k / v tile
     static constexpr int COLS = W > 64 ? 64 : W;              // columns of a TMA box (one swizzle span)
     static constexpr int ROWB = COLS * 2;
     static constexpr int NSUB = W / COLS;
-    static constexpr int SUB = kTile * ROWB;
-    static constexpr int TILE = NSUB * SUB;
-    static constexpr int QB = PAIR ? TILE : 2 * TILE;         // Q of an item
+    static constexpr int QSUB = kTile * ROWB, QTILE = NSUB * QSUB;
+    static constexpr int SUB = KB * ROWB, TILE = NSUB * SUB;  // a K or V block
+    static constexpr int QB = PAIR ? QTILE : 2 * QTILE;       // Q of an item
     static constexpr int QST = QB > 32768 ? 1 : 2;
-    static constexpr int NST = TILE == 32768 ? 5 : 8;         // K / V ring
+    static constexpr int KST = TILE == 32768 ? 3 : 4;         // K ring
+    static constexpr int VST = TILE == 32768 ? 2 : 4;         // V ring
     static constexpr int NV = (PAIR && D == 32) ? 64 : D;     // accumulator columns (N = 32 costs the tensor pipe what N = 64 does)
+    static constexpr int O_COL = NSB * KB, O_STRIDE = NV;
     static constexpr int RING_OFF = QST * QB;
-    static constexpr int ITEM_OFF = RING_OFF + NST * TILE;
-    static constexpr int ANS_OFF = ITEM_OFF + kItemRing * 32;
-    static constexpr int BAR_OFF = ANS_OFF + 16;
-    static constexpr int NBAR = 3 * QST + 3 * NST + 6 + 2 * kItemRing + 1;
+    static constexpr int VRING_OFF = RING_OFF + KST * TILE;
+    static constexpr int ITEM_OFF = VRING_OFF + VST * TILE;
+    static constexpr int BAR_OFF = ITEM_OFF + kItemRing * 32;
+    static constexpr int NBAR = 3 * QST + 3 * KST + 2 * VST + 2 * NSB + 4 + 2 * kItemRing;
     static constexpr int SMEM_BYTES = BAR_OFF + 8 * NBAR + 16 + 1024;
     static constexpr uint64_t SWZ = ROWB == 128 ? 2 : 4;
     static_assert(ROWB == 128 || ROWB == 64, "swizzle span");
+    static_assert(O_COL + 2 * O_STRIDE <= 512, "tensor memory");
     static_assert(SMEM_BYTES <= 227 * 1024, "shared memory");
 
     // Q / K operand tile: K-major rows of ROWB bytes
@@ -129,11 +117,8 @@ struct Cfg {
         return (uint64_t)((a & 0x3FFFFu) >> 4) | (uint64_t)(NV > COLS ? SUB >> 4 : 1) << 16 | (uint64_t)((8 * ROWB) >> 4) << 32 |
                (uint64_t)1 << 46 | SWZ << 61;
     }
-    // byte offset of the first column of 16-column step k of tile t's head inside a q / k tile
-    static __device__ __forceinline__ constexpr uint32_t koff(int t, int k) {
-        const int c = (PAIR ? t * D : 0) + 16 * k;
-        return (uint32_t)((c / COLS) * SUB + (c % COLS) * 2);
-    }
+    // byte offset of column c of a q / k tile with `sub` bytes per COLS columns
+    static __device__ __forceinline__ constexpr uint32_t koff(int sub, int c) { return (uint32_t)((c / COLS) * sub + (c % COLS) * 2); }
 };
 
 struct Params {
@@ -165,18 +150,19 @@ template <int D, bool PAIR, bool ROPE>
 __global__ void __launch_bounds__(Threads<ROPE>::N, 1)
 attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
     using C = Cfg<D, PAIR>;
-    constexpr int NST = C::NST, QST = C::QST, NV = C::NV;
+    constexpr int KST = C::KST, VST = C::VST, QST = C::QST, NV = C::NV, NSB = C::NSB, KB = C::KB;
     extern __shared__ unsigned char smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     unsigned char* gbase = smem_raw + (base - raw);
-    const uint32_t ring = base + C::RING_OFF;
+    const uint32_t kring = base + C::RING_OFF, vring = base + C::VRING_OFF;
     volatile int4* items = reinterpret_cast<volatile int4*>(gbase + C::ITEM_OFF);
     const uint32_t bars = base + C::BAR_OFF;
     const uint32_t q_full = bars, q_free = q_full + 8 * QST, q_rot = q_free + 8 * QST;
-    const uint32_t kv_full = q_rot + 8 * QST, kv_free = kv_full + 8 * NST, kv_rot = kv_free + 8 * NST;
-    const uint32_t s_full = kv_rot + 8 * NST, p_ready = s_full + 16, o_full = p_ready + 16;
-    const uint32_t item_full = o_full + 16, item_free = item_full + 8 * kItemRing, ans_bar = item_free + 8 * kItemRing;
+    const uint32_t k_full = q_rot + 8 * QST, k_free = k_full + 8 * KST, k_rot = k_free + 8 * KST;
+    const uint32_t v_full = k_rot + 8 * KST, v_free = v_full + 8 * VST;
+    const uint32_t s_full = v_free + 8 * VST, p_ready = s_full + 8 * NSB, pv_done = p_ready + 8 * NSB, o_full = pv_done + 16;
+    const uint32_t item_full = o_full + 16, item_free = item_full + 8 * kItemRing;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + C::BAR_OFF + 8 * C::NBAR);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
@@ -184,10 +170,11 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
     pdl_launch_dependents();
     if (threadIdx.x == 0) {
         for (int i = 0; i < QST; ++i) { mbar_init(q_full + 8 * i, 1); mbar_init(q_free + 8 * i, 1); mbar_init(q_rot + 8 * i, 4); }
-        for (int i = 0; i < NST; ++i) { mbar_init(kv_full + 8 * i, 1); mbar_init(kv_free + 8 * i, 1); mbar_init(kv_rot + 8 * i, 4); }
-        for (int i = 0; i < 2; ++i) { mbar_init(s_full + 8 * i, 1); mbar_init(p_ready + 8 * i, 4); mbar_init(o_full + 8 * i, 1); }
-        for (int i = 0; i < kItemRing; ++i) { mbar_init(item_full + 8 * i, 1); mbar_init(item_free + 8 * i, ROPE ? 13 : 9); }
-        mbar_init(ans_bar, 1);
+        for (int i = 0; i < KST; ++i) { mbar_init(k_full + 8 * i, 1); mbar_init(k_free + 8 * i, 1); mbar_init(k_rot + 8 * i, 4); }
+        for (int i = 0; i < VST; ++i) { mbar_init(v_full + 8 * i, 1); mbar_init(v_free + 8 * i, 1); }
+        for (int i = 0; i < NSB; ++i) { mbar_init(s_full + 8 * i, 1); mbar_init(p_ready + 8 * i, 4); }
+        for (int i = 0; i < 2; ++i) { mbar_init(pv_done + 8 * i, 1); mbar_init(o_full + 8 * i, 1); }
+        for (int i = 0; i < kItemRing; ++i) { mbar_init(item_full + 8 * i, 1); mbar_init(item_free + 8 * i, ROPE ? 14 : 10); }
         *abort_flag = 0;
         fence_barrier_init();
         prefetch_tmap(&tmap);
@@ -216,196 +203,240 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
 
     if (warp >= 8) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(Threads<ROPE>::REG_REST));
-        if (warp == 8) {
-            // -------------------------------------------------------- items and TMA
-            if (lane == 0) {
-                const uint32_t ans = base + C::ANS_OFF;
-                const int per_tile = p.batch * p.units;
-                int cand = (int)blockIdx.x;
-                uint32_t n = 0, g = 0, n_ans = 0;   // items published, ring slots used, answers read
-                bool ok = true;
-                mbar_expect_tx(ans_bar, 16);
-                steal_request(ans, ans_bar);
-                while (ok) {
-                    Item it{};
-                    if (cand >= 0) {
-                        const int qt = p.qtiles - 1 - cand / per_tile, rem = cand % per_tile;
-                        const int b = rem / p.units;
-                        const int rows = p.rows_mode ? 2 * kTile : kTile;
-                        it.unit = rem % p.units;
-                        it.q0 = qt * rows;
-                        it.len = __ldg(p.seq_len + b);
-                        it.valid = it.q0 < it.len;
-                        it.row0 = __ldg(p.seq_start + b);
-                        it.hi = p.positional ? min(it.len, it.q0 + rows) : it.len;
-                        it.j0 = p.positional ? max(0, it.q0 - p.window + 1) / kTile : 0;
-                        it.nb = (it.hi + kTile - 1) / kTile;
-                    }
-                    if (it.valid || cand < 0) {
-                        const uint32_t slot = n % kItemRing;
-                        if (n >= kItemRing && !(ok = mbar_wait(item_free + 8 * slot, ((n / kItemRing) - 1) & 1, abort_flag))) break;
-                        items[2 * slot].x = it.valid; items[2 * slot].y = it.unit; items[2 * slot].z = it.q0; items[2 * slot].w = it.len;
-                        items[2 * slot + 1].x = it.row0; items[2 * slot + 1].y = it.j0; items[2 * slot + 1].z = it.nb; items[2 * slot + 1].w = it.hi;
-                        mbar_arrive(item_full + 8 * slot);   // release: orders the stores above
-                    }
-                    if (cand < 0) break;
-                    if (it.valid) {
-                        const uint32_t qs = n % QST;
-                        if (n >= QST && !(ok = mbar_wait(q_free + 8 * qs, ((n / QST) - 1) & 1, abort_flag))) break;
-                        const int head0 = (PAIR || !p.rows_mode) ? 2 * it.unit : it.unit;
-                        const int kvh = PAIR ? head0 : head0 / p.kv_group;
-                        mbar_expect_tx(q_full + 8 * qs, C::QB);
+        if (warp == 10) {
+            // -------------------------------------------------------- items (whole warp)
+            const int rows = p.rows_mode ? 2 * kTile : kTile;
+            int qt = p.qtiles - 1, b0 = 0;          // scan position: row tile, first of 32 sequences
+            long long before = 0;                   // tiles that exist in front of it
+            uint32_t n = 0;
+            for (long long i = blockIdx.x;; i += gridDim.x, ++n) {
+                const long long want = i / p.units;
+                int len = 0;
+                unsigned mask = 0;
+                for (; qt >= 0;) {
+                    const int b = b0 + lane;
+                    len = b < p.batch ? __ldg(p.seq_len + b) : 0;
+                    mask = __ballot_sync(0xffffffffu, len > qt * rows);
+                    if (want < before + __popc(mask)) break;
+                    before += __popc(mask);
+                    b0 += 32;
+                    if (b0 >= p.batch) { b0 = 0; --qt; }
+                }
+                Item it{};
+                if (qt >= 0) {
+                    const bool mine = ((mask >> lane) & 1) && __popc(mask & ((1u << lane) - 1u)) == (int)(want - before);
+                    const int src = __ffs(__ballot_sync(0xffffffffu, mine)) - 1;
+                    it.valid = 1;
+                    it.unit = (int)(i % p.units);
+                    it.q0 = qt * rows;
+                    it.len = __shfl_sync(0xffffffffu, len, src);
+                    it.row0 = __ldg(p.seq_start + b0 + src);
+                    it.hi = p.positional ? min(it.len, it.q0 + rows) : it.len;
+                    it.j0 = p.positional ? max(0, it.q0 - p.window + 1) / KB : 0;
+                    it.nb = (it.hi + KB - 1) / KB;
+                }
+                const uint32_t slot = n % kItemRing;
+                if (n >= kItemRing && !mbar_wait_warp(item_free + 8 * slot, ((n / kItemRing) - 1) & 1, abort_flag)) break;
+                if (lane == 0) {
+                    items[2 * slot].x = it.valid; items[2 * slot].y = it.unit; items[2 * slot].z = it.q0; items[2 * slot].w = it.len;
+                    items[2 * slot + 1].x = it.row0; items[2 * slot + 1].y = it.j0; items[2 * slot + 1].z = it.nb; items[2 * slot + 1].w = it.hi;
+                    mbar_arrive(item_full + 8 * slot);   // release: orders the stores above
+                }
+                if (!it.valid) break;
+            }
+        } else if (warp == 8) {
+            // -------------------------------------------------------- TMA (whole warp, one lane issues)
+            uint32_t kst = 0, kph = 1, vst = 0, vph = 1;   // ring positions and the parities of their free barriers
+            bool ok = true;
+            Item it;
+            for (uint32_t n = 0; ok; ++n) {
+                if (next_item(n, it) != 1) break;
+                const uint32_t qs = n % QST;
+                if (n >= QST && !mbar_wait_warp(q_free + 8 * qs, ((n / QST) - 1) & 1, abort_flag)) break;
+                const int head0 = (PAIR || !p.rows_mode) ? 2 * it.unit : it.unit;
+                const int kvh = PAIR ? head0 : head0 / p.kv_group;
+                if (elect_one()) {
+                    mbar_expect_tx(q_full + 8 * qs, C::QB);
 #pragma unroll
-                        for (int t = 0; t < (PAIR ? 1 : 2); ++t)
+                    for (int t = 0; t < (PAIR ? 1 : 2); ++t)
 #pragma unroll
-                            for (int s = 0; s < C::NSUB; ++s)
-                                tma_load_2d(base + qs * C::QB + t * C::TILE + s * C::SUB, &tmap,
-                                            (head0 + (p.rows_mode ? 0 : t)) * D + s * C::COLS, it.row0 + it.q0 + (p.rows_mode ? t * kTile : 0),
-                                            q_full + 8 * qs);
-                        for (int j = it.j0; j < it.nb && ok; ++j) {
+                        for (int s = 0; s < C::NSUB; ++s)
 #pragma unroll
-                            for (int kv = 0; kv < 2; ++kv) {
-                                const uint32_t st = g % NST, use = g / NST;
-                                if (use >= 1 && !(ok = mbar_wait(kv_free + 8 * st, (use - 1) & 1, abort_flag))) break;
-                                mbar_expect_tx(kv_full + 8 * st, C::TILE);
+                            for (int r = 0; r < kTile; r += KB)
+                                tma_load_2d(base + qs * C::QB + t * C::QTILE + s * C::QSUB + r * C::ROWB, &tmap,
+                                            (head0 + (p.rows_mode ? 0 : t)) * D + s * C::COLS,
+                                            it.row0 + it.q0 + (p.rows_mode ? t * kTile : 0) + r, q_full + 8 * qs);
+                }
+                __syncwarp();
+                for (int j = it.j0; j < it.nb && ok; ++j) {
+                    if (!(ok = mbar_wait_warp(k_free + 8 * kst, kph, abort_flag))) break;
+                    if (elect_one()) {
+                        mbar_expect_tx(k_full + 8 * kst, C::TILE);
 #pragma unroll
-                                for (int s = 0; s < C::NSUB; ++s)
-                                    tma_load_2d(ring + st * C::TILE + s * C::SUB, &tmap, p.H + kv * p.Hkv + kvh * D + s * C::COLS,
-                                                it.row0 + j * kTile, kv_full + 8 * st);
-                                ++g;
-                            }
-                        }
-                        if (!ok) break;
-                        ++n;
+                        for (int s = 0; s < C::NSUB; ++s)
+                            tma_load_2d(kring + kst * C::TILE + s * C::SUB, &tmap, p.H + kvh * D + s * C::COLS, it.row0 + j * KB, k_full + 8 * kst);
                     }
-                    if (!(ok = mbar_wait(ans_bar, n_ans & 1, abort_flag))) break;
-                    ++n_ans;
-                    cand = steal_answer(ans);
-                    if (cand >= 0) {
-                        fence_proxy_async();   // the answer has been read before the next one may land on it
-                        mbar_expect_tx(ans_bar, 16);
-                        steal_request(ans, ans_bar);
+                    __syncwarp();
+                    if (++kst == KST) { kst = 0; kph ^= 1; }
+                    if (!(ok = mbar_wait_warp(v_free + 8 * vst, vph, abort_flag))) break;
+                    if (elect_one()) {
+                        mbar_expect_tx(v_full + 8 * vst, C::TILE);
+#pragma unroll
+                        for (int s = 0; s < C::NSUB; ++s)
+                            tma_load_2d(vring + vst * C::TILE + s * C::SUB, &tmap, p.H + p.Hkv + kvh * D + s * C::COLS, it.row0 + j * KB,
+                                        v_full + 8 * vst);
                     }
+                    __syncwarp();
+                    if (++vst == VST) { vst = 0; vph ^= 1; }
                 }
             }
         } else if (warp == 9) {
             // -------------------------------------------------------- MMA issue (whole warp, one lane issues)
-            const uint32_t kv_rdy = ROPE ? kv_rot : kv_full, q_rdy = ROPE ? q_rot : q_full;
-            constexpr uint32_t idesc_o = idesc_attn(kTile, NV, 1);
-            Item it, nx;
-            uint32_t n = 0, slot = 0;       // items opened; ring slots consumed
-            uint32_t gp = 0;                // blocks whose P has been awaited
-            bool ok = true;
-            int state = next_item(0, it);
-            // S of block j of `w` (item number m) for tile t; K in ring slot `ks`
-            auto issue_s = [&](const Item& w, uint32_t m, int j, uint32_t ks, int t) {
-                const int keys = min(kTile, w.hi - j * kTile);
-                const uint32_t idesc = idesc_attn(kTile, (keys + 15) & ~15, 0);
-                const uint32_t q = base + (m % QST) * C::QB + (PAIR ? 0 : t * C::TILE);
-                const uint64_t qd = C::desc_k(q), kd = C::desc_k(ring + ks * C::TILE);
+            // Two cursors over the same jobs: `s` issues scores, up to NSB jobs ahead of `v`, which issues P V.
+            const uint32_t k_rdy = ROPE ? k_rot : k_full, q_rdy = ROPE ? q_rot : q_full;
+            constexpr uint32_t idesc_o = idesc_attn(kTile, NV, 1), idesc_s = idesc_attn(kTile, KB, 0);
+            const uint64_t kd0 = C::desc_k(kring), qd0 = C::desc_k(base), vd0 = C::desc_v(vring);
+            Item it;
+            int s_state = next_item(0, it);     // 1: item open, 0: end of the list, 2: next item not opened yet
+            bool ok = s_state >= 0;
+            uint32_t sn = 0;                    // item number of the score cursor
+            int s_left = it.nb - it.j0, s_keys = it.hi - (it.nb - 1) * KB;   // blocks left, keys of the last one
+            bool s_first = true;                // the item's Q has not been awaited yet
+            uint32_t stile = 0, sbuf = 0, kst = 0, kph = 0, qst = 0, qph = 0;
+            int ahead = 0;                      // score jobs issued and not yet followed by their P V
+            int v_left = s_left, v_keys = s_keys;
+            int f_left[2], f_keys[2], pend = 0; // items the score cursor has opened ahead of the other one
+            f_left[0] = f_left[1] = f_keys[0] = f_keys[1] = 0;
+            // One score job if there is one; at the end of an item the next one is opened only if it has been published,
+            // unless `block`.  Returns 1 issued, 0 none, -1 a wait ran out.
+            auto issue_s = [&](bool block) -> int {
+                if (s_state != 1) {
+                    if (s_state == 0) return 0;
+                    const uint32_t m = sn + 1;
+                    if (!block && !__all_sync(0xffffffffu, mbar_test_wait(item_full + 8 * (m % kItemRing), (m / kItemRing) & 1))) return 0;
+                    s_state = next_item(m, it);
+                    if (s_state <= 0) return s_state;
+                    sn = m;
+                    s_left = it.nb - it.j0;
+                    s_keys = it.hi - (it.nb - 1) * KB;
+                    s_first = true;
+                    if (pend == 0) { f_left[0] = s_left; f_keys[0] = s_keys; }
+                    else { f_left[1] = s_left; f_keys[1] = s_keys; }
+                    ++pend;
+                }
+                if (stile == 0) {
+                    if (s_first) {
+                        if (!mbar_wait_warp(q_rdy + 8 * qst, qph, abort_flag)) return -1;
+                        s_first = false;
+                    }
+                    if (!mbar_wait_warp(k_rdy + 8 * kst, kph, abort_flag)) return -1;
+                    tc_fence_after();
+                }
+                const uint64_t qd = qd0 + (uint64_t)((qst * C::QB + stile * (PAIR ? C::koff(C::QSUB, D) : C::QTILE)) >> 4);
+                const uint64_t kd = kd0 + (uint64_t)((kst * C::TILE + (PAIR ? stile * C::koff(C::SUB, D) : 0)) >> 4);
+                const bool last = s_left == 1;
+                const uint32_t idesc = last ? idesc_attn(kTile, (s_keys + 15) & ~15, 0) : idesc_s;
+                const uint32_t sacc = tmem + sbuf * KB;
                 if (elect_one()) {
 #pragma unroll
                     for (int k = 0; k < D / 16; ++k)
-                        umma_bf16<1>(tmem + t * kTile, qd + (C::koff(t, k) >> 4), kd + (C::koff(PAIR ? t : 0, k) >> 4), idesc, k != 0);
-                    umma_commit<1>(s_full + 8 * t);
+                        umma_bf16<1>(sacc, qd + (C::koff(C::QSUB, 16 * k) >> 4), kd + (C::koff(C::SUB, 16 * k) >> 4), idesc, k != 0);
+                    umma_commit<1>(s_full + 8 * sbuf);
+                    if (stile) {
+                        umma_commit<1>(k_free + 8 * kst);
+                        if (last) umma_commit<1>(q_free + 8 * qst);
+                    }
                 }
                 __syncwarp();
-            };
-            auto wait_slot = [&]() -> bool {
-                const bool r = mbar_wait_warp(kv_rdy + 8 * (slot % NST), (slot / NST) & 1, abort_flag);
-                tc_fence_after();
-                return r;
-            };
-            if (state == 1) {
-                ok = mbar_wait_warp(q_rdy, 0, abort_flag) && wait_slot();
-                if (ok) {
-                    issue_s(it, 0, it.j0, 0, 0);
-                    issue_s(it, 0, it.j0, 0, 1);
-                    if (elect_one()) {
-                        umma_commit<1>(kv_free);
-                        if (it.j0 + 1 == it.nb) umma_commit<1>(q_free);
+                if (++sbuf == NSB) sbuf = 0;
+                ++ahead;
+                if (stile) {
+                    if (++kst == KST) { kst = 0; kph ^= 1; }
+                    if (--s_left == 0) {
+                        s_state = 2;
+                        if (++qst == QST) { qst = 0; qph ^= 1; }
                     }
-                    __syncwarp();
-                    slot = 1;
                 }
-            }
-            int j = state == 1 ? it.j0 : 0;
-            while (ok && state == 1) {
-                const uint32_t vs = slot % NST;
-                const uint32_t vt = ring + vs * C::TILE;
-                const int keys = min(kTile, it.hi - j * kTile), kpad = (keys + 15) & ~15;
-                const bool last = j + 1 == it.nb;
-                if (!(ok = wait_slot())) break;
-                ++slot;
-                if (keys < kpad) {
+                stile ^= 1;
+                return 1;
+            };
+            if (s_state == 1)
+                for (int i = 0; i < NSB && ok; ++i) ok = issue_s(false) >= 0;
+            uint32_t vbuf = 0, pph = 0, vst = 0, vph = 0;
+            bool v_first = true;
+            while (ok) {
+                if (ahead == 0) {      // nothing between the cursors: wait for the next item
+                    if (issue_s(true) <= 0) break;
+                    if (!(ok = issue_s(false) >= 0)) break;
+                }
+                if (v_left == 0) {     // the next item: the score cursor has opened it
+                    v_left = f_left[0]; v_keys = f_keys[0];
+                    f_left[0] = f_left[1]; f_keys[0] = f_keys[1];
+                    --pend;
+                    v_first = true;
+                }
+                const bool last = v_left == 1;
+                const int kpad = last ? (v_keys + 15) & ~15 : KB;
+                if (!(ok = mbar_wait_warp(v_full + 8 * vst, vph, abort_flag))) break;
+                if (last && v_keys < kpad) {
                     // rows past the end of the sequence get probability 0, but whatever lies behind them in memory must
                     // not turn that into a NaN: clear them
-                    for (int i = lane; i < (kpad - keys) * (C::ROWB / 16) * C::NSUB; i += 32) {
-                        const int s = i / ((kpad - keys) * (C::ROWB / 16)), o = i % ((kpad - keys) * (C::ROWB / 16));
-                        st_shared_v4(vt + s * C::SUB + keys * C::ROWB + o * 16, make_uint4(0, 0, 0, 0));
-                    }
+                    const uint32_t vt = vring + vst * C::TILE;
+                    const int chunks = (kpad - v_keys) * (C::ROWB / 16);
+                    for (int i = lane; i < chunks * C::NSUB; i += 32)
+                        st_shared_v4(vt + (i / chunks) * C::SUB + v_keys * C::ROWB + (i % chunks) * 16, make_uint4(0, 0, 0, 0));
                     fence_proxy_async();
                     __syncwarp();
                 }
-                // the block after this one: of this item or of the next
-                uint32_t ks = 0;
-                int nstate = 1, nj = j + 1;
+                const uint64_t vds = vd0 + (uint64_t)((vst * C::TILE) >> 4);
 #pragma unroll
                 for (int t = 0; t < 2; ++t) {
-                    if (!(ok = mbar_wait_warp(p_ready + 8 * t, gp & 1, abort_flag))) break;
+                    if (!(ok = mbar_wait_warp(p_ready + 8 * vbuf, pph, abort_flag))) break;
                     tc_fence_after();
+                    const uint64_t vd = vds + (uint64_t)((PAIR && D == 64 ? t * C::SUB : 0) >> 4);
+                    const uint32_t pa = tmem + vbuf * KB, oa = tmem + C::O_COL + t * C::O_STRIDE;
                     if (elect_one()) {
-                        const uint64_t vd = C::desc_v(vt + (PAIR && D == 64 ? t * C::SUB : 0));
-                        for (int kk = 0; kk < kpad / 16; ++kk)
-                            umma_ts(tmem + 256 + t * kTile, tmem + t * kTile + kk * 8, vd + (uint64_t)((16 * C::ROWB) >> 4) * kk, idesc_o,
-                                    (j != it.j0 || kk != 0) ? 1u : 0u);
-                        if (last) umma_commit<1>(o_full + 8 * t);
-                        if (t == 1) umma_commit<1>(kv_free + 8 * vs);
+                        if (!last) {
+                            umma_ts(oa, pa, vd, idesc_o, v_first ? 0u : 1u);
+#pragma unroll
+                            for (int kk = 1; kk < KB / 16; ++kk) umma_ts(oa, pa + kk * 8, vd + (uint64_t)((16 * C::ROWB) >> 4) * kk, idesc_o, 1u);
+                        } else {
+                            for (int kk = 0; kk < kpad / 16; ++kk)
+                                umma_ts(oa, pa + kk * 8, vd + (uint64_t)((16 * C::ROWB) >> 4) * kk, idesc_o, (!v_first || kk != 0) ? 1u : 0u);
+                            umma_commit<1>(o_full + 8 * t);
+                        }
+                        umma_commit<1>(pv_done + 8 * t);
+                        if (t == 1) umma_commit<1>(v_free + 8 * vst);
                     }
                     __syncwarp();
-                    if (t == 0) {
-                        nx = it;
-                        if (last) {
-                            ++n;
-                            nstate = next_item(n, nx);
-                            nj = nx.j0;
-                            if (nstate == 1 && !mbar_wait_warp(q_rdy + 8 * (n % QST), (n / QST) & 1, abort_flag)) nstate = -1;
-                        }
-                        if (nstate == 1) {
-                            ks = slot % NST;
-                            if (!wait_slot()) nstate = -1;
-                            ++slot;
-                        }
-                        if (nstate < 0) { ok = false; break; }
+                    if (++vbuf == NSB) { vbuf = 0; pph ^= 1; }
+                    --ahead;
+                    // scores into the buffers that are free now: the one just left and any that had no item to fill them
+                    while (ahead < NSB) {
+                        const int r = issue_s(false);
+                        ok = r >= 0;
+                        if (r <= 0) break;
                     }
-                    if (nstate == 1) {
-                        issue_s(nx, n, nj, ks, t);
-                        if (t == 1 && elect_one()) {
-                            umma_commit<1>(kv_free + 8 * ks);
-                            if (nj + 1 == nx.nb) umma_commit<1>(q_free + 8 * (n % QST));
-                        }
-                        __syncwarp();
-                    }
+                    if (!ok) break;
                 }
-                ++gp;
-                it = nx;
-                j = nj;
-                state = nstate;
+                v_first = false;
+                --v_left;
+                if (++vst == VST) { vst = 0; vph ^= 1; }
             }
         } else if (ROPE && warp >= 12) {
             // -------------------------------------------------------- rotary embedding of Q tiles and K blocks
             constexpr int HEADS = PAIR ? 2 : 1, CPR = D / 16;   // heads per tile; (lo, hi) 16-byte chunk pairs per head row
             const int rt = threadIdx.x - 12 * 32;
-            // rows first_pos + r, r < 128, of a tile; positions at or past `len` are left alone
-            auto rotate = [&](uint32_t tile, int first_pos, int len) {
-                for (int i = rt; i < kTile * HEADS * CPR; i += 128) {
+            // rows first_pos + r, r < rows, of a tile with `sub` bytes per 64 columns; positions at or past `len` are left alone
+            auto rotate = [&](uint32_t tile, int sub, int rows, int first_pos, int len) {
+                for (int i = rt; i < rows * HEADS * CPR; i += 128) {
                     const int r = i / (HEADS * CPR), c = i % (HEADS * CPR);
                     const int hd = c / CPR, cc = c % CPR, pos = first_pos + r;
                     if (pos >= len) continue;
                     const int lo_col = hd * D + cc * 8, hi_col = lo_col + D / 2;
                     const uint32_t swz = C::ROWB == 128 ? (uint32_t)(r & 7) : (uint32_t)((r >> 1) & 3);
-                    const uint32_t a = tile + (lo_col / C::COLS) * C::SUB + r * C::ROWB + ((((uint32_t)(lo_col % C::COLS) / 8) ^ swz) << 4);
-                    const uint32_t b = tile + (hi_col / C::COLS) * C::SUB + r * C::ROWB + ((((uint32_t)(hi_col % C::COLS) / 8) ^ swz) << 4);
+                    const uint32_t a = tile + (lo_col / C::COLS) * sub + r * C::ROWB + ((((uint32_t)(lo_col % C::COLS) / 8) ^ swz) << 4);
+                    const uint32_t b = tile + (hi_col / C::COLS) * sub + r * C::ROWB + ((((uint32_t)(hi_col % C::COLS) / 8) ^ swz) << 4);
                     const float4* pc = reinterpret_cast<const float4*>(p.rope_cos + (size_t)pos * (D / 2) + cc * 8);
                     const float4* ps = reinterpret_cast<const float4*>(p.rope_sin + (size_t)pos * (D / 2) + cc * 8);
                     uint4 lo = ld_shared_v4(a), hi = ld_shared_v4(b);
@@ -417,22 +448,21 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
                 __syncwarp();
             };
             Item it;
-            uint32_t slot = 0;
+            uint32_t kst = 0, kph = 0;
             bool ok = true;
             for (uint32_t n = 0; ok; ++n) {
                 if (next_item(n, it) != 1) break;
                 const uint32_t qs = n % QST;
                 if (!mbar_wait_warp(q_full + 8 * qs, (n / QST) & 1, abort_flag)) break;
-                rotate(base + qs * C::QB, it.q0, it.len);
-                if (!PAIR) rotate(base + qs * C::QB + C::TILE, it.q0 + (p.rows_mode ? kTile : 0), it.len);
+                rotate(base + qs * C::QB, C::QSUB, kTile, it.q0, it.len);
+                if (!PAIR) rotate(base + qs * C::QB + C::QTILE, C::QSUB, kTile, it.q0 + (p.rows_mode ? kTile : 0), it.len);
                 if (lane == 0) mbar_arrive(q_rot + 8 * qs);
-                for (int j = it.j0; j < it.nb && ok; ++j)
-                    for (int kv = 0; kv < 2; ++kv, ++slot) {
-                        const uint32_t st = slot % NST;
-                        if (!(ok = mbar_wait_warp(kv_full + 8 * st, (slot / NST) & 1, abort_flag))) break;
-                        if (kv == 0) rotate(ring + st * C::TILE, j * kTile, it.len);
-                        if (lane == 0) mbar_arrive(kv_rot + 8 * st);
-                    }
+                for (int j = it.j0; j < it.nb; ++j) {
+                    if (!(ok = mbar_wait_warp(k_full + 8 * kst, kph, abort_flag))) break;
+                    rotate(kring + kst * C::TILE, C::SUB, KB, j * KB, it.len);
+                    if (lane == 0) mbar_arrive(k_rot + 8 * kst);
+                    if (++kst == KST) { kst = 0; kph ^= 1; }
+                }
             }
         }
     } else {
@@ -440,9 +470,11 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(Threads<ROPE>::REG_SOFTMAX));
         const int t = warp >> 2, quad = warp & 3;
         const uint32_t tl = tmem + ((uint32_t)(quad * 32) << 16);
-        const uint32_t s_col = tl + t * kTile, o_col = tl + 256 + t * kTile + ((PAIR && D == 32) ? t * 32 : 0);
+        const uint32_t o_col = tl + C::O_COL + t * C::O_STRIDE + ((PAIR && D == 32) ? t * 32 : 0);
+        constexpr int NCH = KB / 32;         // 32-key chunks per block
         const float scale = p.scale_log2e;
-        uint32_t gb = 0;    // blocks seen
+        uint32_t buf = t, sph = 0;   // score buffer and its parity; jobs t, t + 2, t + 4, ..
+        uint32_t done = 0;           // blocks of this tile before the current one, over all items
         bool ok = true;
         Item it;
         for (uint32_t n = 0; ok; ++n) {
@@ -453,35 +485,28 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
             const int head = (PAIR || !p.rows_mode) ? 2 * it.unit + t : it.unit;
             float m_ref = -INFINITY;
             uint64_t l2[2] = {0, 0};
-            for (int j = it.j0; j < it.nb; ++j, ++gb) {
-                if (!(ok = mbar_wait_warp(s_full + 8 * t, gb & 1, abort_flag))) break;
+            for (int j = it.j0; j < it.nb; ++j, ++done) {
+                if (!(ok = mbar_wait_warp(s_full + 8 * buf, sph, abort_flag))) break;
                 if (live) {
                     tc_fence_after();
-                    const int k0 = j * kTile;
-                    uint32_t s[4][32];
-                    // 32-key chunks with a key that some row of the warp can see
-                    const int c_lo = p.positional ? max(0, (wr0 - p.window + 1 - k0) >> 5) : 0;
-                    const int c_hi = (min(it.hi, p.positional ? wr0 + 32 : it.hi) - k0 + 31) >> 5;   // one past the last
-                    const bool whole = k0 + kTile <= it.hi &&
-                                       (!p.positional || (k0 + kTile - 1 <= wr0 && k0 > wr0 + 31 - p.window));
-                    const int n_store = (min(kTile, it.hi - k0) + 31) >> 5;
-                    if (whole) {
+                    const uint32_t s_col = tl + buf * KB;
+                    const int k0 = j * KB;
+                    uint32_t s[NCH][32];
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) tmem_ld_32x32(s_col + 32 * c, s[c]);
-                        tmem_ld_wait();
-                    } else {
-#pragma unroll
-                        for (int c = 0; c < 4; ++c)
-                            if (c >= c_lo && c < c_hi) tmem_ld_32x32(s_col + 32 * c, s[c]);
-                        tmem_ld_wait();
+                    for (int c = 0; c < NCH; ++c) tmem_ld_32x32(s_col + 32 * c, s[c]);
+                    tmem_ld_wait();
+                    const bool whole = k0 + KB <= it.hi && (!p.positional || (k0 + KB - 1 <= wr0 && k0 > wr0 + 31 - p.window));
+                    if (!whole) {
+                        // visible keys of this row: columns first .. lim; one bit per column
                         const int first = p.positional ? row - p.window + 1 - k0 : 0;
                         const int lim = min(it.hi - 1, p.positional ? row : it.hi) - k0;
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) {
-                            const bool on = c >= c_lo && c < c_hi;
+                        for (int c = 0; c < NCH; ++c) {
+                            const int a = min(max(first - 32 * c, 0), 32), e = min(max(lim + 1 - 32 * c, 0), 32);
+                            const uint32_t bits = (e > a ? (uint32_t)((1ull << e) - 1) & ~(uint32_t)((1ull << a) - 1) : 0u);
 #pragma unroll
                             for (int i = 0; i < 32; ++i)
-                                if (!on || 32 * c + i < first || 32 * c + i > lim) s[c][i] = 0xFF800000u;   // -inf
+                                if (!((bits >> i) & 1)) s[c][i] = 0xFF800000u;   // -inf
                         }
                     }
                     float m_blk;
@@ -489,9 +514,11 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
                         float mx[4];
 #pragma unroll
                         for (int c = 0; c < 4; ++c) {
-                            mx[c] = fmaxf(__uint_as_float(s[c][0]), __uint_as_float(s[c][1]));
+                            constexpr int R = KB / 4;     // scores per partial maximum
+                            mx[c] = fmaxf(__uint_as_float(s[c * R / 32][c * R % 32]), __uint_as_float(s[c * R / 32][c * R % 32 + 1]));
 #pragma unroll
-                            for (int i = 2; i < 32; i += 2) mx[c] = max3f(mx[c], __uint_as_float(s[c][i]), __uint_as_float(s[c][i + 1]));
+                            for (int i = 2; i < R; i += 2)
+                                mx[c] = max3f(mx[c], __uint_as_float(s[c * R / 32][c * R % 32 + i]), __uint_as_float(s[c * R / 32][c * R % 32 + i + 1]));
                         }
                         m_blk = fmaxf(max3f(mx[0], mx[1], mx[2]), mx[3]) * scale;
                     }
@@ -500,6 +527,9 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
                     } else {
                         const bool need = m_blk > m_ref + kRescaleAbove;
                         if (__any_sync(0xffffffffu, need)) {
+                            // the products issued so far must have landed in O
+                            if (!(ok = mbar_wait_warp(pv_done + 8 * t, (done - 1) & 1, abort_flag))) break;
+                            tc_fence_after();
                             const float alpha = need ? ex2f(m_ref - m_blk) : 1.f;
                             if (need) m_ref = m_blk;
                             const uint64_t a2 = pack_f32x2(alpha, alpha);
@@ -518,23 +548,19 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
                     }
                     const float neg = m_ref == -INFINITY ? 0.f : -m_ref;
                     const uint64_t sc2 = pack_f32x2(scale, scale), ng2 = pack_f32x2(neg, neg);
+                    // straight line over all chunks, masked ones included: a branch per chunk drains the exponential unit
+                    // each time, and a second copy of the code costs more in instruction fetches than it saves
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        if (c >= n_store) break;
+                    for (int c = 0; c < NCH; ++c) {
                         uint32_t pk[16];
-                        if (whole || (c >= c_lo && c < c_hi)) {
 #pragma unroll
-                            for (int i = 0; i < 16; ++i) {
-                                float x0, x1;
-                                unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(s[c][2 * i]), __uint_as_float(s[c][2 * i + 1])), sc2, ng2), x0, x1);
-                                x0 = ex2f(x0);
-                                x1 = ex2f(x1);
-                                l2[i & 1] = add_f32x2(l2[i & 1], pack_f32x2(x0, x1));
-                                pk[i] = pack_bf16(x0, x1);
-                            }
-                        } else {
-#pragma unroll
-                            for (int i = 0; i < 16; ++i) pk[i] = 0;
+                        for (int i = 0; i < 16; ++i) {
+                            float x0, x1;
+                            unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(s[c][2 * i]), __uint_as_float(s[c][2 * i + 1])), sc2, ng2), x0, x1);
+                            x0 = ex2f(x0);
+                            x1 = ex2f(x1);
+                            l2[i & 1] = add_f32x2(l2[i & 1], pack_f32x2(x0, x1));
+                            pk[i] = pack_bf16(x0, x1);
                         }
                         tmem_st_32x16(s_col + 16 * c, pk);
                     }
@@ -542,7 +568,9 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
                     tc_fence_before();
                 }
                 __syncwarp();
-                if (lane == 0) mbar_arrive(p_ready + 8 * t);
+                if (lane == 0) mbar_arrive(p_ready + 8 * buf);
+                buf += 2;
+                if (buf >= NSB) { buf -= NSB; sph ^= 1; }
             }
             if (!ok) break;
             // ---- O / row sum -> bf16 -> global ----

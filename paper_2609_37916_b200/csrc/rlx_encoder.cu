@@ -427,20 +427,19 @@ rlx_status_t launch_attention_fwd(const bf16* qkv, int rows, const int32_t* seq_
     p.qtiles = (max_len + item_rows - 1) / item_rows;
     p.kv_group = kv_group; p.rows_mode = rows_mode; p.positional = positional; p.window = window;
     p.scale_log2e = 1.4426950408889634f / sqrtf((float)d);
-    const long long items = (long long)p.qtiles * B * p.units;
-    if (items > 0x7fffffffll) return RLX_ERR_UNSUPPORTED;
+    const int grid = (int)std::min<long long>((long long)p.qtiles * B * p.units, sm_count());
     CUtensorMap tm;
     const uint32_t cols = (d == 32 && !pair) ? 32 : 64;
-    if (!make_tmap(&tm, qkv, (uint64_t)rows, (uint64_t)p.H + 2 * p.Hkv, tcat::kTile, cols,
+    if (!make_tmap(&tm, qkv, (uint64_t)rows, (uint64_t)p.H + 2 * p.Hkv, d == 128 ? tcat::Cfg<128, false>::KB : tcat::Cfg<64, true>::KB, cols,
                    cols == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B))
         return RLX_ERR_CUDA;
 #define RLX_ATT_FWD(D, PAIR)                                                                                                   \
     do {                                                                                                                       \
         if (rope_cos)                                                                                                          \
-            RLX_CUDA_TRY(launch_ex(tcat::attention_fwd_kernel<D, PAIR, true>, dim3((unsigned)items), tcat::Threads<true>::N,   \
+            RLX_CUDA_TRY(launch_ex(tcat::attention_fwd_kernel<D, PAIR, true>, dim3(grid), tcat::Threads<true>::N,   \
                                    tcat::Cfg<D, PAIR>::SMEM_BYTES, st, tm, p));                                                \
         else                                                                                                                   \
-            RLX_CUDA_TRY(launch_ex(tcat::attention_fwd_kernel<D, PAIR, false>, dim3((unsigned)items), tcat::Threads<false>::N, \
+            RLX_CUDA_TRY(launch_ex(tcat::attention_fwd_kernel<D, PAIR, false>, dim3(grid), tcat::Threads<false>::N, \
                                    tcat::Cfg<D, PAIR>::SMEM_BYTES, st, tm, p));                                                \
     } while (0)
     if (pair) { if (d == 32) RLX_ATT_FWD(32, true); else RLX_ATT_FWD(64, true); }
