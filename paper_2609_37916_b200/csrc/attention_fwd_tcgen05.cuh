@@ -15,18 +15,18 @@
 //                     tensor memory to registers, block maximum, exponentials, P (bf16) back over the scores; at the
 //                     end of an item O / row sum -> global
 //   warp 8            TMA: Q tiles, K and V blocks through a ring each
-//   warp 9            MMA issue.  Score jobs q = 2 * block + tile go round NSB score buffers: PV(q), then S(q + NSB)
-//                     into the buffer that P(q) has left, across item boundaries too (P is read from tensor memory,
-//                     V is MN-major).  This warp is the pace-maker: between two instructions the tensor pipe waits for
-//                     its scalar code, so stage numbers, phases and descriptors are carried, never divided out (3900 ->
-//                     see below cycles per pair of blocks at head_dim 64)
+//   warp 9             issues S(q) = Q_t K^T: score jobs q = 2 * block + tile go round NSB score buffers, across item
+//                     boundaries too, so the scores run ahead of the softmax
+//   warp 11            issues O_t += P(q) V (P read from tensor memory, V MN-major) and hands the buffer back
+//                     One warp for both was the pace-maker: 1750 cycles per job, of which 640 to 770 are tensor time and
+//                     the rest its own scalar code; the softmax takes about 2400 per job and tile
 //   warp 10           items
 //   warps 12..15      (rotary form only) rotate the Q tiles and K blocks in shared memory before they are used
 //
 // The reference maximum of a row stays the one of its first block unless a later block exceeds it by more than 2^8
 // (then P <= 256 is still exact in range); only then does the warp wait for PV_t(j-1) and rescale its rows of O in
-// tensor memory.  Parity waits that skip completions are safe because the tensor pipe completes in issue order: a
-// group that has seen S(q) knows that everything issued before it, PV(q - NSB) included, is complete.
+// tensor memory.  Waits that skip completions of a barrier are safe because either issuer's products complete in
+// order: a group that has seen S(q) knows that S(q - 1), PV(q - NSB) and everything before them are complete.
 // All mbarrier waits are bounded.
 #pragma once
 #include <cuda.h>
@@ -83,8 +83,8 @@ __device__ __forceinline__ float ex2f(float x) {
 }
 template <int D, bool PAIR>
 struct Cfg {
-    static constexpr int KB = 128;                            // keys per block
-    static constexpr int NSB = D == 128 ? 2 : 3;              // score buffers (the accumulators take 2 * D columns)
+    static constexpr int KB = D == 128 ? 64 : 128;            // keys per block
+    static constexpr int NSB = D == 128 ? 4 : 3;              // score buffers (the accumulators take 2 * D columns)
     static constexpr int W = PAIR ? 2 * D : D;                // columns of a q / k / v tile
     static constexpr int COLS = W > 64 ? 64 : W;              // columns of a TMA box (one swizzle span)
     static constexpr int ROWB = COLS * 2;
@@ -101,7 +101,7 @@ struct Cfg {
     static constexpr int VRING_OFF = RING_OFF + KST * TILE;
     static constexpr int ITEM_OFF = VRING_OFF + VST * TILE;
     static constexpr int BAR_OFF = ITEM_OFF + kItemRing * 32;
-    static constexpr int NBAR = 3 * QST + 3 * KST + 2 * VST + 2 * NSB + 4 + 2 * kItemRing;
+    static constexpr int NBAR = 3 * QST + 3 * KST + 2 * VST + 3 * NSB + 2 + 2 * kItemRing;
     static constexpr int SMEM_BYTES = BAR_OFF + 8 * NBAR + 16 + 1024;
     static constexpr uint64_t SWZ = ROWB == 128 ? 2 : 4;
     static_assert(ROWB == 128 || ROWB == 64, "swizzle span");
@@ -161,7 +161,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
     const uint32_t q_full = bars, q_free = q_full + 8 * QST, q_rot = q_free + 8 * QST;
     const uint32_t k_full = q_rot + 8 * QST, k_free = k_full + 8 * KST, k_rot = k_free + 8 * KST;
     const uint32_t v_full = k_rot + 8 * KST, v_free = v_full + 8 * VST;
-    const uint32_t s_full = v_free + 8 * VST, p_ready = s_full + 8 * NSB, pv_done = p_ready + 8 * NSB, o_full = pv_done + 16;
+    const uint32_t s_full = v_free + 8 * VST, p_ready = s_full + 8 * NSB, buf_free = p_ready + 8 * NSB, o_full = buf_free + 8 * NSB;
     const uint32_t item_full = o_full + 16, item_free = item_full + 8 * kItemRing;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + C::BAR_OFF + 8 * C::NBAR);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
@@ -172,9 +172,9 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
         for (int i = 0; i < QST; ++i) { mbar_init(q_full + 8 * i, 1); mbar_init(q_free + 8 * i, 1); mbar_init(q_rot + 8 * i, 4); }
         for (int i = 0; i < KST; ++i) { mbar_init(k_full + 8 * i, 1); mbar_init(k_free + 8 * i, 1); mbar_init(k_rot + 8 * i, 4); }
         for (int i = 0; i < VST; ++i) { mbar_init(v_full + 8 * i, 1); mbar_init(v_free + 8 * i, 1); }
-        for (int i = 0; i < NSB; ++i) { mbar_init(s_full + 8 * i, 1); mbar_init(p_ready + 8 * i, 4); }
-        for (int i = 0; i < 2; ++i) { mbar_init(pv_done + 8 * i, 1); mbar_init(o_full + 8 * i, 1); }
-        for (int i = 0; i < kItemRing; ++i) { mbar_init(item_full + 8 * i, 1); mbar_init(item_free + 8 * i, ROPE ? 14 : 10); }
+        for (int i = 0; i < NSB; ++i) { mbar_init(s_full + 8 * i, 1); mbar_init(p_ready + 8 * i, 4); mbar_init(buf_free + 8 * i, 1); }
+        for (int i = 0; i < 2; ++i) mbar_init(o_full + 8 * i, 1);
+        for (int i = 0; i < kItemRing; ++i) { mbar_init(item_full + 8 * i, 1); mbar_init(item_free + 8 * i, ROPE ? 15 : 11); }
         *abort_flag = 0;
         fence_barrier_init();
         prefetch_tmap(&tmap);
@@ -291,137 +291,89 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
                 }
             }
         } else if (warp == 9) {
-            // -------------------------------------------------------- MMA issue (whole warp, one lane issues)
-            // Two cursors over the same jobs: `s` issues scores, up to NSB jobs ahead of `v`, which issues P V.
+            // -------------------------------------------------------- scores (whole warp, one lane issues)
             const uint32_t k_rdy = ROPE ? k_rot : k_full, q_rdy = ROPE ? q_rot : q_full;
-            constexpr uint32_t idesc_o = idesc_attn(kTile, NV, 1), idesc_s = idesc_attn(kTile, KB, 0);
-            const uint64_t kd0 = C::desc_k(kring), qd0 = C::desc_k(base), vd0 = C::desc_v(vring);
+            constexpr uint32_t idesc_s = idesc_attn(kTile, KB, 0);
+            const uint64_t kd0 = C::desc_k(kring), qd0 = C::desc_k(base);
+            uint32_t sbuf = 0, bph = 1, kst = 0, kph = 0, qst = 0, qph = 0;
+            bool ok = true;
             Item it;
-            int s_state = next_item(0, it);     // 1: item open, 0: end of the list, 2: next item not opened yet
-            bool ok = s_state >= 0;
-            uint32_t sn = 0;                    // item number of the score cursor
-            int s_left = it.nb - it.j0, s_keys = it.hi - (it.nb - 1) * KB;   // blocks left, keys of the last one
-            bool s_first = true;                // the item's Q has not been awaited yet
-            uint32_t stile = 0, sbuf = 0, kst = 0, kph = 0, qst = 0, qph = 0;
-            int ahead = 0;                      // score jobs issued and not yet followed by their P V
-            int v_left = s_left, v_keys = s_keys;
-            int f_left[2], f_keys[2], pend = 0; // items the score cursor has opened ahead of the other one
-            f_left[0] = f_left[1] = f_keys[0] = f_keys[1] = 0;
-            // One score job if there is one; at the end of an item the next one is opened only if it has been published,
-            // unless `block`.  Returns 1 issued, 0 none, -1 a wait ran out.
-            auto issue_s = [&](bool block) -> int {
-                if (s_state != 1) {
-                    if (s_state == 0) return 0;
-                    const uint32_t m = sn + 1;
-                    if (!block && !__all_sync(0xffffffffu, mbar_test_wait(item_full + 8 * (m % kItemRing), (m / kItemRing) & 1))) return 0;
-                    s_state = next_item(m, it);
-                    if (s_state <= 0) return s_state;
-                    sn = m;
-                    s_left = it.nb - it.j0;
-                    s_keys = it.hi - (it.nb - 1) * KB;
-                    s_first = true;
-                    if (pend == 0) { f_left[0] = s_left; f_keys[0] = s_keys; }
-                    else { f_left[1] = s_left; f_keys[1] = s_keys; }
-                    ++pend;
-                }
-                if (stile == 0) {
-                    if (s_first) {
-                        if (!mbar_wait_warp(q_rdy + 8 * qst, qph, abort_flag)) return -1;
-                        s_first = false;
-                    }
-                    if (!mbar_wait_warp(k_rdy + 8 * kst, kph, abort_flag)) return -1;
-                    tc_fence_after();
-                }
-                const uint64_t qd = qd0 + (uint64_t)((qst * C::QB + stile * (PAIR ? C::koff(C::QSUB, D) : C::QTILE)) >> 4);
-                const uint64_t kd = kd0 + (uint64_t)((kst * C::TILE + (PAIR ? stile * C::koff(C::SUB, D) : 0)) >> 4);
-                const bool last = s_left == 1;
-                const uint32_t idesc = last ? idesc_attn(kTile, (s_keys + 15) & ~15, 0) : idesc_s;
-                const uint32_t sacc = tmem + sbuf * KB;
-                if (elect_one()) {
+            for (uint32_t n = 0; ok; ++n) {
+                if (next_item(n, it) != 1 || !mbar_wait_warp(q_rdy + 8 * qst, qph, abort_flag)) break;
+                const uint64_t qd1 = qd0 + (uint64_t)((qst * C::QB) >> 4);
+                for (int left = it.nb - it.j0; left > 0 && ok; --left) {
+                    if (!(ok = mbar_wait_warp(k_rdy + 8 * kst, kph, abort_flag))) break;
+                    const uint64_t kd1 = kd0 + (uint64_t)((kst * C::TILE) >> 4);
+                    const uint32_t idesc = left == 1 ? idesc_attn(kTile, (it.hi - (it.nb - 1) * KB + 15) & ~15, 0) : idesc_s;
+#pragma unroll 1
+                    for (uint32_t t = 0; t < 2; ++t) {
+                        if (!(ok = mbar_wait_warp(buf_free + 8 * sbuf, bph, abort_flag))) break;
+                        tc_fence_after();
+                        const uint64_t qd = qd1 + (uint64_t)((t * (PAIR ? C::koff(C::QSUB, D) : C::QTILE)) >> 4);
+                        const uint64_t kd = kd1 + (uint64_t)((PAIR ? t * C::koff(C::SUB, D) : 0) >> 4);
+                        const uint32_t acc = tmem + sbuf * KB;
+                        if (elect_one()) {
 #pragma unroll
-                    for (int k = 0; k < D / 16; ++k)
-                        umma_bf16<1>(sacc, qd + (C::koff(C::QSUB, 16 * k) >> 4), kd + (C::koff(C::SUB, 16 * k) >> 4), idesc, k != 0);
-                    umma_commit<1>(s_full + 8 * sbuf);
-                    if (stile) {
-                        umma_commit<1>(k_free + 8 * kst);
-                        if (last) umma_commit<1>(q_free + 8 * qst);
-                    }
-                }
-                __syncwarp();
-                if (++sbuf == NSB) sbuf = 0;
-                ++ahead;
-                if (stile) {
-                    if (++kst == KST) { kst = 0; kph ^= 1; }
-                    if (--s_left == 0) {
-                        s_state = 2;
-                        if (++qst == QST) { qst = 0; qph ^= 1; }
-                    }
-                }
-                stile ^= 1;
-                return 1;
-            };
-            if (s_state == 1)
-                for (int i = 0; i < NSB && ok; ++i) ok = issue_s(false) >= 0;
-            uint32_t vbuf = 0, pph = 0, vst = 0, vph = 0;
-            bool v_first = true;
-            while (ok) {
-                if (ahead == 0) {      // nothing between the cursors: wait for the next item
-                    if (issue_s(true) <= 0) break;
-                    if (!(ok = issue_s(false) >= 0)) break;
-                }
-                if (v_left == 0) {     // the next item: the score cursor has opened it
-                    v_left = f_left[0]; v_keys = f_keys[0];
-                    f_left[0] = f_left[1]; f_keys[0] = f_keys[1];
-                    --pend;
-                    v_first = true;
-                }
-                const bool last = v_left == 1;
-                const int kpad = last ? (v_keys + 15) & ~15 : KB;
-                if (!(ok = mbar_wait_warp(v_full + 8 * vst, vph, abort_flag))) break;
-                if (last && v_keys < kpad) {
-                    // rows past the end of the sequence get probability 0, but whatever lies behind them in memory must
-                    // not turn that into a NaN: clear them
-                    const uint32_t vt = vring + vst * C::TILE;
-                    const int chunks = (kpad - v_keys) * (C::ROWB / 16);
-                    for (int i = lane; i < chunks * C::NSUB; i += 32)
-                        st_shared_v4(vt + (i / chunks) * C::SUB + v_keys * C::ROWB + (i % chunks) * 16, make_uint4(0, 0, 0, 0));
-                    fence_proxy_async();
-                    __syncwarp();
-                }
-                const uint64_t vds = vd0 + (uint64_t)((vst * C::TILE) >> 4);
-#pragma unroll
-                for (int t = 0; t < 2; ++t) {
-                    if (!(ok = mbar_wait_warp(p_ready + 8 * vbuf, pph, abort_flag))) break;
-                    tc_fence_after();
-                    const uint64_t vd = vds + (uint64_t)((PAIR && D == 64 ? t * C::SUB : 0) >> 4);
-                    const uint32_t pa = tmem + vbuf * KB, oa = tmem + C::O_COL + t * C::O_STRIDE;
-                    if (elect_one()) {
-                        if (!last) {
-                            umma_ts(oa, pa, vd, idesc_o, v_first ? 0u : 1u);
-#pragma unroll
-                            for (int kk = 1; kk < KB / 16; ++kk) umma_ts(oa, pa + kk * 8, vd + (uint64_t)((16 * C::ROWB) >> 4) * kk, idesc_o, 1u);
-                        } else {
-                            for (int kk = 0; kk < kpad / 16; ++kk)
-                                umma_ts(oa, pa + kk * 8, vd + (uint64_t)((16 * C::ROWB) >> 4) * kk, idesc_o, (!v_first || kk != 0) ? 1u : 0u);
-                            umma_commit<1>(o_full + 8 * t);
+                            for (int k = 0; k < D / 16; ++k)
+                                umma_bf16<1>(acc, qd + (C::koff(C::QSUB, 16 * k) >> 4), kd + (C::koff(C::SUB, 16 * k) >> 4), idesc, k != 0);
+                            umma_commit<1>(s_full + 8 * sbuf);
+                            if (t) {
+                                umma_commit<1>(k_free + 8 * kst);
+                                if (left == 1) umma_commit<1>(q_free + 8 * qst);
+                            }
                         }
-                        umma_commit<1>(pv_done + 8 * t);
-                        if (t == 1) umma_commit<1>(v_free + 8 * vst);
+                        __syncwarp();
+                        if (++sbuf == NSB) { sbuf = 0; bph ^= 1; }
                     }
-                    __syncwarp();
-                    if (++vbuf == NSB) { vbuf = 0; pph ^= 1; }
-                    --ahead;
-                    // scores into the buffers that are free now: the one just left and any that had no item to fill them
-                    while (ahead < NSB) {
-                        const int r = issue_s(false);
-                        ok = r >= 0;
-                        if (r <= 0) break;
-                    }
-                    if (!ok) break;
+                    if (++kst == KST) { kst = 0; kph ^= 1; }
                 }
-                v_first = false;
-                --v_left;
-                if (++vst == VST) { vst = 0; vph ^= 1; }
+                if (++qst == QST) { qst = 0; qph ^= 1; }
+            }
+        } else if (warp == 11) {
+            // -------------------------------------------------------- O += P V (whole warp, one lane issues)
+            constexpr uint32_t idesc_o = idesc_attn(kTile, NV, 1);
+            const uint64_t vd0 = C::desc_v(vring);
+            uint32_t vbuf = 0, pph = 0, vst = 0, vph = 0;
+            bool ok = true;
+            Item it;
+            for (uint32_t n = 0; ok; ++n) {
+                if (next_item(n, it) != 1) break;
+                bool first = true;
+                for (int left = it.nb - it.j0; left > 0 && ok; --left) {
+                    const bool last = left == 1;
+                    const int keys = last ? it.hi - (it.nb - 1) * KB : KB, kpad = (keys + 15) & ~15;
+                    if (!(ok = mbar_wait_warp(v_full + 8 * vst, vph, abort_flag))) break;
+                    if (keys < kpad) {
+                        // rows past the end of the sequence get probability 0, but whatever lies behind them in memory must
+                        // not turn that into a NaN: clear them
+                        const uint32_t vtile = vring + vst * C::TILE;
+                        const int chunks = (kpad - keys) * (C::ROWB / 16);
+                        for (int i = lane; i < chunks * C::NSUB; i += 32)
+                            st_shared_v4(vtile + (i / chunks) * C::SUB + keys * C::ROWB + (i % chunks) * 16, make_uint4(0, 0, 0, 0));
+                        fence_proxy_async();
+                        __syncwarp();
+                    }
+#pragma unroll 1
+                    for (uint32_t t = 0; t < 2; ++t) {
+                        const uint64_t vd = vd0 + (uint64_t)((vst * C::TILE + (PAIR && D == 64 ? t * C::SUB : 0)) >> 4);
+                        const uint32_t pa = tmem + vbuf * KB, oa = tmem + C::O_COL + t * C::O_STRIDE;
+                        if (!(ok = mbar_wait_warp(p_ready + 8 * vbuf, pph, abort_flag))) break;
+                        tc_fence_after();
+                        if (elect_one()) {
+                            umma_ts(oa, pa, vd, idesc_o, first ? 0u : 1u);
+#pragma unroll
+                            for (int kk = 1; kk < KB / 16; ++kk)
+                                if (kk * 16 < kpad) umma_ts(oa, pa + kk * 8, vd + (uint64_t)((16 * C::ROWB) >> 4) * kk, idesc_o, 1u);
+                            umma_commit<1>(buf_free + 8 * vbuf);
+                            if (last) umma_commit<1>(o_full + 8 * t);
+                            if (t) umma_commit<1>(v_free + 8 * vst);
+                        }
+                        __syncwarp();
+                        if (++vbuf == NSB) { vbuf = 0; pph ^= 1; }
+                    }
+                    first = false;
+                    if (++vst == VST) { vst = 0; vph ^= 1; }
+                }
             }
         } else if (ROPE && warp >= 12) {
             // -------------------------------------------------------- rotary embedding of Q tiles and K blocks
@@ -474,7 +426,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
         constexpr int NCH = KB / 32;         // 32-key chunks per block
         const float scale = p.scale_log2e;
         uint32_t buf = t, sph = 0;   // score buffer and its parity; jobs t, t + 2, t + 4, ..
-        uint32_t done = 0;           // blocks of this tile before the current one, over all items
+        uint32_t pbuf = 0, pph = 0;  // the same of this tile's previous block
         bool ok = true;
         Item it;
         for (uint32_t n = 0; ok; ++n) {
@@ -485,7 +437,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
             const int head = (PAIR || !p.rows_mode) ? 2 * it.unit + t : it.unit;
             float m_ref = -INFINITY;
             uint64_t l2[2] = {0, 0};
-            for (int j = it.j0; j < it.nb; ++j, ++done) {
+            for (int j = it.j0; j < it.nb; ++j) {
                 if (!(ok = mbar_wait_warp(s_full + 8 * buf, sph, abort_flag))) break;
                 if (live) {
                     tc_fence_after();
@@ -528,7 +480,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
                         const bool need = m_blk > m_ref + kRescaleAbove;
                         if (__any_sync(0xffffffffu, need)) {
                             // the products issued so far must have landed in O
-                            if (!(ok = mbar_wait_warp(pv_done + 8 * t, (done - 1) & 1, abort_flag))) break;
+                            if (!(ok = mbar_wait_warp(buf_free + 8 * pbuf, pph, abort_flag))) break;
                             tc_fence_after();
                             const float alpha = need ? ex2f(m_ref - m_blk) : 1.f;
                             if (need) m_ref = m_blk;
@@ -569,6 +521,8 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(p_ready + 8 * buf);
+                pbuf = buf;
+                pph = sph;
                 buf += 2;
                 if (buf >= NSB) { buf -= NSB; sph ^= 1; }
             }
