@@ -187,35 +187,49 @@ __device__ __forceinline__ int find_sequence(const int32_t* __restrict__ seq_sta
 }
 
 // Fused QK-RoPE: rotates, in place, the q and k column blocks of packed [rows, ld] projections (v is
-// left alone; ld = 3H, or (hq + 2 hkv) D in the grouped-query layout).  grid = (row tiles of kRopeRows, sequences); one task = eight (j, j + D/2) column pairs
-// of one head of q or k of one row: 2 x 16 bytes in, 2 x 16 bytes out, consecutive lanes on consecutive
-// 16-byte chunks.  A row's position is its index within its sequence.
-constexpr int kRopeRows = 16;
-constexpr int kRopeThreads = 256;
+// left alone; ld = 3H, or (hq + 2 hkv) D in the grouped-query layout).  grid = (row tiles of kRopeRows, sequences); a warp
+// owns a row (its position is its index within its sequence).  A lane keeps to one 16-byte chunk of eight (j, j + D/2)
+// column pairs and walks over the heads with it, so that the row's cosines and sines are loaded once per lane and
+// not once per head (they are twice the bytes of the pairs they rotate), with kRopeBatch heads in flight.
+// HBM-bound: q and k are read and written once.  40,954 rows x (32 + 8) heads x 128: 330 -> 131 us (6.4 TB/s of 6.55 measured).
+constexpr int kRopeRows = 8;
+constexpr int kRopeThreads = 32 * kRopeRows;
+constexpr int kRopeBatch = 4;
 template <int D>
 __global__ void __launch_bounds__(kRopeThreads)
 qk_rope_kernel(__nv_bfloat16* __restrict__ qkv, const int32_t* __restrict__ seq_start,
                const int32_t* __restrict__ seq_len, int rot_heads, int ld, const float* __restrict__ rope_cos,
                const float* __restrict__ rope_sin) {
-    constexpr int CPR = D / 16;                 // tasks per head
-    const int b = blockIdx.y;
-    const int len = __ldg(seq_len + b);
-    const int p0 = blockIdx.x * kRopeRows;
-    if (p0 >= len) return;
-    const size_t row0 = (size_t)__ldg(seq_start + b);
-    const int per_row = rot_heads * CPR;        // q heads then k heads: one contiguous block of rot_heads * D columns
-    const int nrows = min(kRopeRows, len - p0);
-    for (int i = threadIdx.x; i < nrows * per_row; i += kRopeThreads) {
-        const int r = i / per_row, t = i % per_row;
-        const int hd = t / CPR, c = t % CPR;    // hd in [0, rot_heads): a q head, then the k heads
-        const int pos = p0 + r;
-        __nv_bfloat16* base = qkv + (row0 + pos) * (size_t)ld + hd * D + c * 8;
-        uint4 lo = *reinterpret_cast<const uint4*>(base), hi = *reinterpret_cast<const uint4*>(base + D / 2);
-        const float4* pc = reinterpret_cast<const float4*>(rope_cos + (size_t)pos * (D / 2) + c * 8);
-        const float4* ps = reinterpret_cast<const float4*>(rope_sin + (size_t)pos * (D / 2) + c * 8);
-        rope_rotate8(lo, hi, __ldg(pc), __ldg(pc + 1), __ldg(ps), __ldg(ps + 1));
-        *reinterpret_cast<uint4*>(base) = lo;
-        *reinterpret_cast<uint4*>(base + D / 2) = hi;
+    constexpr int CPR = D / 16;                 // chunks per head
+    constexpr int HPW = 32 / CPR;               // heads a warp covers at once
+    const int b = blockIdx.y, lane = threadIdx.x & 31;
+    const int pos = blockIdx.x * kRopeRows + (threadIdx.x >> 5);
+    if (pos >= __ldg(seq_len + b)) return;
+    const int c = lane % CPR;
+    // q heads then k heads: one contiguous block of rot_heads * D columns
+    __nv_bfloat16* base = qkv + ((size_t)__ldg(seq_start + b) + pos) * (size_t)ld + c * 8;
+    const float4* pc = reinterpret_cast<const float4*>(rope_cos + (size_t)pos * (D / 2) + c * 8);
+    const float4* ps = reinterpret_cast<const float4*>(rope_sin + (size_t)pos * (D / 2) + c * 8);
+    const float4 c0 = __ldg(pc), c1 = __ldg(pc + 1), s0 = __ldg(ps), s1 = __ldg(ps + 1);
+    for (int h0 = lane / CPR; h0 < rot_heads; h0 += HPW * kRopeBatch) {
+        uint4 lo[kRopeBatch], hi[kRopeBatch];
+#pragma unroll
+        for (int u = 0; u < kRopeBatch; ++u) {
+            const int h = h0 + u * HPW;
+            if (h < rot_heads) {
+                lo[u] = *reinterpret_cast<const uint4*>(base + h * D);
+                hi[u] = *reinterpret_cast<const uint4*>(base + h * D + D / 2);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < kRopeBatch; ++u) {
+            const int h = h0 + u * HPW;
+            if (h < rot_heads) {
+                rope_rotate8(lo[u], hi[u], c0, c1, s0, s1);
+                *reinterpret_cast<uint4*>(base + h * D) = lo[u];
+                *reinterpret_cast<uint4*>(base + h * D + D / 2) = hi[u];
+            }
+        }
     }
 }
 
