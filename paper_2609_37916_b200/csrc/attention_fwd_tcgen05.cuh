@@ -137,9 +137,9 @@ struct Params {
 template <bool ROPE>
 struct Threads {
     static constexpr int N = ROPE ? 512 : 384;
-    // 256 softmax threads and the rest share what the launch holds: 512 x 128 = 256 x (200 + 56), 384 x 168 > 256 x 208 + 128 x 80
-    static constexpr int REG_SOFTMAX = ROPE ? 200 : 208;
-    static constexpr int REG_REST = ROPE ? 56 : 80;
+    // 256 softmax threads and the rest share what the launch holds: 512 x 128 = 256 x (192 + 64), 384 x 168 > 256 x 208 + 128 x 80
+    static constexpr int REG_SOFTMAX = ROPE ? 192 : 208;
+    static constexpr int REG_REST = ROPE ? 64 : 80;
 };
 
 struct Item {
@@ -378,23 +378,35 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
         } else if (ROPE && warp >= 12) {
             // -------------------------------------------------------- rotary embedding of Q tiles and K blocks
             constexpr int HEADS = PAIR ? 2 : 1, CPR = D / 16;   // heads per tile; (lo, hi) 16-byte chunk pairs per head row
-            const int rt = threadIdx.x - 12 * 32;
-            // rows first_pos + r, r < rows, of a tile with `sub` bytes per 64 columns; positions at or past `len` are left alone
+            // A thread keeps to one chunk pair and walks over rows, with the next row's cosines and sines requested before the
+            // current one is rotated (both heads of a pair share them): 64 KB of tables per 128 x 64 block come from L2.
+            constexpr int STEP = 128 / CPR;                      // rows between a thread's tasks
+            const int rt = threadIdx.x - 12 * 32, cc = rt % CPR, r0 = rt / CPR;
+            // rows first_pos + r, r < rows, of a tile with `sub` bytes per COLS columns; positions at or past `len` are left alone
             auto rotate = [&](uint32_t tile, int sub, int rows, int first_pos, int len) {
-                for (int i = rt; i < rows * HEADS * CPR; i += 128) {
-                    const int r = i / (HEADS * CPR), c = i % (HEADS * CPR);
-                    const int hd = c / CPR, cc = c % CPR, pos = first_pos + r;
-                    if (pos >= len) continue;
-                    const int lo_col = hd * D + cc * 8, hi_col = lo_col + D / 2;
+                const int end = min(rows, len - first_pos);
+                const float4* pc = reinterpret_cast<const float4*>(p.rope_cos + (size_t)(first_pos + r0) * (D / 2) + cc * 8);
+                const float4* ps = reinterpret_cast<const float4*>(p.rope_sin + (size_t)(first_pos + r0) * (D / 2) + cc * 8);
+                float4 c0, c1, s0, s1;
+                if (r0 < end) { c0 = __ldg(pc); c1 = __ldg(pc + 1); s0 = __ldg(ps); s1 = __ldg(ps + 1); }
+#pragma unroll 1
+                for (int r = r0; r < end; r += STEP) {
+                    float4 n0 = c0, n1 = c1, m0 = s0, m1 = s1;
+                    pc += STEP * (D / 8);
+                    ps += STEP * (D / 8);
+                    if (r + STEP < end) { n0 = __ldg(pc); n1 = __ldg(pc + 1); m0 = __ldg(ps); m1 = __ldg(ps + 1); }
                     const uint32_t swz = C::ROWB == 128 ? (uint32_t)(r & 7) : (uint32_t)((r >> 1) & 3);
-                    const uint32_t a = tile + (lo_col / C::COLS) * sub + r * C::ROWB + ((((uint32_t)(lo_col % C::COLS) / 8) ^ swz) << 4);
-                    const uint32_t b = tile + (hi_col / C::COLS) * sub + r * C::ROWB + ((((uint32_t)(hi_col % C::COLS) / 8) ^ swz) << 4);
-                    const float4* pc = reinterpret_cast<const float4*>(p.rope_cos + (size_t)pos * (D / 2) + cc * 8);
-                    const float4* ps = reinterpret_cast<const float4*>(p.rope_sin + (size_t)pos * (D / 2) + cc * 8);
-                    uint4 lo = ld_shared_v4(a), hi = ld_shared_v4(b);
-                    rope_rotate8(lo, hi, __ldg(pc), __ldg(pc + 1), __ldg(ps), __ldg(ps + 1));
-                    st_shared_v4(a, lo);
-                    st_shared_v4(b, hi);
+#pragma unroll
+                    for (int hd = 0; hd < HEADS; ++hd) {
+                        const int lo_col = hd * D + cc * 8, hi_col = lo_col + D / 2;
+                        const uint32_t a = tile + (lo_col / C::COLS) * sub + r * C::ROWB + ((((uint32_t)(lo_col % C::COLS) / 8) ^ swz) << 4);
+                        const uint32_t b = tile + (hi_col / C::COLS) * sub + r * C::ROWB + ((((uint32_t)(hi_col % C::COLS) / 8) ^ swz) << 4);
+                        uint4 lo = ld_shared_v4(a), hi = ld_shared_v4(b);
+                        rope_rotate8(lo, hi, c0, c1, s0, s1);
+                        st_shared_v4(a, lo);
+                        st_shared_v4(b, hi);
+                    }
+                    c0 = n0; c1 = n1; s0 = m0; s1 = m1;
                 }
                 fence_proxy_async();
                 __syncwarp();
