@@ -137,12 +137,12 @@ attention_bf16_kernel(const __nv_bfloat16* __restrict__ qkv, const int32_t* __re
     SM& sm = *reinterpret_cast<SM*>(att_smem_raw);
 
     pdl_launch_dependents();
-    pdl_wait();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int q0 = blockIdx.x * kAttBlockM, head = blockIdx.y, b = blockIdx.z;
     const bool packed = seq_start != nullptr;
-    const size_t row0 = packed ? (size_t)__ldg(seq_start + b) : (size_t)b * S;
-    const int len = packed ? __ldg(seq_len + b) : S;   // rows of this sequence present in memory
+    const size_t row0 = packed ? (size_t)ld_early(seq_start + b) : (size_t)b * S;
+    const int len = packed ? ld_early(seq_len + b) : S;   // rows of this sequence present in memory
+    pdl_wait();
     if (q0 >= len) return;                              // whole CTA outside the sequence (uniform)
     // row layout: H columns of q heads, then H / kv_group of k heads, then as many of v heads
     const int Hkv = H / kind.kv_group;

@@ -33,6 +33,7 @@
 // records RLX_DEVSTAT_TIMEOUT, drains, frees its tensor memory and returns.
 #pragma once
 #include <cuda.h>
+#include <type_traits>
 #include "common.cuh"
 #include "epilogue.cuh"
 
@@ -43,6 +44,7 @@ constexpr int BLOCK_M = 128;
 constexpr int BLOCK_K = 64;   // 64 bf16 = 128 bytes = one swizzle row
 constexpr int UMMA_K = 16;
 constexpr int kStageBufBytes = 32 * 32 * 2;          // one 32-row x 32-column bf16 chunk
+constexpr int kPartBoth = 0, kPartW = 1, kPartA = 2;   // what a producer call requests
 constexpr uint64_t kWaitBudgetNs = 2000000000ull;  // 2 s per wait
 
 template <int BLOCK_N, int CG = 1>
@@ -58,6 +60,7 @@ struct Cfg {
     // the TMA store of a chunk drains while the next chunk is being computed.
     static constexpr int EPI_SPLIT = BLOCK_N >= 128 ? BLOCK_N / 64 : 2;
     static constexpr int EPI_WARPS = 4 * EPI_SPLIT;
+    static constexpr bool SMALL = BLOCK_N == 64 && CG == 1;   // the tile of problems too small to fill the SMs: latency counts
     static constexpr int THREADS = 64 + 32 * EPI_WARPS;
     static constexpr int SLAB = BLOCK_N / EPI_SPLIT;
     static constexpr int STAGING_BYTES = EPI_WARPS * kStageBufBytes;
@@ -457,14 +460,28 @@ struct EpilogueTile {
     static constexpr bool kStatsIn = kFold || EPI == 6;
     static constexpr bool kStatsOut = EPI == 5 || EPI == 6;
     uint4 res[kRes ? NC : 1][4];
+    bool dry = false;               // a rehearsal: same instructions, nothing handed back or stored (see the kernel)
     float ln_a = 1.f, ln_b = 0.f;   // x_norm = x * ln_a + ln_b  (ln_a = rstd, ln_b = -rstd * mu)
 
     // The bias values of a slab (one 128-byte line per chunk) are pulled into L1 a tile ahead of their
     // use by every lane, so that no chunk starts with an L2 round trip.
+    // The LayerNorm vectors of the folding modes likewise: read in place, each chunk cost two L2 round trips (1.0 to 1.3
+    // of the 5 us of a small product).
     static __device__ __forceinline__ void prefetch_bias(const Params& p, int n0) {
-        if (p.bias != nullptr && (threadIdx.x & 31) < NC) asm volatile("prefetch.global.L1 [%0];" ::"l"(p.bias + n0 + (threadIdx.x & 31) * 32));
+        const int lane = threadIdx.x & 31, c = lane % NC, which = lane / NC;
+        const float* v = nullptr;
+        if (kFold) v = which == 0 ? p.cvec : which == 1 ? p.dvec : nullptr;
+        else v = which == 0 ? p.bias : EPI != 6 ? nullptr : which == 1 ? p.ln_gamma : which == 2 ? p.ln_beta : nullptr;
+        if (v != nullptr) asm volatile("prefetch.global.L1 [%0];" ::"l"(v + n0 + c * 32));
     }
 
+    __device__ __forceinline__ void clear() {
+        if (kRes)
+#pragma unroll
+            for (int c = 0; c < NC; ++c)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) res[c][i] = make_uint4(0, 0, 0, 0);
+    }
     __device__ __forceinline__ void prefetch(const Params& p, int M, int m, int n0) {
         if (kRes && m < M) {
             const __nv_bfloat16* rpre = p.residual + (size_t)m * p.N + n0;
@@ -485,7 +502,7 @@ struct EpilogueTile {
     __device__ __forceinline__ void release(uint32_t tempty, uint32_t cta_rank, int lane) {
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) {
+        if (lane == 0 && !dry) {
             if (CG == 1) mbar_arrive_relaxed(tempty);
             else mbar_arrive_cluster_relaxed(map_to_cta(tempty, 0));   // the leader's barrier collects both CTAs' warps
         }
@@ -522,7 +539,7 @@ struct EpilogueTile {
                 uint4 q[4];
                 compute_chunk(p, r[c], n0 + c * 32, c, m, row_ok, brow + c * 32, q);
                 if (trace_slot >= 0 && c < 2) RLX_TRACE_CLK(p, trace_slot + 4 * c + 1);
-                store_chunk(p, tmap_out, q, n0 + c * 32, m_row0, stg, lane, row_off, swz);
+                store_chunk(p, tmap_out, q, n0 + c * 32, m_row0, stg, lane, row_off, swz, dry);
                 if (trace_slot >= 0 && c < 2) RLX_TRACE_CLK(p, trace_slot + 4 * c + 3);
             }
         } else {
@@ -536,7 +553,7 @@ struct EpilogueTile {
                 uint4 q[4];
                 compute_chunk(p, r[c & 1], n0 + c * 32, c, m, row_ok, brow + c * 32, q);
                 if (trace_slot >= 0 && c < 2) RLX_TRACE_CLK(p, trace_slot + 4 * c + 1);
-                store_chunk(p, tmap_out, q, n0 + c * 32, m_row0, stg, lane, row_off, swz);
+                store_chunk(p, tmap_out, q, n0 + c * 32, m_row0, stg, lane, row_off, swz, dry);
                 if (trace_slot >= 0 && c < 2) RLX_TRACE_CLK(p, trace_slot + 4 * c + 3);
             }
         }
@@ -612,17 +629,17 @@ struct EpilogueTile {
         }
         if (kStatsOut && row_ok) {
             // partial statistics of this row's 32 results (two-pass inside the chunk)
-            float sm = 0.f;
+            // (four interleaved sums: one chain of 64 dependent additions per chunk is 0.2 us of a small product)
+            float sm[4] = {0.f, 0.f, 0.f, 0.f}, sq[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-            for (int i = 0; i < 32; ++i) sm += v[i];
-            const float mean = sm * (1.0f / 32.0f);
-            float m2 = 0.f;
+            for (int i = 0; i < 32; ++i) sm[i & 3] += v[i];
+            const float mean = ((sm[0] + sm[1]) + (sm[2] + sm[3])) * (1.0f / 32.0f);
 #pragma unroll
             for (int i = 0; i < 32; ++i) {
                 const float dl = v[i] - mean;
-                m2 = fmaf(dl, dl, m2);
+                sq[i & 3] = fmaf(dl, dl, sq[i & 3]);
             }
-            p.stats_out[(size_t)m * (p.N / 32) + ncol / 32] = make_float2(mean, m2);
+            if (!dry) p.stats_out[(size_t)m * (p.N / 32) + ncol / 32] = make_float2(mean, (sq[0] + sq[1]) + (sq[2] + sq[3]));
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -637,14 +654,14 @@ struct EpilogueTile {
     // of arithmetic ago, must be done reading it) and hand it to the TMA engine.
     static __device__ __forceinline__ void store_chunk(const Params& p, const CUtensorMap* tmap_out, const uint4 (&q)[4],
                                                        int ncol, int m_row0, uint32_t stg, int lane, uint32_t row_off,
-                                                       uint32_t swz) {
+                                                       uint32_t swz, bool dry = false) {
         if (lane == 0) bulk_wait_read<0>();
         __syncwarp();
 #pragma unroll
         for (int i = 0; i < 4; ++i) st_shared_v4(stg + row_off + (((uint32_t)i ^ swz) << 4), q[i]);
         fence_proxy_async();   // the writes above become visible to the TMA engine
         __syncwarp();
-        if (lane == 0 && !RLX_DBG(p, kDbgNoStore)) {
+        if (lane == 0 && !dry && !RLX_DBG(p, kDbgNoStore)) {
             tma_store_2d(tmap_out, ncol, m_row0, stg);
             bulk_commit();
         }
@@ -707,12 +724,12 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
 
-    // everything above is independent of the previous kernel; its outputs are read only from here on
+    // The row count and the weights do not come from the previous kernel (see ld_early): they are read, and the first
+    // stages' W tiles requested, before the wait; A, the residual and the row statistics behind it.
     if (threadIdx.x == 0) RLX_TRACE(p, 1);
-    pdl_wait();
-    if (threadIdx.x == 0) RLX_TRACE(p, 2);
     int M = p.M;
-    if (p.m_ptr != nullptr) M = min(M, __ldg(p.m_ptr));   // packed activations: only sum(len) rows exist
+    if (p.m_ptr != nullptr) M = min(M, ld_early(p.m_ptr));   // packed activations: only sum(len) rows exist
+    if (threadIdx.x == 64) RLX_TRACE(p, 2);
     const int n_tiles = p.N / BLOCK_N;
     const int m_tiles = (M + TILE_M - 1) / TILE_M;
     const int num_tiles = n_tiles * m_tiles;
@@ -722,6 +739,57 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer (whole warp, one lane issues)
         {
+            // Request a stage's tiles: kPartW expects all of its bytes and requests W, kPartA requests A, kPartBoth does both.
+            // cta_group::2: both CTAs' copies complete on the LEADER's full barrier, which expects all bytes.
+            auto load = [&](auto part, int m_blk, int n_blk, int kb, int stage) {
+                constexpr bool A = decltype(part)::value != kPartW, W = decltype(part)::value != kPartA;
+                const int cnt = min(C::KPS, num_kb - kb);             // k-blocks in this stage
+                const uint32_t st0 = base + stage * C::STAGE_BYTES;   // [A k-blocks][W k-blocks]
+                const uint32_t sb0 = st0 + C::KPS * C::A_BYTES;
+                // 3-D maps: one load per operand brings all KPS k-blocks (a k-block past the end of K arrives as zeros and
+                // still counts its bytes)
+                const bool k3 = p.kblock_maps != 0;
+                const int nbytes = k3 ? C::KPS * C::KB_BYTES : cnt * C::KB_BYTES;
+                if (RLX_DBG(p, kDbgNoLoad)) {
+                    if (W && cta_rank == 0) mbar_arrive(full_bar + 8 * stage);
+                } else if constexpr (CG == 1) {
+                    if (W) mbar_expect_tx(full_bar + 8 * stage, nbytes);
+                    if (k3) {
+                        if (A) tma_load_3d(st0, &tmap_a, 0, m_blk * BLOCK_M, kb, full_bar + 8 * stage);
+                        if (W) tma_load_3d(sb0, &tmap_b, 0, n_blk * BLOCK_N, kb, full_bar + 8 * stage);
+                    } else {
+                        for (int i = 0; i < cnt; ++i) {
+                            if (A) tma_load_2d(st0 + i * C::A_BYTES, &tmap_a, (kb + i) * BLOCK_K, m_blk * BLOCK_M, full_bar + 8 * stage);
+                            if (W) tma_load_2d(sb0 + i * C::B_BYTES, &tmap_b, (kb + i) * BLOCK_K, n_blk * BLOCK_N, full_bar + 8 * stage);
+                        }
+                    }
+                } else {
+                    const uint32_t lead_full = map_to_cta(full_bar + 8 * stage, 0);
+                    if (W && cta_rank == 0) mbar_expect_tx(full_bar + 8 * stage, 2 * nbytes);
+                    const int arow = m_blk * TILE_M + (int)cta_rank * BLOCK_M, brow = n_blk * BLOCK_N + (int)cta_rank * C::B_ROWS;
+                    if (k3) {
+                        if (A) tma_load_3d_cg2(st0, &tmap_a, 0, arow, kb, lead_full);
+                        if (W) tma_load_3d_cg2(sb0, &tmap_b, 0, brow, kb, lead_full);
+                    } else {
+                        for (int i = 0; i < cnt; ++i) {
+                            if (A) tma_load_2d_cg2(st0 + i * C::A_BYTES, &tmap_a, (kb + i) * BLOCK_K, arow, lead_full);
+                            if (W) tma_load_2d_cg2(sb0 + i * C::B_BYTES, &tmap_b, (kb + i) * BLOCK_K, brow, lead_full);
+                        }
+                    }
+                }
+            };
+            // Narrow tiles (a handful of rows, one tile per CTA): the first tile's W, as far as the ring reaches, in front of the
+            // wait for the previous kernel. Wider tiles keep to the order of use: a ring full of W in front of the first A
+            // tile delays the first product (18432 x 768 x 768: 29.6 -> 33.5 us).
+            int early = 0;
+            if constexpr (C::SMALL) {
+                if (tile0 < num_tiles)
+                    for (; early < C::STAGES && early * C::KPS < num_kb; ++early) {
+                        if (elect_one()) load(std::integral_constant<int, kPartW>(), 0, tile0 % n_tiles, early * C::KPS, early);
+                        __syncwarp();
+                    }
+            }
+            pdl_wait();
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true;
@@ -729,46 +797,17 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
             for (int tile = tile0; tile < num_tiles && ok; tile += tile_step, ++pit) {
                 const int m_blk = tile / n_tiles, n_blk = tile % n_tiles;
                 for (int kb = 0; kb < num_kb; kb += C::KPS) {
-                    const int cnt = min(C::KPS, num_kb - kb);   // k-blocks in this stage
                     if (pit == 2 && kb == 0 && lane == 0) RLX_TRACE_CLK(p, 58);   // about to wait for a free stage
-                    if (!mbar_wait_warp(empty_bar + 8 * stage, phase ^ 1, abort_flag)) { ok = false; break; }
-                    if (pit == 2 && kb == 0 && lane == 0) RLX_TRACE_CLK(p, 59);   // stage free: loads issued now
-                    const uint32_t st0 = base + stage * C::STAGE_BYTES;   // [A k-blocks][W k-blocks]
-                    const uint32_t sb0 = st0 + C::KPS * C::A_BYTES;
-                    if (elect_one()) {
-                        // 3-D maps: one load per operand brings all KPS k-blocks (a k-block past the end of K
-                        // arrives as zeros and still counts its bytes)
-                        const bool k3 = p.kblock_maps != 0;
-                        const int nbytes = k3 ? C::KPS * C::KB_BYTES : cnt * C::KB_BYTES;
-                        if (RLX_DBG(p, kDbgNoLoad)) {
-                            if (cta_rank == 0) mbar_arrive(full_bar + 8 * stage);
-                        } else if constexpr (CG == 1) {
-                            mbar_expect_tx(full_bar + 8 * stage, nbytes);
-                            if (k3) {
-                                tma_load_3d(st0, &tmap_a, 0, m_blk * BLOCK_M, kb, full_bar + 8 * stage);
-                                tma_load_3d(sb0, &tmap_b, 0, n_blk * BLOCK_N, kb, full_bar + 8 * stage);
-                            } else {
-                                for (int i = 0; i < cnt; ++i) {
-                                    tma_load_2d(st0 + i * C::A_BYTES, &tmap_a, (kb + i) * BLOCK_K, m_blk * BLOCK_M, full_bar + 8 * stage);
-                                    tma_load_2d(sb0 + i * C::B_BYTES, &tmap_b, (kb + i) * BLOCK_K, n_blk * BLOCK_N, full_bar + 8 * stage);
-                                }
-                            }
-                        } else {
-                            // both CTAs' copies complete on the LEADER's full barrier, which expects all bytes
-                            const uint32_t lead_full = map_to_cta(full_bar + 8 * stage, 0);
-                            if (cta_rank == 0) mbar_expect_tx(full_bar + 8 * stage, 2 * nbytes);
-                            const int arow = m_blk * TILE_M + (int)cta_rank * BLOCK_M, brow = n_blk * BLOCK_N + (int)cta_rank * C::B_ROWS;
-                            if (k3) {
-                                tma_load_3d_cg2(st0, &tmap_a, 0, arow, kb, lead_full);
-                                tma_load_3d_cg2(sb0, &tmap_b, 0, brow, kb, lead_full);
-                            } else {
-                                for (int i = 0; i < cnt; ++i) {
-                                    tma_load_2d_cg2(st0 + i * C::A_BYTES, &tmap_a, (kb + i) * BLOCK_K, arow, lead_full);
-                                    tma_load_2d_cg2(sb0 + i * C::B_BYTES, &tmap_b, (kb + i) * BLOCK_K, brow, lead_full);
-                                }
-                            }
+                    if (C::SMALL && early > 0) {
+                        --early;               // a fresh stage whose W is under way
+                        if (elect_one()) load(std::integral_constant<int, kPartA>(), m_blk, n_blk, kb, stage);
+                    } else {
+                        if (!mbar_wait_warp(empty_bar + 8 * stage, phase ^ 1, abort_flag)) { ok = false; break; }
+                        if (pit == 2 && kb == 0 && lane == 0) RLX_TRACE_CLK(p, 59);   // stage free: loads issued now
+                        if (elect_one()) {
+                            load(std::integral_constant<int, kPartBoth>(), m_blk, n_blk, kb, stage);
+                            if (tile == tile0 && kb == 0) RLX_TRACE(p, 3);
                         }
-                        if (tile == tile0 && kb == 0) RLX_TRACE(p, 3);
                     }
                     __syncwarp();
                     if (++stage == C::STAGES) { stage = 0; phase ^= 1; }
@@ -843,24 +882,45 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
         const uint32_t stg = staging + ew * kStageBufBytes;
         int it = 0;
         bool ok = true;
-        if (tile0 < num_tiles) EpilogueTile<EPI, C::SLAB / 32>::prefetch_bias(p, (tile0 % n_tiles) * BLOCK_N + half * C::SLAB);
-        for (int tile = tile0; tile < num_tiles && ok; tile += tile_step, ++it) {
+        // While the previous kernel drains, the epilogue of the first tile is rehearsed on whatever the accumulator holds: the
+        // same instructions with every effect switched off. A kernel of a few microseconds otherwise spends about one of
+        // them fetching these instructions, and the vectors they read, for the first time.
+        // Only the narrowest tiles do it (the products of at most a few hundred rows: 1 x 128 tokens 170.6 -> 166.6 us per
+        // forward); for wider ones the longer-lived registers cost more than it saves.
+        constexpr bool kRehearse = C::SMALL;
+        bool dry = kRehearse;
+        if (!kRehearse) {
+            if (tile0 < num_tiles) EpilogueTile<EPI, C::SLAB / 32>::prefetch_bias(p, (tile0 % n_tiles) * BLOCK_N + half * C::SLAB);
+            pdl_wait();
+        }
+        for (int tile = tile0; tile < num_tiles && ok;) {
             const int m_blk = tile / n_tiles, n_blk = tile % n_tiles;
-            if (tile + tile_step < num_tiles)
-                EpilogueTile<EPI, C::SLAB / 32>::prefetch_bias(p, ((tile + tile_step) % n_tiles) * BLOCK_N + half * C::SLAB);
+            const int next = tile + tile_step;
+            if (!(kRehearse && dry) && next < num_tiles) EpilogueTile<EPI, C::SLAB / 32>::prefetch_bias(p, (next % n_tiles) * BLOCK_N + half * C::SLAB);
             const int as = it & 1;
             const uint32_t aphase = (it >> 1) & 1;
             const int m_row0 = m_blk * TILE_M + (int)cta_rank * BLOCK_M + quad * 32;
             const int n0 = n_blk * BLOCK_N + half * C::SLAB;
             const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + as * BLOCK_N + half * C::SLAB;
             EpilogueTile<EPI, C::SLAB / 32> et;
-            et.prefetch(p, M, m_row0 + lane, n0);   // residual / row statistics: issued before the accumulator wait
-            if (!mbar_wait(tfull_bar + 8 * as, aphase, abort_flag)) { ok = false; break; }
-            tc_fence_after();
+            et.dry = kRehearse && dry;
+            if (kRehearse && dry) et.clear();
+            if (!et.dry) {
+                et.prefetch(p, M, m_row0 + lane, n0);   // residual / row statistics: issued before the accumulator wait
+                if (!mbar_wait(tfull_bar + 8 * as, aphase, abort_flag)) { ok = false; break; }
+                tc_fence_after();
+            }
             if (ew == 0 && lane == 0 && it < 12) RLX_TRACE(p, 16 + it);
             et.template drain<CG>(p, &tmap_out, M, m_row0, n0, taddr, stg, lane, tempty_bar + 8 * as, cta_rank,
                                   (ew == 0 && lane == 0 && (it == 1 || it == 5)) ? 40 + 2 * (it - 1) : -1);
             if (ew == 0 && lane == 0 && it < 12) RLX_TRACE(p, 28 + it);
+            if (kRehearse && dry) {
+                dry = false;
+                pdl_wait();
+            } else {
+                tile = next;
+                ++it;
+            }
         }
         EpilogueTile<EPI, C::SLAB / 32>::finish(lane);
         if (ew == 0 && lane == 0) RLX_TRACE(p, 8);
