@@ -21,6 +21,7 @@
 #include "gemm_ares_tcgen05.cuh"
 #include "gemm_ln_tcgen05.cuh"
 #include "gemm_cln_tcgen05.cuh"
+#include "gemm_splitk_tcgen05.cuh"
 #include "rowwise.cuh"
 
 namespace {
@@ -207,6 +208,12 @@ cudaError_t init_kernels_for_current_device() {
         if ((e = cudaOccupancyMaxActiveClusters(&n, rlx::tc::gemm_tcgen05_kernel<256, 0, 2>, &cfg)) != cudaSuccess) return e;
         if (dev < 64) g_max_pairs[dev] = n;
     }
+#define RLX_SPLITK_ATTR(EPI)                                                                                   \
+    if ((e = cudaFuncSetAttribute(rlx::tcsk::gemm_splitk_tcgen05_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                                  rlx::tcsk::kSmemBytes)) != cudaSuccess)                                       \
+        return e;
+    RLX_SPLITK_ATTR(0) RLX_SPLITK_ATTR(1) RLX_SPLITK_ATTR(2) RLX_SPLITK_ATTR(5) RLX_SPLITK_ATTR(6)
+#undef RLX_SPLITK_ATTR
 #define RLX_ARES_ATTR(BN, EPI)                                                                                  \
     if ((e = cudaFuncSetAttribute(rlx::tcar::gemm_ares_tcgen05_kernel<BN, EPI>,                                \
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, rlx::tcar::Cfg<BN>::SMEM_BYTES)) != \
@@ -646,6 +653,35 @@ struct LnFold {
     float eps = 0.f;
 };
 
+// CTAs per 128 x 64 tile along K (1: do not split).  A long contraction on a few tiles is bound by one SM's operand feed;
+// four CTAs per tile while they all fit beside each other, two while two thirds of them do -- the row count is the
+// padded one, and a batch whose every position is valid then runs two half-length rounds instead of one.
+int pick_split_k(int M, int N, int K, int epi) {
+    if (K < 1536 || N % rlx::tcsk::kBN != 0 || (epi > 2 && epi < 5)) return 1;
+    const int tiles = (M + rlx::tc::BLOCK_M - 1) / rlx::tc::BLOCK_M * (N / rlx::tcsk::kBN), sms = sm_count();
+    return 4 * tiles <= sms ? 4 : 3 * tiles < 2 * sms - 8 ? 2 : 1;
+}
+
+rlx_status_t launch_gemm_splitk(const bf16* A, const bf16* W, const rlx::tc::Params& p, const CUtensorMap& to, int epi, int split,
+                                cudaStream_t st) {
+    CUtensorMap ta, tb;
+    if (!make_tmap(&ta, A, (uint64_t)p.M, (uint64_t)p.K, 32) || !make_tmap(&tb, W, (uint64_t)p.N, (uint64_t)p.K, rlx::tcsk::kBN))
+        return RLX_ERR_CUDA;
+    const int grid = split * ((p.M + rlx::tc::BLOCK_M - 1) / rlx::tc::BLOCK_M) * (p.N / rlx::tcsk::kBN);
+    struct ClusterScope {
+        explicit ClusterScope(int x) { g_cluster_x = x; }
+        ~ClusterScope() { g_cluster_x = 1; }
+    } scope(split);
+    switch (epi) {
+#define RLX_CASE(E) case E: RLX_CUDA_TRY(launch_ex(rlx::tcsk::gemm_splitk_tcgen05_kernel<E>, grid, rlx::tcsk::kThreads, rlx::tcsk::kSmemBytes, st, ta, tb, to, p)); break;
+        RLX_CASE(0) RLX_CASE(1) RLX_CASE(2) RLX_CASE(5) RLX_CASE(6)
+#undef RLX_CASE
+        default: return RLX_ERR_INVALID_ARG;
+    }
+    RLX_CUDA_TRY(cudaGetLastError());
+    return RLX_OK;
+}
+
 rlx_status_t launch_gemm(const bf16* A, const bf16* W, const float* bias, const bf16* residual, int epi, int M, int N,
                          int K, bf16* out, bool simt, int32_t* status, cudaStream_t st,
                          const int32_t* m_ptr = nullptr, int want_cg = 0, const LnFold* lf = nullptr) {
@@ -671,6 +707,13 @@ rlx_status_t launch_gemm(const bf16* A, const bf16* W, const float* bias, const 
     CUtensorMap ta, tb, to;
     // output chunks: 32 x 32 bf16 boxes with the 64-byte swizzle of the epilogue's staging buffers
     if (!make_tmap(&to, out, (uint64_t)M, (uint64_t)N, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B)) return RLX_ERR_CUDA;
+    if (epi >= 3) {
+        if (!lf || N % 32 != 0) return RLX_ERR_INVALID_ARG;
+        p.cvec = lf->cvec; p.dvec = lf->dvec; p.stats_in = lf->stats_in; p.stats_in_p = lf->stats_in_p;
+        p.ln_gamma = lf->gamma; p.ln_beta = lf->beta; p.stats_out = lf->stats_out; p.ln_eps = lf->eps;
+    }
+    const int split = want_cg == 0 ? pick_split_k(M, N, K, epi) : 1;
+    if (split > 1) return launch_gemm_splitk(A, W, p, to, epi, split, st);
     // want_cg == 3: the A-resident CTA-pair kernel, forced; 0: chosen when the problem is large enough
     if (want_cg == 3 || (want_cg == 0 && g_exp_resident >= 0)) {
         const int rbn = pick_resident_bn(M, N, K, epi, want_cg == 3 || g_exp_resident > 0);
@@ -702,11 +745,6 @@ rlx_status_t launch_gemm(const bf16* A, const bf16* W, const float* bias, const 
     p.kblock_maps = make_operand_tmaps(&ta, &tb, A, W, (uint64_t)M, (uint64_t)N, (uint64_t)K, rlx::tc::BLOCK_M,
                                        (uint32_t)(bn / tc.cg), kps);
     if (p.kblock_maps < 0) return RLX_ERR_CUDA;
-    if (epi >= 3) {
-        if (!lf || N % 32 != 0) return RLX_ERR_INVALID_ARG;
-        p.cvec = lf->cvec; p.dvec = lf->dvec; p.stats_in = lf->stats_in; p.stats_in_p = lf->stats_in_p;
-        p.ln_gamma = lf->gamma; p.ln_beta = lf->beta; p.stats_out = lf->stats_out; p.ln_eps = lf->eps;
-    }
     if (tc.cg == 2) {
         switch (bn) {
             case 128: return launch_gemm_tc_bn<128, 2>(ta, tb, to, p, epi, st);
