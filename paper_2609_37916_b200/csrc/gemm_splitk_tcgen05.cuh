@@ -33,7 +33,8 @@ constexpr int kThreads = 64 + 32 * kEpiWarps;
 constexpr int kXchOff = kStages * kStageBytes; // partial sums received: [local unit][source rank]
 constexpr int kXchBytes = 8 * kUnitBytes;      // 8 / S units from S sources
 constexpr int kStagingOff = kXchOff + kXchBytes;
-constexpr int kBarOff = kStagingOff + kEpiWarps * kStageBufBytes;
+constexpr int kVecOff = kStagingOff + kEpiWarps * kStageBufBytes;   // per-column vectors, see EpilogueTile
+constexpr int kBarOff = kVecOff + kEpiWarps * 384;
 constexpr int kSmemBytes = kBarOff + 8 * (2 * kStages + 2) + 16 + 1024;
 static_assert(kSmemBytes <= 227 * 1024, "shared memory");
 
@@ -163,9 +164,9 @@ gemm_splitk_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __g
         const bool finish = e < mine;
         const int m_row0 = m_blk * BLOCK_M + ug * 32, n0 = n_blk * kBN + uh * 32;
         const uint32_t stg = base + kStagingOff + e * kStageBufBytes;
-        using ET = EpilogueTile<EPI, 1>;
+        using ET = EpilogueTile<EPI, 1, true>;
         ET et;
-        if (finish) ET::prefetch_bias(p, n0);
+        if (finish) et.load_vectors(p, n0, base + kVecOff + e * 384);
         pdl_wait();
         if (finish) et.prefetch(p, M, m_row0 + lane, n0);
         bool ok = true;

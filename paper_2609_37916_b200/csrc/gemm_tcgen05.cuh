@@ -47,7 +47,7 @@ constexpr int kStageBufBytes = 32 * 32 * 2;          // one 32-row x 32-column b
 constexpr int kPartBoth = 0, kPartW = 1, kPartA = 2;   // what a producer call requests
 constexpr uint64_t kWaitBudgetNs = 2000000000ull;  // 2 s per wait
 
-template <int BLOCK_N, int CG = 1>
+template <int BLOCK_N, int CG = 1, bool FOLD = false>
 struct Cfg {
     static constexpr int A_BYTES = BLOCK_M * BLOCK_K * 2;
     static constexpr int B_ROWS = BLOCK_N / CG;                  // W rows this CTA loads per k-block
@@ -64,8 +64,14 @@ struct Cfg {
     static constexpr int THREADS = 64 + 32 * EPI_WARPS;
     static constexpr int SLAB = BLOCK_N / EPI_SPLIT;
     static constexpr int STAGING_BYTES = EPI_WARPS * kStageBufBytes;
+    // A warp's 32 columns of the two or three per-column vectors of the LayerNorm-folding modes, see EpilogueTile.  There is
+    // no room for them beside 256-wide tiles, and one vector alone is better read in place (36736 x 1152 x 384 with a
+    // bias: 33.3 us, through shared memory 36.9).
+    static constexpr bool VEC = FOLD && BLOCK_N <= 192;
+    static constexpr int VEC_WARP_BYTES = VEC ? 3 * 128 : 0;
+    static constexpr int VEC_BYTES = EPI_WARPS * VEC_WARP_BYTES;
     static constexpr int BAR_BYTES = 256;
-    static constexpr int RING_BUDGET = 227 * 1024 - 1024 - BAR_BYTES - STAGING_BYTES;
+    static constexpr int RING_BUDGET = 227 * 1024 - 1024 - BAR_BYTES - STAGING_BYTES - VEC_BYTES;
     // A stage holds KPS k-blocks behind ONE full / empty barrier pair.  A barrier round costs the issuing
     // thread a couple of hundred cycles whether or not the barrier is already complete (measured: 4 MMAs
     // + wait + commit take ~430 cycles of the thread, 8 MMAs ~620), so with one k-block per round the
@@ -84,7 +90,7 @@ struct Cfg {
     static constexpr int STAGES = (RING_BUDGET / STAGE_BYTES) > 8 ? 8 : (RING_BUDGET / STAGE_BYTES);
     static constexpr int TMEM_COLS = (2 * BLOCK_N <= 32) ? 32 : (2 * BLOCK_N <= 64) ? 64 : (2 * BLOCK_N <= 128) ? 128
                                      : (2 * BLOCK_N <= 256) ? 256 : 512;
-    static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + STAGING_BYTES + BAR_BYTES + 1024;  // +1024: manual alignment
+    static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + STAGING_BYTES + VEC_BYTES + BAR_BYTES + 1024;  // +1024: manual alignment
     static_assert(BLOCK_N % 16 == 0 && BLOCK_N >= 16 && BLOCK_N <= 256, "UMMA N for M=128 / M=256");
     static_assert(CG == 1 || CG == 2, "cta_group");
     static_assert(B_BYTES % 1024 == 0, "stage tiles must stay 1024-byte aligned");
@@ -453,13 +459,21 @@ constexpr int kDbgNoLoad = 8;       // the producer only arrives (tensor pipe al
 // TMA reads the staged tile itself and writes whole lines.  Rows at or beyond the matrix's row count
 // are clipped by the tensor map; rows between a smaller device-side row count (packed batches) and the
 // end of the last tile are written with values nobody reads.
-template <int EPI, int NC>
+//
+// The per-column vectors (VEC): every thread of a warp needs the same 32 values of each, and reading them in place
+// is eight 16-byte global loads per vector and chunk that take about 45 cycles each, L1 hit or not (a third of the epilogue
+// with one vector, two thirds with three). With two or three of them a lane instead loads ONE column's values ahead of time, and the warp
+// spreads them through its slot in shared memory, from where eight 16-byte broadcasts cost a few cycles each.
+template <int EPI, int NC, bool VEC = false>
 struct EpilogueTile {
     static constexpr bool kRes = EPI == 2 || EPI == 5 || EPI == 6;     // a residual tile is added
     static constexpr bool kFold = EPI == 3 || EPI == 4;                // LayerNorm folded into this GEMM's input
     static constexpr bool kStatsIn = kFold || EPI == 6;
     static constexpr bool kStatsOut = EPI == 5 || EPI == 6;
     uint4 res[kRes ? NC : 1][4];
+    static constexpr int NV = kFold ? 2 : EPI == 6 ? 3 : 1;             // per-column vectors
+    float vv[VEC ? NC : 1][VEC ? NV : 1];   // this lane's column of each, per chunk
+    uint32_t vslot = 0;                     // the warp's slot: NV x 32 floats
     bool dry = false;               // a rehearsal: same instructions, nothing handed back or stored (see the kernel)
     float ln_a = 1.f, ln_b = 0.f;   // x_norm = x * ln_a + ln_b  (ln_a = rstd, ln_b = -rstd * mu)
 
@@ -475,6 +489,26 @@ struct EpilogueTile {
         if (v != nullptr) asm volatile("prefetch.global.L1 [%0];" ::"l"(v + n0 + c * 32));
     }
 
+    __device__ __forceinline__ void load_vectors(const Params& p, int n0, uint32_t slot) {
+        if constexpr (VEC) {
+            vslot = slot;
+            const int lane = threadIdx.x & 31;
+            const float* src[3] = {kFold ? p.cvec : p.bias, kFold ? p.dvec : p.ln_gamma, p.ln_beta};
+#pragma unroll
+            for (int c = 0; c < NC; ++c)
+#pragma unroll
+                for (int k = 0; k < NV; ++k) vv[c][k] = src[k] != nullptr ? __ldg(src[k] + n0 + c * 32 + lane) : 0.f;
+        }
+    }
+    // eight values of vector k, columns 4i .. 4i + 3 and so on: from the slot (VEC) or in place
+    __device__ __forceinline__ float4 vec4(int k, int i, const float* in_place) const {
+        if constexpr (VEC) {
+            const uint4 q = ld_shared_v4(vslot + k * 128 + i * 16);
+            return make_float4(__uint_as_float(q.x), __uint_as_float(q.y), __uint_as_float(q.z), __uint_as_float(q.w));
+        } else {
+            return __ldg(reinterpret_cast<const float4*>(in_place) + i);
+        }
+    }
     __device__ __forceinline__ void clear() {
         if (kRes)
 #pragma unroll
@@ -563,13 +597,20 @@ struct EpilogueTile {
     __device__ __forceinline__ void compute_chunk(const Params& p, const uint32_t (&acc)[32], int ncol, int c, int m,
                                                   bool row_ok, const float* bias32, uint4 (&q)[4]) {
         float v[32];
+        if constexpr (VEC) {
+            const int lane = threadIdx.x & 31;
+            __syncwarp();     // the previous chunk's reads are done
+#pragma unroll
+            for (int k = 0; k < NV; ++k) asm volatile("st.shared.f32 [%0], %1;" ::"r"(vslot + k * 128 + lane * 4), "f"(vv[c][k]) : "memory");
+            __syncwarp();
+        }
         if constexpr (kFold) {
             const float* crow = p.cvec + ncol;
             const float* drow = p.dvec + ncol;
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
-                const float4 c4 = __ldg(reinterpret_cast<const float4*>(crow) + i);
-                const float4 d4 = __ldg(reinterpret_cast<const float4*>(drow) + i);
+                const float4 c4 = vec4(0, i, crow);
+                const float4 d4 = vec4(1, i, drow);
                 v[4 * i + 0] = fmaf(ln_a, __uint_as_float(acc[4 * i + 0]), fmaf(ln_b, c4.x, d4.x));
                 v[4 * i + 1] = fmaf(ln_a, __uint_as_float(acc[4 * i + 1]), fmaf(ln_b, c4.y, d4.y));
                 v[4 * i + 2] = fmaf(ln_a, __uint_as_float(acc[4 * i + 2]), fmaf(ln_b, c4.z, d4.z));
@@ -577,7 +618,10 @@ struct EpilogueTile {
             }
         } else {
             float4 b4[8];
-            if (p.bias != nullptr) {   // uniform; the encoder's GEMMs always carry a bias
+            if constexpr (VEC) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) b4[i] = vec4(0, i, nullptr);
+            } else if (p.bias != nullptr) {   // uniform; the encoder's GEMMs always carry a bias
 #pragma unroll
                 for (int i = 0; i < 8; ++i) b4[i] = ld_global_keep_f4(bias32 + 4 * i);
             } else {
@@ -613,10 +657,8 @@ struct EpilogueTile {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const uint4 w = res[kRes ? c : 0][i];
-                const float4 g0 = __ldg(reinterpret_cast<const float4*>(grow) + 2 * i);
-                const float4 g1 = __ldg(reinterpret_cast<const float4*>(grow) + 2 * i + 1);
-                const float4 e0 = __ldg(reinterpret_cast<const float4*>(berow) + 2 * i);
-                const float4 e1 = __ldg(reinterpret_cast<const float4*>(berow) + 2 * i + 1);
+                const float4 g0 = vec4(1, 2 * i, grow), g1 = vec4(1, 2 * i + 1, grow);
+                const float4 e0 = vec4(2, 2 * i, berow), e1 = vec4(2, 2 * i + 1, berow);
                 v[8 * i + 0] += fmaf(fmaf(bf16lo(w.x), ln_a, ln_b), g0.x, e0.x);
                 v[8 * i + 1] += fmaf(fmaf(bf16hi(w.x), ln_a, ln_b), g0.y, e0.y);
                 v[8 * i + 2] += fmaf(fmaf(bf16lo(w.y), ln_a, ln_b), g0.z, e0.z);
@@ -675,10 +717,10 @@ struct EpilogueTile {
 };
 
 template <int BLOCK_N, int EPI, int CG>
-__global__ void __launch_bounds__((Cfg<BLOCK_N, CG>::THREADS), 1)
+__global__ void __launch_bounds__((Cfg<BLOCK_N, CG, (EPI >= 3)>::THREADS), 1)
 gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
                     const __grid_constant__ CUtensorMap tmap_out, const Params p) {
-    using C = Cfg<BLOCK_N, CG>;
+    using C = Cfg<BLOCK_N, CG, (EPI >= 3)>;
     constexpr int TILE_M = BLOCK_M * CG;   // rows of one output tile (per CTA pair when CG = 2)
     extern __shared__ unsigned char smem_raw[];
     // manual 1024-byte alignment (required by the 128-byte swizzle atoms)
@@ -686,12 +728,12 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
     const uint32_t base = (raw + 1023u) & ~1023u;
     unsigned char* gbase = smem_raw + (base - raw);
     const uint32_t staging = base + C::STAGES * C::STAGE_BYTES;
-    const uint32_t bars = staging + C::STAGING_BYTES;
+    const uint32_t vecs = staging + C::STAGING_BYTES, bars = vecs + C::VEC_BYTES;
     // barrier block: full[STAGES], empty[STAGES], tmem_full[2], tmem_empty[2], tmem slot, abort flag
     const uint32_t full_bar = bars, empty_bar = bars + 8 * C::STAGES;
     const uint32_t tfull_bar = bars + 16 * C::STAGES, tempty_bar = tfull_bar + 16;
     uint32_t* tmem_slot =
-        reinterpret_cast<uint32_t*>(gbase + C::STAGES * C::STAGE_BYTES + C::STAGING_BYTES + 16 * C::STAGES + 32);
+        reinterpret_cast<uint32_t*>(gbase + C::STAGES * C::STAGE_BYTES + C::STAGING_BYTES + C::VEC_BYTES + 16 * C::STAGES + 32);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -882,6 +924,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
         const uint32_t stg = staging + ew * kStageBufBytes;
         int it = 0;
         bool ok = true;
+        using ET = EpilogueTile<EPI, C::SLAB / 32, C::VEC>;
         // While the previous kernel drains, the epilogue of the first tile is rehearsed on whatever the accumulator holds: the
         // same instructions with every effect switched off. A kernel of a few microseconds otherwise spends about one of
         // them fetching these instructions, and the vectors they read, for the first time.
@@ -890,19 +933,20 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
         constexpr bool kRehearse = C::SMALL;
         bool dry = kRehearse;
         if (!kRehearse) {
-            if (tile0 < num_tiles) EpilogueTile<EPI, C::SLAB / 32>::prefetch_bias(p, (tile0 % n_tiles) * BLOCK_N + half * C::SLAB);
+            if (tile0 < num_tiles) ET::prefetch_bias(p, (tile0 % n_tiles) * BLOCK_N + half * C::SLAB);
             pdl_wait();
         }
         for (int tile = tile0; tile < num_tiles && ok;) {
             const int m_blk = tile / n_tiles, n_blk = tile % n_tiles;
             const int next = tile + tile_step;
-            if (!(kRehearse && dry) && next < num_tiles) EpilogueTile<EPI, C::SLAB / 32>::prefetch_bias(p, (next % n_tiles) * BLOCK_N + half * C::SLAB);
+            if (!(kRehearse && dry) && next < num_tiles) ET::prefetch_bias(p, (next % n_tiles) * BLOCK_N + half * C::SLAB);
             const int as = it & 1;
             const uint32_t aphase = (it >> 1) & 1;
             const int m_row0 = m_blk * TILE_M + (int)cta_rank * BLOCK_M + quad * 32;
             const int n0 = n_blk * BLOCK_N + half * C::SLAB;
             const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + as * BLOCK_N + half * C::SLAB;
-            EpilogueTile<EPI, C::SLAB / 32> et;
+            ET et;
+            et.load_vectors(p, n0, vecs + ew * C::VEC_WARP_BYTES);
             et.dry = kRehearse && dry;
             if (kRehearse && dry) et.clear();
             if (!et.dry) {
@@ -922,7 +966,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
                 ++it;
             }
         }
-        EpilogueTile<EPI, C::SLAB / 32>::finish(lane);
+        ET::finish(lane);
         if (ew == 0 && lane == 0) RLX_TRACE(p, 8);
     }
 

@@ -123,7 +123,7 @@ int make_operand_tmaps(CUtensorMap* ta, CUtensorMap* tb, const void* A, const vo
 template <int BN, int EPI, int CG>
 cudaError_t set_gemm_attr() {
     return cudaFuncSetAttribute(rlx::tc::gemm_tcgen05_kernel<BN, EPI, CG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                rlx::tc::Cfg<BN, CG>::SMEM_BYTES);
+                                rlx::tc::Cfg<BN, CG, (EPI >= 3)>::SMEM_BYTES);
 }
 template <int BN, int CG = 1>
 cudaError_t set_gemm_attr_all() {
@@ -580,7 +580,8 @@ rlx_status_t launch_gemm_tc_bn(const CUtensorMap& ta, const CUtensorMap& tb, con
     cudaGetDevice(&dev);
     const int slots = CG == 1 ? sm_count() : ((dev >= 0 && dev < 64) ? g_max_pairs[dev] : 1);
     const int grid = CG * (tiles < slots ? tiles : slots);
-    const int smem = rlx::tc::Cfg<BN, CG>::SMEM_BYTES;
+    static_assert(rlx::tc::Cfg<BN, CG, true>::KPS == rlx::tc::Cfg<BN, CG>::KPS, "one set of tensor maps");
+    const int smem = epi >= 3 ? rlx::tc::Cfg<BN, CG, true>::SMEM_BYTES : rlx::tc::Cfg<BN, CG>::SMEM_BYTES;
     struct ClusterScope {
         explicit ClusterScope(int x) { g_cluster_x = x; }
         ~ClusterScope() { g_cluster_x = 1; }
