@@ -61,7 +61,7 @@ typedef enum {
 #define RLX_FLAG_GEMM_SIMT 0x2u /* use the plain CUDA-core GEMM (bring-up / cross-check only)  */
 #define RLX_FLAG_KERNEL_EVENTS 0x4u /* record a CUDA event between kernels (see rlx_encoder_kernel_times) */
 #define RLX_FLAG_NO_PDL 0x10u   /* plain stream order between kernels (no programmatic dependent launch) */
-#define RLX_FLAG_ATTN_TCGEN05 0x20u /* packed attention on the tcgen05/TMEM kernel instead of the mma.sync one */
+#define RLX_FLAG_ATTN_TCGEN05 0x20u /* packed attention on the tcgen05/TMEM kernel at every size, not only where it is faster */
 #define RLX_FLAG_FUSED_LN 0x40u /* fold the residual LayerNorms into the out-proj / FFN-down GEMMs, whole rows per CTA */
 #define RLX_FLAG_CLUSTER_LN 0x80u /* fold the residual LayerNorms into the GEMMs with cluster-wide row statistics */
 #define RLX_FLAG_NO_PREFETCH 0x100u /* no L2 prefetch of the Linear weights on a side branch of the captured graph */
@@ -414,8 +414,8 @@ rlx_status_t rlx_attention_f32(const float *qkv_f32, const int32_t *attention_ma
  * `rows` rows of [q | k | v]; sequence b owns rows seq_start[b] .. seq_start[b] + seq_len[b], all
  * valid, seq_len[b] <= max_len <= 512; ctx uses the same row numbering.  impl 0: tcgen05/TMEM
  * kernel (TMA-fed, one pass over the keys, S and P in tensor memory, one thread per
- * query row in the softmax); impl 1: warp-level mma.sync kernel (what rlx_encoder_forward runs
- * unless RLX_FLAG_ATTN_TCGEN05 is set).  Rows outside every sequence are not written.
+ * query row in the softmax); impl 1: warp-level mma.sync kernel
+ * (rlx_encoder_forward takes one or the other by head_dim and sequence length).  Rows outside every sequence are not written.
  * status: optional device word, receives RLX_DEVSTAT_TIMEOUT
  * if a bounded wait of impl 0 ran out.
  */

@@ -65,8 +65,8 @@ struct Cfg {
     static constexpr int SLAB = BLOCK_N / EPI_SPLIT;
     static constexpr int STAGING_BYTES = EPI_WARPS * kStageBufBytes;
     // A warp's 32 columns of the two or three per-column vectors of the LayerNorm-folding modes, see EpilogueTile.  There is
-    // no room for them beside 256-wide tiles, and one vector alone is better read in place (36736 x 1152 x 384 with a
-    // bias: 33.3 us, through shared memory 36.9).
+    // no room for them beside 256-wide tiles; a single bias vector is read in place (large products, where that form is
+    // used, are not bound by it).
     static constexpr bool VEC = FOLD && BLOCK_N <= 192;
     static constexpr int VEC_WARP_BYTES = VEC ? 3 * 128 : 0;
     static constexpr int VEC_BYTES = EPI_WARPS * VEC_WARP_BYTES;

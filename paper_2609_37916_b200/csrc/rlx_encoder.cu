@@ -984,6 +984,22 @@ int kernels_in_forward(const rlx_encoder_config_t& c, int B, int S) {
 bool uses_chunks(const rlx_encoder_config_t& c, int B, int S);
 int chunk_batch(int B, int S);
 
+// The tcgen05 attention kernel instead of the mma.sync one: where asked for, and where it pays inside a whole forward
+// (us mma.sync / tcgen05, 6 x 384 with heads of 32 and 12 x 768 with heads of 64; batch x longest sequence):
+//   64: sequences beyond two 128-row tiles everywhere (1 x 512 644 / 569, 64 x 512 4499 / 4119); beyond one tile once
+//       there are enough tokens to fill the chip (100 x 144 2520 / 2434, 70 x 200 1909 / 1889; but 8 x 144 544 / 560,
+//       1 x 256 435 / 474)
+//   32: beyond 384 (128 x 512 1414 / 1360, 60 x 512 832 / 822; 128 x 384 1100 / 1106); two full tiles while an item's
+//       own chain is what a layer waits for (4 x 256 230 / 201, 60 x 256 708 / 690; but 256 x 256 1254 / 1265, and
+//       61 x 203 442 / 459)
+bool uses_attention_fwd(const rlx_encoder_config_t& c, int B, int S) {
+    if (c.flags & RLX_FLAG_ATTN_TCGEN05) return true;
+    const long long tokens = g_whole_call_tokens > 0 ? g_whole_call_tokens : (long long)B * S;
+    constexpr int kT = rlx::tcat::kTile;
+    if (c.hidden / c.num_heads == 64) return S > 2 * kT || (S > kT && tokens >= 8192);
+    return S > 3 * kT || (S >= 2 * kT && tokens <= 16384);
+}
+
 struct GraphEntry {
     int B, S;
     const void *ids, *mask, *out, *ws;
@@ -1203,7 +1219,7 @@ rlx_status_t enqueue_forward(const rlx_encoder* e, const int32_t* ids, const int
                 lf.stats_in = stats_z; lf.stats_in_p = P;
                 RLX_TRY(launch_gemm(z, (const bf16*)(fb + a.f_wqkv), lw.bqkv, nullptr, 3, T, 3 * H, H, qkv, false, status, st, rows, 0, &lf));
             }
-            if (pack && (c.flags & RLX_FLAG_ATTN_TCGEN05))
+            if (pack && uses_attention_fwd(c, B, S))
                 RLX_TRY(launch_attention_fwd(qkv, T, pk.seq_start, pk.seq_len, B, S, h, d, 1, false, 0, nullptr, nullptr, ctx, status, st));
             else
                 RLX_TRY(launch_attention_bf16(qkv, mask, pk.seq_start, pk.seq_len, B, S, h, d, ctx, st));
@@ -1242,7 +1258,7 @@ rlx_status_t enqueue_forward(const rlx_encoder* e, const int32_t* ids, const int
     for (int l = 0; l < c.num_layers; ++l) {
         const rlx_layer_weights_t& lw = w->layers[l];
         RLX_TRY(launch_gemm(x, (const bf16*)lw.wqkv, lw.bqkv, nullptr, RLX_EPI_BIAS, T, 3 * H, H, qkv, simt, status, st, rows));
-        if (pack && (c.flags & RLX_FLAG_ATTN_TCGEN05))
+        if (pack && uses_attention_fwd(c, B, S))
             RLX_TRY(launch_attention_fwd(qkv, T, pk.seq_start, pk.seq_len, B, S, h, d, 1, false, 0, nullptr, nullptr, ctx, status, st));
         else
             RLX_TRY(launch_attention_bf16(qkv, mask, pk.seq_start, pk.seq_len, B, S, h, d, ctx, st));

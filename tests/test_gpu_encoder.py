@@ -229,6 +229,24 @@ def test_random_small_problems_match_oracle(rlx, seed):
             check(other, ref, inp.lengths, tight=(seed % 4 != 0))
 
 
+@pytest.mark.parametrize("name,B,S", [("c1", 3, 255), ("c1", 3, 256), ("c1", 64, 256), ("c1", 65, 256), ("c1", 45, 384),
+                                      ("c1", 45, 385), ("c4", 2, 256), ("c4", 2, 257), ("c4", 64, 128), ("c4", 63, 129),
+                                      ("c4", 64, 129)])
+def test_attention_kernel_choice_at_its_edges(rlx, name, B, S):
+    """Both sides of every line where a forward changes its attention kernel (heads of 32 and of 64), the first, a
+    middle and the last sequence against the oracle; the kernel that may be asked for gives the same at that tolerance."""
+    lengths = np.random.default_rng(B * 1000 + S).integers(0, S + 1, size=B)
+    lengths[0], lengths[-1] = S, S - 1
+    inp = make_inputs(CONFIGS[name], batch=B, seq=S, num_layers=2, lengths=lengths)
+    pick = sorted({0, B // 2, B - 1})
+    ref = oracle.encoder_forward(inp.cfg, inp.ids[pick], inp.mask[pick], inp.params, inp.layers)
+    w = rlx.upload_weights(inp.params, inp.layers)
+    for flags in (0, 0x20):
+        got, status = run_gpu(rlx, inp, weights=w, flags=flags)
+        assert status == 0
+        check(got[pick], ref, inp.lengths[pick])
+
+
 def test_degenerate_lengths_zero_one_full(rlx):
     inp = make_inputs(CONFIGS["c1"], batch=3, seq=40, num_layers=2, lengths=[0, 1, 40])
     got, status = run_gpu(rlx, inp)
