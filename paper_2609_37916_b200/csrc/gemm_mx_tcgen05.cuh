@@ -1,32 +1,32 @@
 // Block-scaled FP8 product on the tensor cores' own block-scaled path (the Blackwell half of
 // ScaledMatMul): out[M,N] = A W^T (+ bias) with BOTH operands given as (8-bit element codes, one E8M0
-// scale byte per 32 consecutive k).  Three kernels (the product has a 128 x 128-tile form, described
-// first, and a persistent 128 x 192-tile form further down for widths that are multiples of 192):
+// scale byte per 32 consecutive k).  Two kernels:
 //
 //  quantise_mx_kernel      bf16 activations -> (codes, scales) by the microscaling rule: per block of 32,
 //                          shared exponent floor(log2 max|x|) - emax(format), elements rounded to the
-//                          nearest even code with saturation.  One thread per block: 64 bytes in, 32 bytes
-//                          of codes and one scale byte out.  Every step is exact (powers of two) except
+//                          nearest even code with saturation.  Every step is exact (powers of two) except
 //                          the final rounding, which is the hardware's round-to-nearest-even conversion.
 //
 //  gemm_mx_tcgen05_kernel  tcgen05.mma.kind::mxf8f6f4.block_scale: the tensor core multiplies the 8-bit
 //                          elements and applies scale_A[row, k/32] * scale_B[col, k/32] per 32-wide
-//                          k-group itself; the scale bytes have to sit in tensor memory.  One CTA = one
-//                          128 x 128 output tile, six warps:
+//                          k-group itself; the scale bytes have to sit in tensor memory.  One persistent CTA
+//                          per SM walks the 128 x BN output tiles, fourteen warps:
 //    warp 0 (1 lane)   TMA: 128 x 128-byte operand tiles (128 k per stage, 128-byte swizzle)
-//    warp 1 (1 lane)   MMA issue: four instructions (K = 32 each) per stage, scale slot selected by
-//                      the instruction descriptor's scale-id fields
-//    warps 2..5        scale feed, then the epilogue.  For every stage each warp copies the 4 scale
-//                      bytes (one 32-bit word = 4 k-groups) of its rows into tensor memory in the layout
-//                      the instruction expects: the 128 rows' words live in 32 lanes x 4 columns (lane l,
-//                      column c = row 32c + l), replicated in all four lane quarters -- so each of the four
-//                      warps writes the same 32 x 4 words into its own quarter with one tcgen05.st (and the
-//                      same again for the 128 columns of W).  After the last stage the same warps read the
-//                      fp32 accumulator (thread = row), add the bias, round to bf16 and store.
+//    warp 1            MMA issue: per stage two or three tcgen05.cp of the stage's scale words from shared into
+//                      tensor memory, then four instructions (K = 32 each), scale byte selected by the
+//                      instruction descriptor's scale-id fields
+//    warps 2..5        scale feed: the 32-bit scale words (4 k-groups each) of the stage's rows into shared memory
+//                      in the order the instruction expects: row l of 32 holds rows l, 32 + l, 64 + l and 96 + l of
+//                      the operand, 16 bytes; tcgen05.cp.32x128b.warpx4 replicates it in all four lane quarters
+//    warps 6..13       epilogue, one lane quarter x one half of the columns each
+//  BN = 192 where N allows (a tile moves 40 KB of operands per 384 tensor-core cycles), else 128 (32 KB per 256).
+//  Accumulators are double-buffered in tensor memory, so that one tile's epilogue overlaps the next main loop.
 //  One mbarrier per stage collects the TMA bytes AND the four scale warps' arrivals, and one commit per
-//  stage frees operands and scale slot together: the issuing thread pays for every barrier round.
-//  TMEM: 128 accumulator columns + 3 scale slots of 8 columns = 152 -> 256 allocated, two CTAs per SM,
-//  which is what overlaps one tile's epilogue with another's main loop.
+//  stage frees operands and scale words together: the issuing thread pays for every barrier round.
+//  What bounds it: the rate at which one SM's operands arrive from L2 (about 80 bytes a clock).  A scale word is
+//  loaded once per tile, four k-blocks per 16-byte load where the row pitch allows; with each of four warps loading
+//  all of a stage's words one by one and writing its own quarter (12 loads of 32 rows each per warp and stage) those
+//  loads took longer than the operands.
 // All mbarrier waits are bounded; on expiry the CTA sets the status bit and leaves.
 #pragma once
 #include <cuda.h>
@@ -38,14 +38,24 @@ namespace tcmx {
 
 using namespace rlx::tc;
 
-constexpr int kThreads = 192;
-constexpr int kTileM = 128, kTileN = 128;
+constexpr int kThreads = 448;           // TMA, MMA, 4 scale warps, 8 epilogue warps
+constexpr int kTileM = 128;
 constexpr int kBlockK = 128;            // 8-bit elements per stage row = 128 bytes = one swizzle row
-constexpr int kStages = 3;              // 3 x 32 KB: two CTAs fit an SM
-constexpr int kTmemCols = 256;
-constexpr int kColSf = kTileN;          // one scale slot (8 columns) per stage, behind the accumulator
 constexpr int kOperandBytes = kTileM * kBlockK;
-constexpr int kSmemBytes = kStages * 2 * kOperandBytes + 256 + 1024;
+constexpr int kSfGroup = 512;           // scale words of 128 operand rows of one stage
+
+template <int BN> struct MxCfg {
+    static_assert(BN == 128 || BN == 192, "");
+    static constexpr int STAGES = BN == 192 ? 5 : 6;
+    static constexpr int STAGE_BYTES = kOperandBytes + BN * kBlockK;
+    static constexpr int W_GROUPS = (BN + 127) / 128;           // 128-row groups of W's scale words; the last may be half used
+    static constexpr int SF_BYTES = (1 + W_GROUPS) * kSfGroup;
+    static constexpr int SF_COLS = 4 * (1 + W_GROUPS);
+    static constexpr int ACC_COLS = 2 * BN;
+    static constexpr int STAGING = 8 * kStageBufBytes;          // one 2 KB chunk buffer per epilogue warp (TMA-store source)
+    static constexpr int SMEM_BYTES = STAGES * (STAGE_BYTES + SF_BYTES) + STAGING + 256 + 1024;
+    static_assert(ACC_COLS + STAGES * SF_COLS <= 512 && SMEM_BYTES <= 232448, "");
+};
 
 // element format ids of the instruction descriptor
 constexpr int kFmtE4M3 = 0, kFmtE5M2 = 1;
@@ -53,8 +63,9 @@ constexpr int kFmtE4M3 = 0, kFmtE5M2 = 1;
 // Instruction descriptor of kind::mxf8f6f4 with block scaling: [4,6) scale id of B, [7,10) A format,
 // [10,13) B format, [15] / [16] A / B major (0 = K-major), [17,23) N >> 3, [23] scale format (1 = E8M0),
 // [24,29) M >> 4, [29,31) scale id of A.  fp32 accumulation is implied.
+template <int BN>
 __device__ __forceinline__ uint32_t idesc_mx(int a_fmt, int b_fmt, int sf_id) {
-    return ((uint32_t)sf_id << 4) | ((uint32_t)a_fmt << 7) | ((uint32_t)b_fmt << 10) | ((uint32_t)(kTileN >> 3) << 17) |
+    return ((uint32_t)sf_id << 4) | ((uint32_t)a_fmt << 7) | ((uint32_t)b_fmt << 10) | ((uint32_t)(BN >> 3) << 17) |
            (1u << 23) | ((uint32_t)(kTileM >> 4) << 24) | ((uint32_t)sf_id << 29);
 }
 __device__ __forceinline__ void umma_mx(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
@@ -66,11 +77,11 @@ __device__ __forceinline__ void umma_mx(uint32_t tmem_d, uint64_t adesc, uint64_
         "tcgen05.mma.cta_group::1.kind::mxf8f6f4.block_scale.scale_vec::1X [%0], %1, %2, %3, [%4], [%5], p;\n"
         "}\n" ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(tmem_sfa), "r"(tmem_sfb), "r"(accumulate) : "memory");
 }
-__device__ __forceinline__ void tmem_st_32x8(uint32_t taddr, const uint32_t (&r)[8]) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
-                 ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
+// 32 rows of 16 bytes (8-row groups 128 bytes apart, no swizzle) into four tensor-memory columns of every lane quarter
+__device__ __forceinline__ void copy_scales(uint32_t tmem_dst, uint32_t smem_src) {
+    const uint64_t desc = (uint64_t)((smem_src & 0x3FFFFu) >> 4) | ((uint64_t)(128 >> 4) << 32) | (1ull << 46);
+    asm volatile("tcgen05.cp.cta_group::1.32x128b.warpx4 [%0], %1;" ::"r"(tmem_dst), "l"(desc) : "memory");
 }
-__device__ __forceinline__ void tmem_st_wait_all() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 struct MxParams {
     const uint8_t* sfa;     // [M, K/32] scale bytes of A
@@ -82,182 +93,31 @@ struct MxParams {
     int32_t* status;
 };
 
-__global__ void __launch_bounds__(kThreads, 2)
-gemm_mx_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_w, MxParams p) {
+template <int BN>
+__global__ void __launch_bounds__(kThreads, 1)
+gemm_mx_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_w,
+                       const __grid_constant__ CUtensorMap tmap_out, MxParams p) {
+    using C = MxCfg<BN>;
+    constexpr int ST = C::STAGES;
     extern __shared__ unsigned char smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     unsigned char* gbase = smem_raw + (base - raw);
-    const uint32_t bars = base + kStages * 2 * kOperandBytes;
-    const uint32_t full = bars, empty = full + 8 * kStages, acc_full = empty + 8 * kStages;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + kStages * 2 * kOperandBytes + 8 * (2 * kStages + 1));
+    const uint32_t staging = base + ST * C::STAGE_BYTES;
+    constexpr int kSfOff = ST * C::STAGE_BYTES + C::STAGING;
+    const uint32_t scales = base + kSfOff;
+    const uint32_t bars = scales + ST * C::SF_BYTES;
+    const uint32_t full = bars, empty = full + 8 * ST, tfull = empty + 8 * ST, tempty = tfull + 16;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + kSfOff + ST * C::SF_BYTES + 8 * (2 * ST + 4));
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n_tiles = p.N / kTileN;
-    const int m0 = (blockIdx.x / n_tiles) * kTileM, n0 = (blockIdx.x % n_tiles) * kTileN;
+    const int n_tiles = p.N / BN, m_tiles = (p.M + kTileM - 1) / kTileM, num_tiles = n_tiles * m_tiles;
     const int nkb = p.K / kBlockK;
-    const int sf_ld = p.K / 32;   // scale bytes per row
 
     if (threadIdx.x == 0) {
         // full: the TMA lane's expect_tx arrival + one arrival per scale warp
-        for (int i = 0; i < kStages; ++i) { mbar_init(full + 8 * i, 5); mbar_init(empty + 8 * i, 1); }
-        mbar_init(acc_full, 1);
-        *abort_flag = 0;
-        fence_barrier_init();
-        prefetch_tmap(&tmap_a);
-        prefetch_tmap(&tmap_w);
-    }
-    if (warp == 1) {
-        tmem_alloc<1>(smem_u32(tmem_slot), kTmemCols);
-        tmem_relinquish<1>();
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
-
-    if (warp == 0) {
-        if (lane == 0) {
-            for (int kb = 0; kb < nkb; ++kb) {
-                const int st = kb % kStages, use = kb / kStages;
-                if (use >= 1 && !mbar_wait(empty + 8 * st, (use - 1) & 1, abort_flag)) break;
-                const uint32_t dst = base + st * 2 * kOperandBytes;
-                mbar_expect_tx(full + 8 * st, 2 * kOperandBytes);
-                tma_load_2d(dst, &tmap_a, kb * kBlockK, m0, full + 8 * st);
-                tma_load_2d(dst + kOperandBytes, &tmap_w, kb * kBlockK, n0, full + 8 * st);
-            }
-        }
-    } else if (warp == 1) {
-        // warp-uniform loop, one elected lane issues (cheaper per instruction than a lone lane under a branch)
-        bool ok = true;
-        for (int kb = 0; kb < nkb && ok; ++kb) {
-            const int st = kb % kStages;
-            if (!(ok = mbar_wait_warp(full + 8 * st, (kb / kStages) & 1, abort_flag))) break;
-            tc_fence_after();
-            if (elect_one()) {
-                const uint64_t adesc = make_smem_desc(base + st * 2 * kOperandBytes);
-                const uint64_t bdesc = make_smem_desc(base + st * 2 * kOperandBytes + kOperandBytes);
-                const uint32_t sfa = tmem + kColSf + st * 8, sfb = sfa + 4;
-#pragma unroll
-                for (int k = 0; k < kBlockK / 32; ++k)   // 32 bytes of k per instruction: descriptor start + 2
-                    umma_mx(tmem, adesc + 2 * k, bdesc + 2 * k, idesc_mx(p.a_fmt, p.w_fmt, k), sfa, sfb, (kb | k) != 0 ? 1u : 0u);
-                umma_commit<1>(empty + 8 * st);
-                if (kb == nkb - 1) umma_commit<1>(acc_full);
-            }
-            __syncwarp();
-        }
-    } else {
-        // ------------------------------------------------------------ scale feed, then epilogue
-        const int quad = warp & 3;
-        const uint32_t lane_addr = tmem + ((uint32_t)(quad * 32) << 16);
-        bool ok = true;
-        for (int kb = 0; kb < nkb && ok; ++kb) {
-            const int slot = kb % kStages, use = kb / kStages;
-            uint32_t w[8];
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const int ar = m0 + 32 * c + lane, wr = n0 + 32 * c + lane;
-                // rows past M are zero-filled operand rows: any finite scale will do
-                w[c] = ar < p.M ? __ldg(reinterpret_cast<const uint32_t*>(p.sfa + (size_t)ar * sf_ld) + kb) : 0x7F7F7F7Fu;
-                w[4 + c] = __ldg(reinterpret_cast<const uint32_t*>(p.sfw + (size_t)wr * sf_ld) + kb);
-            }
-            if (use >= 1 && !(ok = mbar_wait(empty + 8 * slot, (use - 1) & 1, abort_flag))) break;
-            tc_fence_after();
-            tmem_st_32x8(lane_addr + kColSf + slot * 8, w);
-            tmem_st_wait_all();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(full + 8 * slot);
-        }
-        if (ok && (ok = mbar_wait(acc_full, 0, abort_flag))) {
-            tc_fence_after();
-            const int row = m0 + quad * 32 + lane;
-            __nv_bfloat16* orow = p.out + (size_t)row * p.N + n0;
-#pragma unroll 1
-            for (int c0 = 0; c0 < kTileN; c0 += 32) {
-                uint32_t r[32];
-                tmem_ld_32x32(lane_addr + c0, r);
-                tmem_ld_wait();
-                if (row < p.M) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        float v[8];
-#pragma unroll
-                        for (int j = 0; j < 8; ++j)
-                            v[j] = __uint_as_float(r[8 * i + j]) + (p.bias ? __ldg(p.bias + n0 + c0 + 8 * i + j) : 0.f);
-                        uint4 q;
-                        q.x = pack_bf16(v[0], v[1]); q.y = pack_bf16(v[2], v[3]);
-                        q.z = pack_bf16(v[4], v[5]); q.w = pack_bf16(v[6], v[7]);
-                        *(reinterpret_cast<uint4*>(orow + c0) + i) = q;
-                    }
-                }
-            }
-        }
-    }
-    // ---------------------------------------------------------------- teardown
-    if (*abort_flag) {
-        if (threadIdx.x == 0 && p.status) atomicOr(p.status, RLX_DEVSTAT_TIMEOUT_BIT);
-        const uint64_t t0 = global_timer_ns();
-        while (global_timer_ns() - t0 < 200000ull) __nanosleep(1000);
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 1) {
-        __syncwarp();
-        tc_fence_after();
-        tmem_dealloc<1>(tmem, kTmemCols);
-    }
-}
-
-// ---------------------------------------------------------------------------- persistent 128 x 192 tiles
-// The same product for N % 192 == 0 (the encoder's widths 384, 1152, 1536 and multiples): one persistent
-// CTA per SM walks the tile list, the fp32 accumulators are double-buffered in tensor memory so that the
-// epilogue of tile i overlaps the main loop of tile i + 1, the scale feed has its own four warps and the
-// epilogue eight (one lane quarter x one 96-column half each).  A 128 x 192 tile moves 40 KB of operands
-// per 384 tensor-core cycles (the 128 x 128 tile: 32 KB per 256), which is what the SM's fill rate can
-// sustain.  TMEM: 2 x 192 accumulator columns + 4 scale slots of 12 columns (A's 4, W's 8) = 432 -> 512.
-namespace wide {
-constexpr int kTileNW = 192;
-constexpr int kStagesW = 4;
-constexpr int kThreadsW = 448;   // TMA, MMA, 4 scale warps, 8 epilogue warps
-constexpr int kAccCols = 2 * kTileNW;
-constexpr int kSfCols = 12;
-constexpr int kWBytes = kTileNW * kBlockK;
-constexpr int kStageBytesW = kOperandBytes + kWBytes;
-constexpr int kEpiWarpsW = 8;
-constexpr int kStagingW = kEpiWarpsW * kStageBufBytes;   // one 2 KB chunk buffer per epilogue warp (TMA-store source)
-constexpr int kSmemBytesW = kStagesW * kStageBytesW + kStagingW + 256 + 1024;
-
-__device__ __forceinline__ uint32_t idesc_mx_w(int a_fmt, int b_fmt, int sf_id) {
-    return ((uint32_t)sf_id << 4) | ((uint32_t)a_fmt << 7) | ((uint32_t)b_fmt << 10) | ((uint32_t)(kTileNW >> 3) << 17) |
-           (1u << 23) | ((uint32_t)(kTileM >> 4) << 24) | ((uint32_t)sf_id << 29);
-}
-__device__ __forceinline__ void tmem_st_32x4(uint32_t taddr, const uint32_t (&r)[4]) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};"
-                 ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
-}
-
-__global__ void __launch_bounds__(kThreadsW, 1)
-gemm_mx192_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_w,
-                          const __grid_constant__ CUtensorMap tmap_out, MxParams p) {
-    extern __shared__ unsigned char smem_raw[];
-    const uint32_t raw = smem_u32(smem_raw);
-    const uint32_t base = (raw + 1023u) & ~1023u;
-    unsigned char* gbase = smem_raw + (base - raw);
-    const uint32_t staging = base + kStagesW * kStageBytesW;
-    const uint32_t bars = staging + kStagingW;
-    const uint32_t full = bars, empty = full + 8 * kStagesW, tfull = empty + 8 * kStagesW, tempty = tfull + 16;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + kStagesW * kStageBytesW + kStagingW + 8 * (2 * kStagesW + 4));
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n_tiles = p.N / kTileNW, m_tiles = (p.M + kTileM - 1) / kTileM, num_tiles = n_tiles * m_tiles;
-    const int nkb = p.K / kBlockK;
-    const int sf_ld = p.K / 32;
-
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < kStagesW; ++i) { mbar_init(full + 8 * i, 5); mbar_init(empty + 8 * i, 1); }
+        for (int i = 0; i < ST; ++i) { mbar_init(full + 8 * i, 5); mbar_init(empty + 8 * i, 1); }
         for (int i = 0; i < 2; ++i) { mbar_init(tfull + 8 * i, 1); mbar_init(tempty + 8 * i, 8); }
         *abort_flag = 0;
         fence_barrier_init();
@@ -276,94 +136,107 @@ gemm_mx192_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gr
 
     if (warp == 0) {
         if (lane == 0) {
-            uint32_t it = 0;   // stages issued so far
+            uint32_t st = 0, ph = 1;   // a fresh barrier passes the wait for the phase before its first
             bool ok = true;
             for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
-                const int m0 = (tile / n_tiles) * kTileM, n0 = (tile % n_tiles) * kTileNW;
-                for (int kb = 0; kb < nkb; ++kb, ++it) {
-                    const uint32_t st = it % kStagesW, use = it / kStagesW;
-                    if (use >= 1 && !(ok = mbar_wait(empty + 8 * st, (use - 1) & 1, abort_flag))) break;
-                    const uint32_t dst = base + st * kStageBytesW;
-                    mbar_expect_tx(full + 8 * st, kStageBytesW);
+                const int m0 = (tile / n_tiles) * kTileM, n0 = (tile % n_tiles) * BN;
+                for (int kb = 0; kb < nkb; ++kb) {
+                    if (!(ok = mbar_wait(empty + 8 * st, ph, abort_flag))) break;
+                    const uint32_t dst = base + st * C::STAGE_BYTES;
+                    mbar_expect_tx(full + 8 * st, C::STAGE_BYTES);
                     tma_load_2d(dst, &tmap_a, kb * kBlockK, m0, full + 8 * st);
                     tma_load_2d(dst + kOperandBytes, &tmap_w, kb * kBlockK, n0, full + 8 * st);
+                    if (++st == ST) { st = 0; ph ^= 1; }
                 }
             }
         }
     } else if (warp == 1) {
-        uint32_t it = 0, tcount = 0;
+        uint32_t st = 0, ph = 0, tcount = 0;
         bool ok = true;
         for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++tcount) {
             const uint32_t as = tcount & 1, ause = tcount >> 1;
             if (ause >= 1 && !(ok = mbar_wait_warp(tempty + 8 * as, (ause - 1) & 1, abort_flag))) break;
-            for (int kb = 0; kb < nkb; ++kb, ++it) {
-                const uint32_t st = it % kStagesW;
-                if (!(ok = mbar_wait_warp(full + 8 * st, (it / kStagesW) & 1, abort_flag))) break;
+            for (int kb = 0; kb < nkb; ++kb) {
+                if (!(ok = mbar_wait_warp(full + 8 * st, ph, abort_flag))) break;
                 tc_fence_after();
                 if (elect_one()) {
-                    const uint64_t adesc = make_smem_desc(base + st * kStageBytesW);
-                    const uint64_t bdesc = make_smem_desc(base + st * kStageBytesW + kOperandBytes);
-                    const uint32_t sfa = tmem + kAccCols + st * kSfCols, sfb = sfa + 4;
+                    const uint64_t adesc = make_smem_desc(base + st * C::STAGE_BYTES);
+                    const uint64_t bdesc = make_smem_desc(base + st * C::STAGE_BYTES + kOperandBytes);
+                    const uint32_t sfa = tmem + C::ACC_COLS + st * C::SF_COLS, sfb = sfa + 4;
 #pragma unroll
-                    for (int k = 0; k < kBlockK / 32; ++k)
-                        umma_mx(tmem + as * kTileNW, adesc + 2 * k, bdesc + 2 * k, idesc_mx_w(p.a_fmt, p.w_fmt, k), sfa, sfb,
+                    for (int g = 0; g <= C::W_GROUPS; ++g) copy_scales(sfa + 4 * g, scales + st * C::SF_BYTES + g * kSfGroup);
+#pragma unroll
+                    for (int k = 0; k < kBlockK / 32; ++k)   // 32 bytes of k per instruction: descriptor start + 2
+                        umma_mx(tmem + as * BN, adesc + 2 * k, bdesc + 2 * k, idesc_mx<BN>(p.a_fmt, p.w_fmt, k), sfa, sfb,
                                 (kb | k) != 0 ? 1u : 0u);
                     umma_commit<1>(empty + 8 * st);
                     if (kb == nkb - 1) umma_commit<1>(tfull + 8 * as);
                 }
                 __syncwarp();
+                if (++st == ST) { st = 0; ph ^= 1; }
             }
         }
     } else if (warp < 6) {
-        // ------------------------------------------------------------ scale feed (one warp per lane quarter)
-        // The scale words of a stage are requested kAhead stages before they are written to tensor memory,
-        // so that their global-memory latency stays off the pipeline's critical path.
-        constexpr int kAhead = 3;
-        const int quad = warp & 3;
-        const uint32_t lane_addr = tmem + ((uint32_t)(quad * 32) << 16);
-        const int my_tiles = blockIdx.x < num_tiles ? (num_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
-        const long long total = (long long)my_tiles * nkb;
-        uint32_t wa[kAhead][4], wb[kAhead][8];
-        auto fetch = [&](long long i, uint32_t (&a4)[4], uint32_t (&b8)[8]) {
-            const int tile = blockIdx.x + (int)(i / nkb) * gridDim.x, kb = (int)(i % nkb);
-            const int m0 = (tile / n_tiles) * kTileM, n0 = (tile % n_tiles) * kTileNW;
+        // ------------------------------------------------------------ scale feed: 32 rows of every 128 per warp
+        // Four k-blocks of a row at a time, requested while the four before them are handed over, across tiles too.
+        const int q = warp - 2;
+        const int ld = p.K / 128;                      // scale words per row
+        const bool vec = (ld & 3) == 0;                // 16-byte loads: rows start on 16 bytes
+        const uint32_t* sfa = reinterpret_cast<const uint32_t*>(p.sfa);
+        const uint32_t* sfw = reinterpret_cast<const uint32_t*>(p.sfw);
+        auto load4 = [&](const uint32_t* row, int kb0, uint32_t (&r)[4]) {
+            if (vec) {
+                const uint4 v = __ldg(reinterpret_cast<const uint4*>(row + kb0));
+                r[0] = v.x; r[1] = v.y; r[2] = v.z; r[3] = v.w;
+            } else {
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const int ar = m0 + 32 * c + lane;
-                // rows past M are zero-filled operand rows: any finite scale will do
-                a4[c] = ar < p.M ? __ldg(reinterpret_cast<const uint32_t*>(p.sfa + (size_t)ar * sf_ld) + kb) : 0x7F7F7F7Fu;
-            }
-#pragma unroll
-            for (int c = 0; c < 8; ++c) {   // two 128-row groups of W's rows; the second is half used
-                const int wr = 32 * c + lane;
-                b8[c] = wr < kTileNW ? __ldg(reinterpret_cast<const uint32_t*>(p.sfw + (size_t)(n0 + wr) * sf_ld) + kb) : 0x7F7F7F7Fu;
+                for (int u = 0; u < 4; ++u)
+                    if (kb0 + u < nkb) r[u] = __ldg(row + kb0 + u);
             }
         };
+        auto fetch = [&](int tile, int kb0, uint32_t (&r)[1 + C::W_GROUPS][4]) {
+            const int ar = (tile / n_tiles) * kTileM + 32 * q + lane, n0 = (tile % n_tiles) * BN;
+            // rows past M are zero-filled operand rows: any finite scale will do
+            if (ar < p.M) load4(sfa + (size_t)ar * ld, kb0, r[0]);
+            else r[0][0] = r[0][1] = r[0][2] = r[0][3] = 0x7F7F7F7Fu;
 #pragma unroll
-        for (int i = 0; i < kAhead; ++i)
-            if (i < total) fetch(i, wa[i], wb[i]);
+            for (int g = 0; g < C::W_GROUPS; ++g)
+                if (128 * g + 32 * q < BN) load4(sfw + (size_t)(n0 + 128 * g + 32 * q + lane) * ld, kb0, r[1 + g]);
+        };
+        uint32_t cur[1 + C::W_GROUPS][4] = {}, nxt[1 + C::W_GROUPS][4] = {};
+        const uint32_t slot_addr = scales + lane * 16 + q * 4;
+        uint32_t st = 0, ph = 1;
+        int tile = blockIdx.x, kb0 = 0;
         bool ok = true;
-        for (long long i0 = 0; i0 < total && ok; i0 += kAhead) {
+        if (tile < num_tiles) fetch(tile, 0, cur);
+        while (tile < num_tiles && ok) {
+            int ntile = tile, nkb0 = kb0 + 4;
+            if (nkb0 >= nkb) { ntile += gridDim.x; nkb0 = 0; }
+            if (ntile < num_tiles) fetch(ntile, nkb0, nxt);
 #pragma unroll
-            for (int u = 0; u < kAhead; ++u) {
-                const long long i = i0 + u;
-                if (i >= total) break;
-                const uint32_t slot = (uint32_t)(i % kStagesW), use = (uint32_t)(i / kStagesW);
-                if (use >= 1 && !(ok = mbar_wait(empty + 8 * slot, (use - 1) & 1, abort_flag))) break;
-                tc_fence_after();
-                tmem_st_32x4(lane_addr + kAccCols + slot * kSfCols, wa[u]);
-                tmem_st_32x8(lane_addr + kAccCols + slot * kSfCols + 4, wb[u]);
-                tmem_st_wait_all();
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(full + 8 * slot);
-                if (i + kAhead < total) fetch(i + kAhead, wa[u], wb[u]);
+            for (int u = 0; u < 4; ++u) {
+                if (kb0 + u < nkb && ok) {
+                    if (!(ok = mbar_wait(empty + 8 * st, ph, abort_flag))) break;
+#pragma unroll
+                    for (int g = 0; g <= C::W_GROUPS; ++g)
+                        asm volatile("st.shared.b32 [%0], %1;" ::"r"(slot_addr + st * C::SF_BYTES + g * kSfGroup), "r"(cur[g][u]) : "memory");
+                    fence_proxy_async();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(full + 8 * st);
+                    if (++st == ST) { st = 0; ph ^= 1; }
+                }
             }
+#pragma unroll
+            for (int g = 0; g <= C::W_GROUPS; ++g)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) cur[g][u] = nxt[g][u];
+            tile = ntile; kb0 = nkb0;
         }
     } else {
-        // ------------------------------------------------------------ epilogue: lane quarter x 96-column half
-        // the bf16 GEMM's epilogue tile: all three chunks to registers, accumulator handed back, bias, one
+        // ------------------------------------------------------------ epilogue: lane quarter x half of the columns
+        // the bf16 GEMM's epilogue tile: all chunks to registers, accumulator handed back, bias, one
         // TMA store per 32 x 32 chunk out of the warp's swizzled staging buffer
+        constexpr int NC = BN / 64;
         const int quad = warp & 3, half = (warp - 6) >> 2, ew = warp - 6;
         const uint32_t stg = staging + ew * kStageBufBytes;
         Params gp = {};
@@ -371,16 +244,17 @@ gemm_mx192_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gr
         uint32_t tcount = 0;
         bool ok = true;
         for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++tcount) {
-            const int m_row0 = (tile / n_tiles) * kTileM + quad * 32, n0 = (tile % n_tiles) * kTileNW + half * 96;
+            const int m_row0 = (tile / n_tiles) * kTileM + quad * 32, n0 = (tile % n_tiles) * BN + half * (BN / 2);
             const uint32_t as = tcount & 1;
             if (!(ok = mbar_wait(tfull + 8 * as, (tcount >> 1) & 1, abort_flag))) break;
             tc_fence_after();
-            EpilogueTile<0, 3> et;
-            et.template drain<1>(gp, &tmap_out, p.M, m_row0, n0, tmem + ((uint32_t)(quad * 32) << 16) + as * kTileNW + half * 96,
+            EpilogueTile<0, NC> et;
+            et.template drain<1>(gp, &tmap_out, p.M, m_row0, n0, tmem + ((uint32_t)(quad * 32) << 16) + as * BN + half * (BN / 2),
                                  stg, lane, tempty + 8 * as, 0u);
         }
-        EpilogueTile<0, 3>::finish(lane);
+        EpilogueTile<0, NC>::finish(lane);
     }
+    // ---------------------------------------------------------------- teardown
     if (*abort_flag) {
         if (threadIdx.x == 0 && p.status) atomicOr(p.status, RLX_DEVSTAT_TIMEOUT_BIT);
         const uint64_t t0 = global_timer_ns();
@@ -394,7 +268,6 @@ gemm_mx192_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gr
         tmem_dealloc<1>(tmem, 512);
     }
 }
-}  // namespace wide
 
 // ---------------------------------------------------------------------------- activation quantiser
 template <bool E5M2>
@@ -406,33 +279,56 @@ __device__ __forceinline__ uint16_t cvt_fp8x2(float lo, float hi) {
 }
 
 constexpr int kQuantThreads = 256;
+constexpr int kQuantIters = 4;                                       // 16-byte loads in flight per lane
+constexpr int kQuantWarpBlocks = 8 * kQuantIters;                    // 32-element blocks per warp
+constexpr int kQuantCtaBlocks = kQuantThreads / 32 * kQuantWarpBlocks;
 
-// x bf16 [M, K] -> codes [M, K] bytes, scales [M, K/32] bytes; one thread per 32-element block.
+// x bf16 [M, K] -> codes [M, K] bytes, scales [M, K/32] bytes.  Bound by DRAM: 2 bytes in and 1 + 1/32 out per element.
+// Four lanes share a block of 32, so that a warp's loads (16 bytes a lane) and its stores (8 bytes) are contiguous, and
+// the shared exponent comes from the exponent field of the packed maximum; the warp's 32 scale bytes leave as one store.
+// (One thread per block of 64 bytes, with ilogbf and scalbnf per element, took 46 us for 36736 x 1536.)
 template <bool E5M2>
 __global__ void __launch_bounds__(kQuantThreads)
 quantise_mx_kernel(const __nv_bfloat16* __restrict__ x, uint8_t* __restrict__ codes, uint8_t* __restrict__ scales,
                    long long blocks) {
-    const long long b = (long long)blockIdx.x * kQuantThreads + threadIdx.x;
-    if (b >= blocks) return;
     constexpr int kEmax = E5M2 ? 15 : 8;
-    const uint4* src = reinterpret_cast<const uint4*>(x + b * 32);
-    uint4 in[4];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long long b0 = (long long)blockIdx.x * kQuantCtaBlocks + warp * kQuantWarpBlocks;
+    uint4 in[kQuantIters];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) in[i] = __ldg(src + i);
-    const uint32_t* w = reinterpret_cast<const uint32_t*>(in);
-    float amax = 0.f;
+    for (int i = 0; i < kQuantIters; ++i) {
+        const long long b = b0 + 8 * i + (lane >> 2);
+        in[i] = b < blocks ? __ldcs(reinterpret_cast<const uint4*>(x + b * 32) + (lane & 3)) : make_uint4(0, 0, 0, 0);
+    }
+    uint32_t mine = 0;
 #pragma unroll
-    for (int i = 0; i < 16; ++i) amax = fmaxf(amax, fmaxf(fabsf(bf16lo(w[i])), fabsf(bf16hi(w[i]))));
-    int s = amax > 0.f ? ilogbf(amax) - kEmax : 0;
-    s = max(-127, min(127, s));
-    uint4 out[2];
-    uint16_t* o = reinterpret_cast<uint16_t*>(out);
+    for (int i = 0; i < kQuantIters; ++i) {
+        const uint32_t* w = reinterpret_cast<const uint32_t*>(&in[i]);
+        // packed maximum of the magnitudes; a NaN loses against any number, as in fmaxf
+        __nv_bfloat162 m2 = __floats2bfloat162_rn(0.f, 0.f);
 #pragma unroll
-    for (int i = 0; i < 16; ++i) o[i] = cvt_fp8x2<E5M2>(scalbnf(bf16lo(w[i]), -s), scalbnf(bf16hi(w[i]), -s));
-    uint4* dst = reinterpret_cast<uint4*>(codes + b * 32);
-    dst[0] = out[0];
-    dst[1] = out[1];
-    scales[b] = (uint8_t)(s + 127);
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t a = w[j] & 0x7FFF7FFFu;
+            m2 = __hmax2(m2, *reinterpret_cast<const __nv_bfloat162*>(&a));
+        }
+        uint32_t m = *reinterpret_cast<uint32_t*>(&m2);
+        m = max(m & 0xFFFFu, m >> 16);                 // non-negative numbers: their bits order as they do
+        m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
+        m = max(m, __shfl_xor_sync(0xffffffffu, m, 2));
+        const int e = (int)(m >> 7);                   // exponent field; zero for a subnormal maximum
+        int s = m == 0 ? 0 : e == 255 ? 127 : max(e - 127 - kEmax, -127);   // infinity takes the largest scale
+        // 2^-s; 2^-127 is subnormal
+        const float f = s == 127 ? __uint_as_float(0x00400000u) : __uint_as_float((uint32_t)(127 - s) << 23);
+        uint2 o;
+        o.x = cvt_fp8x2<E5M2>(bf16lo(w[0]) * f, bf16hi(w[0]) * f) | (uint32_t)cvt_fp8x2<E5M2>(bf16lo(w[1]) * f, bf16hi(w[1]) * f) << 16;
+        o.y = cvt_fp8x2<E5M2>(bf16lo(w[2]) * f, bf16hi(w[2]) * f) | (uint32_t)cvt_fp8x2<E5M2>(bf16lo(w[3]) * f, bf16hi(w[3]) * f) << 16;
+        const long long b = b0 + 8 * i + (lane >> 2);
+        if (b < blocks) *(reinterpret_cast<uint2*>(codes + b * 32) + (lane & 3)) = o;
+        // lane l keeps the byte of block 8 (l & 3) + (l >> 2): its own four-lane group's, of iteration l & 3
+        if ((lane & 3) == i) mine = (uint32_t)(s + 127);
+    }
+    const long long b = b0 + 8 * (lane & 3) + (lane >> 2);
+    if (b < blocks) scales[b] = (uint8_t)mine;
 }
 
 }  // namespace tcmx

@@ -247,10 +247,10 @@ cudaError_t init_kernels_for_current_device() {
             if ((e = cudaFuncSetAttribute(ffn_kernels[i], cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           i < 3 ? rlx::tcff::Cfg<384>::SMEM_BYTES : rlx::tcff::Cfg<256>::SMEM_BYTES)) != cudaSuccess) return e;
     }
-    if ((e = cudaFuncSetAttribute(rlx::tcmx::gemm_mx_tcgen05_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  rlx::tcmx::kSmemBytes)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(rlx::tcmx::wide::gemm_mx192_tcgen05_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  rlx::tcmx::wide::kSmemBytesW)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(rlx::tcmx::gemm_mx_tcgen05_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  rlx::tcmx::MxCfg<128>::SMEM_BYTES)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(rlx::tcmx::gemm_mx_tcgen05_kernel<192>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  rlx::tcmx::MxCfg<192>::SMEM_BYTES)) != cudaSuccess) return e;
 #define RLX_ATT_FWD_ATTR(D, PAIR)                                                                              \
     if ((e = cudaFuncSetAttribute(rlx::tcat::attention_fwd_kernel<D, PAIR, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
                                   rlx::tcat::Cfg<D, PAIR>::SMEM_BYTES)) != cudaSuccess ||                       \
@@ -1915,7 +1915,7 @@ rlx_status_t rlx_quantise_mx(const void* x_bf16, int32_t M, int32_t K, int32_t f
     const int fmt = mx_element_format(format);
     if (fmt < 0 || K % 32 != 0) return RLX_ERR_UNSUPPORTED;
     const long long blocks = (long long)M * (K / 32);
-    const unsigned grid = (unsigned)((blocks + rlx::tcmx::kQuantThreads - 1) / rlx::tcmx::kQuantThreads);
+    const unsigned grid = (unsigned)((blocks + rlx::tcmx::kQuantCtaBlocks - 1) / rlx::tcmx::kQuantCtaBlocks);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (fmt == rlx::tcmx::kFmtE5M2)
         rlx::tcmx::quantise_mx_kernel<true><<<grid, rlx::tcmx::kQuantThreads, 0, st>>>((const bf16*)x_bf16, (uint8_t*)codes, (uint8_t*)scales, blocks);
@@ -1933,30 +1933,25 @@ rlx_status_t rlx_mx_matmul_bf16(const void* a_codes, const void* a_scales, int32
         (bias && !aligned16(bias)))
         return RLX_ERR_INVALID_ARG;
     const int af = mx_element_format(a_format), wf = mx_element_format(w_format);
-    if (af < 0 || wf < 0 || K % rlx::tcmx::kBlockK != 0 || (N % rlx::tcmx::kTileN != 0 && N % rlx::tcmx::wide::kTileNW != 0))
-        return RLX_ERR_UNSUPPORTED;
+    if (af < 0 || wf < 0 || K % rlx::tcmx::kBlockK != 0 || (N % 128 != 0 && N % 192 != 0)) return RLX_ERR_UNSUPPORTED;
     RLX_CUDA_TRY(init_kernels_for_current_device());
-    const bool wide_tiles = N % rlx::tcmx::wide::kTileNW == 0;   // persistent 128 x 192 tiles when N allows
-    CUtensorMap ta, tw;
+    const int bn = N % 192 == 0 ? 192 : 128;   // the wider tile moves fewer bytes per product
+    const long long tiles = (M + rlx::tcmx::kTileM - 1ll) / rlx::tcmx::kTileM * (N / bn);
+    if (tiles > 0x7fffffffLL) return RLX_ERR_UNSUPPORTED;
+    CUtensorMap ta, tw, to;   // output chunks: 32 x 32 bf16 boxes with the 64-byte swizzle of the staging buffers
     if (!make_tmap_u8(&ta, a_codes, (uint64_t)M, (uint64_t)K, rlx::tcmx::kTileM) ||
-        !make_tmap_u8(&tw, w_codes, (uint64_t)N, (uint64_t)K, wide_tiles ? rlx::tcmx::wide::kTileNW : rlx::tcmx::kTileN))
+        !make_tmap_u8(&tw, w_codes, (uint64_t)N, (uint64_t)K, bn) ||
+        !make_tmap(&to, out, (uint64_t)M, (uint64_t)N, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B))
         return RLX_ERR_CUDA;
     rlx::tcmx::MxParams p;
     p.sfa = (const uint8_t*)a_scales; p.sfw = (const uint8_t*)w_scales; p.bias = bias; p.out = (bf16*)out;
     p.M = M; p.N = N; p.K = K; p.a_fmt = af; p.w_fmt = wf; p.status = status;
-    const long long m_tiles = (M + rlx::tcmx::kTileM - 1) / rlx::tcmx::kTileM;
-    const long long tiles = m_tiles * (wide_tiles ? N / rlx::tcmx::wide::kTileNW : N / rlx::tcmx::kTileN);
-    if (tiles > 0x7fffffffLL) return RLX_ERR_UNSUPPORTED;
-    if (wide_tiles) {
-        const unsigned grid = (unsigned)std::min<long long>(tiles, sm_count());
-        CUtensorMap to;   // output chunks: 32 x 32 bf16 boxes with the 64-byte swizzle of the staging buffers
-        if (!make_tmap(&to, out, (uint64_t)M, (uint64_t)N, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B)) return RLX_ERR_CUDA;
-        rlx::tcmx::wide::gemm_mx192_tcgen05_kernel<<<grid, rlx::tcmx::wide::kThreadsW, rlx::tcmx::wide::kSmemBytesW,
-                                                     static_cast<cudaStream_t>(stream)>>>(ta, tw, to, p);
-    } else {
-        rlx::tcmx::gemm_mx_tcgen05_kernel<<<(unsigned)tiles, rlx::tcmx::kThreads, rlx::tcmx::kSmemBytes,
-                                            static_cast<cudaStream_t>(stream)>>>(ta, tw, p);
-    }
+    const unsigned grid = (unsigned)std::min<long long>(tiles, sm_count());
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (bn == 192)
+        rlx::tcmx::gemm_mx_tcgen05_kernel<192><<<grid, rlx::tcmx::kThreads, rlx::tcmx::MxCfg<192>::SMEM_BYTES, st>>>(ta, tw, to, p);
+    else
+        rlx::tcmx::gemm_mx_tcgen05_kernel<128><<<grid, rlx::tcmx::kThreads, rlx::tcmx::MxCfg<128>::SMEM_BYTES, st>>>(ta, tw, to, p);
     RLX_CUDA_TRY(cudaGetLastError());
     return RLX_OK;
 }

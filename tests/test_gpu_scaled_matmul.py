@@ -203,6 +203,45 @@ def test_mx_matmul_places_every_scale_byte_and_operand_where_the_definition_says
     assert np.array_equal(got, round_to_bf16(exact).astype(np.float64))
 
 
+@pytest.mark.parametrize("blocks_m,blocks_k", [(1, 1), (1, 7), (33, 1), (255, 1), (1, 256), (257, 1), (19, 27)])
+def test_quantise_mx_at_the_edges_of_a_warp_and_a_cta(rlx, blocks_m, blocks_k):
+    """Block counts on both sides of a warp's 32 and a CTA's 256: bit for bit the definition.  Infinity takes the
+    largest scale and saturates, a NaN keeps its code and does not take part in the block's maximum."""
+    rng = np.random.default_rng(blocks_m * 1000 + blocks_k)
+    x = round_to_bf16((rng.standard_normal((blocks_m, 32 * blocks_k)) * 3).astype(np.float32))
+    word = _mx_word(rlx, "fp8_e4m3")
+    codes, scales = (t.cpu().numpy() for t in rlx.quantise_mx(bf16_dev(x), word))
+    want_codes, want_scales = osm.quantise_mx(x.astype(np.float64), osm.E4M3)
+    assert np.array_equal(scales, want_scales) and np.array_equal(codes, want_codes)
+    x[-1, -1] = np.nan
+    want_codes, want_scales = osm.quantise_mx(np.nan_to_num(x, nan=0.0).astype(np.float64), osm.E4M3)
+    codes, scales = (t.cpu().numpy() for t in rlx.quantise_mx(bf16_dev(x), word))
+    assert codes[-1, -1] & 0x7F == 0x7F
+    codes[-1, -1] = want_codes[-1, -1]
+    assert np.array_equal(scales, want_scales) and np.array_equal(codes, want_codes)
+    x[-1, -1], x[-1, -2] = -np.inf, 1.0
+    codes, scales = (t.cpu().numpy() for t in rlx.quantise_mx(bf16_dev(x), word))
+    assert scales[-1, -1] == 254 and codes[-1, -1] == 0xFE and codes[-1, -2] == 0
+
+
+@pytest.mark.parametrize("M,N,K", [(1, 128, 128), (127, 192, 256), (129, 128, 512), (130, 192, 640), (257, 576, 1536),
+                                   (128, 1024, 384), (19073, 192, 128), (19073, 128, 640), (9500, 384, 768)])
+def test_mx_matmul_at_the_edges_of_its_tiles_and_rings(rlx, M, N, K):
+    """One k-block, scale words in 16-byte loads and one by one, a remainder of k-blocks behind a group of four, rings
+    that wrap, more tiles than CTAs.  Every element is 1, so out = 32 sum_g 2^(a + w): exact in fp32, rounded once."""
+    rng = np.random.default_rng(M + N + K)
+    a = rng.integers(-3, 4, size=(M, K // 32))
+    w = rng.integers(-3, 4, size=(N, K // 32))
+    ones = [np.full((r, K), 0x38, np.uint8) for r in (M, N)]
+    word = _mx_word(rlx, "fp8_e4m3")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    got = to_np64(rlx.mx_matmul_bf16(_u8_dev(ones[0]), _u8_dev(a + 127), word, _u8_dev(ones[1]), _u8_dev(w + 127), word,
+                                     status=status))
+    assert int(status.item()) == 0
+    want = 32.0 * (np.exp2(a) @ np.exp2(w).T)
+    assert np.array_equal(got, round_to_bf16(want.astype(np.float32)).astype(np.float64))
+
+
 @pytest.mark.parametrize("a_name,w_name", [("fp8_e4m3", "fp8_e4m3"), ("fp8_e4m3", "fp8_e5m2"), ("fp8_e5m2", "fp8_e4m3")])
 @pytest.mark.parametrize("M,N,K", [(128, 128, 128), (517, 384, 384), (2000, 1536, 384), (1000, 384, 1536)])
 def test_quantise_then_mx_matmul_matches_oracle(rlx, a_name, w_name, M, N, K):
