@@ -21,8 +21,8 @@
 //    warps 6..13       epilogue, one lane quarter x one half of the columns each
 //  BN = 192 where N allows (a tile moves 40 KB of operands per 384 tensor-core cycles), else 128 (32 KB per 256).
 //  Accumulators are double-buffered in tensor memory, so that one tile's epilogue overlaps the next main loop.
-//  One mbarrier per stage collects the TMA bytes AND the four scale warps' arrivals, and one commit per
-//  stage frees operands and scale words together: the issuing thread pays for every barrier round.
+//  Scale words are handed over four k-blocks at a time, through two slots with barriers of their own; one commit per
+//  stage frees its operands.
 //  What bounds it: the rate at which one SM's operands arrive from L2 (about 80 bytes a clock).  A scale word is
 //  loaded once per tile, four k-blocks per 16-byte load where the row pitch allows; with each of four warps loading
 //  all of a stage's words one by one and writing its own quarter (12 loads of 32 rows each per warp and stage) those
@@ -42,19 +42,21 @@ constexpr int kThreads = 448;           // TMA, MMA, 4 scale warps, 8 epilogue w
 constexpr int kTileM = 128;
 constexpr int kBlockK = 128;            // 8-bit elements per stage row = 128 bytes = one swizzle row
 constexpr int kOperandBytes = kTileM * kBlockK;
-constexpr int kSfGroup = 512;           // scale words of 128 operand rows of one stage
+constexpr int kSfGroup = 512;           // scale words of 128 operand rows of one k-block
+constexpr int kSfAhead = 4;             // k-blocks whose scale words are handed over together
 
 template <int BN> struct MxCfg {
-    static_assert(BN == 128 || BN == 192, "");
-    static constexpr int STAGES = BN == 192 ? 5 : 6;
+    static_assert((BN == 128 || BN == 192) && kSfAhead == 4, "");
+    static constexpr int STAGES = kSfAhead;                     // stage = k-block modulo kSfAhead, from a tile's first on
     static constexpr int STAGE_BYTES = kOperandBytes + BN * kBlockK;
     static constexpr int W_GROUPS = (BN + 127) / 128;           // 128-row groups of W's scale words; the last may be half used
-    static constexpr int SF_BYTES = (1 + W_GROUPS) * kSfGroup;
+    static constexpr int SF_BYTES = (1 + W_GROUPS) * kSfGroup;  // one k-block's scale words
+    static constexpr int SF_SLOT_BYTES = kSfAhead * SF_BYTES;
     static constexpr int SF_COLS = 4 * (1 + W_GROUPS);
     static constexpr int ACC_COLS = 2 * BN;
     static constexpr int STAGING = 8 * kStageBufBytes;          // one 2 KB chunk buffer per epilogue warp (TMA-store source)
-    static constexpr int SMEM_BYTES = STAGES * (STAGE_BYTES + SF_BYTES) + STAGING + 256 + 1024;
-    static_assert(ACC_COLS + STAGES * SF_COLS <= 512 && SMEM_BYTES <= 232448, "");
+    static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 2 * SF_SLOT_BYTES + STAGING + 256 + 1024;
+    static_assert(ACC_COLS + 2 * kSfAhead * SF_COLS <= 512 && SMEM_BYTES <= 232448, "");
 };
 
 // element format ids of the instruction descriptor
@@ -68,19 +70,37 @@ __device__ __forceinline__ uint32_t idesc_mx(int a_fmt, int b_fmt, int sf_id) {
     return ((uint32_t)sf_id << 4) | ((uint32_t)a_fmt << 7) | ((uint32_t)b_fmt << 10) | ((uint32_t)(BN >> 3) << 17) |
            (1u << 23) | ((uint32_t)(kTileM >> 4) << 24) | ((uint32_t)sf_id << 29);
 }
-__device__ __forceinline__ void umma_mx(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+// The issuing instructions take the elected lane as a predicate instead of standing under a branch: in converged code
+// the compiler keeps their operands in uniform registers, under a branch it moves each one there again for every
+// instruction.
+__device__ __forceinline__ void umma_mx(uint32_t elected, uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                         uint32_t tmem_sfa, uint32_t tmem_sfb, uint32_t accumulate) {
     asm volatile(
         "{\n"
-        ".reg .pred p;\n"
+        ".reg .pred p, q;\n"
         "setp.ne.b32 p, %6, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::mxf8f6f4.block_scale.scale_vec::1X [%0], %1, %2, %3, [%4], [%5], p;\n"
-        "}\n" ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(tmem_sfa), "r"(tmem_sfb), "r"(accumulate) : "memory");
+        "setp.ne.b32 q, %7, 0;\n"
+        "@q tcgen05.mma.cta_group::1.kind::mxf8f6f4.block_scale.scale_vec::1X [%0], %1, %2, %3, [%4], [%5], p;\n"
+        "}\n" ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(tmem_sfa), "r"(tmem_sfb), "r"(accumulate), "r"(elected)
+        : "memory");
 }
 // 32 rows of 16 bytes (8-row groups 128 bytes apart, no swizzle) into four tensor-memory columns of every lane quarter
-__device__ __forceinline__ void copy_scales(uint32_t tmem_dst, uint32_t smem_src) {
+__device__ __forceinline__ void copy_scales(uint32_t elected, uint32_t tmem_dst, uint32_t smem_src) {
     const uint64_t desc = (uint64_t)((smem_src & 0x3FFFFu) >> 4) | ((uint64_t)(128 >> 4) << 32) | (1ull << 46);
-    asm volatile("tcgen05.cp.cta_group::1.32x128b.warpx4 [%0], %1;" ::"r"(tmem_dst), "l"(desc) : "memory");
+    asm volatile(
+        "{\n"
+        ".reg .pred q;\n"
+        "setp.ne.b32 q, %2, 0;\n"
+        "@q tcgen05.cp.cta_group::1.32x128b.warpx4 [%0], %1;\n"
+        "}\n" ::"r"(tmem_dst), "l"(desc), "r"(elected) : "memory");
+}
+__device__ __forceinline__ void commit_if(uint32_t elected, uint32_t bar) {
+    asm volatile(
+        "{\n"
+        ".reg .pred q;\n"
+        "setp.ne.b32 q, %1, 0;\n"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n"
+        "}\n" ::"r"(bar), "r"(elected) : "memory");
 }
 
 struct MxParams {
@@ -106,9 +126,10 @@ gemm_mx_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
     const uint32_t staging = base + ST * C::STAGE_BYTES;
     constexpr int kSfOff = ST * C::STAGE_BYTES + C::STAGING;
     const uint32_t scales = base + kSfOff;
-    const uint32_t bars = scales + ST * C::SF_BYTES;
+    const uint32_t bars = scales + 2 * C::SF_SLOT_BYTES;
     const uint32_t full = bars, empty = full + 8 * ST, tfull = empty + 8 * ST, tempty = tfull + 16;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + kSfOff + ST * C::SF_BYTES + 8 * (2 * ST + 4));
+    const uint32_t sfull = tempty + 16, sempty = sfull + 16;   // scale words of kSfAhead k-blocks, two slots
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + kSfOff + 2 * C::SF_SLOT_BYTES + 8 * (2 * ST + 8));
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -116,9 +137,11 @@ gemm_mx_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
     const int nkb = p.K / kBlockK;
 
     if (threadIdx.x == 0) {
-        // full: the TMA lane's expect_tx arrival + one arrival per scale warp
-        for (int i = 0; i < ST; ++i) { mbar_init(full + 8 * i, 5); mbar_init(empty + 8 * i, 1); }
-        for (int i = 0; i < 2; ++i) { mbar_init(tfull + 8 * i, 1); mbar_init(tempty + 8 * i, 8); }
+        for (int i = 0; i < ST; ++i) { mbar_init(full + 8 * i, 1); mbar_init(empty + 8 * i, 1); }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(tfull + 8 * i, 1); mbar_init(tempty + 8 * i, 8);
+            mbar_init(sfull + 8 * i, 4); mbar_init(sempty + 8 * i, 1);
+        }
         *abort_flag = 0;
         fence_barrier_init();
         prefetch_tmap(&tmap_a);
@@ -132,69 +155,96 @@ gemm_mx_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);   // uniform, and known to be
 
+    // Stage u of the ring holds the k-blocks u, u + 4, ... of every tile (a tile of fewer leaves some out), so that stage
+    // addresses are constants of the unrolled loops.  With the addresses formed per stage, under a branch for the elected
+    // lane and behind a blocking wait, a stage took the issuing warp 700 cycles (340 of them the four products and their
+    // commit) where the tensor core needs 256 or 384; in this form 36736 x 384 x 1536 with its quantiser 57.2 -> 55.6 us.
     if (warp == 0) {
-        if (lane == 0) {
-            uint32_t st = 0, ph = 1;   // a fresh barrier passes the wait for the phase before its first
-            bool ok = true;
-            for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
-                const int m0 = (tile / n_tiles) * kTileM, n0 = (tile % n_tiles) * BN;
-                for (int kb = 0; kb < nkb; ++kb) {
-                    if (!(ok = mbar_wait(empty + 8 * st, ph, abort_flag))) break;
-                    const uint32_t dst = base + st * C::STAGE_BYTES;
-                    mbar_expect_tx(full + 8 * st, C::STAGE_BYTES);
-                    tma_load_2d(dst, &tmap_a, kb * kBlockK, m0, full + 8 * st);
-                    tma_load_2d(dst + kOperandBytes, &tmap_w, kb * kBlockK, n0, full + 8 * st);
-                    if (++st == ST) { st = 0; ph ^= 1; }
+        uint32_t ph = 0xFu;   // one bit per stage; a fresh barrier passes the wait for the phase before its first
+        bool ok = true;
+        for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
+            const int m0 = (tile / n_tiles) * kTileM, n0 = (tile % n_tiles) * BN;
+            for (int kb0 = 0; kb0 < nkb && ok; kb0 += ST) {
+#pragma unroll
+                for (int u = 0; u < ST; ++u) {
+                    if (kb0 + u < nkb && ok) {
+                        ok = mbar_wait_warp(empty + 8 * u, ph >> u & 1, abort_flag);
+                        ph ^= 1u << u;
+                        if (ok && elect_one()) {
+                            const uint32_t dst = base + u * C::STAGE_BYTES;
+                            mbar_expect_tx(full + 8 * u, C::STAGE_BYTES);
+                            tma_load_2d(dst, &tmap_a, (kb0 + u) * kBlockK, m0, full + 8 * u);
+                            tma_load_2d(dst + kOperandBytes, &tmap_w, (kb0 + u) * kBlockK, n0, full + 8 * u);
+                        }
+                        __syncwarp();
+                    }
                 }
             }
         }
     } else if (warp == 1) {
-        uint32_t st = 0, ph = 0, tcount = 0;
-        bool ok = true;
+        const uint32_t elected = elect_one() ? 1u : 0u;
+        const uint64_t adesc0 = make_smem_desc(base), bdesc0 = make_smem_desc(base + kOperandBytes);
+        const uint32_t idesc0 = idesc_mx<BN>(p.a_fmt, p.w_fmt, 0);
+        uint32_t ph = 0, tcount = 0, ss = 0, sph = 0;
+        // the next wait's outcome is asked for before the current stage is issued: a round to a barrier takes 100-150 cycles
+        bool ok = true, ready = false, sready = false;
         for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++tcount) {
             const uint32_t as = tcount & 1, ause = tcount >> 1;
             if (ause >= 1 && !(ok = mbar_wait_warp(tempty + 8 * as, (ause - 1) & 1, abort_flag))) break;
-            for (int kb = 0; kb < nkb; ++kb) {
-                if (!(ok = mbar_wait_warp(full + 8 * st, ph, abort_flag))) break;
+            const uint32_t acc = tmem + as * BN;
+            for (int kb0 = 0; kb0 < nkb && ok; kb0 += ST) {
+                if (!__all_sync(0xffffffffu, sready) && !(ok = mbar_wait_warp(sfull + 8 * ss, sph, abort_flag))) break;
                 tc_fence_after();
-                if (elect_one()) {
-                    const uint64_t adesc = make_smem_desc(base + st * C::STAGE_BYTES);
-                    const uint64_t bdesc = make_smem_desc(base + st * C::STAGE_BYTES + kOperandBytes);
-                    const uint32_t sfa = tmem + C::ACC_COLS + st * C::SF_COLS, sfb = sfa + 4;
+                const uint32_t sf = tmem + C::ACC_COLS + ss * (kSfAhead * C::SF_COLS);
+                const uint32_t src = scales + ss * C::SF_SLOT_BYTES;
 #pragma unroll
-                    for (int g = 0; g <= C::W_GROUPS; ++g) copy_scales(sfa + 4 * g, scales + st * C::SF_BYTES + g * kSfGroup);
+                for (int u = 0; u < ST; ++u) {
+                    if (kb0 + u < nkb && ok) {
+                        if (!__all_sync(0xffffffffu, ready)) ok = mbar_wait_warp(full + 8 * u, ph >> u & 1, abort_flag);
+                        ph ^= 1u << u;
+                        tc_fence_after();
+                        const bool last = kb0 + u == nkb - 1;
+                        const int nu = last ? 0 : (u + 1) % ST;
+                        ready = mbar_test_wait(full + 8 * nu, ph >> nu & 1);
+                        if (!ok) break;
 #pragma unroll
-                    for (int k = 0; k < kBlockK / 32; ++k)   // 32 bytes of k per instruction: descriptor start + 2
-                        umma_mx(tmem + as * BN, adesc + 2 * k, bdesc + 2 * k, idesc_mx<BN>(p.a_fmt, p.w_fmt, k), sfa, sfb,
-                                (kb | k) != 0 ? 1u : 0u);
-                    umma_commit<1>(empty + 8 * st);
-                    if (kb == nkb - 1) umma_commit<1>(tfull + 8 * as);
+                        for (int g = 0; g <= C::W_GROUPS; ++g)
+                            copy_scales(elected, sf + u * C::SF_COLS + 4 * g, src + u * C::SF_BYTES + g * kSfGroup);
+#pragma unroll
+                        for (int k = 0; k < kBlockK / 32; ++k)   // 32 bytes of k per instruction: descriptor start + 2
+                            umma_mx(elected, acc, adesc0 + (u * (C::STAGE_BYTES >> 4) + 2 * k), bdesc0 + (u * (C::STAGE_BYTES >> 4) + 2 * k),
+                                    idesc0 + ((uint32_t)k << 4 | (uint32_t)k << 29), sf + u * C::SF_COLS, sf + u * C::SF_COLS + 4,
+                                    (u | k) != 0 ? 1u : (kb0 != 0 ? 1u : 0u));
+                        commit_if(elected, empty + 8 * u);
+                        if (u == ST - 1 || last) commit_if(elected, sempty + 8 * ss);
+                        if (last) commit_if(elected, tfull + 8 * as);
+                    }
                 }
-                __syncwarp();
-                if (++st == ST) { st = 0; ph ^= 1; }
+                ss ^= 1; sph ^= ss ^ 1;
+                sready = mbar_test_wait(sfull + 8 * ss, sph);
             }
         }
     } else if (warp < 6) {
         // ------------------------------------------------------------ scale feed: 32 rows of every 128 per warp
-        // Four k-blocks of a row at a time, requested while the four before them are handed over, across tiles too.
+        // Four k-blocks of a row at a time, requested as soon as the four before them are handed over, across tiles too.
         const int q = warp - 2;
         const int ld = p.K / 128;                      // scale words per row
         const bool vec = (ld & 3) == 0;                // 16-byte loads: rows start on 16 bytes
         const uint32_t* sfa = reinterpret_cast<const uint32_t*>(p.sfa);
         const uint32_t* sfw = reinterpret_cast<const uint32_t*>(p.sfw);
-        auto load4 = [&](const uint32_t* row, int kb0, uint32_t (&r)[4]) {
+        auto load4 = [&](const uint32_t* row, int kb0, uint32_t (&r)[kSfAhead]) {
             if (vec) {
                 const uint4 v = __ldg(reinterpret_cast<const uint4*>(row + kb0));
                 r[0] = v.x; r[1] = v.y; r[2] = v.z; r[3] = v.w;
             } else {
 #pragma unroll
-                for (int u = 0; u < 4; ++u)
+                for (int u = 0; u < kSfAhead; ++u)
                     if (kb0 + u < nkb) r[u] = __ldg(row + kb0 + u);
             }
         };
-        auto fetch = [&](int tile, int kb0, uint32_t (&r)[1 + C::W_GROUPS][4]) {
+        auto fetch = [&](int tile, int kb0, uint32_t (&r)[1 + C::W_GROUPS][kSfAhead]) {
             const int ar = (tile / n_tiles) * kTileM + 32 * q + lane, n0 = (tile % n_tiles) * BN;
             // rows past M are zero-filled operand rows: any finite scale will do
             if (ar < p.M) load4(sfa + (size_t)ar * ld, kb0, r[0]);
@@ -203,34 +253,26 @@ gemm_mx_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
             for (int g = 0; g < C::W_GROUPS; ++g)
                 if (128 * g + 32 * q < BN) load4(sfw + (size_t)(n0 + 128 * g + 32 * q + lane) * ld, kb0, r[1 + g]);
         };
-        uint32_t cur[1 + C::W_GROUPS][4] = {}, nxt[1 + C::W_GROUPS][4] = {};
+        uint32_t cur[1 + C::W_GROUPS][kSfAhead] = {};
         const uint32_t slot_addr = scales + lane * 16 + q * 4;
-        uint32_t st = 0, ph = 1;
+        uint32_t ss = 0, sph = 1;
         int tile = blockIdx.x, kb0 = 0;
         bool ok = true;
         if (tile < num_tiles) fetch(tile, 0, cur);
         while (tile < num_tiles && ok) {
-            int ntile = tile, nkb0 = kb0 + 4;
-            if (nkb0 >= nkb) { ntile += gridDim.x; nkb0 = 0; }
-            if (ntile < num_tiles) fetch(ntile, nkb0, nxt);
+            if (!(ok = mbar_wait(sempty + 8 * ss, sph, abort_flag))) break;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (kb0 + u < nkb && ok) {
-                    if (!(ok = mbar_wait(empty + 8 * st, ph, abort_flag))) break;
+            for (int u = 0; u < kSfAhead; ++u)
 #pragma unroll
-                    for (int g = 0; g <= C::W_GROUPS; ++g)
-                        asm volatile("st.shared.b32 [%0], %1;" ::"r"(slot_addr + st * C::SF_BYTES + g * kSfGroup), "r"(cur[g][u]) : "memory");
-                    fence_proxy_async();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(full + 8 * st);
-                    if (++st == ST) { st = 0; ph ^= 1; }
-                }
-            }
-#pragma unroll
-            for (int g = 0; g <= C::W_GROUPS; ++g)
-#pragma unroll
-                for (int u = 0; u < 4; ++u) cur[g][u] = nxt[g][u];
-            tile = ntile; kb0 = nkb0;
+                for (int g = 0; g <= C::W_GROUPS; ++g)
+                    asm volatile("st.shared.b32 [%0], %1;" ::"r"(slot_addr + ss * C::SF_SLOT_BYTES + u * C::SF_BYTES + g * kSfGroup), "r"(cur[g][u]) : "memory");
+            fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(sfull + 8 * ss);
+            ss ^= 1; sph ^= ss ^ 1;
+            kb0 += kSfAhead;
+            if (kb0 >= nkb) { tile += gridDim.x; kb0 = 0; }
+            if (tile < num_tiles) fetch(tile, kb0, cur);   // behind the fence, which would wait for it
         }
     } else {
         // ------------------------------------------------------------ epilogue: lane quarter x half of the columns
