@@ -362,6 +362,9 @@ typedef enum {
     RLX_GEMM_SIMT = 1,           /* plain CUDA-core tiles (bring-up / cross-check)                 */
     RLX_GEMM_TCGEN05_PAIR = 2,   /* force the CTA-pair variant (cta_group::2, 256-row tiles); N % 128 == 0 */
     RLX_GEMM_TCGEN05_SINGLE = 3, /* force the one-CTA-per-tile variant                             */
+    RLX_GEMM_TCGEN05_SPLIT_K = 5, /* force the variant that splits K over two or four CTAs per tile, partial sums added in
+                                    a fixed order: few rows, K >= 1536; RLX_ERR_UNSUPPORTED elsewhere.  Another order of
+                                    the fp32 sums than every other variant's, so never taken unasked here         */
     RLX_GEMM_TCGEN05_RESIDENT = 4 /* force the CTA-pair variant that keeps its 256 rows of A resident in
                                     shared memory and streams only W (K <= 384, N % 128 == 0 or
                                     N % 192 == 0); RLX_GEMM_TCGEN05 picks it by itself for such K once

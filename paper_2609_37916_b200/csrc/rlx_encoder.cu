@@ -656,7 +656,9 @@ struct LnFold {
 
 // CTAs per 128 x 64 tile along K (1: do not split).  A long contraction on a few tiles is bound by one SM's operand feed;
 // four CTAs per tile while they all fit beside each other, two while two thirds of them do -- the row count is the
-// padded one, and a batch whose every position is valid then runs two half-length rounds instead of one.
+// padded one, and a batch whose every position is valid then runs two half-length rounds instead of one.  Taken by
+// itself only by the products that fold a LayerNorm: the plain ones keep one order of summation at every size, which the
+// fused feed-forward kernel shares bit for bit.
 int pick_split_k(int M, int N, int K, int epi) {
     if (K < 1536 || N % rlx::tcsk::kBN != 0 || (epi > 2 && epi < 5)) return 1;
     const int tiles = (M + rlx::tc::BLOCK_M - 1) / rlx::tc::BLOCK_M * (N / rlx::tcsk::kBN), sms = sm_count();
@@ -713,7 +715,8 @@ rlx_status_t launch_gemm(const bf16* A, const bf16* W, const float* bias, const 
         p.cvec = lf->cvec; p.dvec = lf->dvec; p.stats_in = lf->stats_in; p.stats_in_p = lf->stats_in_p;
         p.ln_gamma = lf->gamma; p.ln_beta = lf->beta; p.stats_out = lf->stats_out; p.ln_eps = lf->eps;
     }
-    const int split = want_cg == 0 ? pick_split_k(M, N, K, epi) : 1;
+    const int split = want_cg == 4 || (want_cg == 0 && epi >= 5) ? pick_split_k(M, N, K, epi) : 1;
+    if (want_cg == 4 && split == 1) return RLX_ERR_UNSUPPORTED;
     if (split > 1) return launch_gemm_splitk(A, W, p, to, epi, split, st);
     // want_cg == 3: the A-resident CTA-pair kernel, forced; 0: chosen when the problem is large enough
     if (want_cg == 3 || (want_cg == 0 && g_exp_resident >= 0)) {
@@ -1715,13 +1718,13 @@ rlx_status_t rlx_gemm_bf16(const void* A, const void* W, const float* bias, cons
         return RLX_ERR_INVALID_ARG;
     if (N % 64 != 0 || K % 8 != 0) return RLX_ERR_UNSUPPORTED;
     if (impl != RLX_GEMM_TCGEN05 && impl != RLX_GEMM_SIMT && impl != RLX_GEMM_TCGEN05_PAIR &&
-        impl != RLX_GEMM_TCGEN05_SINGLE && impl != RLX_GEMM_TCGEN05_RESIDENT)
+        impl != RLX_GEMM_TCGEN05_SINGLE && impl != RLX_GEMM_TCGEN05_RESIDENT && impl != RLX_GEMM_TCGEN05_SPLIT_K)
         return RLX_ERR_INVALID_ARG;
     if (impl == RLX_GEMM_TCGEN05_PAIR && N % 128 != 0 && N % 192 != 0) return RLX_ERR_UNSUPPORTED;
     if (impl == RLX_GEMM_TCGEN05_RESIDENT && (K > 384 || (N % 128 != 0 && N % 192 != 0))) return RLX_ERR_UNSUPPORTED;
     RLX_CUDA_TRY(init_kernels_for_current_device());
     const int want_cg = impl == RLX_GEMM_TCGEN05_PAIR ? 2 : impl == RLX_GEMM_TCGEN05_SINGLE ? 1
-                        : impl == RLX_GEMM_TCGEN05_RESIDENT ? 3 : 0;
+                        : impl == RLX_GEMM_TCGEN05_RESIDENT ? 3 : impl == RLX_GEMM_TCGEN05_SPLIT_K ? 4 : 0;
     return launch_gemm((const bf16*)A, (const bf16*)W, bias, (const bf16*)residual, (int)epi, M, N, K, (bf16*)out,
                        impl == RLX_GEMM_SIMT, status, static_cast<cudaStream_t>(stream), nullptr, want_cg);
 }

@@ -465,8 +465,7 @@ def test_attention_all_masked_sequence_gives_zeros(rlx):
 @pytest.mark.parametrize("M", [1, 31, 33, 64, 97, 128, 129, 300])
 @pytest.mark.parametrize("N,K", [(64, 1536), (384, 1536), (192, 1544), (768, 3072)])
 def test_gemm_split_along_k(rlx, M, N, K):
-    """Few rows and a long contraction take the split form by themselves: four or two CTAs per tile, at the edges of
-    the 32-row units and of uneven k ranges, against the oracle and the one-CTA-per-tile form, twice (the order of the
+    """Few rows and a long contraction, split on request: four or two CTAs per tile, at the edges of the 32-row units and of uneven k ranges, against the oracle and the one-CTA-per-tile form, twice (the order of the
     partial sums is fixed)."""
     rng = np.random.default_rng(M + N + K)
     a, w = rand_bf16(rng, (M, K)), rand_bf16(rng, (N, K), 0.05)
@@ -474,8 +473,8 @@ def test_gemm_split_along_k(rlx, M, N, K):
     for epi in (0, 1, 2):
         status = torch.zeros(1, dtype=torch.int32, device="cuda")
         args = (bf16_dev(a), bf16_dev(w), f32_dev(bias), bf16_dev(res) if epi == 2 else None, epi)
-        got = rlx.gemm_bf16(*args, status=status)
-        assert torch.equal(got, rlx.gemm_bf16(*args)) and int(status.item()) == 0
+        got = rlx.gemm_bf16(*args, impl=5, status=status)
+        assert torch.equal(got, rlx.gemm_bf16(*args, impl=5)) and int(status.item()) == 0
         ref = oracle.linear(a.astype(np.float64), w, bias)
         ref = oracle.gelu(ref) if epi == 1 else ref + res if epi == 2 else ref
         assert_close_bf16_out(to_np64(got), ref, extra_abs=K * 2.0 ** -24 * 0.2)
