@@ -166,7 +166,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + C::BAR_OFF + 8 * C::NBAR);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     pdl_launch_dependents();
     if (threadIdx.x == 0) {
         for (int i = 0; i < QST; ++i) { mbar_init(q_full + 8 * i, 1); mbar_init(q_free + 8 * i, 1); mbar_init(q_rot + 8 * i, 4); }
@@ -186,7 +186,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = warp_uniform(*tmem_slot);
     pdl_wait();
 
     // A consumer's next item: 1 ready, 0 end of the list, -1 a wait ran out.  All lanes of a warp call.

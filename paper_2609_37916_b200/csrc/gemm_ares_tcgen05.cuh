@@ -92,8 +92,8 @@ gemm_ares_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gri
                                                       16 * C::STAGES + 8 * C::A_GROUPS + 32);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t cta_rank = cluster_ctarank();   // rank 0 leads the pair
+    const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const uint32_t cta_rank = warp_uniform(cluster_ctarank());   // rank 0 leads the pair
     pdl_launch_dependents();
     if (threadIdx.x == 0) RLX_TRACE(p, 0);
 
@@ -121,7 +121,7 @@ gemm_ares_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gri
     __syncthreads();
     cluster_sync_all();   // the peer's barriers are initialised before any remote use
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = warp_uniform(*tmem_slot);
 
     if (threadIdx.x == 0) RLX_TRACE(p, 1);
     pdl_wait();   // the previous kernel's outputs are read only from here on

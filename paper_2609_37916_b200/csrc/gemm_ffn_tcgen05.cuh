@@ -333,8 +333,8 @@ ffn_fused_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_x, const __gri
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + C::BAR_OFF + 8 * 32);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t cta_rank = cluster_ctarank();
+    const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const uint32_t cta_rank = warp_uniform(cluster_ctarank());
     pdl_launch_dependents();
     if (threadIdx.x == 0) {
         for (int i = 0; i < C::KB1; ++i) mbar_init(x_full + 8 * i, 1);
@@ -362,7 +362,7 @@ ffn_fused_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_x, const __gri
     __syncthreads();
     cluster_sync_all();
     tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = warp_uniform(*tmem_slot);
 
     pdl_wait();
     int M = p.M;

@@ -132,7 +132,7 @@ gemm_mx_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + kSfOff + 2 * C::SF_SLOT_BYTES + 8 * (2 * ST + 8));
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     const int n_tiles = p.N / BN, m_tiles = (p.M + kTileM - 1) / kTileM, num_tiles = n_tiles * m_tiles;
     const int nkb = p.K / kBlockK;
 
@@ -155,7 +155,7 @@ gemm_mx_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);   // uniform, and known to be
+    const uint32_t tmem = warp_uniform(*tmem_slot);
 
     // Stage u of the ring holds the k-blocks u, u + 4, ... of every tile (a tile of fewer leaves some out), so that stage
     // addresses are constants of the unrolled loops.  With the addresses formed per stage, under a branch for the elected

@@ -55,8 +55,8 @@ gemm_splitk_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __g
     const uint32_t xch_bar = acc_bar + 8;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + kBarOff + 8 * (2 * kStages + 2));
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int rank = (int)cluster_ctarank(), S = (int)tccl::cluster_nctarank();
+    const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const int rank = (int)warp_uniform(cluster_ctarank()), S = (int)tccl::cluster_nctarank();
     pdl_launch_dependents();
 
     int M = p.M;
@@ -89,7 +89,7 @@ gemm_splitk_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __g
     __syncthreads();
     cluster_sync_all();      // the peers' barriers exist before anything is sent to them
     tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = warp_uniform(*tmem_slot);
 
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer (whole warp, one lane issues)

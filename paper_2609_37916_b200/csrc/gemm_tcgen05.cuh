@@ -736,8 +736,8 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
         reinterpret_cast<uint32_t*>(gbase + C::STAGES * C::STAGE_BYTES + C::STAGING_BYTES + C::VEC_BYTES + 16 * C::STAGES + 32);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t cta_rank = (CG == 2) ? cluster_ctarank() : 0u;   // rank 0 leads the pair
+    const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const uint32_t cta_rank = (CG == 2) ? warp_uniform(cluster_ctarank()) : 0u;   // rank 0 leads the pair
     pdl_launch_dependents();
     if (threadIdx.x == 0) RLX_TRACE(p, 0);
 
@@ -764,7 +764,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
     __syncthreads();
     if constexpr (CG == 2) cluster_sync_all();   // the peer's barriers are initialised before any remote use
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = warp_uniform(*tmem_slot);
 
     // The row count and the weights do not come from the previous kernel (see ld_early): they are read, and the first
     // stages' W tiles requested, before the wait; A, the residual and the row statistics behind it.

@@ -465,8 +465,9 @@ def test_attention_all_masked_sequence_gives_zeros(rlx):
 @pytest.mark.parametrize("M", [1, 31, 33, 64, 97, 128, 129, 300])
 @pytest.mark.parametrize("N,K", [(64, 1536), (384, 1536), (192, 1544), (768, 3072)])
 def test_gemm_split_along_k(rlx, M, N, K):
-    """Few rows and a long contraction, split on request: four or two CTAs per tile, at the edges of the 32-row units and of uneven k ranges, against the oracle and the one-CTA-per-tile form, twice (the order of the
-    partial sums is fixed)."""
+    """Few rows and a long contraction, split on request: four or two CTAs per tile, at the edges of the 32-row units
+    and of uneven k ranges, against the oracle and the one-CTA-per-tile form, twice (the order of the partial sums is
+    fixed)."""
     rng = np.random.default_rng(M + N + K)
     a, w = rand_bf16(rng, (M, K)), rand_bf16(rng, (N, K), 0.05)
     bias, res = (0.1 * rng.standard_normal(N)).astype(np.float32), rand_bf16(rng, (M, N))
