@@ -132,25 +132,28 @@ gemm_splitk_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __g
         // ------------------------------------------------------------ MMA issuer (whole warp, one lane issues)
         if (groups > 0) {
             constexpr uint32_t idesc = make_idesc(BLOCK_M, kBN);
-            int stage = 0;
-            uint32_t phase = 0;
-            bool ok = true;
+            const uint64_t adesc0 = make_smem_desc(base), bdesc0 = make_smem_desc(base + kKps * kABytes);
+            uint32_t stage = 0, phase = 0;
+            bool ok = true, ready = false;
             for (int kb = kb0; kb < kb1; kb += kKps) {
                 const int cnt = min(kKps, kb1 - kb);
-                if (!(ok = mbar_wait_warp(full_bar + 8 * stage, phase, abort_flag))) break;
+                if (!__all_sync(0xffffffffu, ready) && !(ok = mbar_wait_warp(full_bar + 8 * stage, phase, abort_flag))) break;
                 tc_fence_after();
+                const uint32_t cur = stage;
+                if (++stage == kStages) { stage = 0; phase ^= 1; }
+                ready = mbar_test_wait(full_bar + 8 * stage, phase);
                 if (elect_one()) {
-                    for (int i = 0; i < cnt; ++i) {
-                        const uint64_t ad = make_smem_desc(base + stage * kStageBytes + i * kABytes);
-                        const uint64_t bd = make_smem_desc(base + stage * kStageBytes + kKps * kABytes + i * kBBytes);
+                    const uint64_t ad0 = adesc0 + cur * (kStageBytes >> 4), bd0 = bdesc0 + cur * (kStageBytes >> 4);
 #pragma unroll
-                        for (int k = 0; k < BLOCK_K / UMMA_K; ++k)
-                            umma_bf16<1>(tmem, ad + 2 * k, bd + 2 * k, idesc, (kb != kb0 || (i | k) != 0) ? 1u : 0u);
-                    }
-                    umma_commit<1>(empty_bar + 8 * stage);
+                    for (int i = 0; i < kKps; ++i)
+                        if (i < cnt)
+#pragma unroll
+                            for (int k = 0; k < BLOCK_K / UMMA_K; ++k)
+                                umma_bf16<1>(tmem, ad0 + (i * (kABytes >> 4) + 2 * k), bd0 + (i * (kBBytes >> 4) + 2 * k), idesc,
+                                             (kb != kb0 || (i | k) != 0) ? 1u : 0u);
+                    umma_commit<1>(empty_bar + 8 * cur);
                 }
                 __syncwarp();
-                if (++stage == kStages) { stage = 0; phase ^= 1; }
             }
             if (ok && elect_one()) umma_commit<1>(acc_bar);
             __syncwarp();

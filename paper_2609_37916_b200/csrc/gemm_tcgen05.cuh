@@ -861,10 +861,10 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
         // ------------------------------------------------------------ MMA issuer (whole warp, one lane issues)
         if (cta_rank == 0) {
             constexpr uint32_t idesc = make_idesc(TILE_M, BLOCK_N);
-            int stage = 0;
-            uint32_t phase = 0;
+            const uint64_t adesc0 = make_smem_desc(base), bdesc0 = make_smem_desc(base + C::KPS * C::A_BYTES);
+            uint32_t stage = 0, phase = 0;
             int it = 0;
-            bool ok = true;
+            bool ok = true, ready = false;
             if (lane == 0) { RLX_TRACE(p, 9); RLX_TRACE_CLK(p, 14); }
             RLX_CLK_DECL(clk_full);
             RLX_CLK_DECL(clk_tempty);
@@ -880,28 +880,35 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
                     const int cnt = min(C::KPS, num_kb - kb);
                     bool got_ops;
                     if (it == 2 && kb == 0 && lane == 0) RLX_TRACE_CLK(p, 60);            // MMA thread starts waiting for that stage
-                    RLX_CLK_ADD(clk_full, got_ops = mbar_wait_warp(full_bar + 8 * stage, phase, abort_flag));
+                    RLX_CLK_ADD(clk_full, got_ops = __all_sync(0xffffffffu, ready) || mbar_wait_warp(full_bar + 8 * stage, phase, abort_flag));
                     if (!got_ops) { ok = false; break; }
                     if (it == 2 && kb == 0 && lane == 0) RLX_TRACE_CLK(p, 61);            // operands landed
                     tc_fence_after();
-                    const uint32_t st0 = base + stage * C::STAGE_BYTES;
+                    const uint32_t cur = stage;
+                    if (++stage == C::STAGES) { stage = 0; phase ^= 1; }
+                    // the next wait's outcome, asked for while this stage is issued: a round to a barrier takes 100-150 cycles.
+                    // Where the tensor core is what a stage waits for it costs a little (32 x 128 215.4 -> 216.3 us), so only
+                    // the narrowest tiles ask (1 x 128 144.9 -> 143.5).
+                    if (C::SMALL) ready = mbar_test_wait(full_bar + 8 * stage, phase);
                     if (elect_one()) {
                         if (it == 0 && kb == 0) RLX_TRACE(p, 5);
                         if (!RLX_DBG(p, kDbgNoMma)) {
-                            for (int i = 0; i < cnt; ++i) {
-                                const uint64_t adesc = make_smem_desc(st0 + i * C::A_BYTES);
-                                const uint64_t bdesc = make_smem_desc(st0 + C::KPS * C::A_BYTES + i * C::B_BYTES);
+                            const uint64_t ad0 = adesc0 + cur * (C::STAGE_BYTES >> 4), bd0 = bdesc0 + cur * (C::STAGE_BYTES >> 4);
 #pragma unroll
-                                for (int k = 0; k < BLOCK_K / UMMA_K; ++k) {
-                                    // advancing 16 bf16 = 32 bytes along K inside the swizzle row: +2 in 16-byte units
-                                    umma_bf16<CG>(tmem_d, adesc + 2 * k, bdesc + 2 * k, idesc, (kb | i | k) != 0 ? 1u : 0u);
+                            for (int i = 0; i < C::KPS; ++i) {
+                                if (i < cnt) {
+#pragma unroll
+                                    for (int k = 0; k < BLOCK_K / UMMA_K; ++k) {
+                                        // advancing 16 bf16 = 32 bytes along K inside the swizzle row: +2 in 16-byte units
+                                        umma_bf16<CG>(tmem_d, ad0 + (i * (C::A_BYTES >> 4) + 2 * k), bd0 + (i * (C::B_BYTES >> 4) + 2 * k),
+                                                      idesc, (kb | i | k) != 0 ? 1u : 0u);
+                                    }
                                 }
                             }
                         }
-                        umma_commit<CG>(empty_bar + 8 * stage);  // stage reusable once these MMAs have read it
+                        umma_commit<CG>(empty_bar + 8 * cur);  // stage reusable once these MMAs have read it
                     }
                     __syncwarp();
-                    if (++stage == C::STAGES) { stage = 0; phase ^= 1; }
                 }
                 if (ok && elect_one()) {
                     umma_commit<CG>(tfull_bar + 8 * as);  // accumulator complete
