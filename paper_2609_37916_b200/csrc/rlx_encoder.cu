@@ -989,18 +989,17 @@ int chunk_batch(int B, int S);
 
 // The tcgen05 attention kernel instead of the mma.sync one: where asked for, and where it pays inside a whole forward
 // (us mma.sync / tcgen05, 6 x 384 with heads of 32 and 12 x 768 with heads of 64; batch x longest sequence):
-//   64: sequences beyond two 128-row tiles everywhere (1 x 512 644 / 569, 64 x 512 4499 / 4119); beyond one tile once
-//       there are enough tokens to fill the chip (100 x 144 2520 / 2434, 70 x 200 1909 / 1889; but 8 x 144 544 / 560,
-//       1 x 256 435 / 474)
-//   32: beyond 384 (128 x 512 1414 / 1360, 60 x 512 832 / 822; 128 x 384 1100 / 1106); two full tiles while an item's
-//       own chain is what a layer waits for (4 x 256 230 / 201, 60 x 256 708 / 690; but 256 x 256 1254 / 1265, and
-//       61 x 203 442 / 459)
+//   64: sequences beyond two 128-row tiles everywhere (1 x 512 644 / 569, 64 x 512 4499 / 4119), two full tiles but for a
+//       single sequence (4 x 256 551 / 524; 1 x 256 417 / 442), beyond one tile once there are enough tokens to fill the
+//       chip (100 x 144 2520 / 2434, 70 x 200 1909 / 1889; but 8 x 144 505 / 510)
+//   32: two full tiles (256 x 256 1267 / 1208, 128 x 384 1077 / 1040); less while few tokens leave an item's own chain as
+//       what a layer waits for (16 x 192 218 / 201; but 256 x 192 983 / 1000, 61 x 203 431 / 438)
 bool uses_attention_fwd(const rlx_encoder_config_t& c, int B, int S) {
     if (c.flags & RLX_FLAG_ATTN_TCGEN05) return true;
     const long long tokens = g_whole_call_tokens > 0 ? g_whole_call_tokens : (long long)B * S;
     constexpr int kT = rlx::tcat::kTile;
-    if (c.hidden / c.num_heads == 64) return S > 2 * kT || (S > kT && tokens >= 8192);
-    return S > 3 * kT || (S >= 2 * kT && tokens <= 16384);
+    if (c.hidden / c.num_heads == 64) return S > 2 * kT || (S == 2 * kT && B > 1) || (S > kT && tokens >= 8192);
+    return S >= 2 * kT || (S >= kT + kT / 2 && tokens <= 4096);
 }
 
 struct GraphEntry {

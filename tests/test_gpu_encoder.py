@@ -229,9 +229,9 @@ def test_random_small_problems_match_oracle(rlx, seed):
             check(other, ref, inp.lengths, tight=(seed % 4 != 0))
 
 
-@pytest.mark.parametrize("name,B,S", [("c1", 3, 255), ("c1", 3, 256), ("c1", 64, 256), ("c1", 65, 256), ("c1", 45, 384),
-                                      ("c1", 45, 385), ("c4", 2, 256), ("c4", 2, 257), ("c4", 64, 128), ("c4", 63, 129),
-                                      ("c4", 64, 129)])
+@pytest.mark.parametrize("name,B,S", [("c1", 3, 191), ("c1", 21, 192), ("c1", 22, 192), ("c1", 22, 255), ("c1", 22, 256),
+                                      ("c1", 45, 385), ("c4", 1, 256), ("c4", 2, 256), ("c4", 1, 257), ("c4", 64, 128),
+                                      ("c4", 63, 129), ("c4", 64, 129)])
 def test_attention_kernel_choice_at_its_edges(rlx, name, B, S):
     """Both sides of every line where a forward changes its attention kernel (heads of 32 and of 64), the first, a
     middle and the last sequence against the oracle; the kernel that may be asked for gives the same at that tolerance."""
