@@ -101,7 +101,7 @@ struct Cfg {
     static constexpr int VRING_OFF = RING_OFF + KST * TILE;
     static constexpr int ITEM_OFF = VRING_OFF + VST * TILE;
     static constexpr int BAR_OFF = ITEM_OFF + kItemRing * 32;
-    static constexpr int NBAR = 3 * QST + 3 * KST + 2 * VST + 3 * NSB + 2 + 2 * kItemRing;
+    static constexpr int NBAR = 3 * QST + 3 * KST + 2 * VST + 3 * NSB + 2 + 2 * kItemRing + 8;
     static constexpr int SMEM_BYTES = BAR_OFF + 8 * NBAR + 16 + 1024;
     static constexpr uint64_t SWZ = ROWB == 128 ? 2 : 4;
     static_assert(ROWB == 128 || ROWB == 64, "swizzle span");
@@ -162,7 +162,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
     const uint32_t k_full = q_rot + 8 * QST, k_free = k_full + 8 * KST, k_rot = k_free + 8 * KST;
     const uint32_t v_full = k_rot + 8 * KST, v_free = v_full + 8 * VST;
     const uint32_t s_full = v_free + 8 * VST, p_ready = s_full + 8 * NSB, buf_free = p_ready + 8 * NSB, o_full = buf_free + 8 * NSB;
-    const uint32_t item_full = o_full + 16, item_free = item_full + 8 * kItemRing;
+    const uint32_t item_full = o_full + 16, item_free = item_full + 8 * kItemRing, turn = item_free + 8 * kItemRing;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + C::BAR_OFF + 8 * C::NBAR);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
@@ -174,6 +174,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
         for (int i = 0; i < VST; ++i) { mbar_init(v_full + 8 * i, 1); mbar_init(v_free + 8 * i, 1); }
         for (int i = 0; i < NSB; ++i) { mbar_init(s_full + 8 * i, 1); mbar_init(p_ready + 8 * i, 4); mbar_init(buf_free + 8 * i, 1); }
         for (int i = 0; i < 2; ++i) mbar_init(o_full + 8 * i, 1);
+        for (int i = 0; i < 8; ++i) mbar_init(turn + 8 * i, 1);
         for (int i = 0; i < kItemRing; ++i) { mbar_init(item_full + 8 * i, 1); mbar_init(item_free + 8 * i, ROPE ? 15 : 11); }
         *abort_flag = 0;
         fence_barrier_init();
@@ -439,6 +440,13 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
         const float scale = p.scale_log2e;
         uint32_t buf = t, sph = 0;   // score buffer and its parity; jobs t, t + 2, t + 4, ..
         uint32_t pbuf = 0, pph = 0;  // the same of this tile's previous block
+        // With short blocks the two tiles' warps of a scheduler take turns on the exponential unit, handing over a chunk before
+        // the end: they otherwise fall into step, load and reduce at the same time and leave the unit idle meanwhile
+        // (32 q / 8 kv heads of 128, 8 x 2048: 479 -> 462 us).  A block of 128 keys is long enough for that not to matter,
+        // and a lone warp does not fill the unit (heads of 64 181 -> 205), so there they share it freely.
+        constexpr bool TURNS = KB == 64;
+        const uint32_t my_turn = turn + 8 * (t * 4 + quad), other_turn = turn + 8 * ((t ^ 1) * 4 + quad);
+        uint32_t tph = t ^ 1;        // tile 0 begins: a fresh barrier passes the wait for the phase before its first
         bool ok = true;
         Item it;
         for (uint32_t n = 0; ok; ++n) {
@@ -512,10 +520,12 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
                     }
                     const float neg = m_ref == -INFINITY ? 0.f : -m_ref;
                     const uint64_t sc2 = pack_f32x2(scale, scale), ng2 = pack_f32x2(neg, neg);
+                    if (TURNS && !(ok = mbar_wait_warp(my_turn, tph, abort_flag))) break;
                     // straight line over all chunks, masked ones included: a branch per chunk drains the exponential unit
                     // each time, and a second copy of the code costs more in instruction fetches than it saves
 #pragma unroll
                     for (int c = 0; c < NCH; ++c) {
+                        if (TURNS && c == NCH - 1 && lane == 0) mbar_arrive(other_turn);
                         uint32_t pk[16];
 #pragma unroll
                         for (int i = 0; i < 16; ++i) {
@@ -530,7 +540,11 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
                     }
                     tmem_st_wait();
                     tc_fence_before();
+                } else if (TURNS) {
+                    if (!(ok = mbar_wait_warp(my_turn, tph, abort_flag))) break;
+                    if (lane == 0) mbar_arrive(other_turn);
                 }
+                tph ^= 1;
                 __syncwarp();
                 if (lane == 0) mbar_arrive(p_ready + 8 * buf);
                 pbuf = buf;
