@@ -15,8 +15,12 @@
 //                     tensor memory to registers, block maximum, exponentials, P (bf16) back over the scores; at the
 //                     end of an item O / row sum -> global
 //   warp 8            TMA: Q tiles, K and V blocks through a ring each
-//   warp 9             issues S(q) = Q_t K^T: score jobs q = 2 * block + tile go round NSB score buffers, across item
-//                     boundaries too, so the scores run ahead of the softmax
+//   warp 9             issues S(q) = Q_t K^T: score jobs q = 2 * block + tile go round the score buffers, across item
+//                     boundaries too, so the scores run ahead of the softmax.  Heads of 32 and 64 have three buffers, and P
+//                     is written over the scores.  Heads of 128 leave room for one, which is free again as soon as a
+//                     softmax group has its scores in registers, and a buffer for each tile's P: with 64-key blocks and
+//                     four buffers instead, S came as 16 products of N = 64 per 128 keys, which take the tensor core 46
+//                     cycles each where N = 128 takes 63 (32 q / 8 kv heads, 8 x 2048: 465 -> 429 us)
 //   warp 11            issues O_t += P(q) V (P read from tensor memory, V MN-major) and hands the buffer back
 //                     One warp for both was the pace-maker: 1750 cycles per job, of which 640 to 770 are tensor time and
 //                     the rest its own scalar code; the softmax takes about 2400 per job and tile
@@ -26,7 +30,8 @@
 // The reference maximum of a row stays the one of its first block unless a later block exceeds it by more than 2^8
 // (then P <= 256 is still exact in range); only then does the warp wait for PV_t(j-1) and rescale its rows of O in
 // tensor memory.  Waits that skip completions of a barrier are safe because either issuer's products complete in
-// order: a group that has seen S(q) knows that S(q - 1), PV(q - NSB) and everything before them are complete.
+// order: a group that has seen S(q) knows that S(q - 1), PV(q - 3) and everything before them are complete (heads of 128 wait
+// for the tile's previous PV in every block).
 // All mbarrier waits are bounded.
 #pragma once
 #include <cuda.h>
@@ -83,8 +88,12 @@ __device__ __forceinline__ float ex2f(float x) {
 }
 template <int D, bool PAIR>
 struct Cfg {
-    static constexpr int KB = D == 128 ? 64 : 128;            // keys per block
-    static constexpr int NSB = D == 128 ? 4 : 3;              // score buffers (the accumulators take 2 * D columns)
+    static constexpr int KB = 128;                            // keys per block
+    // The accumulators take 2 * D columns of tensor memory.  Heads of 128 leave room for one score buffer and a buffer for
+    // P per tile (APART); otherwise three score buffers, over which P is written.
+    static constexpr bool APART = D == 128;
+    static constexpr int NSB = APART ? 1 : 3;
+    static constexpr int NPB = APART ? 2 : NSB;               // P buffers, in order of use
     static constexpr int W = PAIR ? 2 * D : D;                // columns of a q / k / v tile
     static constexpr int COLS = W > 64 ? 64 : W;              // columns of a TMA box (one swizzle span)
     static constexpr int ROWB = COLS * 2;
@@ -96,12 +105,13 @@ struct Cfg {
     static constexpr int KST = TILE == 32768 ? 3 : 4;         // K ring
     static constexpr int VST = TILE == 32768 ? 2 : 4;         // V ring
     static constexpr int NV = (PAIR && D == 32) ? 64 : D;     // accumulator columns (N = 32 costs the tensor pipe what N = 64 does)
-    static constexpr int O_COL = NSB * KB, O_STRIDE = NV;
+    static constexpr int P_COL = APART ? KB : 0, P_STRIDE = APART ? KB / 2 : KB;
+    static constexpr int O_COL = APART ? 2 * KB : NSB * KB, O_STRIDE = NV;
     static constexpr int RING_OFF = QST * QB;
     static constexpr int VRING_OFF = RING_OFF + KST * TILE;
     static constexpr int ITEM_OFF = VRING_OFF + VST * TILE;
     static constexpr int BAR_OFF = ITEM_OFF + kItemRing * 32;
-    static constexpr int NBAR = 3 * QST + 3 * KST + 2 * VST + 3 * NSB + 2 + 2 * kItemRing + 8;
+    static constexpr int NBAR = 3 * QST + 3 * KST + 2 * VST + 2 * NPB + NSB + 2 + 2 + 2 * kItemRing;
     static constexpr int SMEM_BYTES = BAR_OFF + 8 * NBAR + 16 + 1024;
     static constexpr uint64_t SWZ = ROWB == 128 ? 2 : 4;
     static_assert(ROWB == 128 || ROWB == 64, "swizzle span");
@@ -150,7 +160,8 @@ template <int D, bool PAIR, bool ROPE>
 __global__ void __launch_bounds__(Threads<ROPE>::N, 1)
 attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
     using C = Cfg<D, PAIR>;
-    constexpr int KST = C::KST, VST = C::VST, QST = C::QST, NV = C::NV, NSB = C::NSB, KB = C::KB;
+    constexpr int KST = C::KST, VST = C::VST, QST = C::QST, NV = C::NV, NSB = C::NSB, NPB = C::NPB, KB = C::KB;
+    constexpr bool APART = C::APART;
     extern __shared__ unsigned char smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
@@ -161,8 +172,8 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
     const uint32_t q_full = bars, q_free = q_full + 8 * QST, q_rot = q_free + 8 * QST;
     const uint32_t k_full = q_rot + 8 * QST, k_free = k_full + 8 * KST, k_rot = k_free + 8 * KST;
     const uint32_t v_full = k_rot + 8 * KST, v_free = v_full + 8 * VST;
-    const uint32_t s_full = v_free + 8 * VST, p_ready = s_full + 8 * NSB, buf_free = p_ready + 8 * NSB, o_full = buf_free + 8 * NSB;
-    const uint32_t item_full = o_full + 16, item_free = item_full + 8 * kItemRing, turn = item_free + 8 * kItemRing;
+    const uint32_t s_full = v_free + 8 * VST, p_ready = s_full + 8 * NPB, buf_free = p_ready + 8 * NPB, o_full = buf_free + 8 * NSB;
+    const uint32_t item_full = o_full + 16, item_free = item_full + 8 * kItemRing, p_free = item_free + 8 * kItemRing;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + C::BAR_OFF + 8 * C::NBAR);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
@@ -172,9 +183,10 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
         for (int i = 0; i < QST; ++i) { mbar_init(q_full + 8 * i, 1); mbar_init(q_free + 8 * i, 1); mbar_init(q_rot + 8 * i, 4); }
         for (int i = 0; i < KST; ++i) { mbar_init(k_full + 8 * i, 1); mbar_init(k_free + 8 * i, 1); mbar_init(k_rot + 8 * i, 4); }
         for (int i = 0; i < VST; ++i) { mbar_init(v_full + 8 * i, 1); mbar_init(v_free + 8 * i, 1); }
-        for (int i = 0; i < NSB; ++i) { mbar_init(s_full + 8 * i, 1); mbar_init(p_ready + 8 * i, 4); mbar_init(buf_free + 8 * i, 1); }
+        for (int i = 0; i < NPB; ++i) { mbar_init(s_full + 8 * i, 1); mbar_init(p_ready + 8 * i, 4); }
+        for (int i = 0; i < NSB; ++i) mbar_init(buf_free + 8 * i, APART ? 4 : 1);
         for (int i = 0; i < 2; ++i) mbar_init(o_full + 8 * i, 1);
-        for (int i = 0; i < 8; ++i) mbar_init(turn + 8 * i, 1);
+        for (int i = 0; i < 2; ++i) mbar_init(p_free + 8 * i, 1);
         for (int i = 0; i < kItemRing; ++i) { mbar_init(item_full + 8 * i, 1); mbar_init(item_free + 8 * i, ROPE ? 15 : 11); }
         *abort_flag = 0;
         fence_barrier_init();
@@ -317,7 +329,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
 #pragma unroll
                             for (int k = 0; k < D / 16; ++k)
                                 umma_bf16<1>(acc, qd + (C::koff(C::QSUB, 16 * k) >> 4), kd + (C::koff(C::SUB, 16 * k) >> 4), idesc, k != 0);
-                            umma_commit<1>(s_full + 8 * sbuf);
+                            umma_commit<1>(s_full + 8 * (APART ? t : sbuf));
                             if (t) {
                                 umma_commit<1>(k_free + 8 * kst);
                                 if (left == 1) umma_commit<1>(q_free + 8 * qst);
@@ -357,7 +369,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
 #pragma unroll 1
                     for (uint32_t t = 0; t < 2; ++t) {
                         const uint64_t vd = vd0 + (uint64_t)((vst * C::TILE + (PAIR && D == 64 ? t * C::SUB : 0)) >> 4);
-                        const uint32_t pa = tmem + vbuf * KB, oa = tmem + C::O_COL + t * C::O_STRIDE;
+                        const uint32_t pa = tmem + C::P_COL + vbuf * C::P_STRIDE, oa = tmem + C::O_COL + t * C::O_STRIDE;
                         if (!(ok = mbar_wait_warp(p_ready + 8 * vbuf, pph, abort_flag))) break;
                         tc_fence_after();
                         if (elect_one()) {
@@ -365,12 +377,12 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
 #pragma unroll
                             for (int kk = 1; kk < KB / 16; ++kk)
                                 if (kk * 16 < kpad) umma_ts(oa, pa + kk * 8, vd + (uint64_t)((16 * C::ROWB) >> 4) * kk, idesc_o, 1u);
-                            umma_commit<1>(buf_free + 8 * vbuf);
+                            umma_commit<1>((APART ? p_free : buf_free) + 8 * vbuf);
                             if (last) umma_commit<1>(o_full + 8 * t);
                             if (t) umma_commit<1>(v_free + 8 * vst);
                         }
                         __syncwarp();
-                        if (++vbuf == NSB) { vbuf = 0; pph ^= 1; }
+                        if (++vbuf == NPB) { vbuf = 0; pph ^= 1; }
                     }
                     first = false;
                     if (++vst == VST) { vst = 0; vph ^= 1; }
@@ -440,13 +452,6 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
         const float scale = p.scale_log2e;
         uint32_t buf = t, sph = 0;   // score buffer and its parity; jobs t, t + 2, t + 4, ..
         uint32_t pbuf = 0, pph = 0;  // the same of this tile's previous block
-        // With short blocks the two tiles' warps of a scheduler take turns on the exponential unit, handing over a chunk before
-        // the end: they otherwise fall into step, load and reduce at the same time and leave the unit idle meanwhile
-        // (32 q / 8 kv heads of 128, 8 x 2048: 479 -> 462 us).  A block of 128 keys is long enough for that not to matter,
-        // and a lone warp does not fill the unit (heads of 64 181 -> 205), so there they share it freely.
-        constexpr bool TURNS = KB == 64;
-        const uint32_t my_turn = turn + 8 * (t * 4 + quad), other_turn = turn + 8 * ((t ^ 1) * 4 + quad);
-        uint32_t tph = t ^ 1;        // tile 0 begins: a fresh barrier passes the wait for the phase before its first
         bool ok = true;
         Item it;
         for (uint32_t n = 0; ok; ++n) {
@@ -459,14 +464,28 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
             uint64_t l2[2] = {0, 0};
             for (int j = it.j0; j < it.nb; ++j) {
                 if (!(ok = mbar_wait_warp(s_full + 8 * buf, sph, abort_flag))) break;
+                if (APART && !live) {
+                    if (lane == 0) mbar_arrive(buf_free);
+                    if (!(ok = mbar_wait_warp(p_free + 8 * t, sph ^ 1, abort_flag))) break;
+                }
                 if (live) {
                     tc_fence_after();
-                    const uint32_t s_col = tl + buf * KB;
+                    const uint32_t s_col = tl + (APART ? 0 : buf * KB);
+                    const uint32_t p_col = APART ? tl + C::P_COL + t * C::P_STRIDE : s_col;
                     const int k0 = j * KB;
                     uint32_t s[NCH][32];
 #pragma unroll
                     for (int c = 0; c < NCH; ++c) tmem_ld_32x32(s_col + 32 * c, s[c]);
                     tmem_ld_wait();
+                    bool p_done = false;
+                    if (APART) {
+                        // the scores are in registers: their buffer is the other tile's
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(buf_free);
+                        // this tile's previous product: P's buffer is free and O complete (asked for ahead of its use)
+                        p_done = mbar_test_wait(p_free + 8 * t, sph ^ 1);
+                    }
                     const bool whole = k0 + KB <= it.hi && (!p.positional || (k0 + KB - 1 <= wr0 && k0 > wr0 + 31 - p.window));
                     if (!whole) {
                         // visible keys of this row: columns first .. lim; one bit per column
@@ -494,13 +513,17 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
                         }
                         m_blk = fmaxf(max3f(mx[0], mx[1], mx[2]), mx[3]) * scale;
                     }
+                    if (APART) {
+                        if (!__all_sync(0xffffffffu, p_done) && !(ok = mbar_wait_warp(p_free + 8 * t, sph ^ 1, abort_flag))) break;
+                        tc_fence_after();
+                    }
                     if (j == it.j0) {
                         m_ref = m_blk;
                     } else {
                         const bool need = m_blk > m_ref + kRescaleAbove;
                         if (__any_sync(0xffffffffu, need)) {
                             // the products issued so far must have landed in O
-                            if (!(ok = mbar_wait_warp(buf_free + 8 * pbuf, pph, abort_flag))) break;
+                            if (!APART && !(ok = mbar_wait_warp(buf_free + 8 * pbuf, pph, abort_flag))) break;
                             tc_fence_after();
                             const float alpha = need ? ex2f(m_ref - m_blk) : 1.f;
                             if (need) m_ref = m_blk;
@@ -520,12 +543,10 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
                     }
                     const float neg = m_ref == -INFINITY ? 0.f : -m_ref;
                     const uint64_t sc2 = pack_f32x2(scale, scale), ng2 = pack_f32x2(neg, neg);
-                    if (TURNS && !(ok = mbar_wait_warp(my_turn, tph, abort_flag))) break;
                     // straight line over all chunks, masked ones included: a branch per chunk drains the exponential unit
                     // each time, and a second copy of the code costs more in instruction fetches than it saves
 #pragma unroll
                     for (int c = 0; c < NCH; ++c) {
-                        if (TURNS && c == NCH - 1 && lane == 0) mbar_arrive(other_turn);
                         uint32_t pk[16];
 #pragma unroll
                         for (int i = 0; i < 16; ++i) {
@@ -536,21 +557,18 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
                             l2[i & 1] = add_f32x2(l2[i & 1], pack_f32x2(x0, x1));
                             pk[i] = pack_bf16(x0, x1);
                         }
-                        tmem_st_32x16(s_col + 16 * c, pk);
+                        tmem_st_32x16(p_col + 16 * c, pk);
                     }
                     tmem_st_wait();
                     tc_fence_before();
-                } else if (TURNS) {
-                    if (!(ok = mbar_wait_warp(my_turn, tph, abort_flag))) break;
-                    if (lane == 0) mbar_arrive(other_turn);
                 }
-                tph ^= 1;
                 __syncwarp();
                 if (lane == 0) mbar_arrive(p_ready + 8 * buf);
                 pbuf = buf;
                 pph = sph;
-                buf += 2;
-                if (buf >= NSB) { buf -= NSB; sph ^= 1; }
+                if (!APART) buf += 2;
+                if (APART) sph ^= 1;
+                else if (buf >= NSB) { buf -= NSB; sph ^= 1; }
             }
             if (!ok) break;
             // ---- O / row sum -> bf16 -> global ----

@@ -437,7 +437,7 @@ rlx_status_t launch_attention_fwd(const bf16* qkv, int rows, const int32_t* seq_
     const int grid = (int)std::min<long long>((long long)p.qtiles * B * p.units, sm_count());
     CUtensorMap tm;
     const uint32_t cols = (d == 32 && !pair) ? 32 : 64;
-    if (!make_tmap(&tm, qkv, (uint64_t)rows, (uint64_t)p.H + 2 * p.Hkv, d == 128 ? tcat::Cfg<128, false>::KB : tcat::Cfg<64, true>::KB, cols,
+    if (!make_tmap(&tm, qkv, (uint64_t)rows, (uint64_t)p.H + 2 * p.Hkv, tcat::Cfg<64, true>::KB, cols,
                    cols == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B))
         return RLX_ERR_CUDA;
 #define RLX_ATT_FWD(D, PAIR)                                                                                                   \
@@ -460,11 +460,11 @@ rlx_status_t launch_attention_fwd(const bf16* qkv, int rows, const int32_t* seq_
 }
 
 // Where the tcgen05 kernel replaces the mma.sync one (measured on packed batches, us old / new):
-//   head_dim 128: everywhere (16 prompts of 1024..4096, causal, 32 q / 8 kv heads 3561 / 1044; 64 of 16..256 75 / 43)
-//   head_dim 64: longer than one 128-row tile (causal 1024..4096, 16 heads 907 / 477; 16..256 39.6 / 35.2; window 64
-//     over 100..1500 67 / 66; but 16..128 21.1 / 22.3: one tile and one block per item are all set-up and latency)
+//   head_dim 128: everywhere (16 prompts of 1024..4096, causal, 32 q / 8 kv heads 3561 / 873; 64 of 16..256 75 / 43)
+//   head_dim 64: longer than one 128-row tile (causal 1024..4096, 16 heads 907 / 369; 16..256 39.6 / 33.6; window 512
+//     over 100..1500 140 / 80; but 16..128 21.1 / 23.1: one tile and one block per item are all set-up and latency)
 //   head_dim 32: only where many blocks per tile pay for its fixed costs: longer than 512 keys, no short window
-//     (causal 400..2000 156 / 124; 16..256 25.8 / 29.3; window 64 over 100..1500 48 / 54)
+//     (causal 400..2000 156 / 107; 16..256 25.8 / 28.2; window 64 over 100..1500 47.7 / 48.5)
 bool attention_fwd_pays(int d, int max_len, bool positional, int window) {
     if (d == 128) return true;
     if (d == 64) return max_len > rlx::tcat::kTile;
