@@ -622,7 +622,7 @@ def run_attention_kind(args):
                                f"mask {args.mask}" + (f"({args.window})" if args.mask == "sliding" else "") +
                                (", rotary q,k" if args.rope else ""), "l2": "256 MiB flush write between steps"},
         "gpu_launches": args.steps, "clocks": sampler.summary(),
-        "roofline": {"kernel": f"attention_bf16_kernel<{d}>", "bound": "alu", "achieved": exps / (p50 * 1e-3) / 1e12,
+        "roofline": {"kernel": "attention_bf16_kernel<32>" if d == 32 and args.mask == "sliding" and args.window <= 256 else f"attention_fwd_kernel<{d}>", "bound": "alu", "achieved": exps / (p50 * 1e-3) / 1e12,
                      "peak": EXP_PEAK_TEXP_S, "unit": "Texp/s", "frac": exps / (p50 * 1e-3) / 1e12 / EXP_PEAK_TEXP_S,
                      "traffic": None, "tensor_tflops": flops / (p50 * 1e-3) / 1e12,
                      "tensor_frac_of_" + peak_kind: flops / (p50 * 1e-3) / 1e12 / peaks["bf16_tflops"],
@@ -773,7 +773,7 @@ def run_mx_matmul(args):
         "config": {"workload": "M=36736 tokens, N=384, K=1536 (FFN-down shape), both operands FP8 E4M3 with E8M0 scales per 32; "
                                "the other shapes are in `shapes`", "l2": "256 MiB flush write between steps"},
         "gpu_launches": args.steps, "clocks": sampler.summary(),
-        "roofline": {"kernel": "gemm_mx192_tcgen05_kernel", "bound": "tensor", "achieved": r["tflops"], "peak": fp8_peak,
+        "roofline": {"kernel": "gemm_mx_tcgen05_kernel", "bound": "tensor", "achieved": r["tflops"], "peak": fp8_peak,
                      "unit": "TFLOP/s", "frac": r["frac_of_fp8_peak"], "traffic": None,
                      "peak_source": peak_kind + "; FP8 peak taken as 2 x the measured bf16 figure (no FP8 peak measured)"},
         "e2e": None, "cpu_baseline": None, "shapes": rows,
