@@ -147,9 +147,10 @@ struct Params {
 template <bool ROPE>
 struct Threads {
     static constexpr int N = ROPE ? 512 : 384;
-    // 256 softmax threads and the rest share what the launch holds: 512 x 128 = 256 x (192 + 64), 384 x 168 > 256 x 208 + 128 x 80
-    static constexpr int REG_SOFTMAX = ROPE ? 192 : 208;
-    static constexpr int REG_REST = ROPE ? 64 : 80;
+    // 256 softmax threads and the rest share what the launch holds: 512 x 128 = 256 x (176 + 80), 384 x 168 > 256 x 208 + 128 x 80
+    // (with 192 + 64 the rotators, and with 168 + 88 the softmax, spilled: windowed prompts of heads of 64 104.6 -> 100.4 us)
+    static constexpr int REG_SOFTMAX = ROPE ? 176 : 208;
+    static constexpr int REG_REST = 80;
 };
 
 struct Item {
