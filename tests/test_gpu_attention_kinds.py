@@ -256,3 +256,26 @@ def test_tile_and_block_edges_of_the_tcgen05_kernel(rlx, d, hq, hkv, kind, windo
         err = np.abs(got[:total] - ref)
         assert np.isfinite(err).all() and err.max() <= tol, (float(err.max()), tol)
         assert np.sqrt((err ** 2).mean()) <= 2 * BF16_U * vmax
+
+
+@pytest.mark.parametrize("d,hq,hkv", [(32, 2, 2), (64, 2, 2), (64, 3, 3), (64, 4, 2), (128, 4, 2)])
+@pytest.mark.parametrize("kind,window", [(NONE, 0), (CAUSAL, 0), (SLIDING, 300)])
+def test_row_sums_are_those_of_the_rounded_probabilities(rlx, d, hq, hkv, kind, window):
+    """v is 1 or the next bf16 number, 1 + 2^-7, so an output says which of the two the weighted mean is nearer to.
+
+    A weight's rounding to bf16 (u relative) that stands in the numerator and in the row sum alike moves the mean by at
+    most u max|v - mean| <= u 2^-7; the fp32 sums (at most 45 accumulation steps of 2^-23 and 180 additions of 2^-24, relative
+    to a mean of one) by less than 2^-15.  A row sum of the unrounded weights moves it by up to u itself, 128 times as much."""
+    rng = np.random.default_rng(d + hq)
+    lengths = [700, 130, 517]
+    total, start = sum(lengths), np.array([0, 700, 830], np.int32)
+    qkv = rand_bf16(rng, (total, (hq + 2 * hkv) * d))
+    qkv[:, :hq * d] *= 2                       # a few keys carry most of a row's weight
+    qkv[:, (hq + hkv) * d:] = 1 + 2.0 ** -7 * rng.integers(0, 2, (total, hkv * d))
+    got = to_np64(rlx.attention_kind_bf16(bf16_dev(qkv), i32_dev(start), i32_dev(np.array(lengths)), 700, hq, kind, window,
+                                          num_kv_heads=hkv))
+    ref = ak.attention_packed(qkv.astype(np.float64), start, np.array(lengths), hq, kind, window, None, num_kv_heads=hkv)
+    clear = np.abs(ref - (1 + 2.0 ** -8)) > BF16_U * 2.0 ** -7 + 2.0 ** -15
+    assert clear.mean() > 0.9
+    want = np.where(ref > 1 + 2.0 ** -8, 1 + 2.0 ** -7, 1.0)
+    assert np.array_equal(got[clear], want[clear]), float((got[clear] != want[clear]).mean())
