@@ -447,8 +447,9 @@ rlx_status_t rlx_attention_packed_bf16(const void *qkv_bf16, int32_t rows, const
  * memory, 16-byte aligned; seq_len[b] <= max_len <= RLX_ATTENTION_KIND_MAX_LEN).  rope_cos and
  * rope_sin are device fp32 tables [max_len, head_dim/2] (row = position, 16-byte aligned) holding
  * cos / sin of position * theta^(-2j/head_dim), or both NULL for no rotation.  `window` is read for
- * RLX_MASK_SLIDING_WINDOW only.  head_dim in {32, 64, 128}.  Key blocks that no row of a 128-row query
- * tile can see are neither loaded nor multiplied.  Asynchronous on cuda_stream; the caller owns
+ * RLX_MASK_SLIDING_WINDOW only.  head_dim in {32, 64, 128}.  128-key blocks that no row of a 128-row query
+ * tile can see are not multiplied for that tile.  In the blocks that it does see, a masked key has weight zero, so an
+ * infinite or NaN v there can reach any row of the tile (0 x inf).  Asynchronous on cuda_stream; the caller owns
  * every buffer; nothing is allocated.  Errors: RLX_ERR_INVALID_ARG for null / misaligned pointers,
  * a lone rope table, an unknown kind or window < 1; RLX_ERR_UNSUPPORTED for other head sizes or
  * lengths beyond the maximum.

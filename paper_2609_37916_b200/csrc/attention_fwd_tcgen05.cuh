@@ -97,7 +97,7 @@ __device__ __forceinline__ void add_bf16x2(float& lo, float& hi, uint32_t v) {
 }
 template <int D, bool PAIR>
 struct Cfg {
-    static constexpr int KB = 128;                            // keys per block
+    static constexpr int KB = kTile;                          // keys per block
     // The accumulators take 2 * D columns of tensor memory.  Heads of 128 leave room for one score buffer and a buffer for
     // P per tile (APART); otherwise three score buffers, over which P is written.
     static constexpr bool APART = D == 128;
@@ -165,6 +165,17 @@ struct Threads {
 struct Item {
     int valid, unit, q0, len, row0, j0, nb, hi;
 };
+// Two row tiles of one head walk the item's blocks j0 .. nb - 1 together, but a block that no row of a tile can see is not
+// multiplied for it: a non-finite v there would reach it (0 x inf).  Tile 0 has the blocks in front of the first one's end, tile 1
+// those from the second one's start on.
+__device__ __forceinline__ int tile0_end(const Params& p, const Item& it) {
+    return p.rows_mode && p.positional ? min(it.nb, it.q0 / kTile + 1) : it.nb;
+}
+__device__ __forceinline__ int tile1_begin(const Params& p, const Item& it) {
+    if (!p.rows_mode) return it.j0;
+    if (it.len <= it.q0 + kTile) return it.nb;   // no row of it exists
+    return p.positional ? max(0, it.q0 + kTile - p.window + 1) / kTile : it.j0;
+}
 
 template <int D, bool PAIR, bool ROPE>
 __global__ void __launch_bounds__(Threads<ROPE>::N, 1)
@@ -324,6 +335,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
             for (uint32_t n = 0; ok; ++n) {
                 if (next_item(n, it) != 1 || !mbar_wait_warp(q_rdy + 8 * qst, qph, abort_flag)) break;
                 const uint64_t qd1 = qd0 + (uint64_t)((qst * C::QB) >> 4);
+                const int end0 = tile0_end(p, it), begin1 = tile1_begin(p, it);
                 for (int left = it.nb - it.j0; left > 0 && ok; --left) {
                     if (!(ok = mbar_wait_warp(k_rdy + 8 * kst, kph, abort_flag))) break;
                     const uint64_t kd1 = kd0 + (uint64_t)((kst * C::TILE) >> 4);
@@ -335,10 +347,13 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
                         const uint64_t qd = qd1 + (uint64_t)((t * (PAIR ? C::koff(C::QSUB, D) : C::QTILE)) >> 4);
                         const uint64_t kd = kd1 + (uint64_t)((PAIR ? t * C::koff(C::SUB, D) : 0) >> 4);
                         const uint32_t acc = tmem + sbuf * KB;
+                        const bool seen = t ? it.nb - left >= begin1 : it.nb - left < end0;
                         if (elect_one()) {
+                            if (seen) {
 #pragma unroll
-                            for (int k = 0; k < D / 16; ++k)
-                                umma_bf16<1>(acc, qd + (C::koff(C::QSUB, 16 * k) >> 4), kd + (C::koff(C::SUB, 16 * k) >> 4), idesc, k != 0);
+                                for (int k = 0; k < D / 16; ++k)
+                                    umma_bf16<1>(acc, qd + (C::koff(C::QSUB, 16 * k) >> 4), kd + (C::koff(C::SUB, 16 * k) >> 4), idesc, k != 0);
+                            }
                             umma_commit<1>(s_full + 8 * (APART ? t : sbuf));
                             if (t) {
                                 umma_commit<1>(k_free + 8 * kst);
@@ -361,7 +376,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
             Item it;
             for (uint32_t n = 0; ok; ++n) {
                 if (next_item(n, it) != 1) break;
-                bool first = true;
+                const int end0 = tile0_end(p, it), begin1 = tile1_begin(p, it);
                 for (int left = it.nb - it.j0; left > 0 && ok; --left) {
                     const bool last = left == 1;
                     const int keys = last ? it.hi - (it.nb - 1) * KB : KB, kpad = (keys + 15) & ~15;
@@ -382,11 +397,14 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
                         const uint32_t pa = tmem + C::P_COL + vbuf * C::P_STRIDE, oa = tmem + C::O_COL + t * C::O_STRIDE;
                         if (!(ok = mbar_wait_warp(p_ready + 8 * vbuf, pph, abort_flag))) break;
                         tc_fence_after();
+                        const int j = it.nb - left;
                         if (elect_one()) {
-                            umma_ts(oa, pa, vd, idesc_o, first ? 0u : 1u);
+                            if (t ? j >= begin1 : j < end0) {
+                                umma_ts(oa, pa, vd, idesc_o, j == (t ? begin1 : it.j0) ? 0u : 1u);
 #pragma unroll
-                            for (int kk = 1; kk < KB / 16; ++kk)
-                                if (kk * 16 < kpad) umma_ts(oa, pa + kk * 8, vd + (uint64_t)((16 * C::ROWB) >> 4) * kk, idesc_o, 1u);
+                                for (int kk = 1; kk < KB / 16; ++kk)
+                                    if (kk * 16 < kpad) umma_ts(oa, pa + kk * 8, vd + (uint64_t)((16 * C::ROWB) >> 4) * kk, idesc_o, 1u);
+                            }
                             umma_commit<1>((APART ? p_free : buf_free) + 8 * vbuf);
                             if (last) umma_commit<1>(o_full + 8 * t);
                             if (t) umma_commit<1>(v_free + 8 * vst);
@@ -394,7 +412,6 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
                         __syncwarp();
                         if (++vbuf == NPB) { vbuf = 0; pph ^= 1; }
                     }
-                    first = false;
                     if (++vst == VST) { vst = 0; vph ^= 1; }
                 }
             }
@@ -470,15 +487,17 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
             const int wr0 = q0 + quad * 32, row = wr0 + lane;      // rows of this warp, of this thread (position in the sequence)
             const bool live = wr0 < it.len;
             const int head = (PAIR || !p.rows_mode) ? 2 * it.unit + t : it.unit;
+            const int jb = t ? tile1_begin(p, it) : it.j0, je = t ? it.nb : tile0_end(p, it);
             float m_ref = -INFINITY;
             float l4[4] = {0.f, 0.f, 0.f, 0.f};
             for (int j = it.j0; j < it.nb; ++j) {
                 if (!(ok = mbar_wait_warp(s_full + 8 * buf, sph, abort_flag))) break;
-                if (APART && !live) {
+                const bool seen = live && j >= jb && j < je;
+                if (APART && !seen) {
                     if (lane == 0) mbar_arrive(buf_free);
                     if (!(ok = mbar_wait_warp(p_free + 8 * t, sph ^ 1, abort_flag))) break;
                 }
-                if (live) {
+                if (seen) {
                     tc_fence_after();
                     const uint32_t s_col = tl + (APART ? 0 : buf * KB);
                     const uint32_t p_col = APART ? tl + C::P_COL + t * C::P_STRIDE : s_col;
@@ -527,7 +546,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
                         if (!__all_sync(0xffffffffu, p_done) && !(ok = mbar_wait_warp(p_free + 8 * t, sph ^ 1, abort_flag))) break;
                         tc_fence_after();
                     }
-                    if (j == it.j0) {
+                    if (j == jb) {
                         m_ref = m_blk;
                     } else {
                         const bool need = m_blk > m_ref + kRescaleAbove;

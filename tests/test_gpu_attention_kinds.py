@@ -279,3 +279,34 @@ def test_row_sums_are_those_of_the_rounded_probabilities(rlx, d, hq, hkv, kind, 
     assert clear.mean() > 0.9
     want = np.where(ref > 1 + 2.0 ** -8, 1 + 2.0 ** -7, 1.0)
     assert np.array_equal(got[clear], want[clear]), float((got[clear] != want[clear]).mean())
+
+
+@pytest.mark.parametrize("d,hq,hkv", [(32, 3, 3), (64, 2, 2), (64, 1, 1), (64, 6, 2), (64, 4, 2), (128, 1, 1), (128, 4, 4), (128, 5, 1),
+                                      (128, 4, 2)])
+@pytest.mark.parametrize("theta", [None, 10000.0])
+def test_blocks_that_a_row_tile_cannot_see_are_not_multiplied(rlx, d, hq, hkv, theta):
+    """Infinite and NaN v in 128-key blocks that no row of a 128-row tile can see leave its rows as they are, bit for bit:
+    later blocks under the causal mask, earlier ones under a window, in the first and the second tile of 256 rows."""
+    rng = np.random.default_rng(d + hq)
+    lengths = np.array([900, 640], np.int32)
+    start = np.array([0, 900], np.int32)
+    qkv = rand_bf16(rng, (1540, (hq + 2 * hkv) * d))
+    rope = None if theta is None else rlx.rope_tables(900, d, theta)
+
+    def run(a, kind, window):
+        return to_np64(rlx.attention_kind_bf16(bf16_dev(a), i32_dev(start), i32_dev(lengths), 900, hq, kind, window, rope,
+                                               num_kv_heads=hkv))
+    v = slice((hq + hkv) * d, None)
+    for tile in (1, 2, 3, 4):
+        for kind, window, bad, rows in ((CAUSAL, 0, slice(128 * tile, None), slice(0, 128 * tile)),
+                                        (SLIDING, 300, slice(128 * tile, None), slice(0, 128 * tile)),
+                                        # rows from 128 t + 256 on see keys from 128 t + 1 on
+                                        (SLIDING, 256, slice(0, 128 * tile), slice(128 * tile + 256, None))):
+            clean = run(qkv, kind, window)
+            poisoned = qkv.copy()
+            for s0, n in zip(start, lengths):
+                poisoned[s0:s0 + n][bad, v] = np.inf
+                poisoned[s0:s0 + n][bad, v][::3] = np.nan
+            got = run(poisoned, kind, window)
+            for s0, n in zip(start, lengths):
+                assert np.array_equal(got[s0:s0 + n][rows], clean[s0:s0 + n][rows]), (tile, kind, window)
