@@ -4,7 +4,6 @@
 // on registers (mean, then centred sum of squares), biased variance, eps inside the square root.
 #pragma once
 #include "common.cuh"
-#include "gemm_tcgen05.cuh"
 
 namespace rlx {
 
@@ -524,6 +523,7 @@ ln_fold_weights_kernel(const __grid_constant__ FoldList fl) {
 // z * rstd over its rows for its 8 columns; sum_r LN(z)_rc = gamma_c * (sum_r z_rc rstd_r + sum_r b_r)
 // + n * beta_c.  Fixed-order reductions (deterministic).
 constexpr int kPoolMaxRows = 512;
+constexpr int kPoolMaxPartials = 32;   // hidden <= 1024, a multiple of 128: 4, 8, .. 32 partials a row
 __global__ void __launch_bounds__(kPoolThreads)
 pool_ln_l2norm_kernel(const __nv_bfloat16* __restrict__ z, const int32_t* __restrict__ mask, float* __restrict__ out, int S,
                       int H, const int32_t* __restrict__ seq_start, const int32_t* __restrict__ seq_len,
@@ -548,8 +548,25 @@ pool_ln_l2norm_kernel(const __nv_bfloat16* __restrict__ z, const int32_t* __rest
     for (int r = threadIdx.x; r < nrows; r += kPoolThreads) {
         float a = 0.f, bb = 0.f;
         if (packed || __ldg(mb + r) != 0) {
-            float mu, rstd;
-            tc::row_stats_from_partials(stats + (row0 + r) * (size_t)P, P, eps, mu, rstd);
+            // Chan's combination of the row's partials, centred: the mean first, then the squares of the distances from it.  In one
+            // pass (mean of the squares less the square of the mean) a row with a mean of 256 deviations loses 1e-3 of its
+            // variance.  All partials are requested together and kept: read again in a loop they cost 4 us at 12 x 768.
+            const float4* sp = reinterpret_cast<const float4*>(stats + (row0 + r) * (size_t)P);
+            float4 q[kPoolMaxPartials / 2];
+#pragma unroll
+            for (int i = 0; i < kPoolMaxPartials / 2; ++i) q[i] = 2 * i < P ? __ldg(sp + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+            float sm = 0.f, m2 = 0.f;
+#pragma unroll
+            for (int i = 0; i < kPoolMaxPartials / 2; ++i) sm = sm + q[i].x + q[i].z;
+            const float mu = sm / (float)P;
+#pragma unroll
+            for (int i = 0; i < kPoolMaxPartials / 2; ++i)
+                if (2 * i < P) {
+                    const float d0 = q[i].x - mu, d1 = q[i].z - mu;
+                    m2 += q[i].y + 32.f * d0 * d0;
+                    m2 += q[i].w + 32.f * d1 * d1;
+                }
+            const float rstd = 1.0f / sqrtf(m2 / (32.f * (float)P) + eps);
             a = rstd;
             bb = -rstd * mu;
             ++cnt;

@@ -9,7 +9,7 @@ torch = pytest.importorskip("torch")
 
 from gpu_common import cosine_rows, i32_dev, to_np64  # noqa: E402
 from oracle import oracle  # noqa: E402
-from synth.inputs import CONFIGS, EncoderConfig, make_inputs  # noqa: E402
+from synth.inputs import CONFIGS, make_inputs  # noqa: E402
 
 pytestmark = pytest.mark.gpu
 
@@ -245,6 +245,27 @@ def test_attention_kernel_choice_at_its_edges(rlx, name, B, S):
         got, status = run_gpu(rlx, inp, weights=w, flags=flags)
         assert status == 0
         check(got[pick], ref, inp.lengths[pick])
+
+
+@pytest.mark.parametrize("seed", range(4))
+def test_last_layernorm_of_rows_with_a_large_mean(rlx, seed):
+    """Rows in front of the last LayerNorm with a mean of 256 deviations: the LayerNorm folded into the pooling keeps its
+    fp32 precision.  The layer is set up so that those rows are b2 alone (w2 = 0, ln1 = 0), numbers that bf16 holds exactly.
+
+    Bound: z a and the sum of b are of the size of the mean, 258 deviations, and are rounded to fp32 at most four times in all;
+    the embedding is that over the length of the unscaled row, at least sqrt(H)."""
+    rng = np.random.default_rng(seed)
+    inp = make_inputs(CONFIGS["c1"], batch=3, seq=16, num_layers=1, lengths=[1, 1, 1])
+    H, layer = inp.cfg.hidden, inp.layers[0]
+    layer["b2"] = (256 + 2 * rng.integers(0, 2, H)).astype(np.float32)
+    layer["ln2_b"] = (0.5 * rng.choice((-1.0, 1.0), H)).astype(np.float32)
+    layer["ln2_g"] = np.ones(H, np.float32)
+    for name in ("w2", "ln1_g", "ln1_b", "b1"):
+        layer[name] = np.zeros_like(layer[name])
+    ref = oracle.encoder_forward(inp.cfg, inp.ids, inp.mask, inp.params, inp.layers)
+    got, status = run_gpu(rlx, inp, flags=0x200)
+    assert status == 0
+    assert np.abs(got - ref).max() <= 4 * 258 * 2.0 ** -24 / np.sqrt(H), np.abs(got - ref).max()
 
 
 def test_degenerate_lengths_zero_one_full(rlx):
