@@ -654,6 +654,11 @@ struct LnFold {
     float eps = 0.f;
 };
 
+// Sub-batches of a chunked call take the kernel choice of the whole call (its padded token count): a short last one would
+// otherwise fold its LayerNorms, split its contractions or attend with another kernel, and chunking would change results.
+thread_local long long g_whole_call_tokens = 0;
+long long call_tokens(int B, int S) { return g_whole_call_tokens > 0 ? g_whole_call_tokens : (long long)B * S; }
+
 // CTAs per 128 x 64 tile along K (1: do not split).  A long contraction on a few tiles is bound by one SM's operand feed;
 // four CTAs per tile while they all fit beside each other, two while two thirds of them do -- the row count is the
 // padded one, and a batch whose every position is valid then runs two half-length rounds instead of one.  Taken by
@@ -661,7 +666,8 @@ struct LnFold {
 // fused feed-forward kernel shares bit for bit.
 int pick_split_k(int M, int N, int K, int epi) {
     if (K < 1536 || N % rlx::tcsk::kBN != 0 || (epi > 2 && epi < 5)) return 1;
-    const int tiles = (M + rlx::tc::BLOCK_M - 1) / rlx::tc::BLOCK_M * (N / rlx::tcsk::kBN), sms = sm_count();
+    const long long rows = std::max<long long>(M, g_whole_call_tokens);
+    const long long tiles = (rows + rlx::tc::BLOCK_M - 1) / rlx::tc::BLOCK_M * (N / rlx::tcsk::kBN), sms = sm_count();
     return 4 * tiles <= sms ? 4 : 3 * tiles < 2 * sms - 8 ? 2 : 1;
 }
 
@@ -912,7 +918,7 @@ Arena plan_arena(int B, int S, int H, int F, int L = 0, bool fold = false) {
 bool uses_fused_ln(const rlx_encoder_config_t& c, int B, int S) {
     if ((c.flags & RLX_FLAG_GEMM_SIMT) || !(c.flags & RLX_FLAG_FUSED_LN)) return false;
     if (c.hidden != 256 && c.hidden != 384 && c.hidden != 512) return false;
-    return (long long)B * S >= 128ll * sm_count_of(c.device);
+    return call_tokens(B, S) >= 128ll * sm_count_of(c.device);
 }
 
 // Everything of a layer behind the attention in one kernel (out-projection, residual, LayerNorm, FFN-up, GELU,
@@ -923,9 +929,6 @@ bool uses_fused_ln(const rlx_encoder_config_t& c, int B, int S) {
 // valid rows on (8972 valid: -1 %, 37 k: -15 %) and loses up to 20 % on a heavily padded batch (20480 padded,
 // 2729 valid: 393 against 330 us), so the padded threshold is set where a half-empty batch still breaks even.
 constexpr long long kAutoFusedFfnMinTokens = 32768;
-// Sub-batches of a chunked call take the kernel choice of the whole call (its padded token count), so that
-// chunking never changes which kernels compute a row.
-thread_local long long g_whole_call_tokens = 0;
 // Bodies of the IF / ELSE node of a captured forward are recorded with the choice forced (1: layer tail, 0: separate
 // kernels; -1: the host's rule).
 thread_local int g_force_layer_tail = -1;
@@ -940,8 +943,7 @@ bool uses_fold_ln(const rlx_encoder_config_t& c, int B, int S);
 bool uses_fused_ffn(const rlx_encoder_config_t& c, int B, int S) {
     if (g_force_layer_tail >= 0) return g_force_layer_tail == 1;
     if (c.flags & (RLX_FLAG_GEMM_SIMT | RLX_FLAG_FUSED_LN | RLX_FLAG_CLUSTER_LN | RLX_FLAG_NO_FUSED_FFN)) return false;
-    const long long tokens = g_whole_call_tokens > 0 ? g_whole_call_tokens : (long long)B * S;
-    if (!(c.flags & RLX_FLAG_FUSED_FFN) && tokens < kAutoFusedFfnMinTokens) return false;
+    if (!(c.flags & RLX_FLAG_FUSED_FFN) && call_tokens(B, S) < kAutoFusedFfnMinTokens) return false;
     return ffn_fused_supported(c.hidden, c.ffn) && !uses_fold_ln(c, B, S);
 }
 
@@ -976,7 +978,7 @@ bool uses_fold_ln(const rlx_encoder_config_t& c, int B, int S) {
     if (!can) return false;
     if (c.flags & RLX_FLAG_FOLD_LN) return true;
     const bool other_fusion = (c.flags & (RLX_FLAG_FUSED_LN | RLX_FLAG_CLUSTER_LN)) != 0;
-    return !g_no_auto_fold && !(c.flags & RLX_FLAG_NO_AUTO_FOLD) && !other_fusion && (long long)B * S <= kAutoFoldMaxTokens;
+    return !g_no_auto_fold && !(c.flags & RLX_FLAG_NO_AUTO_FOLD) && !other_fusion && call_tokens(B, S) <= kAutoFoldMaxTokens;
 }
 
 int kernels_in_forward(const rlx_encoder_config_t& c, int B, int S) {
@@ -996,9 +998,9 @@ int chunk_batch(int B, int S);
 //       what a layer waits for (16 x 192 218 / 201; but 256 x 192 983 / 1000, 61 x 203 431 / 438)
 bool uses_attention_fwd(const rlx_encoder_config_t& c, int B, int S) {
     if (c.flags & RLX_FLAG_ATTN_TCGEN05) return true;
-    const long long tokens = g_whole_call_tokens > 0 ? g_whole_call_tokens : (long long)B * S;
+    const long long tokens = call_tokens(B, S);
     constexpr int kT = rlx::tcat::kTile;
-    if (c.hidden / c.num_heads == 64) return S > 2 * kT || (S == 2 * kT && B > 1) || (S > kT && tokens >= 8192);
+    if (c.hidden / c.num_heads == 64) return S > 2 * kT || (S == 2 * kT && tokens > S) || (S > kT && tokens >= 8192);
     return S >= 2 * kT || (S >= kT + kT / 2 && tokens <= 4096);
 }
 

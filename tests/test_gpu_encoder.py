@@ -9,7 +9,7 @@ torch = pytest.importorskip("torch")
 
 from gpu_common import cosine_rows, i32_dev, to_np64  # noqa: E402
 from oracle import oracle  # noqa: E402
-from synth.inputs import CONFIGS, make_inputs  # noqa: E402
+from synth.inputs import CONFIGS, EncoderConfig, make_inputs  # noqa: E402
 
 pytestmark = pytest.mark.gpu
 
@@ -245,6 +245,21 @@ def test_attention_kernel_choice_at_its_edges(rlx, name, B, S):
         got, status = run_gpu(rlx, inp, weights=w, flags=flags)
         assert status == 0
         check(got[pick], ref, inp.lengths[pick])
+
+
+@pytest.mark.parametrize("heads", [2, 4])
+@pytest.mark.parametrize("flags", [0, 0x200, 0x400])   # the host's choice, folded LayerNorm, none folded
+def test_a_short_last_chunk_takes_the_kernels_of_the_whole_call(rlx, heads, flags):
+    """4033 x 256 positions run as 63 sub-batches of 64 sequences and one of a single sequence, a size at which a call of its own
+    would fold the LayerNorms, split the long contraction and take another attention kernel."""
+    cfg = EncoderConfig("chunks", 1, 128, heads, 1536, 4033, 256, 1, 256, 7)
+    inp = make_inputs(cfg)
+    w = rlx.upload_weights(inp.params, inp.layers)
+    whole, status = run_gpu(rlx, inp, flags=flags, weights=w)
+    chunked, cstatus = run_gpu(rlx, inp, flags=flags | 0x800, weights=w)
+    assert status == 0 and cstatus == 0
+    bad = np.flatnonzero((whole != chunked).any(1))
+    assert bad.size == 0, bad
 
 
 @pytest.mark.parametrize("seed", range(4))
