@@ -453,6 +453,10 @@ rlx_status_t rlx_attention_packed_bf16(const void *qkv_bf16, int32_t rows, const
  * every buffer; nothing is allocated.  Errors: RLX_ERR_INVALID_ARG for null / misaligned pointers,
  * a lone rope table, an unknown kind or window < 1; RLX_ERR_UNSUPPORTED for other head sizes or
  * lengths beyond the maximum.
+ * rlx_attention_kind_status_bf16 is the same call with a status word: optional device int32, receives
+ * RLX_DEVSTAT_TIMEOUT if a bounded wait of the tcgen05 kernel ran out (heads of 128, longer sequences of
+ * heads of 64 and 32; the mma.sync kernel has no such waits).  The rows of ctx that the block which gave up
+ * was to write are NaN then, with and without the word.
  */
 #define RLX_MASK_NONE 0
 #define RLX_MASK_CAUSAL 1
@@ -463,6 +467,11 @@ rlx_status_t rlx_attention_kind_bf16(const void *qkv_bf16, int32_t rows, const i
                                      int32_t num_heads, int32_t num_kv_heads, int32_t head_dim, int32_t mask_kind,
                                      int32_t window, const float *rope_cos, const float *rope_sin,
                                      void *ctx_bf16, void *cuda_stream);
+rlx_status_t rlx_attention_kind_status_bf16(const void *qkv_bf16, int32_t rows, const int32_t *seq_start,
+                                            const int32_t *seq_len, int32_t batch, int32_t max_len,
+                                            int32_t num_heads, int32_t num_kv_heads, int32_t head_dim,
+                                            int32_t mask_kind, int32_t window, const float *rope_cos,
+                                            const float *rope_sin, void *ctx_bf16, int32_t *status, void *cuda_stream);
 
 /*
  * Tables for the rotary embedding of rlx_attention_kind_bf16 / rlx_qk_rope_bf16 (Section 3.2 names the

@@ -42,7 +42,7 @@ EXPORTS = (
     "rlx_encoder_create", "rlx_encoder_destroy", "rlx_encoder_workspace_bytes", "rlx_encoder_forward",
     "rlx_encoder_forward_host", "rlx_encoder_forward_tp", "rlx_encoder_forward_static", "rlx_encoder_last_device_status", "rlx_encoder_kernels_per_forward", "rlx_encoder_kernel_times",
     "rlx_status_string", "rlx_pack_sequences", "rlx_embed_layernorm", "rlx_layernorm", "rlx_gemm_bf16", "rlx_gemm_residual_layernorm_bf16", "rlx_attention_bf16",
-    "rlx_attention_f32", "rlx_attention_packed_bf16", "rlx_attention_kind_bf16", "rlx_rope_tables", "rlx_qk_rope_bf16", "rlx_dequant_block_scaled_bf16", "rlx_scaled_matmul_bf16", "rlx_quantise_mx", "rlx_mx_matmul_bf16", "rlx_ffn_fused_bf16", "rlx_layer_tail_bf16", "rlx_selftest_bounded_wait", "rlx_pool_l2norm",
+    "rlx_attention_f32", "rlx_attention_packed_bf16", "rlx_attention_kind_bf16", "rlx_attention_kind_status_bf16", "rlx_rope_tables", "rlx_qk_rope_bf16", "rlx_dequant_block_scaled_bf16", "rlx_scaled_matmul_bf16", "rlx_quantise_mx", "rlx_mx_matmul_bf16", "rlx_ffn_fused_bf16", "rlx_layer_tail_bf16", "rlx_selftest_bounded_wait", "rlx_pool_l2norm",
 )
 
 
@@ -345,18 +345,19 @@ def rope_tables(max_len: int, head_dim: int, theta: float = 10000.0, device="cud
 
 
 def attention_kind_bf16(qkv, seq_start, seq_len, max_len: int, num_heads: int, mask_kind: int, window: int = 0,
-                        rope=None, out=None, stream=None, num_kv_heads: Optional[int] = None):
+                        rope=None, out=None, stream=None, num_kv_heads: Optional[int] = None, status=None):
     """qkv: packed [rows, (hq + 2 hkv) d] bf16 (hkv = hq unless num_kv_heads is given); rope: None or the
     (cos, sin) pair of rope_tables; returns ctx [rows, hq d] (a fresh zero-filled tensor, or `out` with rows
-    outside every sequence left as they were)."""
+    outside every sequence left as they were).  status: optional int32 device tensor, receives the time-out bit if a
+    bounded wait ran out (rows of ctx are NaN then)."""
     rows, W = qkv.shape
     hkv = num_heads if num_kv_heads is None else num_kv_heads
     d = W // (num_heads + 2 * hkv)
     ctx = torch.zeros((rows, num_heads * d), dtype=torch.bfloat16, device=qkv.device) if out is None else out
     cos, sin = rope if rope is not None else (None, None)
-    _check(_load().rlx_attention_kind_bf16(_ptr(qkv), rows, _ptr(seq_start), _ptr(seq_len), seq_len.numel(), max_len,
-                                           num_heads, hkv, d, mask_kind, window, _ptr(cos), _ptr(sin),
-                                           _ptr(ctx), _stream(stream)),
+    _check(_load().rlx_attention_kind_status_bf16(_ptr(qkv), rows, _ptr(seq_start), _ptr(seq_len), seq_len.numel(), max_len,
+                                                  num_heads, hkv, d, mask_kind, window, _ptr(cos), _ptr(sin),
+                                                  _ptr(ctx), _ptr(status), _stream(stream)),
            "rlx_attention_kind_bf16")
     return ctx
 

@@ -32,7 +32,8 @@
 // tensor memory.  Waits that skip completions of a barrier are safe because either issuer's products complete in
 // order: a group that has seen S(q) knows that S(q - 1), PV(q - 3) and everything before them are complete (heads of 128 wait
 // for the tile's previous PV in every block).
-// All mbarrier waits are bounded.
+// All mbarrier waits are bounded: a CTA whose wait runs out records RLX_DEVSTAT_TIMEOUT, drains, frees its tensor memory and
+// leaves NaN in its rows.
 #pragma once
 #include <cuda.h>
 #include "common.cuh"
@@ -175,6 +176,27 @@ __device__ __forceinline__ int tile1_begin(const Params& p, const Item& it) {
     if (!p.rows_mode) return it.j0;
     if (it.len <= it.q0 + kTile) return it.nb;   // no row of it exists
     return p.positional ? max(0, it.q0 + kTile - p.window + 1) / kTile : it.j0;
+}
+
+// A CTA that gave up leaves NaN in every row of its items, written before or not: its callers need not hold a status word.
+// `cols`: columns of ctx that belong to an item.
+// Out of line and with its arguments by value: in place it changed the softmax loop, 32 q / 8 kv heads of 128, causal: 1021 -> 1084 us.
+__device__ __noinline__ void fill_nan(__nv_bfloat16* ctx, int H, const int32_t* seq_start, const int32_t* seq_len, int batch, int qtiles,
+                                      int units, int rows, int cols) {
+    const int vecs = cols / 8;                // 16-byte pieces of a row
+    long long i = blockIdx.x, tiles = 0;      // next item of this CTA; row tiles that exist so far, in the order of the items
+    for (int qt = qtiles - 1; qt >= 0; --qt)
+        for (int b = 0; b < batch; ++b) {
+            const int n = min(rows, __ldg(seq_len + b) - qt * rows);
+            if (n <= 0) continue;
+            ++tiles;
+            for (; i < tiles * units; i += gridDim.x) {
+                __nv_bfloat16* o = ctx + ((size_t)__ldg(seq_start + b) + qt * rows) * H + (i % units) * cols;
+                for (int k = threadIdx.x; k < n * vecs; k += blockDim.x)
+                    *reinterpret_cast<uint4*>(o + (size_t)(k / vecs) * H + k % vecs * 8) =
+                        make_uint4(0x7FFF7FFFu, 0x7FFF7FFFu, 0x7FFF7FFFu, 0x7FFF7FFFu);
+            }
+        }
 }
 
 template <int D, bool PAIR, bool ROPE>
@@ -645,6 +667,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
         tc_fence_after();
         tmem_dealloc<1>(tmem, 512);
     }
+    if (*abort_flag) fill_nan(p.ctx, p.H, p.seq_start, p.seq_len, p.batch, p.qtiles, p.units, p.rows_mode ? 2 * kTile : kTile, p.rows_mode ? D : 2 * D);
 }
 
 }  // namespace tcat

@@ -1772,10 +1772,10 @@ rlx_status_t rlx_attention_packed_bf16(const void* qkv, int32_t rows, const int3
     return RLX_ERR_INVALID_ARG;
 }
 
-rlx_status_t rlx_attention_kind_bf16(const void* qkv, int32_t rows, const int32_t* seq_start, const int32_t* seq_len,
-                                     int32_t B, int32_t max_len, int32_t h, int32_t hkv, int32_t d, int32_t mask_kind,
-                                     int32_t window, const float* rope_cos, const float* rope_sin, void* ctx,
-                                     void* stream) {
+rlx_status_t rlx_attention_kind_status_bf16(const void* qkv, int32_t rows, const int32_t* seq_start, const int32_t* seq_len,
+                                            int32_t B, int32_t max_len, int32_t h, int32_t hkv, int32_t d, int32_t mask_kind,
+                                            int32_t window, const float* rope_cos, const float* rope_sin, void* ctx,
+                                            int32_t* status, void* stream) {
     if (!qkv || !seq_start || !seq_len || !ctx || B <= 0 || max_len <= 0 || h <= 0 || rows <= 0) return RLX_ERR_INVALID_ARG;
     if (!aligned16(qkv) || !aligned16(ctx) || !aligned16(rope_cos) || !aligned16(rope_sin)) return RLX_ERR_INVALID_ARG;
     if ((rope_cos == nullptr) != (rope_sin == nullptr)) return RLX_ERR_INVALID_ARG;
@@ -1790,9 +1790,17 @@ rlx_status_t rlx_attention_kind_bf16(const void* qkv, int32_t rows, const int32_
     const int w = mask_kind == RLX_MASK_SLIDING_WINDOW ? window : (1 << 30);   // causal: the window never cuts
     if (attention_fwd_pays(d, max_len, positional, w))
         return launch_attention_fwd((const bf16*)qkv, rows, seq_start, seq_len, B, max_len, h, d, h / hkv, positional, w, rope_cos,
-                                    rope_sin, (bf16*)ctx, nullptr, static_cast<cudaStream_t>(stream));
+                                    rope_sin, (bf16*)ctx, status, static_cast<cudaStream_t>(stream));
     return launch_attention_bf16((const bf16*)qkv, nullptr, seq_start, seq_len, B, max_len, h, d, (bf16*)ctx,
                                  static_cast<cudaStream_t>(stream), positional, w, rope_cos, rope_sin, h / hkv);
+}
+
+rlx_status_t rlx_attention_kind_bf16(const void* qkv, int32_t rows, const int32_t* seq_start, const int32_t* seq_len,
+                                     int32_t B, int32_t max_len, int32_t h, int32_t hkv, int32_t d, int32_t mask_kind,
+                                     int32_t window, const float* rope_cos, const float* rope_sin, void* ctx,
+                                     void* stream) {
+    return rlx_attention_kind_status_bf16(qkv, rows, seq_start, seq_len, B, max_len, h, hkv, d, mask_kind, window, rope_cos, rope_sin,
+                                          ctx, nullptr, stream);
 }
 
 rlx_status_t rlx_qk_rope_bf16(void* qkv, int32_t rows, const int32_t* seq_start, const int32_t* seq_len, int32_t B,

@@ -5,6 +5,7 @@ import os
 import re
 
 import pytest
+import torch
 
 from paper_2609_37916_b200 import binding
 from paper_2609_37916_b200.build import build
@@ -171,6 +172,29 @@ def test_attention_kind_validates_on_the_host(lib):
     assert run(h=6, hkv=4) == 1 and run(hkv=0) == 1       # k/v heads must divide the q heads
     assert run(d=48) == 2 and run(d=256) == 2              # head sizes other than 32 / 64 / 128
     assert run(max_len=32769) == 2                         # beyond RLX_ATTENTION_KIND_MAX_LEN
+
+
+def test_attention_kind_hands_on_its_status_word(lib, monkeypatch):
+    """The form with a status word validates like the plain one, and the binding passes the word in its place."""
+    fake = C.c_void_p(0x1000)
+    call = lib.rlx_attention_kind_status_bf16
+    assert call(fake, 64, fake, fake, 1, 64, 2, 2, 32, 3, 0, None, None, fake, fake, None) == 1     # unknown kind
+    assert call(fake, 64, fake, fake, 1, 64, 2, 2, 48, 1, 0, None, None, fake, fake, None) == 2     # head size
+    seen = []
+
+    class Recorder:
+        @staticmethod
+        def rlx_attention_kind_status_bf16(*args):
+            seen.append(args)
+            return 0
+
+    monkeypatch.setattr(binding, "_lib", Recorder)
+    qkv = torch.zeros(8, 192, dtype=torch.bfloat16)
+    start, length, word = (torch.zeros(1, dtype=torch.int32) for _ in range(3))
+    out = torch.zeros(8, 64, dtype=torch.bfloat16)
+    binding.attention_kind_bf16(qkv, start, length, 8, 2, binding.MASK_CAUSAL, out=out, stream=0, status=word)
+    binding.attention_kind_bf16(qkv, start, length, 8, 2, binding.MASK_CAUSAL, out=out, stream=0)
+    assert [a[-2].value for a in seen] == [word.data_ptr(), None] and seen[0][-3].value == out.data_ptr()
 
 
 def test_qk_rope_validates_on_the_host(lib):
