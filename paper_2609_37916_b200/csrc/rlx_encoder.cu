@@ -212,7 +212,7 @@ cudaError_t init_kernels_for_current_device() {
     if ((e = cudaFuncSetAttribute(rlx::tcsk::gemm_splitk_tcgen05_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
                                   rlx::tcsk::kSmemBytes)) != cudaSuccess)                                       \
         return e;
-    RLX_SPLITK_ATTR(0) RLX_SPLITK_ATTR(1) RLX_SPLITK_ATTR(2) RLX_SPLITK_ATTR(5) RLX_SPLITK_ATTR(6)
+    RLX_SPLITK_ATTR(0) RLX_SPLITK_ATTR(1) RLX_SPLITK_ATTR(2) RLX_SPLITK_ATTR(6)
 #undef RLX_SPLITK_ATTR
 #define RLX_ARES_ATTR(BN, EPI)                                                                                  \
     if ((e = cudaFuncSetAttribute(rlx::tcar::gemm_ares_tcgen05_kernel<BN, EPI>,                                \
@@ -265,10 +265,10 @@ cudaError_t init_kernels_for_current_device() {
                                   (int)sizeof(rlx::AttSmem<D>))) != \
         cudaSuccess)                                                                                        \
         return e;
-    RLX_ATT_SMEM_ATTR(32, 0, false) RLX_ATT_SMEM_ATTR(64, 0, false)
     if ((e = cudaFuncSetAttribute(rlx::attention_bf16_kernel<32, 0, false, 32, 4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)sizeof(rlx::AttSmem<32, rlx::AttRing<true>::BN, rlx::AttRing<true>::ST>))) != cudaSuccess)
         return e;
+    RLX_ATT_SMEM_ATTR(64, 0, false)
     RLX_ATT_SMEM_ATTR(32, 0, true) RLX_ATT_SMEM_ATTR(64, 0, true)
     RLX_ATT_SMEM_ATTR(32, 1, false) RLX_ATT_SMEM_ATTR(64, 1, false)
     RLX_ATT_SMEM_ATTR(32, 1, true) RLX_ATT_SMEM_ATTR(64, 1, true)
@@ -398,11 +398,10 @@ rlx_status_t launch_attention_bf16(const bf16* qkv, const int32_t* mask, const i
                            sizeof(rlx::AttSmem<D>),                                                                 \
                            st, qkv, mask, seq_start, seq_len, ctx, S, H, scale_log2e, kind))
     if (d == 32) {
-        if (!positional && !rope && S <= rlx::kAttMaxSeq)   // the encoder's shape: 128-key stages, two deep
+        if (!positional && !rope)   // the encoder's shape, at most 512 keys (longer ones take tcgen05): 128-key stages, two deep
             RLX_CUDA_TRY(launch_ex(rlx::attention_bf16_kernel<32, 0, false, 32, 4, true>, grid, rlx::kAttThreads,
                                    sizeof(rlx::AttSmem<32, rlx::AttRing<true>::BN, rlx::AttRing<true>::ST>), st, qkv, mask, seq_start,
                                    seq_len, ctx, S, H, scale_log2e, kind));
-        else if (!positional && !rope) RLX_ATT_LAUNCH(32, 0, false);
         else if (!positional) RLX_ATT_LAUNCH(32, 0, true);
         else if (!rope) RLX_ATT_LAUNCH(32, 1, false);
         else RLX_ATT_LAUNCH(32, 1, true);
@@ -665,7 +664,7 @@ long long call_tokens(int B, int S) { return g_whole_call_tokens > 0 ? g_whole_c
 // itself only by the products that fold a LayerNorm: the plain ones keep one order of summation at every size, which the
 // fused feed-forward kernel shares bit for bit.
 int pick_split_k(int M, int N, int K, int epi) {
-    if (K < 1536 || N % rlx::tcsk::kBN != 0 || (epi > 2 && epi < 5)) return 1;
+    if (K < 1536 || N % rlx::tcsk::kBN != 0 || (epi > 2 && epi != 6)) return 1;
     const long long rows = std::max<long long>(M, g_whole_call_tokens);
     const long long tiles = (rows + rlx::tc::BLOCK_M - 1) / rlx::tc::BLOCK_M * (N / rlx::tcsk::kBN), sms = sm_count();
     return 4 * tiles <= sms ? 4 : 3 * tiles < 2 * sms - 8 ? 2 : 1;
@@ -683,7 +682,7 @@ rlx_status_t launch_gemm_splitk(const bf16* A, const bf16* W, const rlx::tc::Par
     } scope(split);
     switch (epi) {
 #define RLX_CASE(E) case E: RLX_CUDA_TRY(launch_ex(rlx::tcsk::gemm_splitk_tcgen05_kernel<E>, grid, rlx::tcsk::kThreads, rlx::tcsk::kSmemBytes, st, ta, tb, to, p)); break;
-        RLX_CASE(0) RLX_CASE(1) RLX_CASE(2) RLX_CASE(5) RLX_CASE(6)
+        RLX_CASE(0) RLX_CASE(1) RLX_CASE(2) RLX_CASE(6)
 #undef RLX_CASE
         default: return RLX_ERR_INVALID_ARG;
     }
@@ -721,7 +720,7 @@ rlx_status_t launch_gemm(const bf16* A, const bf16* W, const float* bias, const 
         p.cvec = lf->cvec; p.dvec = lf->dvec; p.stats_in = lf->stats_in; p.stats_in_p = lf->stats_in_p;
         p.ln_gamma = lf->gamma; p.ln_beta = lf->beta; p.stats_out = lf->stats_out; p.ln_eps = lf->eps;
     }
-    const int split = want_cg == 4 || (want_cg == 0 && epi >= 5) ? pick_split_k(M, N, K, epi) : 1;
+    const int split = want_cg == 4 || (want_cg == 0 && epi == 6) ? pick_split_k(M, N, K, epi) : 1;
     if (want_cg == 4 && split == 1) return RLX_ERR_UNSUPPORTED;
     if (split > 1) return launch_gemm_splitk(A, W, p, to, epi, split, st);
     // want_cg == 3: the A-resident CTA-pair kernel, forced; 0: chosen when the problem is large enough

@@ -230,11 +230,11 @@ def test_empty_sequences_and_a_long_one(rlx):
 
 
 @pytest.mark.parametrize("d,hq,hkv", [(32, 2, 2), (32, 3, 3), (32, 4, 2), (64, 2, 2), (64, 1, 1), (64, 6, 2), (128, 1, 1), (128, 4, 1)])
-@pytest.mark.parametrize("kind,window", [(NONE, 0), (CAUSAL, 0), (SLIDING, 127), (SLIDING, 129), (SLIDING, 300)])
+@pytest.mark.parametrize("kind,window", [(NONE, 0), (CAUSAL, 0), (SLIDING, 127), (SLIDING, 129), (SLIDING, 257), (SLIDING, 300), (SLIDING, 383)])
 def test_tile_and_block_edges_of_the_tcgen05_kernel(rlx, d, hq, hkv, kind, window):
     """Lengths at the edges of the 128-row tiles and 128-key blocks, in each pairing of tiles (two heads, two heads of
-    one k/v head, two row tiles), with a sequence long enough that every head size takes that kernel; junk behind
-    the last sequence."""
+    one k/v head, two row tiles), with a sequence long enough that every head size takes that kernel (heads of 32 with
+    a window of 127 or 129 keep to the mma.sync kernel); junk behind the last sequence."""
     rng = np.random.default_rng(d + 10 * hq + window)
     lengths = [1, 127, 128, 129, 255, 256, 257, 0, 383, 520, 16]
     total, W = sum(lengths), (hq + 2 * hkv) * d

@@ -247,6 +247,23 @@ def test_attention_kernel_choice_at_its_edges(rlx, name, B, S):
         check(got[pick], ref, inp.lengths[pick])
 
 
+@pytest.mark.parametrize("name,B,S", [("c1", 6, 128), ("c1", 7, 110), ("c1", 15, 128), ("c1", 16, 121), ("c4", 3, 128), ("c4", 4, 97),
+                                      ("c4", 7, 128), ("c4", 9, 100)])
+def test_folded_forward_splits_its_long_contraction(rlx, name, B, S):
+    """FFN-down of a small folded forward (residual through LayerNorm, row statistics out) on four CTAs per tile, on two, and
+    on one, at the first and last row counts of each on 148 SMs, against the oracle; and twice the same bits."""
+    lengths = np.random.default_rng(B * S).integers(1, S + 1, size=B)
+    lengths[0] = lengths[-1] = S
+    inp = make_inputs(CONFIGS[name], batch=B, seq=S, num_layers=2, lengths=lengths)
+    ref = oracle.encoder_forward(inp.cfg, inp.ids, inp.mask, inp.params, inp.layers)
+    w = rlx.upload_weights(inp.params, inp.layers)
+    got, status = run_gpu(rlx, inp, weights=w)
+    assert status == 0
+    check(got, ref, inp.lengths)
+    again, _ = run_gpu(rlx, inp, weights=w)
+    assert np.array_equal(got, again)
+
+
 @pytest.mark.parametrize("heads", [2, 4])
 @pytest.mark.parametrize("flags", [0, 0x200, 0x400])   # the host's choice, folded LayerNorm, none folded
 def test_a_short_last_chunk_takes_the_kernels_of_the_whole_call(rlx, heads, flags):

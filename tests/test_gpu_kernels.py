@@ -462,11 +462,12 @@ def test_attention_all_masked_sequence_gives_zeros(rlx):
 
 
 # ------------------------------------------------------------------ GEMM split along K over a cluster
-@pytest.mark.parametrize("M", [1, 31, 33, 64, 97, 128, 129, 300])
-@pytest.mark.parametrize("N,K", [(64, 1536), (384, 1536), (192, 1544), (768, 3072)])
+@pytest.mark.parametrize("M,N,K", [(m, n, k) for m in (1, 31, 33, 64, 97, 128, 129, 300)
+                                   for n, k in ((64, 1536), (384, 1536), (192, 1544), (768, 3072))] +
+                         [(1000, 384, 1536), (1900, 384, 1544), (897, 384, 3072), (500, 768, 1608)])
 def test_gemm_split_along_k(rlx, M, N, K):
-    """Few rows and a long contraction, split on request: four or two CTAs per tile, at the edges of the 32-row units
-    and of uneven k ranges, against the oracle and the one-CTA-per-tile form, twice (the order of the partial sums is
+    """Few rows and a long contraction, split on request: four CTAs per tile (up to 37 tiles on 148 SMs) or two (the last
+    four shapes: 48, 90, 48 and 48 tiles), at the edges of the 32-row units and of uneven k ranges, against the oracle and the one-CTA-per-tile form, twice (the order of the partial sums is
     fixed)."""
     rng = np.random.default_rng(M + N + K)
     a, w = rand_bf16(rng, (M, K)), rand_bf16(rng, (N, K), 0.05)
