@@ -1,7 +1,7 @@
 // bf16 "Linear" GEMM for few rows and a long contraction: out[M,N] = epilogue(A[M,K] W[N,K]^T + bias), split along K
 // over a cluster.
 //
-// The `S` CTAs of a cluster take one 128 x 64 tile and K / S of its contraction each (TMA -> tcgen05, as in
+// `S` CTAs, a cluster or a part of one, take one 128 x 64 tile and K / S of its contraction each (TMA -> tcgen05, as in
 // gemm_tcgen05.cuh; the W tiles are requested in front of the wait for the previous kernel). The tile's
 // 32 x 32 units are dealt out to the CTAs: every CTA sends its partial sums of a unit to the unit's owner with
 // st.async (data and arrival in one, no fence), and the owner adds them in rank order -- the result does not
@@ -56,12 +56,18 @@ gemm_splitk_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __g
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + kBarOff + 8 * (2 * kStages + 2));
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
-    const int rank = (int)warp_uniform(cluster_ctarank()), S = (int)tccl::cluster_nctarank();
     pdl_launch_dependents();
 
     int M = p.M;
     if (p.m_ptr != nullptr) M = min(M, ld_early(p.m_ptr));
     const int n_tiles = p.N / kBN;
+    // CTAs per tile: as many as there are in a cluster, fewer when the tiles that exist (the host knows the padded row count
+    // only) would not all run beside each other; the cluster then holds several tiles.
+    const int existing = (M + BLOCK_M - 1) / BLOCK_M * n_tiles, crank = (int)warp_uniform(cluster_ctarank());
+    int S = (int)tccl::cluster_nctarank();
+    if (S == 4 && existing > p.split_tiles4) S = 2;
+    if (S == 2 && existing > p.split_tiles2) S = 1;
+    const int rank = crank % S, first = crank - rank;        // rank among the tile's CTAs, cluster rank of its first one
     const int tile = blockIdx.x / S, m_blk = tile / n_tiles, n_blk = tile % n_tiles;
     const int rows = min(BLOCK_M, M - m_blk * BLOCK_M);      // rows of this tile that exist (<= 0: none)
     const int groups = rows > 0 ? (rows + 31) / 32 : 0;      // 32-row groups
@@ -183,8 +189,8 @@ gemm_splitk_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __g
                 if (kb0 >= kb1)
 #pragma unroll
                     for (int i = 0; i < 32; ++i) r[i] = 0;
-                const uint32_t dst = map_to_cta(base + kXchOff + ((unit / S) * S + rank) * kUnitBytes + lane * 16, unit % S);
-                const uint32_t bar = map_to_cta(xch_bar, unit % S);
+                const uint32_t dst = map_to_cta(base + kXchOff + ((unit / S) * S + rank) * kUnitBytes + lane * 16, first + unit % S);
+                const uint32_t bar = map_to_cta(xch_bar, first + unit % S);
 #pragma unroll
                 for (int i = 0; i < 8; ++i) st_async_v4(dst + i * 512, bar, r + 4 * i);   // [column quad][row]: no bank conflicts
                 tc_fence_before();

@@ -388,6 +388,7 @@ struct Params {
     const int32_t* m_ptr;            // optional device row count: rows >= *m_ptr are not computed
     int kblock_maps;                 // the operand tensor maps are 3-D views [K/64][rows][64]: one TMA load brings a
                                      // whole stage's k-blocks of an operand (needs K % 64 == 0); else 2-D, one per k-block
+    int split_tiles4, split_tiles2;  // split-K form: up to so many existing tiles get four / two CTAs each
 #ifdef RLX_EXPERIMENTS
     int debug;                       // ablation switches of the experiments build (kDbg* bits)
     unsigned long long* trace;       // experiments build: 64 timestamp slots per CTA (or null)

@@ -140,6 +140,7 @@ cudaError_t set_gemm_attr_all() {
 // Number of CTA pairs that can be resident at once (pairs must sit in one GPC), per device.
 int g_max_pairs[64] = {};
 int g_max_pairs_resident[64] = {};   // the same for the A-resident kernel (its own shared-memory footprint)
+int g_max_split2[64] = {}, g_max_split4[64] = {};   // clusters of two and four of the split-K kernel
 
 // Multiprocessor count of the current device (grids of the persistent kernels are sized from it).
 constexpr int kNominalSMs = 148;   // B200; used only when no device can be queried (host-only callers)
@@ -214,6 +215,22 @@ cudaError_t init_kernels_for_current_device() {
         return e;
     RLX_SPLITK_ATTR(0) RLX_SPLITK_ATTR(1) RLX_SPLITK_ATTR(2) RLX_SPLITK_ATTR(6)
 #undef RLX_SPLITK_ATTR
+    for (int size = 2; size <= 4; size *= 2) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(size * sm_count());
+        cfg.blockDim = dim3(rlx::tcsk::kThreads);
+        cfg.dynamicSmemBytes = rlx::tcsk::kSmemBytes;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = size;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if ((e = cudaOccupancyMaxActiveClusters(&n, rlx::tcsk::gemm_splitk_tcgen05_kernel<6>, &cfg)) != cudaSuccess) return e;
+        if (dev < 64) (size == 2 ? g_max_split2 : g_max_split4)[dev] = n;
+    }
 #define RLX_ARES_ATTR(BN, EPI)                                                                                  \
     if ((e = cudaFuncSetAttribute(rlx::tcar::gemm_ares_tcgen05_kernel<BN, EPI>,                                \
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, rlx::tcar::Cfg<BN>::SMEM_BYTES)) != \
@@ -658,16 +675,27 @@ struct LnFold {
 thread_local long long g_whole_call_tokens = 0;
 long long call_tokens(int B, int S) { return g_whole_call_tokens > 0 ? g_whole_call_tokens : (long long)B * S; }
 
-// CTAs per 128 x 64 tile along K (1: do not split).  A long contraction on a few tiles is bound by one SM's operand feed;
-// four CTAs per tile while they all fit beside each other, two while two thirds of them do -- the row count is the
-// padded one, and a batch whose every position is valid then runs two half-length rounds instead of one.  Taken by
-// itself only by the products that fold a LayerNorm: the plain ones keep one order of summation at every size, which the
-// fused feed-forward kernel shares bit for bit.
-int pick_split_k(int M, int N, int K, int epi) {
+// CTAs per 128 x 64 tile along K that a cluster of the split form holds (1: do not split); the kernel takes fewer when the
+// tiles that exist would not all run beside each other, at most `fit` clusters of two or four of them at once (74 and 33 on
+// 148 SMs; the host knows the padded row count only).  A long contraction on a few tiles is bound by one SM's operand feed.
+// Whole forwards, us without / with the split, half and all of the positions valid:
+//   four, up to a quarter of the SMs: 1 x 128 143.6 / 141.7 and 151 / 150, 5 x 128 155 / 148 and 167 / 160, 6 x 128 170 / 154 and
+//     178 / 168 (201 when all of 36 tiles are split in four), 3 x 128 through 12 x 768 438 / 374 and 453 / 419 (487); the smaller model
+//     at an even number of 128-row tiles loses (2 x 128 150 / 165, 4 x 128 149 / 165) for a reason that is not known: without
+//     programmatic launches four is ahead there too (189 / 182, 191 / 186)
+//   two, K >= 3072, while a batch four fifths valid fits: 6 x 128 479 / 460 and 531 / 523, 7 x 120 468 / 457 and 544 / 571 (615 split);
+//     beyond, the full batch's loss grows (8 x 128 497 / 479, 555 / 583)
+//   two, shorter K, up to a third of the SMs: 7 x 128 165 / 163 and 187 / 188; beyond, halves of 768 gain nothing (10 x 128 176 / 181,
+//     15 x 128 189 / 193 and 211 / 251)
+// Taken by itself only by the product that folds a LayerNorm and reads its residual through one: the plain ones keep one
+// order of summation at every size, which the fused feed-forward kernel shares bit for bit.  `asked`: up to two thirds
+// of the SMs, whatever K.
+int pick_split_k(int M, int N, int K, int epi, int fit2, bool asked) {
     if (K < 1536 || N % rlx::tcsk::kBN != 0 || (epi > 2 && epi != 6)) return 1;
     const long long rows = std::max<long long>(M, g_whole_call_tokens);
     const long long tiles = (rows + rlx::tc::BLOCK_M - 1) / rlx::tc::BLOCK_M * (N / rlx::tcsk::kBN), sms = sm_count();
-    return 4 * tiles <= sms ? 4 : 3 * tiles < 2 * sms - 8 ? 2 : 1;
+    if (4 * tiles <= sms) return 4;
+    return (asked ? 3 * tiles <= 2 * sms : K >= 3072 ? 4 * tiles <= 5 * fit2 : 3 * tiles <= sms) ? 2 : 1;
 }
 
 rlx_status_t launch_gemm_splitk(const bf16* A, const bf16* W, const rlx::tc::Params& p, const CUtensorMap& to, int epi, int split,
@@ -720,9 +748,17 @@ rlx_status_t launch_gemm(const bf16* A, const bf16* W, const float* bias, const 
         p.cvec = lf->cvec; p.dvec = lf->dvec; p.stats_in = lf->stats_in; p.stats_in_p = lf->stats_in_p;
         p.ln_gamma = lf->gamma; p.ln_beta = lf->beta; p.stats_out = lf->stats_out; p.ln_eps = lf->eps;
     }
-    const int split = want_cg == 4 || (want_cg == 0 && epi == 6) ? pick_split_k(M, N, K, epi) : 1;
-    if (want_cg == 4 && split == 1) return RLX_ERR_UNSUPPORTED;
-    if (split > 1) return launch_gemm_splitk(A, W, p, to, epi, split, st);
+    if (want_cg == 4 || (want_cg == 0 && epi == 6)) {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        const bool known = dev >= 0 && dev < 64;
+        const int fit2 = known ? g_max_split2[dev] : sm_count() / 2, fit4 = known ? g_max_split4[dev] : sm_count() / 8;
+        const int split = pick_split_k(M, N, K, epi, fit2, want_cg == 4);
+        if (want_cg == 4 && split == 1) return RLX_ERR_UNSUPPORTED;
+        p.split_tiles2 = want_cg == 4 ? 1 << 30 : fit2;   // asked for: whatever the number of tiles
+        p.split_tiles4 = want_cg == 4 ? 1 << 30 : fit4;
+        if (split > 1) return launch_gemm_splitk(A, W, p, to, epi, split, st);
+    }
     // want_cg == 3: the A-resident CTA-pair kernel, forced; 0: chosen when the problem is large enough
     if (want_cg == 3 || (want_cg == 0 && g_exp_resident >= 0)) {
         const int rbn = pick_resident_bn(M, N, K, epi, want_cg == 3 || g_exp_resident > 0);

@@ -247,13 +247,17 @@ def test_attention_kernel_choice_at_its_edges(rlx, name, B, S):
         check(got[pick], ref, inp.lengths[pick])
 
 
-@pytest.mark.parametrize("name,B,S", [("c1", 6, 128), ("c1", 7, 110), ("c1", 15, 128), ("c1", 16, 121), ("c4", 3, 128), ("c4", 4, 97),
-                                      ("c4", 7, 128), ("c4", 9, 100)])
-def test_folded_forward_splits_its_long_contraction(rlx, name, B, S):
+@pytest.mark.parametrize("name,B,S", [("c1", 5, 128), ("c1", 6, 128), ("c1", 7, 110), ("c1", 8, 128), ("c1", 9, 120), ("c4", 2, 128),
+                                      ("c4", 3, 128), ("c4", 4, 97), ("c4", 6, 128), ("c4", 7, 128), ("c4", 8, 120)])
+@pytest.mark.parametrize("full", [False, True])
+def test_folded_forward_splits_its_long_contraction(rlx, name, B, S, full):
     """FFN-down of a small folded forward (residual through LayerNorm, row statistics out) on four CTAs per tile, on two, and
-    on one, at the first and last row counts of each on 148 SMs, against the oracle; and twice the same bits."""
+    on one, at the first and last row counts of each on 148 SMs, against the oracle; and twice the same bits.  With every
+    position valid clusters of four (36 tiles) and of two (84 tiles) take more tiles and fewer CTAs for each."""
     lengths = np.random.default_rng(B * S).integers(1, S + 1, size=B)
     lengths[0] = lengths[-1] = S
+    if full:
+        lengths[:] = S
     inp = make_inputs(CONFIGS[name], batch=B, seq=S, num_layers=2, lengths=lengths)
     ref = oracle.encoder_forward(inp.cfg, inp.ids, inp.mask, inp.params, inp.layers)
     w = rlx.upload_weights(inp.params, inp.layers)
