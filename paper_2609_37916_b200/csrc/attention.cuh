@@ -8,7 +8,9 @@
 //    shuffles, the row sums come from an extra ones column of the PV product; the 1/sqrt(d)*log2(e)
 //    scale is folded into the exp2 argument.  At head_dim 32 the online-softmax step is 32 keys (half a
 //    staged block): 64 registers per thread, four CTAs per SM instead of three (-6 % on the 256 x 256
-//    workload; at head_dim 64, and in the mask-kind / rotary modes, the 64-key step is kept).  Key blocks beyond the
+//    workload; at head_dim 64, and in the mask-kind / rotary modes, the 64-key step is kept).  head_dim 128
+//    (mask-kind entry point only) runs one CTA per SM with the 32-key step: 64 output accumulators and
+//    32 Q-fragment registers per thread leave no room for more.  Key blocks beyond the
 //    last valid key are never loaded; masking runs only in blocks that contain an invalid key.
 //  attention_f32_kernel: fp32 in/out CUDA-core kernel, one warp per query row, K/V staged in shared
 //    memory 32 keys at a time, warp-shuffle reductions.  Reference-precision mode for testing.
@@ -80,7 +82,7 @@ constexpr int kAttMaxSeq = 512;
 // Keys per shared-memory stage and depth of the K/V ring.  The encoder's own shape (head_dim 32, at most 512 keys,
 // no window, no rotation: the launcher's choice, kernel parameter WIDE) takes 128-key stages in a two-deep ring: a sequence is one to four stages, so half as
 // many CTA-wide barriers are crossed for the same shared memory (-5 % at 256 x 256).  Long sequences (the mask
-// kinds, rotary q/k, head_dim 64) keep 64-key stages four deep: with thousands of keys the prefetch
+// kinds, rotary q/k, head_dim 64 / 128) keep 64-key stages four deep: with thousands of keys the prefetch
 // distance matters more than the barrier count (the 128 x 2 ring measured 30-50 % slower there).
 template <bool WIDE>
 struct AttRing {
@@ -121,8 +123,8 @@ struct AttKind {
 // Two addressing modes share the kernel:
 //   padded: seq_start == nullptr.  Sequence b occupies rows b*S .. b*S+S; `mask` flags valid keys.
 //   packed: rows of sequence b are seq_start[b] .. seq_start[b]+seq_len[b], all valid (mask unused).
-template <int D, int MK = 0, bool ROPE = false, int KS = ((D == 32 && MK == 0 && !ROPE) ? 32 : 64),
-          int MINB = (D == 32 ? (KS == 32 ? 4 : 3) : 2), bool WIDE = false>
+template <int D, int MK = 0, bool ROPE = false, int KS = (((D == 32 && MK == 0 && !ROPE) || D == 128) ? 32 : 64),
+          int MINB = (D == 32 ? (KS == 32 ? 4 : 3) : D == 64 ? 2 : 1), bool WIDE = false>
 __global__ void __launch_bounds__(kAttThreads, MINB)
 attention_bf16_kernel(const __nv_bfloat16* __restrict__ qkv, const int32_t* __restrict__ mask,
                       const int32_t* __restrict__ seq_start, const int32_t* __restrict__ seq_len,

@@ -289,6 +289,7 @@ cudaError_t init_kernels_for_current_device() {
     RLX_ATT_SMEM_ATTR(32, 0, true) RLX_ATT_SMEM_ATTR(64, 0, true)
     RLX_ATT_SMEM_ATTR(32, 1, false) RLX_ATT_SMEM_ATTR(64, 1, false)
     RLX_ATT_SMEM_ATTR(32, 1, true) RLX_ATT_SMEM_ATTR(64, 1, true)
+    RLX_ATT_SMEM_ATTR(128, 0, false) RLX_ATT_SMEM_ATTR(128, 0, true) RLX_ATT_SMEM_ATTR(128, 1, false) RLX_ATT_SMEM_ATTR(128, 1, true)
 #undef RLX_ATT_SMEM_ATTR
     if (dev < 64) done[dev] = true;
     return cudaSuccess;
@@ -409,7 +410,7 @@ rlx_status_t launch_attention_bf16(const bf16* qkv, const int32_t* mask, const i
     dim3 grid((S + rlx::kAttBlockM - 1) / rlx::kAttBlockM, h, B);
     const rlx::AttKind kind{window, rope_cos, rope_sin, kv_group};
     const bool rope = rope_cos != nullptr;
-    if (d != 32 && d != 64) return RLX_ERR_UNSUPPORTED;
+    if (d != 32 && d != 64 && d != 128) return RLX_ERR_UNSUPPORTED;
 #define RLX_ATT_LAUNCH(D, MK, ROPE)                                                                              \
     RLX_CUDA_TRY(launch_ex(rlx::attention_bf16_kernel<D, MK, ROPE>, grid, rlx::kAttThreads,                      \
                            sizeof(rlx::AttSmem<D>),                                                                 \
@@ -422,11 +423,16 @@ rlx_status_t launch_attention_bf16(const bf16* qkv, const int32_t* mask, const i
         else if (!positional) RLX_ATT_LAUNCH(32, 0, true);
         else if (!rope) RLX_ATT_LAUNCH(32, 1, false);
         else RLX_ATT_LAUNCH(32, 1, true);
-    } else {
+    } else if (d == 64) {
         if (!positional && !rope) RLX_ATT_LAUNCH(64, 0, false);
         else if (!positional) RLX_ATT_LAUNCH(64, 0, true);
         else if (!rope) RLX_ATT_LAUNCH(64, 1, false);
         else RLX_ATT_LAUNCH(64, 1, true);
+    } else {
+        if (!positional && !rope) RLX_ATT_LAUNCH(128, 0, false);
+        else if (!positional) RLX_ATT_LAUNCH(128, 0, true);
+        else if (!rope) RLX_ATT_LAUNCH(128, 1, false);
+        else RLX_ATT_LAUNCH(128, 1, true);
     }
 #undef RLX_ATT_LAUNCH
     RLX_CUDA_TRY(cudaGetLastError());
@@ -475,16 +481,30 @@ rlx_status_t launch_attention_fwd(const bf16* qkv, int rows, const int32_t* seq_
     return RLX_OK;
 }
 
-// Where the tcgen05 kernel replaces the mma.sync one (measured on packed batches, us old / new):
-//   head_dim 128: everywhere (16 prompts of 1024..4096, causal, 32 q / 8 kv heads 3561 / 873; 64 of 16..256 75 / 43)
-//   head_dim 64: longer than one 128-row tile (causal 1024..4096, 16 heads 907 / 369; 16..256 39.6 / 33.6; window 512
-//     over 100..1500 140 / 80; but 16..128 21.1 / 23.1: one tile and one block per item are all set-up and latency)
-//   head_dim 32: only where many blocks per tile pay for its fixed costs: longer than 512 keys, no short window
-//     (causal 400..2000 156 / 107; 16..256 25.8 / 28.2; window 64 over 100..1500 47.7 / 48.5)
-bool attention_fwd_pays(int d, int max_len, bool positional, int window) {
-    if (d == 128) return true;
-    if (d == 64) return max_len > rlx::tcat::kTile;
-    return max_len > rlx::kAttMaxSeq && (!positional || window > 2 * rlx::tcat::kTile);
+// Where the tcgen05 kernel replaces the mma.sync one in calls by mask kind (us mma.sync / tcgen05; the longest sequence, the
+// keys that a row tile can see, and whether its 128-row tiles of heads fill the chip).  A tcgen05 item is one long chain (load,
+// scores, softmax, P V, store: 7 us, with a window's three blocks 12), the mma.sync kernel a short one per tile, so few
+// tiles that see few keys are left to the latter.  Not a matter of the rotation: rotating first gives the same bits.
+//   heads of 128: everywhere (16 prompts of 1024..4096, causal, 32 q / 8 kv heads 3566 / 1061; 64 of 16..256 138 / 62) but
+//     within a wave of mma.sync CTAs, one per SM, where tiles see at most 192 keys (1 x 20 3.7 / 7.0, 1 x 128 7.0 / 9.2, window 64
+//     over 1 x 1024 with 8 heads 8.8 / 12.4, but 32 heads 16.5 / 12.7; 1 x 200 10.4 / 9.6) or a window shows them at most 256
+//     (128 over 1 x 512 10.6 / 12.0)
+//   heads of 64: longer than one tile (causal 1024..4096, 16 heads 907 / 371; 16..256 36.5 / 25.4; 16..128 6.5 / 7.8 in 16 sequences) but
+//     up to four waves of 148 for at most 192 positions (64 x 10..160, 8 heads 13.8 / 15.2), up to two where
+//     tiles see at most 192 keys (window 64 over 1 x 4096, 8 heads 9.2 / 12.7, but 16 heads 16.5 / 16.4), one up to 448 keys (1 x 256
+//     7.6 / 8.8, window 300 over 1 x 1024 11.9 / 12.9, 512 15.6 / 13.8)
+//   heads of 32: longer than 512 positions, no window up to 256 (causal 400..2000 152 / 103; window 64 over 16 x 1024..4096, 8 heads
+//     48.5 / 47.2), but for a wave of tiles that see at most 640 keys (window 512 over 1 x 1024 12.0 / 13.1, over 1 x 4096 17.6 / 15.9)
+bool attention_fwd_pays(int d, int rows, int B, int max_len, int h, bool positional, int window) {
+    constexpr int kT = rlx::tcat::kTile;
+    const long long sms = sm_count();
+    const int keys = positional && window < max_len ? std::min(max_len, window + kT - 1) : max_len;   // that a tile can see
+    const long long grid = (long long)h * B * ((max_len + kT - 1) / kT);
+    const long long tiles = std::min(grid, h * ((long long)rows / kT + B / 2 + 1));   // about so many exist
+    if (d == 128) return tiles > sms || (keys > 192 && (keys > 256 || max_len <= 256));
+    if (d == 64)
+        return max_len > kT && (grid > sms || keys > 448) && (tiles > 2 * sms || keys > 192) && (tiles > 4 * sms || max_len > 192);
+    return max_len > rlx::kAttMaxSeq && (!positional || (window > 2 * kT && (grid > sms || keys > 640)));
 }
 
 // Feed-forward block in one kernel (hidden 256 or 384, F % 64 == 0): out = gelu(x W1^T + b1) W2^T + b2 + x.
@@ -1823,7 +1843,7 @@ rlx_status_t rlx_attention_kind_status_bf16(const void* qkv, int32_t rows, const
     RLX_CUDA_TRY(init_kernels_for_current_device());
     const bool positional = mask_kind != RLX_MASK_NONE;
     const int w = mask_kind == RLX_MASK_SLIDING_WINDOW ? window : (1 << 30);   // causal: the window never cuts
-    if (attention_fwd_pays(d, max_len, positional, w))
+    if (attention_fwd_pays(d, rows, B, max_len, h, positional, w))
         return launch_attention_fwd((const bf16*)qkv, rows, seq_start, seq_len, B, max_len, h, d, h / hkv, positional, w, rope_cos,
                                     rope_sin, (bf16*)ctx, status, static_cast<cudaStream_t>(stream));
     return launch_attention_bf16((const bf16*)qkv, nullptr, seq_start, seq_len, B, max_len, h, d, (bf16*)ctx,

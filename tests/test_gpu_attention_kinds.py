@@ -236,7 +236,7 @@ def test_tile_and_block_edges_of_the_tcgen05_kernel(rlx, d, hq, hkv, kind, windo
     one k/v head, two row tiles), with a sequence long enough that every head size takes that kernel (heads of 32 with
     a window of 127 or 129 keep to the mma.sync kernel); junk behind the last sequence."""
     rng = np.random.default_rng(d + 10 * hq + window)
-    lengths = [1, 127, 128, 129, 255, 256, 257, 0, 383, 520, 16]
+    lengths = [1, 127, 128, 129, 255, 256, 257, 0, 383, 520, 16] * (8 if hq == 1 else 3)   # enough of them for that kernel
     total, W = sum(lengths), (hq + 2 * hkv) * d
     qkv = rand_bf16(rng, (total + 3, W))
     qkv[total:] = np.float32("nan")
@@ -267,8 +267,8 @@ def test_row_sums_are_those_of_the_rounded_probabilities(rlx, d, hq, hkv, kind, 
     most u max|v - mean| <= u 2^-7; the fp32 sums (at most 45 accumulation steps of 2^-23 and 180 additions of 2^-24, relative
     to a mean of one) by less than 2^-15.  A row sum of the unrounded weights moves it by up to u itself, 128 times as much."""
     rng = np.random.default_rng(d + hq)
-    lengths = [700, 130, 517]
-    total, start = sum(lengths), np.array([0, 700, 830], np.int32)
+    lengths = [700, 130, 517] * 5              # enough of them for the tcgen05 kernel
+    total, start = sum(lengths), (np.cumsum(lengths) - lengths).astype(np.int32)
     qkv = rand_bf16(rng, (total, (hq + 2 * hkv) * d))
     qkv[:, :hq * d] *= 2                       # a few keys carry most of a row's weight
     qkv[:, (hq + hkv) * d:] = 1 + 2.0 ** -7 * rng.integers(0, 2, (total, hkv * d))
@@ -288,9 +288,9 @@ def test_blocks_that_a_row_tile_cannot_see_are_not_multiplied(rlx, d, hq, hkv, t
     """Infinite and NaN v in 128-key blocks that no row of a 128-row tile can see leave its rows as they are, bit for bit:
     later blocks under the causal mask, earlier ones under a window, in the first and the second tile of 256 rows."""
     rng = np.random.default_rng(d + hq)
-    lengths = np.array([900, 640], np.int32)
-    start = np.array([0, 900], np.int32)
-    qkv = rand_bf16(rng, (1540, (hq + 2 * hkv) * d))
+    lengths = np.array([900, 640] * (10 // hq + 1), np.int32)       # enough of them for the tcgen05 kernel
+    start = (np.cumsum(lengths) - lengths).astype(np.int32)
+    qkv = rand_bf16(rng, (int(lengths.sum()), (hq + 2 * hkv) * d))
     rope = None if theta is None else rlx.rope_tables(900, d, theta)
 
     def run(a, kind, window):
@@ -310,3 +310,26 @@ def test_blocks_that_a_row_tile_cannot_see_are_not_multiplied(rlx, d, hq, hkv, t
             got = run(poisoned, kind, window)
             for s0, n in zip(start, lengths):
                 assert np.array_equal(got[s0:s0 + n][rows], clean[s0:s0 + n][rows]), (tile, kind, window)
+
+
+@pytest.mark.parametrize("d,hq,hkv,n,length,kind,window", [
+    (128, 4, 2, 1, 192, NONE, 0), (128, 4, 2, 1, 193, NONE, 0), (128, 3, 3, 1, 257, SLIDING, 129), (128, 3, 3, 1, 257, SLIDING, 130),
+    (128, 8, 8, 18, 128, CAUSAL, 0), (128, 8, 8, 19, 128, CAUSAL, 0), (64, 2, 2, 1, 448, CAUSAL, 0), (64, 2, 2, 1, 449, CAUSAL, 0),
+    (64, 8, 4, 2, 1100, SLIDING, 321), (64, 8, 4, 2, 1100, SLIDING, 322), (64, 8, 4, 19, 192, NONE, 0), (64, 8, 4, 50, 192, NONE, 0),
+    (64, 8, 4, 3, 1100, SLIDING, 65), (64, 8, 4, 3, 1100, SLIDING, 66), (32, 2, 2, 1, 640, CAUSAL, 0), (32, 2, 2, 1, 641, CAUSAL, 0),
+    (32, 4, 2, 7, 640, SLIDING, 300), (32, 4, 2, 8, 640, SLIDING, 300)])
+def test_kernel_choice_at_its_edges(rlx, d, hq, hkv, n, length, kind, window):
+    """Both sides of the lines between the two attention kernels, plain and with the rotation, which is bit for bit the rotation
+    in place followed by the plain call on either."""
+    rng = np.random.default_rng(d + n + length)
+    lengths, start = np.full(n, length, np.int32), (length * np.arange(n)).astype(np.int32)
+    lengths[-1] -= 1
+    qkv = rand_bf16(rng, (n * length, (hq + 2 * hkv) * d))
+    args = (i32_dev(start), i32_dev(lengths), length, hq)
+    got = to_np64(rlx.attention_kind_bf16(bf16_dev(qkv), *args, kind, window, num_kv_heads=hkv))
+    ref = ak.attention_packed(qkv.astype(np.float64), start, lengths, hq, kind, window, None, num_kv_heads=hkv)
+    assert np.abs(got - ref).max() <= 2 * BF16_U * (np.abs(qkv[:, (hq + hkv) * d:]).max() + np.abs(ref).max())
+    rope = rlx.rope_tables(length, d)
+    inside = rlx.attention_kind_bf16(bf16_dev(qkv), *args, kind, window, rope, num_kv_heads=hkv)
+    turned = rlx.binding.qk_rope_bf16(bf16_dev(qkv), *args, rope, num_kv_heads=hkv)
+    assert torch.equal(inside, rlx.attention_kind_bf16(turned, *args, kind, window, num_kv_heads=hkv))
