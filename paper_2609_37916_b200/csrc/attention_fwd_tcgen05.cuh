@@ -76,6 +76,12 @@ __device__ __forceinline__ void tmem_ld_32x16(uint32_t taddr, uint32_t (&r)[16])
           "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
         : "r"(taddr) : "memory");
 }
+__device__ __forceinline__ void tmem_ld_32x1(uint32_t taddr, uint32_t& r) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void tmem_st_32x1(uint32_t taddr, uint32_t r) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x1.b32 [%0], {%1};" ::"r"(taddr), "r"(r) : "memory");
+}
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ float max3f(float a, float b, float c) {
     float d;
@@ -114,17 +120,25 @@ struct Cfg {
     static constexpr int QST = QB > 32768 ? 1 : 2;
     static constexpr int KST = TILE == 32768 ? 3 : 4;         // K ring
     static constexpr int VST = TILE == 32768 ? 2 : 4;         // V ring
-    static constexpr int NV = (PAIR && D == 32) ? 64 : D;     // accumulator columns (N = 32 costs the tensor pipe what N = 64 does)
+    // Heads of 32 leave tensor memory for 16 more accumulator columns, and N = 48 costs the tensor pipe what N = 32 does: the
+    // row sums come as further columns of P V, whose V columns are ones.  V tiles then have one head's columns each.
+    static constexpr bool SUMS = D == 32;
+    static constexpr int NV = SUMS ? D + 16 : D;              // accumulator columns
+    static constexpr int VROWB = SUMS ? 2 * D : ROWB;         // bytes of a row of a V tile
+    static constexpr int VCOLS = VROWB / 2, VSUBS = W / VCOLS, VSUB = KB * VROWB;
+    static constexpr int ONES_BYTES = SUMS ? 16 * VROWB : 0;  // 16 keys: what one product reads
     static constexpr int P_COL = APART ? KB : 0, P_STRIDE = APART ? KB / 2 : KB;
     static constexpr int O_COL = APART ? 2 * KB : NSB * KB, O_STRIDE = NV;
     static constexpr int RING_OFF = QST * QB;
     static constexpr int VRING_OFF = RING_OFF + KST * TILE;
-    static constexpr int ITEM_OFF = VRING_OFF + VST * TILE;
+    static constexpr int ONES_OFF = VRING_OFF + VST * TILE;
+    static constexpr int ITEM_OFF = ONES_OFF + ONES_BYTES;
     static constexpr int BAR_OFF = ITEM_OFF + kItemRing * 32;
     static constexpr int NBAR = 3 * QST + 3 * KST + 2 * VST + 2 * NPB + NSB + 2 + 2 + 2 * kItemRing;
     static constexpr int SMEM_BYTES = BAR_OFF + 8 * NBAR + 16 + 1024;
     static constexpr uint64_t SWZ = ROWB == 128 ? 2 : 4;
     static_assert(ROWB == 128 || ROWB == 64, "swizzle span");
+    static_assert(VSUBS * VSUB == TILE, "V tile");
     static_assert(O_COL + 2 * O_STRIDE <= 512, "tensor memory");
     static_assert(SMEM_BYTES <= 227 * 1024, "shared memory");
 
@@ -132,10 +146,16 @@ struct Cfg {
     static __device__ __forceinline__ uint64_t desc_k(uint32_t a) {
         return (uint64_t)((a & 0x3FFFFu) >> 4) | (uint64_t)1 << 16 | (uint64_t)((8 * ROWB) >> 4) << 32 | (uint64_t)1 << 46 | SWZ << 61;
     }
-    // V: the head dimension is contiguous (N), keys run over rows; the second 64 columns are SUB bytes away
+    // V: the head dimension is contiguous (N), keys run over rows; the columns behind a tile's are SUB bytes away, or the ones
     static __device__ __forceinline__ uint64_t desc_v(uint32_t a) {
-        return (uint64_t)((a & 0x3FFFFu) >> 4) | (uint64_t)(NV > COLS ? SUB >> 4 : 1) << 16 | (uint64_t)((8 * ROWB) >> 4) << 32 |
-               (uint64_t)1 << 46 | SWZ << 61;
+        constexpr uint64_t lbo = SUMS ? (ONES_OFF - VRING_OFF) >> 4 : NV > VCOLS ? VSUB >> 4 : 1;
+        return (uint64_t)((a & 0x3FFFFu) >> 4) | lbo << 16 | (uint64_t)((8 * VROWB) >> 4) << 32 | (uint64_t)1 << 46 |
+               (uint64_t)(VROWB == 128 ? 2 : 4) << 61;
+    }
+    // the descriptor `bytes` further on in the ring; the ones stay where they are
+    static __device__ __forceinline__ uint64_t desc_step(uint32_t bytes) {
+        const uint64_t d = bytes >> 4;
+        return SUMS ? d - (d << 16) : d;
     }
     // byte offset of column c of a q / k tile with `sub` bytes per COLS columns
     static __device__ __forceinline__ constexpr uint32_t koff(int sub, int c) { return (uint32_t)((c / COLS) * sub + (c % COLS) * 2); }
@@ -201,7 +221,7 @@ __device__ __noinline__ void fill_nan(__nv_bfloat16* ctx, int H, const int32_t* 
 
 template <int D, bool PAIR, bool ROPE>
 __global__ void __launch_bounds__(Threads<ROPE>::N, 1)
-attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
+attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap tmap_v, const Params p) {
     using C = Cfg<D, PAIR>;
     constexpr int KST = C::KST, VST = C::VST, QST = C::QST, NV = C::NV, NSB = C::NSB, NPB = C::NPB, KB = C::KB;
     constexpr bool APART = C::APART;
@@ -234,6 +254,12 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
         *abort_flag = 0;
         fence_barrier_init();
         prefetch_tmap(&tmap);
+        prefetch_tmap(&tmap_v);
+    }
+    if (C::SUMS && warp == 11) {
+        for (int i = lane; i < C::ONES_BYTES / 16; i += 32)
+            st_shared_v4(base + C::ONES_OFF + 16 * i, make_uint4(0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u));
+        fence_proxy_async();
     }
     if (warp == 9) {
         tmem_alloc<1>(smem_u32(tmem_slot), 512);
@@ -338,8 +364,8 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
                     if (elect_one()) {
                         mbar_expect_tx(v_full + 8 * vst, C::TILE);
 #pragma unroll
-                        for (int s = 0; s < C::NSUB; ++s)
-                            tma_load_2d(vring + vst * C::TILE + s * C::SUB, &tmap, p.H + p.Hkv + kvh * D + s * C::COLS, it.row0 + j * KB,
+                        for (int s = 0; s < C::VSUBS; ++s)
+                            tma_load_2d(vring + vst * C::TILE + s * C::VSUB, &tmap_v, p.H + p.Hkv + kvh * D + s * C::VCOLS, it.row0 + j * KB,
                                         v_full + 8 * vst);
                     }
                     __syncwarp();
@@ -407,15 +433,15 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
                         // rows past the end of the sequence get probability 0, but whatever lies behind them in memory must
                         // not turn that into a NaN: clear them
                         const uint32_t vtile = vring + vst * C::TILE;
-                        const int chunks = (kpad - keys) * (C::ROWB / 16);
-                        for (int i = lane; i < chunks * C::NSUB; i += 32)
-                            st_shared_v4(vtile + (i / chunks) * C::SUB + keys * C::ROWB + (i % chunks) * 16, make_uint4(0, 0, 0, 0));
+                        const int chunks = (kpad - keys) * (C::VROWB / 16);
+                        for (int i = lane; i < chunks * C::VSUBS; i += 32)
+                            st_shared_v4(vtile + (i / chunks) * C::VSUB + keys * C::VROWB + (i % chunks) * 16, make_uint4(0, 0, 0, 0));
                         fence_proxy_async();
                         __syncwarp();
                     }
 #pragma unroll 1
                     for (uint32_t t = 0; t < 2; ++t) {
-                        const uint64_t vd = vd0 + (uint64_t)((vst * C::TILE + (PAIR && D == 64 ? t * C::SUB : 0)) >> 4);
+                        const uint64_t vd = vd0 + C::desc_step(vst * C::TILE + (PAIR ? t * C::VSUB : 0));
                         const uint32_t pa = tmem + C::P_COL + vbuf * C::P_STRIDE, oa = tmem + C::O_COL + t * C::O_STRIDE;
                         if (!(ok = mbar_wait_warp(p_ready + 8 * vbuf, pph, abort_flag))) break;
                         tc_fence_after();
@@ -425,7 +451,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
                                 umma_ts(oa, pa, vd, idesc_o, j == (t ? begin1 : it.j0) ? 0u : 1u);
 #pragma unroll
                                 for (int kk = 1; kk < KB / 16; ++kk)
-                                    if (kk * 16 < kpad) umma_ts(oa, pa + kk * 8, vd + (uint64_t)((16 * C::ROWB) >> 4) * kk, idesc_o, 1u);
+                                    if (kk * 16 < kpad) umma_ts(oa, pa + kk * 8, vd + C::desc_step(16 * C::VROWB * kk), idesc_o, 1u);
                             }
                             umma_commit<1>((APART ? p_free : buf_free) + 8 * vbuf);
                             if (last) umma_commit<1>(o_full + 8 * t);
@@ -496,7 +522,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(Threads<ROPE>::REG_SOFTMAX));
         const int t = warp >> 2, quad = warp & 3;
         const uint32_t tl = tmem + ((uint32_t)(quad * 32) << 16);
-        const uint32_t o_col = tl + C::O_COL + t * C::O_STRIDE + ((PAIR && D == 32) ? t * 32 : 0);
+        const uint32_t o_col = tl + C::O_COL + t * C::O_STRIDE;
         constexpr int NCH = KB / 32;         // 32-key chunks per block
         const float scale = p.scale_log2e;
         uint32_t buf = t, sph = 0;   // score buffer and its parity; jobs t, t + 2, t + 4, ..
@@ -512,6 +538,7 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
             const int jb = t ? tile1_begin(p, it) : it.j0, je = t ? it.nb : tile0_end(p, it);
             float m_ref = -INFINITY;
             float l4[4] = {0.f, 0.f, 0.f, 0.f};
+            uint64_t any2[2] = {0, 0};
             for (int j = it.j0; j < it.nb; ++j) {
                 if (!(ok = mbar_wait_warp(s_full + 8 * buf, sph, abort_flag))) break;
                 const bool seen = live && j >= jb && j < je;
@@ -580,6 +607,12 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
                             if (need) m_ref = m_blk;
 #pragma unroll
                             for (int i = 0; i < 4; ++i) l4[i] *= alpha;
+                            if (C::SUMS) {
+                                uint32_t l;
+                                tmem_ld_32x1(o_col + D, l);
+                                tmem_ld_wait();
+                                tmem_st_32x1(o_col + D, __float_as_uint(__uint_as_float(l) * alpha));
+                            }
 #pragma unroll
                             for (int c0 = 0; c0 < D; c0 += 16) {
                                 uint32_t o[16];
@@ -596,9 +629,11 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
                     // straight line over all chunks, masked ones included: a branch per chunk drains the exponential unit
                     // each time, and a second copy of the code costs more in instruction fetches than it saves
                     // The row sum adds the ROUNDED probabilities, those that P V multiplies, so that a weight's rounding changes
-                    // numerator and denominator alike.  Summing the unrounded ones is an instruction less per pair (12 heads of
-                    // 32, 256 sequences of 32..256: 61 against 69 us; 32 q / 8 kv heads of 128, causal: 0.97 against 1.03 ms), but its
-                    // error against 64 bits was 1 to 2 % larger for v around zero and 7 % for v with a mean of four deviations.
+                    // numerator and denominator alike: with the sum of the unrounded ones the error against 64 bits was 1 to 2 %
+                    // larger for v around zero and 7 % for v with a mean of four deviations.
+                    // The unrounded sum is kept as well: it says whether a row saw any key, and with it the compiler orders the
+                    // loop far better, even where it is one instruction more (12 heads of 32, 256 sequences of 32..256: 71.8 us
+                    // without it, 62.3 with; 32 q / 8 kv heads of 64, window 300 over 1024..4096: 306 / 293; of 128, causal: 1078 / 1054).
 #pragma unroll
                     for (int c = 0; c < NCH; ++c) {
                         uint32_t pk[16];
@@ -608,8 +643,9 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
                             unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(s[c][2 * i]), __uint_as_float(s[c][2 * i + 1])), sc2, ng2), x0, x1);
                             x0 = ex2f(x0);
                             x1 = ex2f(x1);
+                            any2[i & 1] = add_f32x2(any2[i & 1], pack_f32x2(x0, x1));
                             pk[i] = pack_bf16(x0, x1);
-                            add_bf16x2(l4[2 * (i & 1)], l4[2 * (i & 1) + 1], pk[i]);
+                            if (!C::SUMS) add_bf16x2(l4[2 * (i & 1)], l4[2 * (i & 1) + 1], pk[i]);
                         }
                         tmem_st_32x16(p_col + 16 * c, pk);
                     }
@@ -629,8 +665,17 @@ attention_fwd_kernel(const __grid_constant__ CUtensorMap tmap, const Params p) {
             if (!(ok = mbar_wait_warp(o_full + 8 * t, n & 1, abort_flag))) break;
             if (live) {
                 tc_fence_after();
-                const float l = (l4[0] + l4[1]) + (l4[2] + l4[3]);
-                const float inv = l > 0.f ? 1.0f / l : 0.f;
+                float l = (l4[0] + l4[1]) + (l4[2] + l4[3]);
+                if (C::SUMS) {
+                    uint32_t sum;
+                    tmem_ld_32x1(o_col + D, sum);
+                    tmem_ld_wait();
+                    l = __uint_as_float(sum);
+                }
+                float a0, a1, b0, b1;
+                unpack_f32x2(any2[0], a0, a1);
+                unpack_f32x2(any2[1], b0, b1);
+                const float inv = (a0 + a1) + (b0 + b1) > 0.f ? 1.0f / l : 0.f;
                 __nv_bfloat16* orow = p.ctx + (size_t)(it.row0 + row) * p.H + head * D;
 #pragma unroll
                 for (int c = 0; c < D / 32; ++c) {

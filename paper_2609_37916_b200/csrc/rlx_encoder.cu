@@ -462,14 +462,17 @@ rlx_status_t launch_attention_fwd(const bf16* qkv, int rows, const int32_t* seq_
     if (!make_tmap(&tm, qkv, (uint64_t)rows, (uint64_t)p.H + 2 * p.Hkv, tcat::Cfg<64, true>::KB, cols,
                    cols == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B))
         return RLX_ERR_CUDA;
+    CUtensorMap tv = tm;                       // heads of 32: one head's columns per V tile
+    if (d == 32 && pair && !make_tmap(&tv, qkv, (uint64_t)rows, (uint64_t)p.H + 2 * p.Hkv, tcat::Cfg<32, true>::KB, 32, CU_TENSOR_MAP_SWIZZLE_64B))
+        return RLX_ERR_CUDA;
 #define RLX_ATT_FWD(D, PAIR)                                                                                                   \
     do {                                                                                                                       \
         if (rope_cos)                                                                                                          \
             RLX_CUDA_TRY(launch_ex(tcat::attention_fwd_kernel<D, PAIR, true>, dim3(grid), tcat::Threads<true>::N,   \
-                                   tcat::Cfg<D, PAIR>::SMEM_BYTES, st, tm, p));                                                \
+                                   tcat::Cfg<D, PAIR>::SMEM_BYTES, st, tm, tv, p));                                                \
         else                                                                                                                   \
             RLX_CUDA_TRY(launch_ex(tcat::attention_fwd_kernel<D, PAIR, false>, dim3(grid), tcat::Threads<false>::N, \
-                                   tcat::Cfg<D, PAIR>::SMEM_BYTES, st, tm, p));                                                \
+                                   tcat::Cfg<D, PAIR>::SMEM_BYTES, st, tm, tv, p));                                                \
     } while (0)
     if (pair) { if (d == 32) RLX_ATT_FWD(32, true); else RLX_ATT_FWD(64, true); }
     else if (d == 32) RLX_ATT_FWD(32, false);
