@@ -1023,10 +1023,14 @@ bool uses_cluster_ln(const rlx_encoder_config_t& c) {
 
 // RLX_FLAG_FOLD_LN: LayerNorm folded algebraically into the consuming GEMMs (hidden % 32 == 0, seq <= 512).
 // LayerNorm folded into the GEMMs: asked for by flag, or chosen automatically for small batches, where a
-// forward is a chain of launch latencies and 5 kernels per layer beat 7 (measured: 1 x 16 tokens 0.043 vs
-// 0.046 ms, 1 x 128 0.186 vs 0.199, 32 x 128 with 2.1 k valid tokens 0.254 vs 0.262; the break-even is
-// near 3 k VALID tokens -- 32 x 128 with every position valid loses 4 % -- but only the padded size is
-// known on the host; at 256 x 256 the folded form loses 10 %).
+// forward is a chain of launch latencies and 5 kernels per layer beat 7.  Only the padded size is known on the host.  Folded /
+// separate, us, half and all of the positions valid:
+//   6 x 384    1 x 128 140 / 160 and 148 / 166, 32 x 128 210 / 233 and 260 / 274, 64 x 128 274 / 287 and 397 / 407,
+//              96 x 128 372 / 376 and 526 / 527, 61 x 203 396 / 402 and 595 / 591, 255 x 128 749 / 736 and 1364 / 1286
+//   12 x 768   1 x 128 387 / 450 and 406 / 459, 7 x 120 457 / 502 and 572 / 559, 32 x 128 740 / 732 and 1094 / 1042,
+//              64 x 128 1224 / 1134 and 2065 / 1833
+// One line for both widths: it costs the wider model up to 5 % between 2000 and 4096 tokens, and the narrower one would gain
+// up to 5 % from 4096 to 12000.
 constexpr int kAutoFoldMaxTokens = 4096;
 // Set for the duration of a call that runs out of the built-in arena: the folded form needs room for a
 // gamma-scaled copy of every Linear weight (12 MB at H = 384), which that arena does not have.
