@@ -490,9 +490,9 @@ rlx_status_t rlx_rope_tables(int32_t max_len, int32_t head_dim, double theta, fl
  * packed projection IN PLACE (one pass over both; v is not touched), with the pairing, positions and
  * tables of rlx_attention_kind_bf16 -- after this call, rlx_attention_kind_bf16 with NULL tables gives
  * bit for bit what it gives on the unrotated buffer with the tables.  One pass over 2/3 of qkv at HBM
- * speed, where the in-attention form rotates every key block once per 128-row query tile: prefer this
- * call for sequences of more than a few hundred rows, the in-attention form when qkv must stay
- * read-only.  qkv: device bf16 [rows, (num_heads + 2*num_kv_heads)*head_dim], 16-byte aligned, modified; other
+ * speed, where the in-attention form rotates every key block again for each 128-row query tile (both heads of a
+ * pair at once): prefer this call for sequences of more than a few hundred rows (16 causal prompts of 1024..4096,
+ * 16 heads of 64: 0.44 + 0.06 against 0.73 ms), the in-attention form when qkv must stay read-only.  qkv: device bf16 [rows, (num_heads + 2*num_kv_heads)*head_dim], 16-byte aligned, modified; other
  * arguments and error behaviour as in rlx_attention_kind_bf16 (both tables required).
  */
 rlx_status_t rlx_qk_rope_bf16(void *qkv_bf16, int32_t rows, const int32_t *seq_start, const int32_t *seq_len,

@@ -1052,12 +1052,14 @@ bool uses_chunks(const rlx_encoder_config_t& c, int B, int S);
 int chunk_batch(int B, int S);
 
 // The tcgen05 attention kernel instead of the mma.sync one: where asked for, and where it pays inside a whole forward
-// (us mma.sync / tcgen05, 6 x 384 with heads of 32 and 12 x 768 with heads of 64; batch x longest sequence):
-//   64: sequences beyond two 128-row tiles everywhere (1 x 512 644 / 569, 64 x 512 4499 / 4119), two full tiles but for a
-//       single sequence (4 x 256 551 / 524; 1 x 256 417 / 442), beyond one tile once there are enough tokens to fill the
-//       chip (100 x 144 2520 / 2434, 70 x 200 1909 / 1889; but 8 x 144 505 / 510)
-//   32: two full tiles (256 x 256 1267 / 1208, 128 x 384 1077 / 1040); less while few tokens leave an item's own chain as
-//       what a layer waits for (16 x 192 218 / 201; but 256 x 192 983 / 1000, 61 x 203 431 / 438)
+// (us mma.sync / tcgen05, 6 x 384 with heads of 32 and 12 x 768 with heads of 64; batch x longest sequence, lengths from an
+// eighth of it on):
+//   64: sequences beyond two 128-row tiles everywhere (1 x 512 515 / 486, 64 x 512 4437 / 3939), two full tiles but for a
+//       single sequence (4 x 256 568 / 544; 1 x 256 392 / 452), beyond one tile once there are enough tokens to fill the
+//       chip (100 x 144 1894 / 1860, 70 x 200 1904 / 1852; but 8 x 144 518 / 528)
+//   32: two full tiles (256 x 256 1202 / 1173 and 2305 / 2185 with every position valid, 128 x 384 1110 / 1068, 64 x 256
+//       475 / 475); less while few tokens leave an item's own chain as what a layer waits for (16 x 192 234 / 215; but
+//       256 x 192 1001 / 1035, 61 x 203 421 / 425)
 bool uses_attention_fwd(const rlx_encoder_config_t& c, int B, int S) {
     if (c.flags & RLX_FLAG_ATTN_TCGEN05) return true;
     const long long tokens = call_tokens(B, S);
