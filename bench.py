@@ -323,6 +323,8 @@ class EncoderRun:
         self.out_h = torch.empty((B, H), dtype=torch.float32).pin_memory()
         self.flush = torch.empty(256 << 20, dtype=torch.uint8, device="cuda")
         self.n_kernels = self.enc.kernels_per_forward(B, S)
+        # the timed forward may run QKV GEMM and attention as one kernel; the instrumented one keeps them apart
+        self.n_launches = self.enc.launches_per_forward(B, S)
         per_layer = (self.n_kernels - 3) // cfg.num_layers
         # 7 = plain layer; 5 = both LayerNorms fused into the GEMMs; 3 = QKV GEMM, attention, one kernel for the rest
         fused_ffn = per_layer == 3
@@ -517,7 +519,7 @@ def run_ours(args):
                     "h2d_bytes_per_step": 2 * B * S * 4, "d2h_bytes_per_step": B * H * 4,
                     "timing": "host wall clock around rlx_encoder_forward_host with pinned host buffers: the kernels read ids / mask from, and write the embeddings to, host memory over the bus (no separate copy operations), then the stream is synchronised"},
             # main chain + the side-branch weight prefetch kernel (models whose Linear weights fit in L2)
-            "gpu_launches": args.steps * (run.n_kernels + (1 if cfg.num_layers * 24 * cfg.hidden * cfg.hidden <= (48 << 20)
+            "gpu_launches": args.steps * (run.n_launches + (1 if cfg.num_layers * 24 * cfg.hidden * cfg.hidden <= (48 << 20)
                                                            and cfg.ffn == 4 * cfg.hidden else 0)),
             "clocks": sampler.summary(),
             "roofline": roofline,

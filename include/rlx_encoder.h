@@ -290,8 +290,12 @@ rlx_status_t rlx_encoder_forward_static(rlx_encoder_t *encoder, const int32_t *t
  */
 rlx_status_t rlx_encoder_last_device_status(rlx_encoder_t *encoder, void *workspace, void *cuda_stream);
 
-/* Number of kernels one forward of (batch, seq) launches (for launch accounting). */
+/* Number of kernels of one forward of (batch, seq), the steps of its layers counted apart: the entries of
+ * rlx_encoder_kernel_times.  A forward of at most 4096 positions in sequences of at most 128 runs a layer's QKV GEMM and
+ * attention as one kernel unless RLX_FLAG_KERNEL_EVENTS, _NO_PACK or _ATTN_TCGEN05 is set (bit for bit the same result);
+ * rlx_encoder_launches_per_forward counts those as one. */
 int32_t rlx_encoder_kernels_per_forward(const rlx_encoder_t *encoder, int32_t batch, int32_t seq);
+int32_t rlx_encoder_launches_per_forward(const rlx_encoder_t *encoder, int32_t batch, int32_t seq);
 
 /*
  * Self-test of the device-side failure path (no fault is provoked): a one-thread kernel waits on a

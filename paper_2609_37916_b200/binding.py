@@ -40,7 +40,7 @@ STATIC_WORKSPACE_BYTES = 16 << 20
 
 EXPORTS = (
     "rlx_encoder_create", "rlx_encoder_destroy", "rlx_encoder_workspace_bytes", "rlx_encoder_forward",
-    "rlx_encoder_forward_host", "rlx_encoder_forward_tp", "rlx_encoder_forward_static", "rlx_encoder_last_device_status", "rlx_encoder_kernels_per_forward", "rlx_encoder_kernel_times",
+    "rlx_encoder_forward_host", "rlx_encoder_forward_tp", "rlx_encoder_forward_static", "rlx_encoder_last_device_status", "rlx_encoder_kernels_per_forward", "rlx_encoder_launches_per_forward", "rlx_encoder_kernel_times",
     "rlx_status_string", "rlx_pack_sequences", "rlx_embed_layernorm", "rlx_layernorm", "rlx_gemm_bf16", "rlx_gemm_residual_layernorm_bf16", "rlx_attention_bf16",
     "rlx_attention_f32", "rlx_attention_packed_bf16", "rlx_attention_kind_bf16", "rlx_attention_kind_status_bf16", "rlx_rope_tables", "rlx_qk_rope_bf16", "rlx_dequant_block_scaled_bf16", "rlx_scaled_matmul_bf16", "rlx_quantise_mx", "rlx_mx_matmul_bf16", "rlx_ffn_fused_bf16", "rlx_layer_tail_bf16", "rlx_selftest_bounded_wait", "rlx_pool_l2norm",
 )
@@ -180,6 +180,9 @@ class Encoder:
 
     def kernels_per_forward(self, batch: int, seq: int) -> int:
         return int(_load().rlx_encoder_kernels_per_forward(self._h, batch, seq))
+
+    def launches_per_forward(self, batch: int, seq: int) -> int:
+        return int(_load().rlx_encoder_launches_per_forward(self._h, batch, seq))
 
     def alloc_workspace(self, batch: int, seq: int, device="cuda") -> torch.Tensor:
         n = self.workspace_bytes(batch, seq)

@@ -1,0 +1,341 @@
+// QKV projection and attention of short sequences in one kernel: ctx = attention(x Wqkv^T + b), or with the LayerNorm in front
+// folded in (epilogue mode 3 of gemm_tcgen05.cuh).
+//
+// A CTA takes a bin (consecutive whole sequences with at most 128 packed rows together, see pack_sequences_kernel) and HPC
+// heads: it multiplies the bin's rows with those heads' rows of Wqkv (TMA -> tcgen05, accumulators in tensor memory), puts q,
+// k and v as bf16 where the operand ring was, and attends from there with mma.sync, a warp per 16 rows of a sequence.  Every
+// number is formed as the two separate kernels form it (same order along K, same epilogue, same softmax steps), so the
+// result is bit for bit theirs, and a sequence's does not depend on its bin.
+//
+// What bounds it: latency, as everything in a small forward; the point is the link that is not there.  A kernel boundary
+// costs the store of q, k, v, the hand-over and the round trip of the loads behind it.
+//
+// All waits are bounded.
+#pragma once
+#include "attention.cuh"
+#include "gemm_tcgen05.cuh"
+
+namespace rlx {
+namespace tcqa {
+
+using namespace rlx::tc;
+
+constexpr int kRows = kBinRows;
+constexpr int kWarps = 12;                    // epilogue: a 32-row quadrant of q, of k or of v; then attention
+constexpr int kThreads = 64 + 32 * kWarps;
+constexpr int kMaxTasks = kRows / 16 + kBinSeqs;   // 16-row groups of a bin's sequences
+
+template <int D, int HPC>
+struct Cfg {
+    static constexpr int N = 3 * D * HPC;                     // columns: q of the heads, then k, then v
+    static constexpr int NC = N / 96;                         // 32-column chunks of a warp
+    static constexpr int KPS = N == 96 ? 2 : 1;               // k-blocks per stage
+    static constexpr int STAGES = N == 96 ? 3 : 5;
+    static constexpr int A_BYTES = kRows * BLOCK_K * 2, B_BYTES = N * BLOCK_K * 2, KB_BYTES = A_BYTES + B_BYTES;
+    static constexpr int STAGE_BYTES = KPS * KB_BYTES;
+    static constexpr int TMEM_COLS = N <= 128 ? 128 : 256;
+    static constexpr int STR = D + 8;                         // elements per q / k / v row: conflict-free ldmatrix
+    static constexpr int VEC_OFF = STAGES * STAGE_BYTES;
+    static constexpr int ZERO_OFF = VEC_OFF + kWarps * 384;   // a row of zeros, read in place of v past a sequence's end
+    static constexpr int TASK_OFF = ZERO_OFF + (STR * 2 + 15) / 16 * 16;
+    static constexpr int BAR_OFF = TASK_OFF + kMaxTasks * 16;
+    static constexpr int SMEM_BYTES = BAR_OFF + 8 * (2 * STAGES + 1) + 16 + 1024;
+    static_assert(N == 96 || N == 192, "tile");
+    static_assert(3 * HPC * kRows * STR * 2 <= STAGES * STAGE_BYTES, "q, k and v over the ring");
+    static_assert(SMEM_BYTES <= 227 * 1024, "shared memory");
+};
+
+// Attention of 16 query rows of one sequence, as attention_bf16_kernel computes it: online softmax in steps of 32 (heads of 32) or
+// 64 keys.  q: the first query row, k / v: the sequence's first key, all with STR elements per row; keys: length of the
+// sequence, rows: query rows that exist.  The result replaces the q rows and goes to ctx from there.
+template <int D, int STR>
+__device__ __forceinline__ void attend16(__nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v, uint32_t zero_row, int keys,
+                                         int rows, float scale_log2e, __nv_bfloat16* ctx, size_t ldc) {
+    constexpr int KT = D / 16, ND = D / 8, KS = D == 32 ? 32 : 64, NT = KS / 8;
+    const int lane = threadIdx.x & 31, g = lane >> 2, t4 = lane & 3, mi = lane >> 3;
+    uint32_t qf[KT][4];
+#pragma unroll
+    for (int kt = 0; kt < KT; ++kt)
+        ldmatrix_x4(smem_u32(q + ((lane & 7) + (mi & 1) * 8) * STR + kt * 16 + (lane >> 4) * 8), qf[kt][0], qf[kt][1], qf[kt][2], qf[kt][3]);
+    float o[ND][4];
+#pragma unroll
+    for (int i = 0; i < ND; ++i) { o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f; }
+    float m_run[2] = {-INFINITY, -INFINITY};
+    float l_acc[4] = {0.f, 0.f, 0.f, 0.f};
+    constexpr uint32_t kOnesBf16x2 = 0x3F803F80u;
+#pragma unroll 1
+    for (int k0 = 0; k0 < keys; k0 += KS) {
+        float s[NT][4];
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) {
+            s[nt][0] = s[nt][1] = s[nt][2] = s[nt][3] = 0.f;
+#pragma unroll
+            for (int kp = 0; kp < KT / 2; ++kp) {
+                uint32_t b0, b1, b2, b3;
+                ldmatrix_x4(smem_u32(k + (k0 + nt * 8 + (lane & 7)) * STR + kp * 32 + (mi & 1) * 8 + (mi >> 1) * 16), b0, b1, b2, b3);
+                mma_bf16_16816(s[nt], qf[2 * kp][0], qf[2 * kp][1], qf[2 * kp][2], qf[2 * kp][3], b0, b1);
+                mma_bf16_16816(s[nt], qf[2 * kp + 1][0], qf[2 * kp + 1][1], qf[2 * kp + 1][2], qf[2 * kp + 1][3], b2, b3);
+            }
+        }
+        if (k0 + KS > keys) {
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) {
+                const int kk = k0 + nt * 8 + 2 * t4;
+                if (kk >= keys) { s[nt][0] = -INFINITY; s[nt][2] = -INFINITY; }
+                if (kk + 1 >= keys) { s[nt][1] = -INFINITY; s[nt][3] = -INFINITY; }
+            }
+        }
+        float mx[2] = {fmaxf(s[0][0], s[0][1]), fmaxf(s[0][2], s[0][3])};
+#pragma unroll
+        for (int nt = 1; nt < NT; ++nt) {
+            mx[0] = fmax3(mx[0], s[nt][0], s[nt][1]);
+            mx[1] = fmax3(mx[1], s[nt][2], s[nt][3]);
+        }
+        float alpha[2], msub[2];
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], 1));
+            mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], 2));
+            const float m_new = fmaxf(m_run[r], mx[r] * scale_log2e);
+            msub[r] = (m_new == -INFINITY) ? 0.f : m_new;
+            alpha[r] = fast_exp2(m_run[r] - msub[r]);
+            m_run[r] = m_new;
+        }
+        const uint64_t a0 = att_pack2(alpha[0], alpha[0]), a1 = att_pack2(alpha[1], alpha[1]);
+#pragma unroll
+        for (int nd = 0; nd < ND; ++nd) {
+            att_unpack2(att_mul2(att_pack2(o[nd][0], o[nd][1]), a0), o[nd][0], o[nd][1]);
+            att_unpack2(att_mul2(att_pack2(o[nd][2], o[nd][3]), a1), o[nd][2], o[nd][3]);
+        }
+        l_acc[0] *= alpha[0];
+        l_acc[2] *= alpha[1];
+        uint32_t pf[NT / 2][4];
+        const uint64_t c2 = att_pack2(scale_log2e, scale_log2e);
+        const uint64_t nm0 = att_pack2(-msub[0], -msub[0]), nm1 = att_pack2(-msub[1], -msub[1]);
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) {
+            float x0, x1, x2, x3;
+            att_unpack2(att_fma2(att_pack2(s[nt][0], s[nt][1]), c2, nm0), x0, x1);
+            att_unpack2(att_fma2(att_pack2(s[nt][2], s[nt][3]), c2, nm1), x2, x3);
+            pf[nt >> 1][(nt & 1) * 2 + 0] = pack_bf16(fast_exp2(x0), fast_exp2(x1));
+            pf[nt >> 1][(nt & 1) * 2 + 1] = pack_bf16(fast_exp2(x2), fast_exp2(x3));
+        }
+#pragma unroll
+        for (int kk = 0; kk < NT / 2; ++kk) {
+            mma_bf16_16816(l_acc, pf[kk][0], pf[kk][1], pf[kk][2], pf[kk][3], kOnesBf16x2, kOnesBf16x2);
+            // behind the sequence's end lie another's rows: probability 0 times whatever they hold must stay 0
+            const int r = k0 + kk * 16 + (mi & 1) * 8 + (lane & 7);
+            const uint32_t vrow = r < keys ? smem_u32(v + r * STR) : zero_row;
+#pragma unroll
+            for (int np = 0; np < ND / 2; ++np) {
+                uint32_t b0, b1, b2, b3;
+                ldmatrix_x4_trans(vrow + (np * 16 + (mi >> 1) * 8) * 2, b0, b1, b2, b3);
+                mma_bf16_16816(o[2 * np], pf[kk][0], pf[kk][1], pf[kk][2], pf[kk][3], b0, b1);
+                mma_bf16_16816(o[2 * np + 1], pf[kk][0], pf[kk][1], pf[kk][2], pf[kk][3], b2, b3);
+            }
+        }
+    }
+    float l_run[2] = {l_acc[0], l_acc[2]};
+#pragma unroll
+    for (int r = 0; r < 2; ++r) l_run[r] = l_run[r] > 0.f ? 1.0f / l_run[r] : 0.f;
+    // rows past the sequence's end are the next one's queries: left alone
+#pragma unroll
+    for (int nd = 0; nd < ND; ++nd) {
+        if (g < rows) *reinterpret_cast<uint32_t*>(q + g * STR + nd * 8 + 2 * t4) = pack_bf16(o[nd][0] * l_run[0], o[nd][1] * l_run[0]);
+        if (g + 8 < rows)
+            *reinterpret_cast<uint32_t*>(q + (g + 8) * STR + nd * 8 + 2 * t4) = pack_bf16(o[nd][2] * l_run[1], o[nd][3] * l_run[1]);
+    }
+    __syncwarp();
+    constexpr int CH = D / 8;
+    for (int i = lane; i < 16 * CH; i += 32) {
+        const int r = i / CH, c = i % CH;
+        if (r < rows) *reinterpret_cast<uint4*>(ctx + r * ldc + c * 8) = *reinterpret_cast<const uint4*>(q + r * STR + c * 8);
+    }
+}
+
+struct AttParams {
+    const int32_t *bins, *seq_start;   // pack_sequences_kernel's
+    __nv_bfloat16* ctx;                // [rows, H]
+    float scale_log2e;
+};
+
+// grid (heads / HPC, bins that there can be); tmap_a: x as k-blocks of 128 rows, tmap_w: Wqkv as [q | k | v][row][column], boxes of
+// 3 x D HPC x 64.  p: bias / folding vectors and row statistics of the product, K = H.
+template <int D, int HPC, int EPI>
+__global__ void __launch_bounds__(kThreads, 1)
+qkv_attention_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_w, const Params p,
+                     const AttParams ap) {
+    using C = Cfg<D, HPC>;
+    extern __shared__ unsigned char smem_raw[];
+    const uint32_t raw = smem_u32(smem_raw);
+    const uint32_t base = (raw + 1023u) & ~1023u;
+    unsigned char* gbase = smem_raw + (base - raw);
+    const uint32_t full_bar = base + C::BAR_OFF, empty_bar = full_bar + 8 * C::STAGES, acc_bar = empty_bar + 8 * C::STAGES;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + C::BAR_OFF + 8 * (2 * C::STAGES + 1));
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    int4* tasks = reinterpret_cast<int4*>(gbase + C::TASK_OFF);   // first row in the bin, query row offset, length
+    const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const int bin = blockIdx.y, head0 = blockIdx.x * HPC, H = p.K, num_kb = H / BLOCK_K;
+    pdl_launch_dependents();
+
+    const bool exists = bin < ld_early(ap.bins);
+    const int b0 = exists ? ld_early(ap.bins + 1 + bin) : 0, b1 = exists ? ld_early(ap.bins + 2 + bin) : 0;
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < C::STAGES; ++i) { mbar_init(full_bar + 8 * i, 1); mbar_init(empty_bar + 8 * i, 1); }
+        mbar_init(acc_bar, 1);
+        *abort_flag = 0;
+        fence_barrier_init();
+        prefetch_tmap(&tmap_a);
+        prefetch_tmap(&tmap_w);
+    }
+    if (warp == 1) {
+        tmem_alloc<1>(smem_u32(tmem_slot), C::TMEM_COLS);
+        tmem_relinquish<1>();
+    }
+    const int row0 = exists ? ld_early(ap.seq_start + b0) : 0, rows = exists ? ld_early(ap.seq_start + b1) - row0 : 0;
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = warp_uniform(*tmem_slot);
+
+    if (warp == 0) {
+        // ------------------------------------------------------------ TMA producer (whole warp, one lane issues)
+        auto load_w = [&](int kb, int stage) {
+            mbar_expect_tx(full_bar + 8 * stage, C::STAGE_BYTES);
+            for (int i = 0; i < C::KPS; ++i)
+                tma_load_3d(base + stage * C::STAGE_BYTES + C::KPS * C::A_BYTES + i * C::B_BYTES, &tmap_w, (kb + i) * BLOCK_K, head0 * D, 0,
+                            full_bar + 8 * stage);
+        };
+        auto load_a = [&](int kb, int stage) { tma_load_3d(base + stage * C::STAGE_BYTES, &tmap_a, 0, row0, kb, full_bar + 8 * stage); };
+        int early = 0;   // weights do not come from the previous kernel
+        if (rows > 0)
+            for (; early < C::STAGES && early * C::KPS < num_kb; ++early) {
+                if (elect_one()) load_w(early * C::KPS, early);
+                __syncwarp();
+            }
+        pdl_wait();
+        if (rows > 0) {
+            int stage = 0;
+            uint32_t phase = 0;
+            for (int kb = 0; kb < num_kb; kb += C::KPS) {
+                if (early > 0) {
+                    --early;
+                    if (elect_one()) load_a(kb, stage);
+                } else {
+                    if (!mbar_wait_warp(empty_bar + 8 * stage, phase ^ 1, abort_flag)) break;
+                    if (elect_one()) { load_w(kb, stage); load_a(kb, stage); }
+                }
+                __syncwarp();
+                if (++stage == C::STAGES) { stage = 0; phase ^= 1; }
+            }
+        }
+    } else if (warp == 1) {
+        // ------------------------------------------------------------ MMA issuer (whole warp, one lane issues)
+        if (rows > 0) {
+            constexpr uint32_t idesc = make_idesc(kRows, C::N);
+            const uint64_t adesc0 = make_smem_desc(base), bdesc0 = make_smem_desc(base + C::KPS * C::A_BYTES);
+            uint32_t stage = 0, phase = 0;
+            bool ok = true, ready = false;
+            for (int kb = 0; kb < num_kb; kb += C::KPS) {
+                if (!__all_sync(0xffffffffu, ready) && !(ok = mbar_wait_warp(full_bar + 8 * stage, phase, abort_flag))) break;
+                tc_fence_after();
+                const uint32_t cur = stage;
+                if (++stage == C::STAGES) { stage = 0; phase ^= 1; }
+                ready = mbar_test_wait(full_bar + 8 * stage, phase);
+                if (elect_one()) {
+                    const uint64_t ad0 = adesc0 + cur * (C::STAGE_BYTES >> 4), bd0 = bdesc0 + cur * (C::STAGE_BYTES >> 4);
+#pragma unroll
+                    for (int i = 0; i < C::KPS; ++i)
+#pragma unroll
+                        for (int k = 0; k < BLOCK_K / UMMA_K; ++k)
+                            umma_bf16<1>(tmem, ad0 + (i * (C::A_BYTES >> 4) + 2 * k), bd0 + (i * (C::B_BYTES >> 4) + 2 * k), idesc,
+                                         (kb | i | k) != 0 ? 1u : 0u);
+                    umma_commit<1>(empty_bar + 8 * cur);
+                }
+                __syncwarp();
+            }
+            if (ok && elect_one()) umma_commit<1>(acc_bar);
+            __syncwarp();
+        }
+    } else {
+        // ------------------------------------------------------------ q, k, v, then attention
+        const int e = warp - 2, quad = warp & 3, part = e >> 2;
+        const int n0 = part * H + head0 * D;
+        using ET = EpilogueTile<EPI, C::NC, true>;
+        ET et;
+        et.load_vectors(p, n0, base + C::VEC_OFF + e * 384);
+        // the bin's row groups and the row of zeros
+        int ntasks = 0;
+        {
+            const int i = b0 + lane, nseq = b1 - b0;
+            const int first = lane < nseq ? ld_early(ap.seq_start + i) - row0 : 0;
+            const int len = lane < nseq ? ld_early(ap.seq_start + i + 1) - row0 - first : 0;
+            const int mine = (len + 15) / 16;
+            int incl = mine;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int n = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += n;
+            }
+            ntasks = __shfl_sync(0xffffffffu, incl, 31);
+            if (e == 0)
+                for (int j = 0; j < mine; ++j) tasks[incl - mine + j] = make_int4(first, 16 * j, len, 0);
+            if (e == 1 && lane < (C::STR * 2 + 15) / 16) st_shared_v4(base + C::ZERO_OFF + lane * 16, make_uint4(0, 0, 0, 0));
+        }
+        pdl_wait();
+        const int row = quad * 32 + lane;
+        const bool live = quad * 32 < rows;
+        bool ok = true;
+        if (live) {
+            et.prefetch(p, row0 + rows, row0 + row, n0);
+            ok = mbar_wait_warp(acc_bar, 0, abort_flag);
+            tc_fence_after();
+            uint32_t r[C::NC][32];
+#pragma unroll
+            for (int c = 0; c < C::NC; ++c) tmem_ld_32x32(tmem + ((uint32_t)(quad * 32) << 16) + part * (D * HPC) + c * 32, r[c]);
+            tmem_ld_wait();
+#pragma unroll
+            for (int c = 0; c < C::NC; ++c) {
+                uint4 v[4];
+                et.compute_chunk(p, r[c], n0 + c * 32, c, row0 + row, row < rows, p.bias + n0 + c * 32, v);
+                // column c * 32 of the part: head c (heads of 32), or column 32 c of the one head
+                const int hh = D == 32 ? c : 0, col = D == 32 ? 0 : c * 32;
+                const uint32_t dst = base + (uint32_t)(((part * HPC + hh) * kRows + row) * C::STR + col) * 2;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) st_shared_v4(dst + 16 * i, v[i]);
+            }
+            tc_fence_before();
+        } else if (rows > 0) {
+            ok = mbar_wait_warp(acc_bar, 0, abort_flag);   // the ring is free
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * kWarps) : "memory");
+        if (ok) {
+            __nv_bfloat16* qkv = reinterpret_cast<__nv_bfloat16*>(gbase);
+            for (int t = e; t < ntasks * HPC; t += kWarps) {
+                const int hh = t / ntasks;
+                const int4 task = tasks[t - hh * ntasks];
+                __nv_bfloat16* qh = qkv + hh * kRows * C::STR;
+                attend16<D, C::STR>(qh + (task.x + task.y) * C::STR, qh + (HPC * kRows + task.x) * C::STR,
+                                    qh + (2 * HPC * kRows + task.x) * C::STR, base + C::ZERO_OFF, task.z, min(16, task.z - task.y),
+                                    ap.scale_log2e, ap.ctx + (size_t)(row0 + task.x + task.y) * H + (head0 + hh) * D, (size_t)H);
+            }
+        }
+    }
+    // ---------------------------------------------------------------- teardown
+    __syncwarp();
+    if (*abort_flag) {
+        if (threadIdx.x == 0 && p.status) atomicOr(p.status, RLX_DEVSTAT_TIMEOUT_BIT);
+        const uint64_t t0 = global_timer_ns();
+        while (global_timer_ns() - t0 < 200000ull) __nanosleep(1000);
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        __syncwarp();
+        tc_fence_after();
+        tmem_dealloc<1>(tmem, C::TMEM_COLS);
+    }
+}
+
+}  // namespace tcqa
+}  // namespace rlx

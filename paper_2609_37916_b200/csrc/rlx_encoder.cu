@@ -23,6 +23,7 @@
 #include "gemm_cln_tcgen05.cuh"
 #include "gemm_splitk_tcgen05.cuh"
 #include "rowwise.cuh"
+#include "qkv_attention_tcgen05.cuh"
 
 namespace {
 
@@ -268,6 +269,12 @@ cudaError_t init_kernels_for_current_device() {
                                   rlx::tcmx::MxCfg<128>::SMEM_BYTES)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(rlx::tcmx::gemm_mx_tcgen05_kernel<192>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   rlx::tcmx::MxCfg<192>::SMEM_BYTES)) != cudaSuccess) return e;
+#define RLX_QA_ATTR(D, HPC, EPI)                                                                               \
+    if ((e = cudaFuncSetAttribute(rlx::tcqa::qkv_attention_kernel<D, HPC, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                                  rlx::tcqa::Cfg<D, HPC>::SMEM_BYTES)) != cudaSuccess)                          \
+        return e;
+    RLX_QA_ATTR(32, 1, 0) RLX_QA_ATTR(32, 1, 3) RLX_QA_ATTR(32, 2, 0) RLX_QA_ATTR(32, 2, 3) RLX_QA_ATTR(64, 1, 0) RLX_QA_ATTR(64, 1, 3)
+#undef RLX_QA_ATTR
 #define RLX_ATT_FWD_ATTR(D, PAIR)                                                                              \
     if ((e = cudaFuncSetAttribute(rlx::tcat::attention_fwd_kernel<D, PAIR, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
                                   rlx::tcat::Cfg<D, PAIR>::SMEM_BYTES)) != cudaSuccess ||                       \
@@ -333,15 +340,16 @@ struct Packing {   // device arrays written by pack_sequences_kernel; all null i
     const int32_t* seq_len = nullptr;
     const int32_t* seq_start = nullptr;    // [B+1]; seq_start[B] = number of packed rows
     const int32_t* pos_of_rank = nullptr;
+    const int32_t* bins = nullptr;         // sequences by bins of at most 128 rows (QKV projection and attention in one kernel)
     int B = 0;
     const int32_t* total() const { return seq_start ? seq_start + B : nullptr; }
 };
 
 rlx_status_t launch_pack(const int32_t* mask, int B, int S, int32_t* seq_len, int32_t* seq_start,
                          int32_t* pos_of_rank, unsigned int* ticket, cudaStream_t st,
-                         cudaGraphConditionalHandle cond = 0, int cond_min_rows = 0) {
+                         cudaGraphConditionalHandle cond = 0, int cond_min_rows = 0, int32_t* bins = nullptr) {
     rlx::pack_sequences_kernel<<<B, rlx::kPackThreads, 0, st>>>(mask, B, S, seq_len, seq_start, pos_of_rank, ticket, cond,
-                                                                cond_min_rows);
+                                                                cond_min_rows, bins);
     RLX_CUDA_TRY(cudaGetLastError());
     return RLX_OK;
 }
@@ -830,6 +838,51 @@ rlx_status_t launch_gemm(const bf16* A, const bf16* W, const float* bias, const 
     return RLX_ERR_UNSUPPORTED;
 }
 
+// [q | k | v][row][column] view of Wqkv [3 H, H]: one box brings the same rows of all three.
+bool make_tmap_qkv(CUtensorMap* map, const void* ptr, uint64_t H, uint32_t box_rows) {
+    encode_tiled_fn fn = get_encode_fn();
+    if (!fn) return false;
+    cuuint64_t dims[3] = {H, H, 3};
+    cuuint64_t strides[2] = {H * sizeof(bf16), H * H * sizeof(bf16)};
+    cuuint32_t box[3] = {(cuuint32_t)rlx::tc::BLOCK_K, box_rows, 3};
+    cuuint32_t estr[3] = {1, 1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// QKV projection and attention in one kernel: ctx = attention(x Wqkv^T + bias), epi 0, or with a LayerNorm folded in, epi 3.
+// Bins that there can be: two consecutive ones closed for their rows have more than kBinRows together, the others hold
+// kBinSeqs sequences.
+int max_bins(int B, int S) {
+    return (int)std::min<long long>(B, 2ll * B * S / rlx::kBinRows + B / rlx::kBinSeqs + 1);
+}
+template <int D, int HPC>
+rlx_status_t launch_qkv_attention_d(const bf16* x, const bf16* w, const rlx::tc::Params& p, const rlx::tcqa::AttParams& ap, int epi,
+                                    int heads, int bins, cudaStream_t st) {
+    using C = rlx::tcqa::Cfg<D, HPC>;
+    CUtensorMap ta, tw;
+    if (!make_tmap_kblocks(&ta, x, (uint64_t)p.M, (uint64_t)p.K, rlx::tcqa::kRows, C::KPS) || !make_tmap_qkv(&tw, w, (uint64_t)p.K, D * HPC))
+        return RLX_ERR_CUDA;
+    const dim3 grid(heads / HPC, bins);
+    if (epi == 0) RLX_CUDA_TRY(launch_ex(rlx::tcqa::qkv_attention_kernel<D, HPC, 0>, grid, rlx::tcqa::kThreads, C::SMEM_BYTES, st, ta, tw, p, ap));
+    else RLX_CUDA_TRY(launch_ex(rlx::tcqa::qkv_attention_kernel<D, HPC, 3>, grid, rlx::tcqa::kThreads, C::SMEM_BYTES, st, ta, tw, p, ap));
+    RLX_CUDA_TRY(cudaGetLastError());
+    return RLX_OK;
+}
+rlx_status_t launch_qkv_attention(const bf16* x, const bf16* w, const float* bias, int epi, int B, int S, int H, int heads, bf16* ctx,
+                                  int32_t* status, cudaStream_t st, const Packing& pk, const LnFold* lf = nullptr) {
+    rlx::tc::Params p{};
+    p.bias = bias; p.M = B * S; p.N = 3 * H; p.K = H; p.status = status;
+    if (lf) { p.cvec = lf->cvec; p.dvec = lf->dvec; p.stats_in = lf->stats_in; p.stats_in_p = lf->stats_in_p; p.ln_eps = lf->eps; }
+    const int d = H / heads, bins = max_bins(B, S);
+    const rlx::tcqa::AttParams ap{pk.bins, pk.seq_start, ctx, 1.4426950408889634f / sqrtf((float)d)};
+    if (d == 64) return launch_qkv_attention_d<64, 1>(x, w, p, ap, epi, heads, bins, st);
+    // one head per CTA while every bin there can be finds its SMs, else two: a row's x is then loaded half as often
+    if (heads * bins <= sm_count()) return launch_qkv_attention_d<32, 1>(x, w, p, ap, epi, heads, bins, st);
+    return launch_qkv_attention_d<32, 2>(x, w, p, ap, epi, heads, bins, st);
+}
+
 // out = LN(A W^T + bias + residual): whole rows per CTA (N = 256, 384 or 512).
 rlx_status_t launch_gemm_ln(const bf16* A, const bf16* W, const float* bias, const bf16* residual, const float* gamma,
                             const float* beta, float eps, int M, int N, int K, bf16* out, int32_t* status,
@@ -1068,6 +1121,19 @@ bool uses_attention_fwd(const rlx_encoder_config_t& c, int B, int S) {
     return S >= 2 * kT || (S >= kT + kT / 2 && tokens <= 4096);
 }
 
+// QKV projection and attention in one kernel: no sequence longer than a bin, and few enough bins that they run beside each other (a
+// CTA does not overlap one bin's attention with the next one's products, as the separate kernels do).  Whole forwards, us
+// separate / in one:
+//   6 x 384    1 x 32 128 / 107, 1 x 128 142 / 119 and 150 / 126 (half and all of the positions valid), 4 x 128 160 / 125,
+//              16 x 64 155 / 145, 32 x 128 212 / 186 and 262 / 267, 256 x 16 276 / 227, 64 x 128 297 / 283, 128 x 64 296 / 304,
+//              96 x 128 374 / 387, 200 x 128 625 / 673
+//   12 x 768   1 x 128 386 / 349, 7 x 120 458 / 408 and 572 / 493, 32 x 128 745 / 706 and 1085 / 1073, 64 x 128 1107 / 1147
+constexpr long long kQkvAttentionMaxTokens = 4096;
+bool uses_qkv_attention(const rlx_encoder_config_t& c, int B, int S) {
+    if (c.flags & (RLX_FLAG_GEMM_SIMT | RLX_FLAG_KERNEL_EVENTS | RLX_FLAG_NO_PACK | RLX_FLAG_ATTN_TCGEN05)) return false;
+    return S <= rlx::kBinRows && call_tokens(B, S) <= kQkvAttentionMaxTokens && !uses_fused_ffn(c, B, S) && !uses_attention_fwd(c, B, S);
+}
+
 struct GraphEntry {
     int B, S;
     const void *ids, *mask, *out, *ws;
@@ -1173,11 +1239,13 @@ rlx_status_t enqueue_forward(const rlx_encoder* e, const int32_t* ids, const int
         }
     }
     Packing pk;
+    const bool fuse_qa = pack && uses_qkv_attention(c, B, S);
     if (pack) {
         int32_t* seq_len = reinterpret_cast<int32_t*>(ws + a.seq_len);
         int32_t* seq_start = reinterpret_cast<int32_t*>(ws + a.seq_start);
         int32_t* pos_of_rank = reinterpret_cast<int32_t*>(ws + a.pos_of_rank);
-        pk.seq_len = seq_len; pk.seq_start = seq_start; pk.pos_of_rank = pos_of_rank; pk.B = B;
+        int32_t* bins = fuse_qa ? reinterpret_cast<int32_t*>(qkv) : nullptr;   // the projection stays on the chip: its buffer is free
+        pk.seq_len = seq_len; pk.seq_start = seq_start; pk.pos_of_rank = pos_of_rank; pk.bins = bins; pk.B = B;
         // The tickets live in the status block, which the caller zeroes once before the first call; each
         // kernel leaves its own at zero again, so no memset node sits in front of the first kernel.
         unsigned int* ticket = reinterpret_cast<unsigned int*>(ws + a.status + kTicketOffset);
@@ -1192,7 +1260,7 @@ rlx_status_t enqueue_forward(const rlx_encoder* e, const int32_t* ids, const int
             if (cstat != cudaStreamCaptureStatusActive || gcap == nullptr) return RLX_ERR_CUDA;
             cudaGraphConditionalHandle cond;
             RLX_CUDA_TRY(cudaGraphConditionalHandleCreate(&cond, gcap, 0, cudaGraphCondAssignDefault));
-            RLX_TRY(launch_pack(mask, B, S, seq_len, seq_start, pos_of_rank, ticket, st, cond, kDeviceChoiceMinRows));
+            RLX_TRY(launch_pack(mask, B, S, seq_len, seq_start, pos_of_rank, ticket, st, cond, kDeviceChoiceMinRows, bins));
             RLX_CUDA_TRY(cudaStreamGetCaptureInfo_v2(st, &cstat, nullptr, &gcap, &deps, &ndeps));
             cudaGraphNodeParams np = {};
             np.type = cudaGraphNodeTypeConditional;
@@ -1217,7 +1285,7 @@ rlx_status_t enqueue_forward(const rlx_encoder* e, const int32_t* ids, const int
             if (forked) RLX_CUDA_TRY(cudaStreamWaitEvent(st, e->join_event, 0));   // join the side branch
             return RLX_OK;
         }
-        if (!body_only) RLX_TRY(launch_pack(mask, B, S, seq_len, seq_start, pos_of_rank, ticket, st));
+        if (!body_only) RLX_TRY(launch_pack(mask, B, S, seq_len, seq_start, pos_of_rank, ticket, st, 0, 0, bins));
     }
     const int32_t* rows = pk.total();
     const bool fuse_ln = !fold && uses_fused_ln(c, B, S);
@@ -1280,14 +1348,20 @@ rlx_status_t enqueue_forward(const rlx_encoder* e, const int32_t* ids, const int
             unsigned char* fb = ws + a.fold + (size_t)l * a.fold_layer;
             LnFold lf;
             lf.eps = c.ln_eps;
-            if (l == 0) {
-                RLX_TRY(launch_gemm(x, (const bf16*)lw.wqkv, lw.bqkv, nullptr, RLX_EPI_BIAS, T, 3 * H, H, qkv, false, status, st, rows));
-            } else {
+            if (l > 0) {
                 lf.cvec = (const float*)(fb + a.f_cqkv); lf.dvec = (const float*)(fb + a.f_dqkv);
                 lf.stats_in = stats_z; lf.stats_in_p = P;
+            }
+            if (fuse_qa) {
+                RLX_TRY(launch_qkv_attention(l == 0 ? x : z, l == 0 ? (const bf16*)lw.wqkv : (const bf16*)(fb + a.f_wqkv), lw.bqkv,
+                                             l == 0 ? RLX_EPI_BIAS : 3, B, S, H, h, ctx, status, st, pk, l == 0 ? nullptr : &lf));
+            } else if (l == 0) {
+                RLX_TRY(launch_gemm(x, (const bf16*)lw.wqkv, lw.bqkv, nullptr, RLX_EPI_BIAS, T, 3 * H, H, qkv, false, status, st, rows));
+            } else {
                 RLX_TRY(launch_gemm(z, (const bf16*)(fb + a.f_wqkv), lw.bqkv, nullptr, 3, T, 3 * H, H, qkv, false, status, st, rows, 0, &lf));
             }
-            if (pack && uses_attention_fwd(c, B, S))
+            if (fuse_qa) {
+            } else if (pack && uses_attention_fwd(c, B, S))
                 RLX_TRY(launch_attention_fwd(qkv, T, pk.seq_start, pk.seq_len, B, S, h, d, 1, false, 0, nullptr, nullptr, ctx, status, st));
             else
                 RLX_TRY(launch_attention_bf16(qkv, mask, pk.seq_start, pk.seq_len, B, S, h, d, ctx, st));
@@ -1325,8 +1399,10 @@ rlx_status_t enqueue_forward(const rlx_encoder* e, const int32_t* ids, const int
                             w->emb_ln_g, w->emb_ln_b, T, S, H, c.vocab, c.ln_eps, x, status, st, pk));
     for (int l = 0; l < c.num_layers; ++l) {
         const rlx_layer_weights_t& lw = w->layers[l];
-        RLX_TRY(launch_gemm(x, (const bf16*)lw.wqkv, lw.bqkv, nullptr, RLX_EPI_BIAS, T, 3 * H, H, qkv, simt, status, st, rows));
-        if (pack && uses_attention_fwd(c, B, S))
+        if (fuse_qa) RLX_TRY(launch_qkv_attention(x, (const bf16*)lw.wqkv, lw.bqkv, RLX_EPI_BIAS, B, S, H, h, ctx, status, st, pk));
+        else RLX_TRY(launch_gemm(x, (const bf16*)lw.wqkv, lw.bqkv, nullptr, RLX_EPI_BIAS, T, 3 * H, H, qkv, simt, status, st, rows));
+        if (fuse_qa) {
+        } else if (pack && uses_attention_fwd(c, B, S))
             RLX_TRY(launch_attention_fwd(qkv, T, pk.seq_start, pk.seq_len, B, S, h, d, 1, false, 0, nullptr, nullptr, ctx, status, st));
         else
             RLX_TRY(launch_attention_bf16(qkv, mask, pk.seq_start, pk.seq_len, B, S, h, d, ctx, st));
@@ -1587,6 +1663,11 @@ size_t rlx_encoder_workspace_bytes(const rlx_encoder_t* e, int32_t batch, int32_
 int32_t rlx_encoder_kernels_per_forward(const rlx_encoder_t* e, int32_t batch, int32_t seq) {
     if (!e || batch <= 0 || seq <= 0) return 0;
     return kernels_in_forward(e->cfg, batch, seq);
+}
+
+int32_t rlx_encoder_launches_per_forward(const rlx_encoder_t* e, int32_t batch, int32_t seq) {
+    if (!e || batch <= 0 || seq <= 0) return 0;
+    return kernels_in_forward(e->cfg, batch, seq) - (uses_qkv_attention(e->cfg, batch, seq) ? e->cfg.num_layers : 0);
 }
 
 rlx_status_t rlx_encoder_forward(rlx_encoder_t* e, const int32_t* ids, const int32_t* mask, int32_t B, int32_t S,

@@ -85,14 +85,18 @@ __device__ __forceinline__ void ln_normalise_store(float (&v)[NV * 4], const LnA
 //   seq_len[b]            number of valid positions of sequence b
 //   seq_start[0..B]       exclusive prefix sum of seq_len (seq_start[B] = total packed rows)
 //   pos_of_rank[b*S + r]  original position s of the r-th valid token of sequence b
+//   bins (optional)       consecutive sequences that have at most kBinRows rows, and are at most kBinSeqs, together: bins[0]
+//                         their number n, bins[1 + j] the first sequence of bin j, bins[1 + n] = B
 // One CTA per sequence; the last CTA to finish (ticket counter, reset for the next launch) scans
 // seq_len.  Integer work only.
 constexpr int kPackThreads = 128;
+constexpr int kBinRows = 128, kBinSeqs = 16;
 
 __global__ void __launch_bounds__(kPackThreads)
 pack_sequences_kernel(const int32_t* __restrict__ mask, int B, int S, int32_t* __restrict__ seq_len,
                       int32_t* __restrict__ seq_start, int32_t* __restrict__ pos_of_rank,
-                      unsigned int* __restrict__ ticket, cudaGraphConditionalHandle cond, int cond_min_rows) {
+                      unsigned int* __restrict__ ticket, cudaGraphConditionalHandle cond, int cond_min_rows,
+                      int32_t* __restrict__ bins) {
     __shared__ int warp_cnt[kPackThreads / 32];
     __shared__ int is_last;
     pdl_launch_dependents();
@@ -128,6 +132,7 @@ pack_sequences_kernel(const int32_t* __restrict__ mask, int B, int S, int32_t* _
     // exclusive scan of seq_len by the last CTA: each warp-sized chunk with shuffles, carried serially
     if (warp == 0) {
         int carry = 0;
+        int nbins = 0, in_bin = kBinSeqs, bin_rows = 0;
         for (int base = 0; base < B; base += 32) {
             const int i = base + lane;
             const int v = i < B ? *((volatile int32_t*)seq_len + i) : 0;
@@ -139,6 +144,22 @@ pack_sequences_kernel(const int32_t* __restrict__ mask, int B, int S, int32_t* _
             }
             if (i < B) seq_start[i] = carry + incl - v;
             carry += __shfl_sync(0xffffffffu, incl, 31);
+            if (bins != nullptr)
+                for (int k = 0; k < min(32, B - base); ++k) {
+                    const int len = __shfl_sync(0xffffffffu, v, k);
+                    if (in_bin == kBinSeqs || bin_rows + len > kBinRows) {
+                        if (lane == 0) bins[1 + nbins] = base + k;
+                        ++nbins;
+                        in_bin = 0;
+                        bin_rows = 0;
+                    }
+                    ++in_bin;
+                    bin_rows += len;
+                }
+        }
+        if (bins != nullptr && lane == 0) {
+            bins[0] = nbins;
+            bins[1 + nbins] = B;
         }
         if (lane == 0) {
             seq_start[B] = carry;

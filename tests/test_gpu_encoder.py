@@ -268,6 +268,30 @@ def test_folded_forward_splits_its_long_contraction(rlx, name, B, S, full):
     assert np.array_equal(got, again)
 
 
+@pytest.mark.parametrize("name,B,S,lengths", [
+    ("c1", 1, 1, "full"), ("c1", 1, 128, "full"), ("c1", 1, 16, "ragged"), ("c1", 5, 33, "ragged"),
+    ("c1", 12, 128, "full"), ("c1", 13, 128, "ragged"),                    # one head per CTA, two
+    ("c1", 40, 3, "ragged"), ("c1", 200, 17, "one"),                       # bins that are full by their number of sequences
+    ("c1", 32, 128, "ragged"), ("c1", 32, 128, "full"), ("c1", 31, 130, "ragged"), ("c1", 33, 125, "ragged"),   # the last sizes that take it, the first that do not
+    ("c4", 1, 128, "full"), ("c4", 7, 120, "ragged"), ("c4", 9, 64, "holes"), ("c4", 64, 31, "ragged"), ("c4", 32, 128, "ragged")])
+@pytest.mark.parametrize("flags", [0, 0x400])   # LayerNorm folded into the product, and a kernel of its own
+def test_projection_and_attention_in_one_kernel_give_the_bits_of_two(rlx, name, B, S, lengths, flags):
+    """The instrumented forward (RLX_FLAG_KERNEL_EVENTS) keeps the QKV GEMM and the attention apart.  Bins of several sequences, of
+    one, of empty ones, full and nearly full; heads of 32 and of 64."""
+    rng = np.random.default_rng(B * 1000 + S)
+    n = {"full": np.full(B, S), "one": np.ones(B, int)}.get(lengths, rng.integers(0, S + 1, size=B))
+    n[B // 2] = S
+    inp = make_inputs(CONFIGS[name], batch=B, seq=S, num_layers=2, lengths=n, ln_affine_random=True, mask_holes=0.2 if lengths == "holes" else 0.0)
+    w = rlx.upload_weights(inp.params, inp.layers)
+    one, status = run_gpu(rlx, inp, weights=w, flags=flags)
+    two, tstatus = run_gpu(rlx, inp, weights=w, flags=flags | 4)
+    eager, estatus = run_gpu(rlx, inp, weights=w, flags=flags | 1)
+    assert status == 0 and tstatus == 0 and estatus == 0
+    assert np.array_equal(one, two) and np.array_equal(one, eager)
+    pick = sorted({0, B // 2, B - 1})
+    check(one[pick], oracle.encoder_forward(inp.cfg, inp.ids[pick], inp.mask[pick], inp.params, inp.layers), inp.lengths[pick])
+
+
 @pytest.mark.parametrize("heads", [2, 4])
 @pytest.mark.parametrize("flags", [0, 0x200, 0x400])   # the host's choice, folded LayerNorm, none folded
 def test_a_short_last_chunk_takes_the_kernels_of_the_whole_call(rlx, heads, flags):
