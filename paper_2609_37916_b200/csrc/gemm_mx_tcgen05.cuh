@@ -23,8 +23,9 @@
 //  Accumulators are double-buffered in tensor memory, so that one tile's epilogue overlaps the next main loop.
 //  Scale words are handed over four k-blocks at a time, through two slots with barriers of their own; one commit per
 //  stage frees its operands.
-//  What bounds it is not settled: at 36736 x 384 x 1536 a stage takes about 1100 cycles, where its products need 384 and
-//  its 40 KB of operands, at the 80 bytes a clock that one SM draws from L2, 512.  A scale word is
+//  What bounds it: the operands.  36736 x 384 x 1536 moves 275 MB from L2 in 21 us, 13.1 TB/s; all SMs loading and nothing else
+//  drew 13.2 (32749 x 3072 x 768 in bf16).  128 x 384 tiles (220 MB; three stages, one accumulator) took as long there and longer
+//  at fewer rows (20000 x 384 x 1536 15.9 / 19.9).  A scale word is
 //  loaded once per tile, four k-blocks per 16-byte load where the row pitch allows; with each of four warps loading
 //  all of a stage's words one by one and writing its own quarter (12 loads of 32 rows each per warp and stage) those
 //  loads took longer than the operands.
@@ -189,17 +190,36 @@ gemm_mx_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
         const uint64_t adesc0 = make_smem_desc(base), bdesc0 = make_smem_desc(base + kOperandBytes);
         const uint32_t idesc0 = idesc_mx<BN>(p.a_fmt, p.w_fmt, 0);
         uint32_t ph = 0, tcount = 0, ss = 0, sph = 0;
+        // A group of four k-blocks' scale words goes to tensor memory at once, and a group ahead of its products where the words are
+        // there: copies and products run in the order they are issued, and a product right behind the copy that it needs waits for
+        // all of that copy's latency (product alone, 36736 x 384 x 1536 23.0 -> 21.4 us, 20000 rows 18.8 -> 16.8).
+        auto copy_group = [&](uint32_t slot) {
+#pragma unroll
+            for (int u = 0; u < ST; ++u)
+#pragma unroll
+                for (int g = 0; g <= C::W_GROUPS; ++g)
+                    copy_scales(elected, tmem + C::ACC_COLS + (slot * ST + u) * C::SF_COLS + 4 * g, scales + slot * C::SF_SLOT_BYTES + u * C::SF_BYTES + g * kSfGroup);
+            commit_if(elected, sempty + 8 * slot);
+        };
         // the next wait's outcome is asked for before the current stage is issued: a round to a barrier takes 100-150 cycles
-        bool ok = true, ready = false, sready = false;
+        bool ok = true, ready = false, copied = false;
         for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++tcount) {
             const uint32_t as = tcount & 1, ause = tcount >> 1;
             if (ause >= 1 && !(ok = mbar_wait_warp(tempty + 8 * as, (ause - 1) & 1, abort_flag))) break;
             const uint32_t acc = tmem + as * BN;
             for (int kb0 = 0; kb0 < nkb && ok; kb0 += ST) {
-                if (!__all_sync(0xffffffffu, sready) && !(ok = mbar_wait_warp(sfull + 8 * ss, sph, abort_flag))) break;
-                tc_fence_after();
+                if (!copied) {
+                    if (!(ok = mbar_wait_warp(sfull + 8 * ss, sph, abort_flag))) break;
+                    tc_fence_after();
+                    copy_group(ss);
+                }
                 const uint32_t sf = tmem + C::ACC_COLS + ss * (kSfAhead * C::SF_COLS);
-                const uint32_t src = scales + ss * C::SF_SLOT_BYTES;
+                ss ^= 1; sph ^= ss ^ 1;
+                copied = (kb0 + ST < nkb || tile + (int)gridDim.x < num_tiles) && __all_sync(0xffffffffu, mbar_test_wait(sfull + 8 * ss, sph)) != 0;
+                if (copied) {
+                    tc_fence_after();
+                    copy_group(ss);
+                }
 #pragma unroll
                 for (int u = 0; u < ST; ++u) {
                     if (kb0 + u < nkb && ok) {
@@ -211,20 +231,14 @@ gemm_mx_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
                         ready = mbar_test_wait(full + 8 * nu, ph >> nu & 1);
                         if (!ok) break;
 #pragma unroll
-                        for (int g = 0; g <= C::W_GROUPS; ++g)
-                            copy_scales(elected, sf + u * C::SF_COLS + 4 * g, src + u * C::SF_BYTES + g * kSfGroup);
-#pragma unroll
                         for (int k = 0; k < kBlockK / 32; ++k)   // 32 bytes of k per instruction: descriptor start + 2
                             umma_mx(elected, acc, adesc0 + (u * (C::STAGE_BYTES >> 4) + 2 * k), bdesc0 + (u * (C::STAGE_BYTES >> 4) + 2 * k),
                                     idesc0 + ((uint32_t)k << 4 | (uint32_t)k << 29), sf + u * C::SF_COLS, sf + u * C::SF_COLS + 4,
                                     (u | k) != 0 ? 1u : (kb0 != 0 ? 1u : 0u));
                         commit_if(elected, empty + 8 * u);
-                        if (u == ST - 1 || last) commit_if(elected, sempty + 8 * ss);
                         if (last) commit_if(elected, tfull + 8 * as);
                     }
                 }
-                ss ^= 1; sph ^= ss ^ 1;
-                sready = mbar_test_wait(sfull + 8 * ss, sph);
             }
         }
     } else if (warp < 6) {
