@@ -48,6 +48,7 @@ __global__ void __launch_bounds__(kDequantThreads)
 dequant_block_scaled_kernel(const uint8_t* __restrict__ codes, const uint8_t* __restrict__ scales,
                             __nv_bfloat16* __restrict__ out, int N, int K, MiniFloatFormat fmt) {
     __shared__ float lut[256];
+    pdl_launch_dependents();   // rlx_scaled_matmul_bf16's product sets itself up meanwhile
     const int ncodes = 1 << (1 + fmt.ebits + fmt.mbits);
     if ((int)threadIdx.x < ncodes) lut[threadIdx.x] = minifloat_value(threadIdx.x, fmt);
     __syncthreads();

@@ -158,6 +158,7 @@ gemm_mx_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = warp_uniform(*tmem_slot);
+    pdl_wait();   // codes and scales come from the kernel in front
 
     // Stage u of the ring holds the k-blocks u, u + 4, ... of every tile (a tile of fewer leaves some out), so that stage
     // addresses are constants of the unrolled loops.  With the addresses formed per stage, under a branch for the elected
@@ -349,6 +350,7 @@ __global__ void __launch_bounds__(kQuantThreads)
 quantise_mx_kernel(const __nv_bfloat16* __restrict__ x, uint8_t* __restrict__ codes, uint8_t* __restrict__ scales,
                    long long blocks) {
     constexpr int kEmax = E5M2 ? 15 : 8;
+    pdl_launch_dependents();   // a product behind it sets itself up meanwhile
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long b0 = (long long)blockIdx.x * kQuantCtaBlocks + warp * kQuantWarpBlocks;
     uint4 in[kQuantIters];

@@ -388,6 +388,7 @@ struct Params {
     const int32_t* m_ptr;            // optional device row count: rows >= *m_ptr are not computed
     int kblock_maps;                 // the operand tensor maps are 3-D views [K/64][rows][64]: one TMA load brings a
                                      // whole stage's k-blocks of an operand (needs K % 64 == 0); else 2-D, one per k-block
+    int w_fresh;                     // W comes from the kernel in front: nothing of it is requested ahead of the wait for that
     int split_tiles4, split_tiles2;  // split-K form: up to so many existing tiles get four / two CTAs each
 #ifdef RLX_EXPERIMENTS
     int debug;                       // ablation switches of the experiments build (kDbg* bits)
@@ -826,7 +827,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
             // tile delays the first product (18432 x 768 x 768: 29.6 -> 33.5 us).
             int early = 0;
             if constexpr (C::SMALL) {
-                if (tile0 < num_tiles)
+                if (tile0 < num_tiles && !p.w_fresh)
                     for (; early < C::STAGES && early * C::KPS < num_kb; ++early) {
                         if (elect_one()) load(std::integral_constant<int, kPartW>(), 0, tile0 % n_tiles, early * C::KPS, early);
                         __syncwarp();

@@ -242,6 +242,23 @@ def test_mx_matmul_at_the_edges_of_its_tiles_and_rings(rlx, M, N, K):
     assert np.array_equal(got, round_to_bf16(want.astype(np.float32)).astype(np.float64))
 
 
+@pytest.mark.parametrize("M", [1, 40, 200, 5000])
+@pytest.mark.parametrize("N,K", [(192, 384), (384, 1536)])
+def test_scaled_product_behind_its_decoding_reads_the_decoded_weights(rlx, M, N, K):
+    """The product is launched while the decoding runs: call after call with other codes into the same scratch and output."""
+    rng = np.random.default_rng(M + N + K)
+    x = bf16_dev(rand_bf16(rng, (M, K)))
+    bias = torch.zeros(N, device="cuda")
+    scratch, out = (torch.empty(s, dtype=torch.bfloat16, device="cuda") for s in ((N, K), (M, N)))
+    sets = [(_u8_dev(rng.integers(0, 0x7F, size=(N, K))), _u8_dev(rng.integers(112, 120, size=(N, K // 32)))) for _ in range(3)]
+    want = [rlx.gemm_bf16(x, rlx.dequant_block_scaled_bf16(c, sc, N, K, rlx.binding.FMT_FP8_E4M3), bias) for c, sc in sets]
+    got = []
+    for i in range(12):
+        rlx.scaled_matmul_bf16(x, *sets[i % 3], rlx.binding.FMT_FP8_E4M3, bias, w_scratch=scratch, out=out)
+        got.append(out.clone())
+    assert all(torch.equal(g, want[i % 3]) for i, g in enumerate(got))
+
+
 @pytest.mark.parametrize("a_name,w_name", [("fp8_e4m3", "fp8_e4m3"), ("fp8_e4m3", "fp8_e5m2"), ("fp8_e5m2", "fp8_e4m3")])
 @pytest.mark.parametrize("M,N,K", [(128, 128, 128), (517, 384, 384), (2000, 1536, 384), (1000, 384, 1536)])
 def test_quantise_then_mx_matmul_matches_oracle(rlx, a_name, w_name, M, N, K):
