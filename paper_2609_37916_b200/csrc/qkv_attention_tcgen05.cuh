@@ -21,12 +21,13 @@ namespace tcqa {
 using namespace rlx::tc;
 
 constexpr int kRows = kBinRows;
-constexpr int kWarps = 12;                    // epilogue: a 32-row quadrant of q, of k or of v; then attention
-constexpr int kThreads = 64 + 32 * kWarps;
+constexpr int kEpiWarps = 12;                 // a 32-row quadrant of q, of k or of v each; then they attend
 constexpr int kMaxTasks = kRows / 16 + kBinSeqs;   // 16-row groups of a bin's sequences
 
 template <int D, int HPC>
 struct Cfg {
+    static constexpr int WARPS = HPC == 2 ? 16 : kEpiWarps;   // that attend: two heads of a full bin are sixteen groups of 16 rows
+    static constexpr int THREADS = 64 + 32 * WARPS;
     static constexpr int N = 3 * D * HPC;                     // columns: q of the heads, then k, then v
     static constexpr int NC = N / 96;                         // 32-column chunks of a warp
     static constexpr int KPS = N == 96 ? 2 : 1;               // k-blocks per stage
@@ -36,10 +37,11 @@ struct Cfg {
     static constexpr int TMEM_COLS = N <= 128 ? 128 : 256;
     static constexpr int STR = D + 8;                         // elements per q / k / v row: conflict-free ldmatrix
     static constexpr int VEC_OFF = STAGES * STAGE_BYTES;
-    static constexpr int ZERO_OFF = VEC_OFF + kWarps * 384;   // a row of zeros, read in place of v past a sequence's end
+    static constexpr int ZERO_OFF = VEC_OFF + kEpiWarps * 384;   // a row of zeros, read in place of v past a sequence's end
     static constexpr int TASK_OFF = ZERO_OFF + (STR * 2 + 15) / 16 * 16;
     static constexpr int BAR_OFF = TASK_OFF + kMaxTasks * 16;
-    static constexpr int SMEM_BYTES = BAR_OFF + 8 * (2 * STAGES + 1) + 16 + 1024;
+    static constexpr int NBAR = 2 * STAGES + 1;
+    static constexpr int SMEM_BYTES = BAR_OFF + 8 * NBAR + 16 + 1024;
     static_assert(N == 96 || N == 192, "tile");
     static_assert(3 * HPC * kRows * STR * 2 <= STAGES * STAGE_BYTES, "q, k and v over the ring");
     static_assert(SMEM_BYTES <= 227 * 1024, "shared memory");
@@ -47,10 +49,10 @@ struct Cfg {
 
 // Attention of 16 query rows of one sequence, as attention_bf16_kernel computes it: online softmax in steps of 32 (heads of 32) or
 // 64 keys.  q: the first query row, k / v: the sequence's first key, all with STR elements per row; keys: length of the
-// sequence, rows: query rows that exist.  The result replaces the q rows and goes to ctx from there.
+// sequence, rows: query rows that exist.  The result replaces the q rows.
 template <int D, int STR>
 __device__ __forceinline__ void attend16(__nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v, uint32_t zero_row, int keys,
-                                         int rows, float scale_log2e, __nv_bfloat16* ctx, size_t ldc) {
+                                         int rows, float scale_log2e) {
     constexpr int KT = D / 16, ND = D / 8, KS = D == 32 ? 32 : 64, NT = KS / 8;
     const int lane = threadIdx.x & 31, g = lane >> 2, t4 = lane & 3, mi = lane >> 3;
     uint32_t qf[KT][4];
@@ -146,24 +148,21 @@ __device__ __forceinline__ void attend16(__nv_bfloat16* q, const __nv_bfloat16* 
             *reinterpret_cast<uint32_t*>(q + (g + 8) * STR + nd * 8 + 2 * t4) = pack_bf16(o[nd][2] * l_run[1], o[nd][3] * l_run[1]);
     }
     __syncwarp();
-    constexpr int CH = D / 8;
-    for (int i = lane; i < 16 * CH; i += 32) {
-        const int r = i / CH, c = i % CH;
-        if (r < rows) *reinterpret_cast<uint4*>(ctx + r * ldc + c * 8) = *reinterpret_cast<const uint4*>(q + r * STR + c * 8);
-    }
 }
 
+struct RowMaps {
+    CUtensorMap m[4];                  // x as k-blocks, boxes of 32, 64, 96 and 128 rows: only the 32-row groups that a bin has are loaded
+};
 struct AttParams {
     const int32_t *bins, *seq_start;   // pack_sequences_kernel's
     __nv_bfloat16* ctx;                // [rows, H]
     float scale_log2e;
 };
 
-// grid (heads / HPC, bins that there can be); tmap_a: x as k-blocks of 128 rows, tmap_w: Wqkv as [q | k | v][row][column], boxes of
-// 3 x D HPC x 64.  p: bias / folding vectors and row statistics of the product, K = H.
+// grid (heads / HPC, bins that there can be); tmap_w: Wqkv as [q | k | v][row][column], boxes of 3 x D HPC x 64.  p: bias / folding vectors and row statistics of the product, K = H.
 template <int D, int HPC, int EPI>
-__global__ void __launch_bounds__(kThreads, 1)
-qkv_attention_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_w, const Params p,
+__global__ void __launch_bounds__((Cfg<D, HPC>::THREADS), 1)
+qkv_attention_kernel(const __grid_constant__ RowMaps tmap_a, const __grid_constant__ CUtensorMap tmap_w, const Params p,
                      const AttParams ap) {
     using C = Cfg<D, HPC>;
     extern __shared__ unsigned char smem_raw[];
@@ -171,42 +170,42 @@ qkv_attention_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
     const uint32_t base = (raw + 1023u) & ~1023u;
     unsigned char* gbase = smem_raw + (base - raw);
     const uint32_t full_bar = base + C::BAR_OFF, empty_bar = full_bar + 8 * C::STAGES, acc_bar = empty_bar + 8 * C::STAGES;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + C::BAR_OFF + 8 * (2 * C::STAGES + 1));
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + C::BAR_OFF + 8 * C::NBAR);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     int4* tasks = reinterpret_cast<int4*>(gbase + C::TASK_OFF);   // first row in the bin, query row offset, length
     const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     const int bin = blockIdx.y, head0 = blockIdx.x * HPC, H = p.K, num_kb = H / BLOCK_K;
     pdl_launch_dependents();
 
-    const bool exists = bin < ld_early(ap.bins);
-    const int b0 = exists ? ld_early(ap.bins + 1 + bin) : 0, b1 = exists ? ld_early(ap.bins + 2 + bin) : 0;
     if (threadIdx.x == 0) {
         for (int i = 0; i < C::STAGES; ++i) { mbar_init(full_bar + 8 * i, 1); mbar_init(empty_bar + 8 * i, 1); }
         mbar_init(acc_bar, 1);
         *abort_flag = 0;
         fence_barrier_init();
-        prefetch_tmap(&tmap_a);
         prefetch_tmap(&tmap_w);
     }
     if (warp == 1) {
         tmem_alloc<1>(smem_u32(tmem_slot), C::TMEM_COLS);
         tmem_relinquish<1>();
     }
+    const bool exists = bin < ld_early(ap.bins);
+    const int b0 = exists ? ld_early(ap.bins + 1 + bin) : 0, b1 = exists ? ld_early(ap.bins + 2 + bin) : 0;
     const int row0 = exists ? ld_early(ap.seq_start + b0) : 0, rows = exists ? ld_early(ap.seq_start + b1) - row0 : 0;
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = warp_uniform(*tmem_slot);
+    const int groups = (rows + 31) / 32, a_kb = groups * (C::A_BYTES / 4);   // 32-row groups; bytes of a k-block of them
 
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer (whole warp, one lane issues)
         auto load_w = [&](int kb, int stage) {
-            mbar_expect_tx(full_bar + 8 * stage, C::STAGE_BYTES);
+            mbar_expect_tx(full_bar + 8 * stage, (uint32_t)(C::KPS * (a_kb + C::B_BYTES)));
             for (int i = 0; i < C::KPS; ++i)
                 tma_load_3d(base + stage * C::STAGE_BYTES + C::KPS * C::A_BYTES + i * C::B_BYTES, &tmap_w, (kb + i) * BLOCK_K, head0 * D, 0,
                             full_bar + 8 * stage);
         };
-        auto load_a = [&](int kb, int stage) { tma_load_3d(base + stage * C::STAGE_BYTES, &tmap_a, 0, row0, kb, full_bar + 8 * stage); };
+        auto load_a = [&](int kb, int stage) { tma_load_3d(base + stage * C::STAGE_BYTES, tmap_a.m + groups - 1, 0, row0, kb, full_bar + 8 * stage); };
         int early = 0;   // weights do not come from the previous kernel
         if (rows > 0)
             for (; early < C::STAGES && early * C::KPS < num_kb; ++early) {
@@ -248,7 +247,7 @@ qkv_attention_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
                     for (int i = 0; i < C::KPS; ++i)
 #pragma unroll
                         for (int k = 0; k < BLOCK_K / UMMA_K; ++k)
-                            umma_bf16<1>(tmem, ad0 + (i * (C::A_BYTES >> 4) + 2 * k), bd0 + (i * (C::B_BYTES >> 4) + 2 * k), idesc,
+                            umma_bf16<1>(tmem, ad0 + (i * (uint32_t)(a_kb >> 4) + 2 * k), bd0 + (i * (C::B_BYTES >> 4) + 2 * k), idesc,
                                          (kb | i | k) != 0 ? 1u : 0u);
                     umma_commit<1>(empty_bar + 8 * cur);
                 }
@@ -260,10 +259,10 @@ qkv_attention_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
     } else {
         // ------------------------------------------------------------ q, k, v, then attention
         const int e = warp - 2, quad = warp & 3, part = e >> 2;
-        const int n0 = part * H + head0 * D;
+        const int n0 = part * H + head0 * D;      // part 3: warps that only attend
         using ET = EpilogueTile<EPI, C::NC, true>;
         ET et;
-        et.load_vectors(p, n0, base + C::VEC_OFF + e * 384);
+        if (part < 3) et.load_vectors(p, n0, base + C::VEC_OFF + e * 384);
         // the bin's row groups and the row of zeros
         int ntasks = 0;
         {
@@ -284,20 +283,19 @@ qkv_attention_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
         }
         pdl_wait();
         const int row = quad * 32 + lane;
-        const bool live = quad * 32 < rows;
+        const bool live = quad * 32 < rows && part < 3;
         bool ok = true;
         if (live) {
             et.prefetch(p, row0 + rows, row0 + row, n0);
             ok = mbar_wait_warp(acc_bar, 0, abort_flag);
             tc_fence_after();
-            uint32_t r[C::NC][32];
-#pragma unroll
-            for (int c = 0; c < C::NC; ++c) tmem_ld_32x32(tmem + ((uint32_t)(quad * 32) << 16) + part * (D * HPC) + c * 32, r[c]);
-            tmem_ld_wait();
 #pragma unroll
             for (int c = 0; c < C::NC; ++c) {
+                uint32_t r[32];
+                tmem_ld_32x32(tmem + ((uint32_t)(quad * 32) << 16) + part * (D * HPC) + c * 32, r);
+                tmem_ld_wait();
                 uint4 v[4];
-                et.compute_chunk(p, r[c], n0 + c * 32, c, row0 + row, row < rows, p.bias + n0 + c * 32, v);
+                et.compute_chunk(p, r, n0 + c * 32, c, row0 + row, row < rows, p.bias + n0 + c * 32, v);
                 // column c * 32 of the part: head c (heads of 32), or column 32 c of the one head
                 const int hh = D == 32 ? c : 0, col = D == 32 ? 0 : c * 32;
                 const uint32_t dst = base + (uint32_t)(((part * HPC + hh) * kRows + row) * C::STR + col) * 2;
@@ -308,16 +306,23 @@ qkv_attention_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
         } else if (rows > 0) {
             ok = mbar_wait_warp(acc_bar, 0, abort_flag);   // the ring is free
         }
-        asm volatile("bar.sync 1, %0;" ::"n"(32 * kWarps) : "memory");
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * C::WARPS) : "memory");
         if (ok) {
             __nv_bfloat16* qkv = reinterpret_cast<__nv_bfloat16*>(gbase);
-            for (int t = e; t < ntasks * HPC; t += kWarps) {
+            for (int t = e; t < ntasks * HPC; t += C::WARPS) {
                 const int hh = t / ntasks;
                 const int4 task = tasks[t - hh * ntasks];
                 __nv_bfloat16* qh = qkv + hh * kRows * C::STR;
-                attend16<D, C::STR>(qh + (task.x + task.y) * C::STR, qh + (HPC * kRows + task.x) * C::STR,
-                                    qh + (2 * HPC * kRows + task.x) * C::STR, base + C::ZERO_OFF, task.z, min(16, task.z - task.y),
-                                    ap.scale_log2e, ap.ctx + (size_t)(row0 + task.x + task.y) * H + (head0 + hh) * D, (size_t)H);
+                const int first = task.x + task.y, n = min(16, task.z - task.y);   // query rows, in the bin
+                attend16<D, C::STR>(qh + first * C::STR, qh + (HPC * kRows + task.x) * C::STR, qh + (2 * HPC * kRows + task.x) * C::STR,
+                                    base + C::ZERO_OFF, task.z, n, ap.scale_log2e);
+                constexpr int CH = D / 8;
+                __nv_bfloat16* out = ap.ctx + (size_t)(row0 + first) * H + (head0 + hh) * D;
+                for (int i = lane; i < 16 * CH; i += 32) {
+                    const int r = i / CH, c = i % CH;
+                    if (r < n)
+                        *reinterpret_cast<uint4*>(out + (size_t)r * H + c * 8) = *reinterpret_cast<const uint4*>(qh + (first + r) * C::STR + c * 8);
+                }
             }
         }
     }

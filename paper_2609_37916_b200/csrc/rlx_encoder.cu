@@ -624,8 +624,14 @@ TileChoice pick_tile(int M, int N, int K, int want_cg = 0) {
 }
 
 template <int BN, int CG>
-rlx_status_t launch_gemm_tc_bn(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& to,
+rlx_status_t launch_gemm_tc_bn(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& to, const bf16* A,
                                const rlx::tc::Params& p, int epi, cudaStream_t st) {
+    rlx::tc::RowMaps<rlx::tc::Cfg<BN, CG>::SMALL> rm;
+    if constexpr (rlx::tc::Cfg<BN, CG>::SMALL)
+        for (int i = 0; i < 3; ++i)
+            if (!(p.kblock_maps ? make_tmap_kblocks(rm.m + i, A, p.M, p.K, 32 * (i + 1), rlx::tc::Cfg<BN, CG>::KPS)
+                                : make_tmap(rm.m + i, A, p.M, p.K, 32 * (i + 1))))
+                return RLX_ERR_CUDA;
     const int tile_m = rlx::tc::BLOCK_M * CG;
     const int tiles = ((p.M + tile_m - 1) / tile_m) * (p.N / BN);
     int dev = 0;
@@ -639,13 +645,13 @@ rlx_status_t launch_gemm_tc_bn(const CUtensorMap& ta, const CUtensorMap& tb, con
         ~ClusterScope() { g_cluster_x = 1; }
     } scope(CG);
     switch (epi) {
-        case 0: RLX_CUDA_TRY(launch_ex(rlx::tc::gemm_tcgen05_kernel<BN, 0, CG>, grid, rlx::tc::Cfg<BN, CG>::THREADS, smem, st, ta, tb, to, p)); break;
-        case 1: RLX_CUDA_TRY(launch_ex(rlx::tc::gemm_tcgen05_kernel<BN, 1, CG>, grid, rlx::tc::Cfg<BN, CG>::THREADS, smem, st, ta, tb, to, p)); break;
-        case 2: RLX_CUDA_TRY(launch_ex(rlx::tc::gemm_tcgen05_kernel<BN, 2, CG>, grid, rlx::tc::Cfg<BN, CG>::THREADS, smem, st, ta, tb, to, p)); break;
-        case 3: RLX_CUDA_TRY(launch_ex(rlx::tc::gemm_tcgen05_kernel<BN, 3, CG>, grid, rlx::tc::Cfg<BN, CG>::THREADS, smem, st, ta, tb, to, p)); break;
-        case 4: RLX_CUDA_TRY(launch_ex(rlx::tc::gemm_tcgen05_kernel<BN, 4, CG>, grid, rlx::tc::Cfg<BN, CG>::THREADS, smem, st, ta, tb, to, p)); break;
-        case 5: RLX_CUDA_TRY(launch_ex(rlx::tc::gemm_tcgen05_kernel<BN, 5, CG>, grid, rlx::tc::Cfg<BN, CG>::THREADS, smem, st, ta, tb, to, p)); break;
-        case 6: RLX_CUDA_TRY(launch_ex(rlx::tc::gemm_tcgen05_kernel<BN, 6, CG>, grid, rlx::tc::Cfg<BN, CG>::THREADS, smem, st, ta, tb, to, p)); break;
+        case 0: RLX_CUDA_TRY(launch_ex(rlx::tc::gemm_tcgen05_kernel<BN, 0, CG>, grid, rlx::tc::Cfg<BN, CG>::THREADS, smem, st, ta, tb, to, rm, p)); break;
+        case 1: RLX_CUDA_TRY(launch_ex(rlx::tc::gemm_tcgen05_kernel<BN, 1, CG>, grid, rlx::tc::Cfg<BN, CG>::THREADS, smem, st, ta, tb, to, rm, p)); break;
+        case 2: RLX_CUDA_TRY(launch_ex(rlx::tc::gemm_tcgen05_kernel<BN, 2, CG>, grid, rlx::tc::Cfg<BN, CG>::THREADS, smem, st, ta, tb, to, rm, p)); break;
+        case 3: RLX_CUDA_TRY(launch_ex(rlx::tc::gemm_tcgen05_kernel<BN, 3, CG>, grid, rlx::tc::Cfg<BN, CG>::THREADS, smem, st, ta, tb, to, rm, p)); break;
+        case 4: RLX_CUDA_TRY(launch_ex(rlx::tc::gemm_tcgen05_kernel<BN, 4, CG>, grid, rlx::tc::Cfg<BN, CG>::THREADS, smem, st, ta, tb, to, rm, p)); break;
+        case 5: RLX_CUDA_TRY(launch_ex(rlx::tc::gemm_tcgen05_kernel<BN, 5, CG>, grid, rlx::tc::Cfg<BN, CG>::THREADS, smem, st, ta, tb, to, rm, p)); break;
+        case 6: RLX_CUDA_TRY(launch_ex(rlx::tc::gemm_tcgen05_kernel<BN, 6, CG>, grid, rlx::tc::Cfg<BN, CG>::THREADS, smem, st, ta, tb, to, rm, p)); break;
         default: return RLX_ERR_INVALID_ARG;
     }
     RLX_CUDA_TRY(cudaGetLastError());
@@ -828,17 +834,17 @@ rlx_status_t launch_gemm(const bf16* A, const bf16* W, const float* bias, const 
     if (p.kblock_maps < 0) return RLX_ERR_CUDA;
     if (tc.cg == 2) {
         switch (bn) {
-            case 128: return launch_gemm_tc_bn<128, 2>(ta, tb, to, p, epi, st);
-            case 192: return launch_gemm_tc_bn<192, 2>(ta, tb, to, p, epi, st);
-            case 256: return launch_gemm_tc_bn<256, 2>(ta, tb, to, p, epi, st);
+            case 128: return launch_gemm_tc_bn<128, 2>(ta, tb, to, A, p, epi, st);
+            case 192: return launch_gemm_tc_bn<192, 2>(ta, tb, to, A, p, epi, st);
+            case 256: return launch_gemm_tc_bn<256, 2>(ta, tb, to, A, p, epi, st);
         }
         return RLX_ERR_UNSUPPORTED;
     }
     switch (bn) {
-        case 64: return launch_gemm_tc_bn<64, 1>(ta, tb, to, p, epi, st);
-        case 128: return launch_gemm_tc_bn<128, 1>(ta, tb, to, p, epi, st);
-        case 192: return launch_gemm_tc_bn<192, 1>(ta, tb, to, p, epi, st);
-        case 256: return launch_gemm_tc_bn<256, 1>(ta, tb, to, p, epi, st);
+        case 64: return launch_gemm_tc_bn<64, 1>(ta, tb, to, A, p, epi, st);
+        case 128: return launch_gemm_tc_bn<128, 1>(ta, tb, to, A, p, epi, st);
+        case 192: return launch_gemm_tc_bn<192, 1>(ta, tb, to, A, p, epi, st);
+        case 256: return launch_gemm_tc_bn<256, 1>(ta, tb, to, A, p, epi, st);
     }
     return RLX_ERR_UNSUPPORTED;
 }
@@ -866,12 +872,14 @@ template <int D, int HPC>
 rlx_status_t launch_qkv_attention_d(const bf16* x, const bf16* w, const rlx::tc::Params& p, const rlx::tcqa::AttParams& ap, int epi,
                                     int heads, int bins, cudaStream_t st) {
     using C = rlx::tcqa::Cfg<D, HPC>;
-    CUtensorMap ta, tw;
-    if (!make_tmap_kblocks(&ta, x, (uint64_t)p.M, (uint64_t)p.K, rlx::tcqa::kRows, C::KPS) || !make_tmap_qkv(&tw, w, (uint64_t)p.K, D * HPC))
-        return RLX_ERR_CUDA;
+    rlx::tcqa::RowMaps ta;
+    CUtensorMap tw;
+    for (int i = 0; i < 4; ++i)
+        if (!make_tmap_kblocks(ta.m + i, x, (uint64_t)p.M, (uint64_t)p.K, 32 * (i + 1), C::KPS)) return RLX_ERR_CUDA;
+    if (!make_tmap_qkv(&tw, w, (uint64_t)p.K, D * HPC)) return RLX_ERR_CUDA;
     const dim3 grid(heads / HPC, bins);
-    if (epi == 0) RLX_CUDA_TRY(launch_ex(rlx::tcqa::qkv_attention_kernel<D, HPC, 0>, grid, rlx::tcqa::kThreads, C::SMEM_BYTES, st, ta, tw, p, ap));
-    else RLX_CUDA_TRY(launch_ex(rlx::tcqa::qkv_attention_kernel<D, HPC, 3>, grid, rlx::tcqa::kThreads, C::SMEM_BYTES, st, ta, tw, p, ap));
+    if (epi == 0) RLX_CUDA_TRY(launch_ex(rlx::tcqa::qkv_attention_kernel<D, HPC, 0>, grid, C::THREADS, C::SMEM_BYTES, st, ta, tw, p, ap));
+    else RLX_CUDA_TRY(launch_ex(rlx::tcqa::qkv_attention_kernel<D, HPC, 3>, grid, C::THREADS, C::SMEM_BYTES, st, ta, tw, p, ap));
     RLX_CUDA_TRY(cudaGetLastError());
     return RLX_OK;
 }

@@ -183,6 +183,20 @@ def test_gemm_matches_oracle_linear(rlx, shape, epi, impl):
     assert_close_bf16_out(got, ref, extra_abs=K * 2.0 ** -24 * 0.2)
 
 
+@pytest.mark.parametrize("M", [1, 31, 32, 33, 64, 65, 96, 97, 129, 160, 225])
+@pytest.mark.parametrize("N,K", [(64, 64), (192, 384), (128, 200), (64, 1600)])   # k-blocks in pairs, an odd number of them, part of one
+def test_narrow_tiles_load_the_row_groups_that_exist(rlx, M, N, K):
+    """One to four 32-row groups in the last row block; small integers, so that a row or a k-block out of place is a wrong integer."""
+    rng = np.random.default_rng(M + N + K)
+    a, w = rng.integers(-1, 2, size=(M, K)).astype(np.float32), rng.integers(-1, 2, size=(N, K)).astype(np.float32)
+    bias = rng.integers(-8, 9, size=N).astype(np.float32)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    got = to_np64(rlx.gemm_bf16(bf16_dev(a), bf16_dev(w), f32_dev(bias), status=status))
+    ref = a.astype(np.float64) @ w.astype(np.float64).T + bias
+    assert int(status.item()) == 0 and np.abs(ref).max() < 256
+    assert np.array_equal(got, ref)
+
+
 @pytest.mark.parametrize("M,H,F", [(256, 384, 256), (300, 384, 1536), (5000, 384, 1536), (40000, 384, 1536), (1000, 256, 512),
                                    (37, 384, 128)])
 def test_ffn_fused_matches_oracle(rlx, M, H, F):
