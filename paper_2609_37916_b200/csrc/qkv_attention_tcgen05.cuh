@@ -157,6 +157,7 @@ struct AttParams {
     const int32_t *bins, *seq_start;   // pack_sequences_kernel's
     __nv_bfloat16* ctx;                // [rows, H]
     float scale_log2e;
+    int first;                         // the kernel in front wrote the tables: nothing may be read ahead of it, not by the next kernel either
 };
 
 // grid (heads / HPC, bins that there can be); tmap_w: Wqkv as [q | k | v][row][column], boxes of 3 x D HPC x 64.  p: bias / folding vectors and row statistics of the product, K = H.
@@ -175,7 +176,7 @@ qkv_attention_kernel(const __grid_constant__ RowMaps tmap_a, const __grid_consta
     int4* tasks = reinterpret_cast<int4*>(gbase + C::TASK_OFF);   // first row in the bin, query row offset, length
     const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     const int bin = blockIdx.y, head0 = blockIdx.x * HPC, H = p.K, num_kb = H / BLOCK_K;
-    pdl_launch_dependents();
+    if (!ap.first) pdl_launch_dependents();
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < C::STAGES; ++i) { mbar_init(full_bar + 8 * i, 1); mbar_init(empty_bar + 8 * i, 1); }
@@ -187,6 +188,10 @@ qkv_attention_kernel(const __grid_constant__ RowMaps tmap_a, const __grid_consta
     if (warp == 1) {
         tmem_alloc<1>(smem_u32(tmem_slot), C::TMEM_COLS);
         tmem_relinquish<1>();
+    }
+    if (ap.first) {
+        pdl_wait();
+        pdl_launch_dependents();
     }
     const bool exists = bin < ld_early(ap.bins);
     const int b0 = exists ? ld_early(ap.bins + 1 + bin) : 0, b1 = exists ? ld_early(ap.bins + 2 + bin) : 0;

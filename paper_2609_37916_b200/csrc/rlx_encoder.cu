@@ -373,6 +373,20 @@ rlx_status_t launch_embed_ln(const int32_t* ids, const bf16* word, const bf16* p
     return RLX_OK;
 }
 
+rlx_status_t launch_pack_embed_ln(const int32_t* ids, const int32_t* mask, const bf16* word, const bf16* pos, const bf16* type,
+                                  const float* g, const float* b, int B, int S, int H, int V, float eps, bf16* out, int32_t* status,
+                                  int32_t* seq_len, int32_t* seq_start, int32_t* bins, cudaStream_t st) {
+    const int grid = (B * S + rlx::kRowWarps - 1) / rlx::kRowWarps + 1, thr = rlx::kRowWarps * 32;
+    switch (H / 128) {
+#define RLX_CASE(NV) case NV: rlx::pack_embed_ln_kernel<NV><<<grid, thr, 0, st>>>(ids, mask, word, pos, type, g, b, out, B, S, V, eps, status, seq_len, seq_start, bins); break;
+        RLX_CASE(1) RLX_CASE(2) RLX_CASE(3) RLX_CASE(4) RLX_CASE(5) RLX_CASE(6) RLX_CASE(7) RLX_CASE(8)
+#undef RLX_CASE
+        default: return RLX_ERR_UNSUPPORTED;
+    }
+    RLX_CUDA_TRY(cudaGetLastError());
+    return RLX_OK;
+}
+
 rlx_status_t launch_layernorm(const bf16* x, const float* g, const float* b, int T, int H, float eps, bf16* out,
                               cudaStream_t st, const int32_t* rows_ptr = nullptr) {
     // rows per warp: as many as still leave ~4 CTAs for every SM (static row bound T), so that large
@@ -884,12 +898,12 @@ rlx_status_t launch_qkv_attention_d(const bf16* x, const bf16* w, const rlx::tc:
     return RLX_OK;
 }
 rlx_status_t launch_qkv_attention(const bf16* x, const bf16* w, const float* bias, int epi, int B, int S, int H, int heads, bf16* ctx,
-                                  int32_t* status, cudaStream_t st, const Packing& pk, const LnFold* lf = nullptr) {
+                                  int32_t* status, cudaStream_t st, const Packing& pk, bool first, const LnFold* lf = nullptr) {
     rlx::tc::Params p{};
     p.bias = bias; p.M = B * S; p.N = 3 * H; p.K = H; p.status = status;
     if (lf) { p.cvec = lf->cvec; p.dvec = lf->dvec; p.stats_in = lf->stats_in; p.stats_in_p = lf->stats_in_p; p.ln_eps = lf->eps; }
     const int d = H / heads, bins = max_bins(B, S);
-    const rlx::tcqa::AttParams ap{pk.bins, pk.seq_start, ctx, 1.4426950408889634f / sqrtf((float)d)};
+    const rlx::tcqa::AttParams ap{pk.bins, pk.seq_start, ctx, 1.4426950408889634f / sqrtf((float)d), first};
     if (d == 64) return launch_qkv_attention_d<64, 1>(x, w, p, ap, epi, heads, bins, st);
     // one head per CTA while every bin there can be finds its SMs, else two: a row's x is then loaded half as often
     if (heads * bins <= sm_count()) return launch_qkv_attention_d<32, 1>(x, w, p, ap, epi, heads, bins, st);
@@ -1144,7 +1158,16 @@ bool uses_attention_fwd(const rlx_encoder_config_t& c, int B, int S) {
 constexpr long long kQkvAttentionMaxTokens = 4096;
 bool uses_qkv_attention(const rlx_encoder_config_t& c, int B, int S) {
     if (c.flags & (RLX_FLAG_GEMM_SIMT | RLX_FLAG_KERNEL_EVENTS | RLX_FLAG_NO_PACK | RLX_FLAG_ATTN_TCGEN05)) return false;
-    return S <= rlx::kBinRows && call_tokens(B, S) <= kQkvAttentionMaxTokens && !uses_fused_ffn(c, B, S) && !uses_attention_fwd(c, B, S);
+    return S <= rlx::kBinRows && B <= rlx::kPackEmbedMaxSeqs && call_tokens(B, S) <= kQkvAttentionMaxTokens && !uses_fused_ffn(c, B, S) && !uses_attention_fwd(c, B, S);
+}
+
+// Packing and embedding in one kernel, in front of the above (us apart / in one: 6 x 384 1 x 32 106.5 / 102.6, 1 x 128 118.6 / 113.9,
+// 7 x 128 133 / 129.5, 32 x 128 186.8 / 184.1, 256 x 16 233.2 / 232.3; 12 x 768 1 x 128 346.8 / 337.3, 7 x 120 408 / 405).  Every CTA reads
+// the whole mask, so a mask in host memory is read in place only where few CTAs do (g_host_io: the call's buffers are host memory).
+thread_local bool g_host_io = false;
+constexpr int kPackEmbedMaxHostTokens = 256;
+bool uses_pack_embed(const rlx_encoder_config_t& c, int B, int S) {
+    return uses_qkv_attention(c, B, S) && (long long)B * S <= (g_host_io ? kPackEmbedMaxHostTokens : rlx::kPackEmbedMaxTokens);
 }
 
 struct GraphEntry {
@@ -1250,6 +1273,7 @@ rlx_status_t enqueue_forward(const rlx_encoder* e, const int32_t* ids, const int
     }
     Packing pk;
     const bool fuse_qa = pack && uses_qkv_attention(c, B, S);
+    const bool fuse_pe = fuse_qa && uses_pack_embed(c, B, S);
     if (pack) {
         int32_t* seq_len = reinterpret_cast<int32_t*>(ws + a.seq_len);
         int32_t* seq_start = reinterpret_cast<int32_t*>(ws + a.seq_start);
@@ -1295,7 +1319,10 @@ rlx_status_t enqueue_forward(const rlx_encoder* e, const int32_t* ids, const int
             if (forked) RLX_CUDA_TRY(cudaStreamWaitEvent(st, e->join_event, 0));   // join the side branch
             return RLX_OK;
         }
-        if (!body_only) RLX_TRY(launch_pack(mask, B, S, seq_len, seq_start, pos_of_rank, ticket, st, 0, 0, bins));
+        if (fuse_pe)
+            RLX_TRY(launch_pack_embed_ln(ids, mask, (const bf16*)w->word_emb, (const bf16*)w->pos_emb, (const bf16*)w->type_emb, w->emb_ln_g,
+                                         w->emb_ln_b, B, S, H, c.vocab, c.ln_eps, x, status, seq_len, seq_start, bins, st));
+        else if (!body_only) RLX_TRY(launch_pack(mask, B, S, seq_len, seq_start, pos_of_rank, ticket, st, 0, 0, bins));
     }
     const int32_t* rows = pk.total();
     const bool fuse_ln = !fold && uses_fused_ln(c, B, S);
@@ -1351,8 +1378,9 @@ rlx_status_t enqueue_forward(const rlx_encoder* e, const int32_t* ids, const int
         float2* stats_z = reinterpret_cast<float2*>(ws + a.stats_z);
         bf16* z = x1;   // raw output of the FFN-down projection (pre-LayerNorm), reused across layers
         const int P = H / 32;
-        RLX_TRY(launch_embed_ln(ids, (const bf16*)w->word_emb, (const bf16*)w->pos_emb, (const bf16*)w->type_emb,
-                                w->emb_ln_g, w->emb_ln_b, T, S, H, c.vocab, c.ln_eps, x, status, st, pk));
+        if (!fuse_pe)
+            RLX_TRY(launch_embed_ln(ids, (const bf16*)w->word_emb, (const bf16*)w->pos_emb, (const bf16*)w->type_emb,
+                                    w->emb_ln_g, w->emb_ln_b, T, S, H, c.vocab, c.ln_eps, x, status, st, pk));
         for (int l = 0; l < c.num_layers; ++l) {
             const rlx_layer_weights_t& lw = w->layers[l];
             unsigned char* fb = ws + a.fold + (size_t)l * a.fold_layer;
@@ -1372,7 +1400,7 @@ rlx_status_t enqueue_forward(const rlx_encoder* e, const int32_t* ids, const int
             }
             if (fuse_qa) {
                 RLX_TRY(launch_qkv_attention(l == 0 ? x : z, l == 0 ? (const bf16*)lw.wqkv : (const bf16*)(fb + a.f_wqkv), lw.bqkv,
-                                             l == 0 ? RLX_EPI_BIAS : 3, B, S, H, h, ctx, status, st, pk, l == 0 ? nullptr : &lf));
+                                             l == 0 ? RLX_EPI_BIAS : 3, B, S, H, h, ctx, status, st, pk, fuse_pe && l == 0, l == 0 ? nullptr : &lf));
             } else if (l == 0) {
                 RLX_TRY(launch_gemm(x, (const bf16*)lw.wqkv, lw.bqkv, nullptr, RLX_EPI_BIAS, T, 3 * H, H, qkv, false, status, st, rows));
             } else {
@@ -1403,11 +1431,12 @@ rlx_status_t enqueue_forward(const rlx_encoder* e, const int32_t* ids, const int
         if (forked) RLX_CUDA_TRY(cudaStreamWaitEvent(st, e->join_event, 0));   // join the side branch
         return RLX_OK;
     }
-    RLX_TRY(launch_embed_ln(ids, (const bf16*)w->word_emb, (const bf16*)w->pos_emb, (const bf16*)w->type_emb,
-                            w->emb_ln_g, w->emb_ln_b, T, S, H, c.vocab, c.ln_eps, x, status, st, pk));
+    if (!fuse_pe)
+        RLX_TRY(launch_embed_ln(ids, (const bf16*)w->word_emb, (const bf16*)w->pos_emb, (const bf16*)w->type_emb,
+                                w->emb_ln_g, w->emb_ln_b, T, S, H, c.vocab, c.ln_eps, x, status, st, pk));
     for (int l = 0; l < c.num_layers; ++l) {
         const rlx_layer_weights_t& lw = w->layers[l];
-        if (fuse_qa) RLX_TRY(launch_qkv_attention(x, (const bf16*)lw.wqkv, lw.bqkv, RLX_EPI_BIAS, B, S, H, h, ctx, status, st, pk));
+        if (fuse_qa) RLX_TRY(launch_qkv_attention(x, (const bf16*)lw.wqkv, lw.bqkv, RLX_EPI_BIAS, B, S, H, h, ctx, status, st, pk, fuse_pe && l == 0));
         else RLX_TRY(launch_gemm(x, (const bf16*)lw.wqkv, lw.bqkv, nullptr, RLX_EPI_BIAS, T, 3 * H, H, qkv, simt, status, st, rows));
         if (fuse_qa) {
         } else if (pack && uses_attention_fwd(c, B, S))
@@ -1676,7 +1705,7 @@ int32_t rlx_encoder_kernels_per_forward(const rlx_encoder_t* e, int32_t batch, i
 int32_t rlx_encoder_launches_per_forward(const rlx_encoder_t* e, int32_t batch, int32_t seq) {
     if (!e || batch <= 0 || seq <= 0) return 0;
     return kernels_in_forward(e->cfg, batch, seq) -
-           (uses_qkv_attention(e->cfg, batch, seq) ? e->cfg.num_layers : 0);
+           (uses_qkv_attention(e->cfg, batch, seq) ? e->cfg.num_layers : 0) - (int)uses_pack_embed(e->cfg, batch, seq);
 }
 
 rlx_status_t rlx_encoder_forward(rlx_encoder_t* e, const int32_t* ids, const int32_t* mask, int32_t B, int32_t S,
@@ -1726,6 +1755,10 @@ rlx_status_t rlx_encoder_forward_host(rlx_encoder_t* e, const int32_t* ids_h, co
     const int32_t* mask_z = static_cast<const int32_t*>(device_view_of_pinned(mask_h));
     float* out_z = static_cast<float*>(device_view_of_pinned(out_h));
     if (ids_z && mask_z && out_z && aligned16(ids_z) && aligned16(mask_z) && aligned16(out_z)) {
+        struct HostIo {
+            HostIo() { g_host_io = true; }
+            ~HostIo() { g_host_io = false; }
+        } host_io;
         s = forward_device(e, ids_z, mask_z, B, S, w, out_z, base, st);
         if (s != RLX_OK) return s;
     } else {

@@ -284,6 +284,23 @@ __device__ __forceinline__ int find_sequence_warp(const int32_t* __restrict__ se
     return lo;
 }
 
+// word[id] + pos[s] + type[0], this lane's columns
+template <int NV>
+__device__ __forceinline__ void embed_row(const __nv_bfloat16* __restrict__ wrow, const __nv_bfloat16* __restrict__ prow,
+                                          const __nv_bfloat16* __restrict__ type, int lane, float (&v)[NV * 4]) {
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+        const int col = (i * 32 + lane) * 4;
+        const uint2 a = __ldg(reinterpret_cast<const uint2*>(wrow + col));
+        const uint2 b = __ldg(reinterpret_cast<const uint2*>(prow + col));
+        const uint2 c = __ldg(reinterpret_cast<const uint2*>(type + col));
+        v[i * 4 + 0] = bf16lo(a.x) + bf16lo(b.x) + bf16lo(c.x);
+        v[i * 4 + 1] = bf16hi(a.x) + bf16hi(b.x) + bf16hi(c.x);
+        v[i * 4 + 2] = bf16lo(a.y) + bf16lo(b.y) + bf16lo(c.y);
+        v[i * 4 + 3] = bf16hi(a.y) + bf16hi(b.y) + bf16hi(c.y);
+    }
+}
+
 // x[row] = LN(word[id] + pos[s] + type[0]).  Ids outside [0, V) are clamped and flagged.
 // Padded mode (seq_start == nullptr): row = token t = b*S + s for all T tokens.
 // Packed mode: row p < seq_start[B] belongs to sequence b = find_sequence(p) at position
@@ -313,21 +330,96 @@ embed_ln_kernel(const int32_t* __restrict__ ids, const __nv_bfloat16* __restrict
         if (lane == 0 && status) atomicOr(status, RLX_DEVSTAT_TOKEN_RANGE_BIT);
         id = id < 0 ? 0 : V - 1;
     }
-    const __nv_bfloat16* wrow = word + (size_t)id * H;
-    const __nv_bfloat16* prow = pos + (size_t)s * H;
     float v[NV * 4];
-#pragma unroll
-    for (int i = 0; i < NV; ++i) {
-        const int col = (i * 32 + lane) * 4;
-        const uint2 a = __ldg(reinterpret_cast<const uint2*>(wrow + col));
-        const uint2 b = __ldg(reinterpret_cast<const uint2*>(prow + col));
-        const uint2 c = __ldg(reinterpret_cast<const uint2*>(type + col));
-        v[i * 4 + 0] = bf16lo(a.x) + bf16lo(b.x) + bf16lo(c.x);
-        v[i * 4 + 1] = bf16hi(a.x) + bf16hi(b.x) + bf16hi(c.x);
-        v[i * 4 + 2] = bf16lo(a.y) + bf16lo(b.y) + bf16lo(c.y);
-        v[i * 4 + 3] = bf16hi(a.y) + bf16hi(b.y) + bf16hi(c.y);
-    }
+    embed_row<NV>(word + (size_t)id * H, pos + (size_t)s * H, type, lane, v);
     ln_normalise_store<NV>(v, gamma, beta, eps, lane, out + (size_t)t * H);
+}
+
+// Packing and embedding + LayerNorm of a small call in one kernel: every CTA goes through the whole mask (at most 16 KB) for the
+// positions of its eight rows, so that no table has to come from another kernel; the last CTA writes the tables that later ones
+// read.  Instead of pack (mask, ticket, scan), hand-over and five dependent loads (search, position, id, rows) it is three: mask,
+// id, rows.  Same values as the two kernels.
+constexpr int kPackEmbedMaxTokens = 4096, kPackEmbedMaxSeqs = 512;
+
+template <int NV>
+__global__ void __launch_bounds__(kRowWarps * 32)
+pack_embed_ln_kernel(const int32_t* __restrict__ ids, const int32_t* __restrict__ mask, const __nv_bfloat16* __restrict__ word,
+                     const __nv_bfloat16* __restrict__ pos, const __nv_bfloat16* __restrict__ type, const float* __restrict__ gamma,
+                     const float* __restrict__ beta, __nv_bfloat16* __restrict__ out, int B, int S, int V, float eps, int32_t* status,
+                     int32_t* __restrict__ seq_len, int32_t* __restrict__ seq_start, int32_t* __restrict__ bins) {
+    constexpr int H = NV * 128, kThreads = kRowWarps * 32, kChunks = kPackEmbedMaxTokens / 32;
+    __shared__ unsigned valid[kChunks];     // a bit per position
+    __shared__ int before[kChunks + 1];     // valid positions in front of a chunk
+    __shared__ int starts[kPackEmbedMaxSeqs + 1];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, T = B * S;
+    pdl_launch_dependents();   // the next kernel waits before it reads anything, and before it lets another one start
+#pragma unroll
+    for (int i = 0; i < kChunks / kRowWarps; ++i) {
+        const int t = i * kThreads + tid;
+        const unsigned bal = __ballot_sync(0xffffffffu, t < T && __ldg(mask + t) != 0);
+        if (lane == 0) valid[i * kRowWarps + warp] = bal;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        constexpr int PER = kChunks / 32;   // chunks of a lane
+        int n[PER], sum = 0;
+#pragma unroll
+        for (int i = 0; i < PER; ++i) { n[i] = sum; sum += __popc(valid[lane * PER + i]); }
+        int incl = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
+        }
+#pragma unroll
+        for (int i = 0; i < PER; ++i) before[lane * PER + i] = incl - sum + n[i];
+        if (lane == 31) before[kChunks] = incl;
+    }
+    __syncthreads();
+    auto rank_of = [&](int t) {             // valid positions in front of position t (t <= T)
+        const int c = t >> 5;
+        return c == kChunks ? before[kChunks] : before[c] + __popc(valid[c] & ((1u << (t & 31)) - 1u));
+    };
+    if (blockIdx.x == gridDim.x - 1) {
+        // ---- the tables, as pack_sequences_kernel leaves them
+        for (int b = tid; b <= B; b += kThreads) seq_start[b] = starts[b] = rank_of(b * S);
+        __syncthreads();
+        for (int b = tid; b < B; b += kThreads) seq_len[b] = starts[b + 1] - starts[b];
+        if (tid == 0) {
+            int nbins = 0, first = 0;
+            bins[1] = 0;
+            for (int b = 1; b < B; ++b)
+                if (b - first == kBinSeqs || starts[b + 1] - starts[first] > kBinRows) {
+                    first = b;
+                    bins[1 + ++nbins] = b;
+                }
+            bins[0] = ++nbins;
+            bins[1 + nbins] = B;
+        }
+        return;
+    }
+    const int row = blockIdx.x * kRowWarps + warp;
+    if (row >= before[kChunks]) return;
+    // the position of this row: the last chunk with at most `row` valid positions in front of it that has any
+    int t = 0;
+    for (int c0 = 0; c0 < kChunks; c0 += 32) {
+        const int c = c0 + lane;
+        const unsigned hit = __ballot_sync(0xffffffffu, before[c] <= row && row < before[c + 1]);
+        if (hit) {
+            const int cc = c0 + __ffs(hit) - 1, k = row - before[cc];
+            const unsigned bits = valid[cc];
+            t = cc * 32 + __ffs(__ballot_sync(0xffffffffu, ((bits >> lane) & 1) && __popc(bits & ((1u << lane) - 1u)) == k)) - 1;
+            break;
+        }
+    }
+    int id = __ldg(ids + t);
+    if (id < 0 || id >= V) {
+        if (lane == 0 && status) atomicOr(status, RLX_DEVSTAT_TOKEN_RANGE_BIT);
+        id = id < 0 ? 0 : V - 1;
+    }
+    float v[NV * 4];
+    embed_row<NV>(word + (size_t)id * H, pos + (size_t)(t % S) * H, type, lane, v);
+    ln_normalise_store<NV>(v, gamma, beta, eps, lane, out + (size_t)row * H);
 }
 
 // out = LN(x) row by row (the residual sum was already formed by the producing GEMM's epilogue).

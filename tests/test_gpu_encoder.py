@@ -290,6 +290,9 @@ def test_projection_and_attention_in_one_kernel_give_the_bits_of_two(rlx, name, 
     assert np.array_equal(one, two) and np.array_equal(one, eager)
     pick = sorted({0, B // 2, B - 1})
     check(one[pick], oracle.encoder_forward(inp.cfg, inp.ids[pick], inp.mask[pick], inp.params, inp.layers), inp.lengths[pick])
+    # from pinned host buffers: packing and embedding in one kernel up to 256 positions, apart beyond
+    host, hstatus = run_gpu(rlx, inp, weights=w, flags=flags, host_io=True)
+    assert hstatus == 0 and np.array_equal(host, one)
 
 
 @pytest.mark.parametrize("heads", [2, 4])
