@@ -10,21 +10,33 @@
 // What bounds it: latency, as everything in a small forward; the point is the link that is not there.  A kernel boundary
 // costs the store of q, k, v, the hand-over and the round trip of the loads behind it.
 //
+// With OUT (few bins, heads of 32, one per CTA) the CTAs of a bin's heads are a cluster that goes on to the attention output:
+// y = ctx Wo^T + bias + residual, with its row statistics, epilogue modes 5 / 6.  Every CTA sends its head's context rows to all of
+// them (st.async: data and arrival in one) and multiplies the whole rows with 32 rows of Wo, which have been there since the
+// start.  An SM takes in 16.5 bytes a clock from its peers behind 700 cycles of latency: 32 / 64 / 128 rows of context 1.8 / 3.0 /
+// 5.4 thousand cycles, where another kernel's link costs eight thousand.
+//
 // All waits are bounded.
 #pragma once
 #include "attention.cuh"
+#include "gemm_cln_tcgen05.cuh"
+#include "gemm_splitk_tcgen05.cuh"
 #include "gemm_tcgen05.cuh"
 
 namespace rlx {
 namespace tcqa {
 
 using namespace rlx::tc;
+using rlx::tccl::mbar_wait_cluster;
+using rlx::tcsk::st_async_v4;
 
 constexpr int kRows = kBinRows;
+constexpr int kMaxOutHeads = 12;              // CTAs of a cluster, with OUT
+constexpr int kChunk = kRows * 16;            // 8 columns of the context rows: [column chunk][row][16 B], the layout without swizzle
 constexpr int kEpiWarps = 12;                 // a 32-row quadrant of q, of k or of v each; then they attend
 constexpr int kMaxTasks = kRows / 16 + kBinSeqs;   // 16-row groups of a bin's sequences
 
-template <int D, int HPC>
+template <int D, int HPC, bool OUT = false>
 struct Cfg {
     static constexpr int WARPS = HPC == 2 ? 16 : kEpiWarps;   // that attend: two heads of a full bin are sixteen groups of 16 rows
     static constexpr int THREADS = 64 + 32 * WARPS;
@@ -36,12 +48,15 @@ struct Cfg {
     static constexpr int STAGE_BYTES = KPS * KB_BYTES;
     static constexpr int TMEM_COLS = N <= 128 ? 128 : 256;
     static constexpr int STR = D + 8;                         // elements per q / k / v row: conflict-free ldmatrix
-    static constexpr int VEC_OFF = STAGES * STAGE_BYTES;
+    // OUT: the context rows lie over the ring, behind q, k and v; Wo's rows have room of their own
+    static constexpr int CTX_OFF = 65536, WO_OFF = STAGES * STAGE_BYTES, WO_BYTES = OUT ? kMaxOutHeads * 32 * 32 * 2 : 0;
+    static constexpr int VEC_OFF = WO_OFF + WO_BYTES;
     static constexpr int ZERO_OFF = VEC_OFF + kEpiWarps * 384;   // a row of zeros, read in place of v past a sequence's end
     static constexpr int TASK_OFF = ZERO_OFF + (STR * 2 + 15) / 16 * 16;
     static constexpr int BAR_OFF = TASK_OFF + kMaxTasks * 16;
-    static constexpr int NBAR = 2 * STAGES + 1;
+    static constexpr int NBAR = 2 * STAGES + 5;
     static constexpr int SMEM_BYTES = BAR_OFF + 8 * NBAR + 16 + 1024;
+    static_assert(!OUT || (D == 32 && HPC == 1 && 3 * kRows * STR * 2 <= CTX_OFF && CTX_OFF + kMaxOutHeads * 4 * kChunk <= WO_OFF), "context rows");
     static_assert(N == 96 || N == 192, "tile");
     static_assert(3 * HPC * kRows * STR * 2 <= STAGES * STAGE_BYTES, "q, k and v over the ring");
     static_assert(SMEM_BYTES <= 227 * 1024, "shared memory");
@@ -161,16 +176,18 @@ struct AttParams {
 };
 
 // grid (heads / HPC, bins that there can be); tmap_w: Wqkv as [q | k | v][row][column], boxes of 3 x D HPC x 64.  p: bias / folding vectors and row statistics of the product, K = H.
-template <int D, int HPC, int EPI>
-__global__ void __launch_bounds__((Cfg<D, HPC>::THREADS), 1)
-qkv_attention_kernel(const __grid_constant__ RowMaps tmap_a, const __grid_constant__ CUtensorMap tmap_w, const Params p,
-                     const AttParams ap) {
-    using C = Cfg<D, HPC>;
+// OUT: tmap_wo: Wo as k-blocks, boxes of 32 x H; po: the attention output's epilogue, its result to po.out.
+template <int D, int HPC, int EPI, bool OUT>
+__global__ void __launch_bounds__((Cfg<D, HPC, OUT>::THREADS), 1)
+qkv_attention_kernel(const __grid_constant__ RowMaps tmap_a, const __grid_constant__ CUtensorMap tmap_w,
+                     const __grid_constant__ CUtensorMap tmap_wo, const Params p, const Params po, const AttParams ap) {
+    using C = Cfg<D, HPC, OUT>;
     extern __shared__ unsigned char smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     unsigned char* gbase = smem_raw + (base - raw);
     const uint32_t full_bar = base + C::BAR_OFF, empty_bar = full_bar + 8 * C::STAGES, acc_bar = empty_bar + 8 * C::STAGES;
+    const uint32_t wo_bar = acc_bar + 8, ctx_bar = wo_bar + 8, free_bar = ctx_bar + 8, out_bar = free_bar + 8;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + C::BAR_OFF + 8 * C::NBAR);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     int4* tasks = reinterpret_cast<int4*>(gbase + C::TASK_OFF);   // first row in the bin, query row offset, length
@@ -181,6 +198,12 @@ qkv_attention_kernel(const __grid_constant__ RowMaps tmap_a, const __grid_consta
     if (threadIdx.x == 0) {
         for (int i = 0; i < C::STAGES; ++i) { mbar_init(full_bar + 8 * i, 1); mbar_init(empty_bar + 8 * i, 1); }
         mbar_init(acc_bar, 1);
+        if (OUT) {
+            mbar_init(wo_bar, 1);
+            mbar_init(ctx_bar, 1);
+            mbar_init(free_bar, gridDim.x);
+            mbar_init(out_bar, 1);
+        }
         *abort_flag = 0;
         fence_barrier_init();
         prefetch_tmap(&tmap_w);
@@ -198,6 +221,7 @@ qkv_attention_kernel(const __grid_constant__ RowMaps tmap_a, const __grid_consta
     const int row0 = exists ? ld_early(ap.seq_start + b0) : 0, rows = exists ? ld_early(ap.seq_start + b1) - row0 : 0;
     tc_fence_before();
     __syncthreads();
+    if constexpr (OUT) cluster_sync_all();   // the peers' barriers exist before anything is sent to them
     tc_fence_after();
     const uint32_t tmem = warp_uniform(*tmem_slot);
     const int groups = (rows + 31) / 32, a_kb = groups * (C::A_BYTES / 4);   // 32-row groups; bytes of a k-block of them
@@ -217,6 +241,12 @@ qkv_attention_kernel(const __grid_constant__ RowMaps tmap_a, const __grid_consta
                 if (elect_one()) load_w(early * C::KPS, early);
                 __syncwarp();
             }
+        if constexpr (OUT)
+            if (rows > 0 && elect_one()) {
+                mbar_expect_tx(wo_bar, (uint32_t)(num_kb * 32 * 128));
+                tma_load_3d(base + C::WO_OFF, &tmap_wo, 0, head0 * D, 0, wo_bar);
+            }
+        __syncwarp();
         pdl_wait();
         if (rows > 0) {
             int stage = 0;
@@ -260,6 +290,27 @@ qkv_attention_kernel(const __grid_constant__ RowMaps tmap_a, const __grid_consta
             }
             if (ok && elect_one()) umma_commit<1>(acc_bar);
             __syncwarp();
+            if constexpr (OUT) {
+                // the attention output: 32 columns, once all heads' context rows are here
+                if (elect_one()) mbar_expect_tx(ctx_bar, (uint32_t)(rows * H * 2));
+                __syncwarp();
+                ok = ok && mbar_wait_warp(wo_bar, 0, abort_flag) && __all_sync(0xffffffffu, mbar_wait_cluster(ctx_bar, 0, abort_flag)) != 0;
+                asm volatile("fence.proxy.async;" ::: "memory");   // the peers' stores, for the tensor core
+                tc_fence_after();
+                if (ok && elect_one()) {
+                    // K-major without swizzle: the 16-byte chunks of a K = 16 step are kChunk apart, 8-row groups 128 bytes
+                    const uint64_t cd = (uint64_t)((base + C::CTX_OFF & 0x3FFFFu) >> 4) | (uint64_t)(kChunk >> 4) << 16 | (uint64_t)(128 >> 4) << 32 |
+                                        (uint64_t)1 << 46;
+                    const uint64_t wd = make_smem_desc(base + C::WO_OFF);
+                    for (int kb = 0; kb < num_kb; ++kb)
+#pragma unroll
+                        for (int k = 0; k < BLOCK_K / UMMA_K; ++k)
+                            umma_bf16<1>(tmem + C::N, cd + (kb * 4 + k) * (2 * kChunk >> 4), wd + (kb * (32 * 128 >> 4) + 2 * k), make_idesc(kRows, 32),
+                                         (kb | k) != 0 ? 1u : 0u);
+                    umma_commit<1>(out_bar);
+                }
+                __syncwarp();
+            }
         }
     } else {
         // ------------------------------------------------------------ q, k, v, then attention
@@ -311,6 +362,11 @@ qkv_attention_kernel(const __grid_constant__ RowMaps tmap_a, const __grid_consta
         } else if (rows > 0) {
             ok = mbar_wait_warp(acc_bar, 0, abort_flag);   // the ring is free
         }
+        if constexpr (OUT) {
+            // this CTA's ring is free: its peers may send context rows
+            if (ok && rows > 0 && e == 0 && lane < (int)gridDim.x) mbar_arrive_cluster_release_cta(map_to_cta(free_bar, lane));
+            __syncwarp();
+        }
         asm volatile("bar.sync 1, %0;" ::"n"(32 * C::WARPS) : "memory");
         if (ok) {
             __nv_bfloat16* qkv = reinterpret_cast<__nv_bfloat16*>(gbase);
@@ -321,13 +377,51 @@ qkv_attention_kernel(const __grid_constant__ RowMaps tmap_a, const __grid_consta
                 const int first = task.x + task.y, n = min(16, task.z - task.y);   // query rows, in the bin
                 attend16<D, C::STR>(qh + first * C::STR, qh + (HPC * kRows + task.x) * C::STR, qh + (2 * HPC * kRows + task.x) * C::STR,
                                     base + C::ZERO_OFF, task.z, n, ap.scale_log2e);
-                constexpr int CH = D / 8;
-                __nv_bfloat16* out = ap.ctx + (size_t)(row0 + first) * H + (head0 + hh) * D;
-                for (int i = lane; i < 16 * CH; i += 32) {
-                    const int r = i / CH, c = i % CH;
-                    if (r < n)
-                        *reinterpret_cast<uint4*>(out + (size_t)r * H + c * 8) = *reinterpret_cast<const uint4*>(qh + (first + r) * C::STR + c * 8);
+                if constexpr (!OUT) {
+                    constexpr int CH = D / 8;
+                    __nv_bfloat16* out = ap.ctx + (size_t)(row0 + first) * H + (head0 + hh) * D;
+                    for (int i = lane; i < 16 * CH; i += 32) {
+                        const int r = i / CH, c = i % CH;
+                        if (r < n)
+                            *reinterpret_cast<uint4*>(out + (size_t)r * H + c * 8) = *reinterpret_cast<const uint4*>(qh + (first + r) * C::STR + c * 8);
+                    }
                 }
+            }
+        }
+        if constexpr (OUT) {
+            // a warp per peer: a warp's stores to different CTAs go out one behind the other
+            asm volatile("bar.sync 1, %0;" ::"n"(32 * C::WARPS) : "memory");
+            const int peer = head0 + e < (int)gridDim.x ? head0 + e : head0 + e - (int)gridDim.x;   // not all to the same one at once
+            if (rows > 0 && e < (int)gridDim.x) ok = ok && __all_sync(0xffffffffu, mbar_wait_cluster(free_bar, 0, abort_flag)) != 0;
+            if (ok && e < (int)gridDim.x) {
+                const uint32_t dst = map_to_cta(base + C::CTX_OFF + head0 * 4 * kChunk, peer), bar = map_to_cta(ctx_bar, peer);
+                for (int r = lane; r < rows; r += 32)
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        const uint4 a = ld_shared_v4(base + (uint32_t)(r * C::STR + c * 8) * 2);
+                        const uint32_t w[4] = {a.x, a.y, a.z, a.w};
+                        st_async_v4(dst + c * kChunk + r * 16, bar, w);
+                    }
+            }
+            __syncwarp();
+            if (part == 0 && live) {
+                using EO = EpilogueTile<EPI == 0 ? 5 : 6, 1, true>;
+                EO eo;
+                eo.load_vectors(po, head0 * D, base + C::VEC_OFF + e * 384);
+                eo.prefetch(po, row0 + rows, row0 + row, head0 * D);
+                ok = ok && mbar_wait_warp(out_bar, 0, abort_flag);
+                tc_fence_after();
+                uint32_t r[32];
+                tmem_ld_32x32(tmem + ((uint32_t)(quad * 32) << 16) + C::N, r);
+                tmem_ld_wait();
+                uint4 v[4];
+                eo.compute_chunk(po, r, head0 * D, 0, row0 + row, ok && row < rows, po.bias + head0 * D, v);
+                if (ok && row < rows) {   // the rows behind are another bin's
+                    uint4* y = reinterpret_cast<uint4*>(po.out + (size_t)(row0 + row) * H + head0 * D);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) y[i] = v[i];
+                }
+                tc_fence_before();
             }
         }
     }
@@ -340,6 +434,7 @@ qkv_attention_kernel(const __grid_constant__ RowMaps tmap_a, const __grid_consta
     }
     tc_fence_before();
     __syncthreads();
+    if constexpr (OUT) cluster_sync_all();   // no CTA leaves while a peer may still write into it
     if (warp == 1) {
         __syncwarp();
         tc_fence_after();

@@ -269,11 +269,14 @@ cudaError_t init_kernels_for_current_device() {
                                   rlx::tcmx::MxCfg<128>::SMEM_BYTES)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(rlx::tcmx::gemm_mx_tcgen05_kernel<192>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   rlx::tcmx::MxCfg<192>::SMEM_BYTES)) != cudaSuccess) return e;
-#define RLX_QA_ATTR(D, HPC, EPI)                                                                               \
-    if ((e = cudaFuncSetAttribute(rlx::tcqa::qkv_attention_kernel<D, HPC, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                  rlx::tcqa::Cfg<D, HPC>::SMEM_BYTES)) != cudaSuccess)                          \
+#define RLX_QA_ATTR(D, HPC, EPI, OUT)                                                                          \
+    if ((e = cudaFuncSetAttribute(rlx::tcqa::qkv_attention_kernel<D, HPC, EPI, OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                                  rlx::tcqa::Cfg<D, HPC, OUT>::SMEM_BYTES)) != cudaSuccess ||                   \
+        (OUT && (e = cudaFuncSetAttribute(rlx::tcqa::qkv_attention_kernel<D, HPC, EPI, OUT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != \
+                    cudaSuccess))                                                                              \
         return e;
-    RLX_QA_ATTR(32, 1, 0) RLX_QA_ATTR(32, 1, 3) RLX_QA_ATTR(32, 2, 0) RLX_QA_ATTR(32, 2, 3) RLX_QA_ATTR(64, 1, 0) RLX_QA_ATTR(64, 1, 3)
+    RLX_QA_ATTR(32, 1, 0, false) RLX_QA_ATTR(32, 1, 3, false) RLX_QA_ATTR(32, 2, 0, false) RLX_QA_ATTR(32, 2, 3, false)
+    RLX_QA_ATTR(64, 1, 0, false) RLX_QA_ATTR(64, 1, 3, false) RLX_QA_ATTR(32, 1, 0, true) RLX_QA_ATTR(32, 1, 3, true)
 #undef RLX_QA_ATTR
 #define RLX_ATT_FWD_ATTR(D, PAIR)                                                                              \
     if ((e = cudaFuncSetAttribute(rlx::tcat::attention_fwd_kernel<D, PAIR, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
@@ -882,28 +885,49 @@ bool make_tmap_qkv(CUtensorMap* map, const void* ptr, uint64_t H, uint32_t box_r
 int max_bins(int B, int S) {
     return (int)std::min<long long>(B, 2ll * B * S / rlx::kBinRows + B / rlx::kBinSeqs + 1);
 }
-template <int D, int HPC>
+// The attention output behind it (null: not in the same kernel): y = ctx Wo^T + bo + residual, with its row statistics.
+struct AttOut {
+    const bf16 *wo, *residual;
+    const float* bo;
+    bf16* y;
+    LnFold lf;
+};
+template <int D, int HPC, bool OUT = false>
 rlx_status_t launch_qkv_attention_d(const bf16* x, const bf16* w, const rlx::tc::Params& p, const rlx::tcqa::AttParams& ap, int epi,
-                                    int heads, int bins, cudaStream_t st) {
-    using C = rlx::tcqa::Cfg<D, HPC>;
+                                    int heads, int bins, cudaStream_t st, const AttOut* ao = nullptr) {
+    using C = rlx::tcqa::Cfg<D, HPC, OUT>;
     rlx::tcqa::RowMaps ta;
-    CUtensorMap tw;
+    CUtensorMap tw, two;
+    rlx::tc::Params po{};
     for (int i = 0; i < 4; ++i)
         if (!make_tmap_kblocks(ta.m + i, x, (uint64_t)p.M, (uint64_t)p.K, 32 * (i + 1), C::KPS)) return RLX_ERR_CUDA;
     if (!make_tmap_qkv(&tw, w, (uint64_t)p.K, D * HPC)) return RLX_ERR_CUDA;
+    two = tw;
+    if (OUT) {
+        if (!make_tmap_kblocks(&two, ao->wo, (uint64_t)p.K, (uint64_t)p.K, D, p.K / rlx::tc::BLOCK_K)) return RLX_ERR_CUDA;
+        po.bias = ao->bo; po.residual = ao->residual; po.out = ao->y; po.M = p.M; po.N = po.K = p.K; po.status = p.status;
+        po.stats_in = ao->lf.stats_in; po.stats_in_p = ao->lf.stats_in_p; po.ln_gamma = ao->lf.gamma; po.ln_beta = ao->lf.beta;
+        po.stats_out = ao->lf.stats_out; po.ln_eps = ao->lf.eps;
+    }
+    struct ClusterScope {
+        explicit ClusterScope(int x) { g_cluster_x = x; }
+        ~ClusterScope() { g_cluster_x = 1; }
+    } scope(OUT ? heads : 1);
     const dim3 grid(heads / HPC, bins);
-    if (epi == 0) RLX_CUDA_TRY(launch_ex(rlx::tcqa::qkv_attention_kernel<D, HPC, 0>, grid, C::THREADS, C::SMEM_BYTES, st, ta, tw, p, ap));
-    else RLX_CUDA_TRY(launch_ex(rlx::tcqa::qkv_attention_kernel<D, HPC, 3>, grid, C::THREADS, C::SMEM_BYTES, st, ta, tw, p, ap));
+    if (epi == 0) RLX_CUDA_TRY(launch_ex(rlx::tcqa::qkv_attention_kernel<D, HPC, 0, OUT>, grid, C::THREADS, C::SMEM_BYTES, st, ta, tw, two, p, po, ap));
+    else RLX_CUDA_TRY(launch_ex(rlx::tcqa::qkv_attention_kernel<D, HPC, 3, OUT>, grid, C::THREADS, C::SMEM_BYTES, st, ta, tw, two, p, po, ap));
     RLX_CUDA_TRY(cudaGetLastError());
     return RLX_OK;
 }
 rlx_status_t launch_qkv_attention(const bf16* x, const bf16* w, const float* bias, int epi, int B, int S, int H, int heads, bf16* ctx,
-                                  int32_t* status, cudaStream_t st, const Packing& pk, bool first, const LnFold* lf = nullptr) {
+                                  int32_t* status, cudaStream_t st, const Packing& pk, bool first, const LnFold* lf = nullptr,
+                                  const AttOut* ao = nullptr) {
     rlx::tc::Params p{};
     p.bias = bias; p.M = B * S; p.N = 3 * H; p.K = H; p.status = status;
     if (lf) { p.cvec = lf->cvec; p.dvec = lf->dvec; p.stats_in = lf->stats_in; p.stats_in_p = lf->stats_in_p; p.ln_eps = lf->eps; }
     const int d = H / heads, bins = max_bins(B, S);
     const rlx::tcqa::AttParams ap{pk.bins, pk.seq_start, ctx, 1.4426950408889634f / sqrtf((float)d), first};
+    if (ao) return launch_qkv_attention_d<32, 1, true>(x, w, p, ap, epi, heads, bins, st, ao);
     if (d == 64) return launch_qkv_attention_d<64, 1>(x, w, p, ap, epi, heads, bins, st);
     // one head per CTA while every bin there can be finds its SMs, else two: a row's x is then loaded half as often
     if (heads * bins <= sm_count()) return launch_qkv_attention_d<32, 1>(x, w, p, ap, epi, heads, bins, st);
@@ -1170,6 +1194,15 @@ bool uses_pack_embed(const rlx_encoder_config_t& c, int B, int S) {
     return uses_qkv_attention(c, B, S) && (long long)B * S <= (g_host_io ? kPackEmbedMaxHostTokens : rlx::kPackEmbedMaxTokens);
 }
 
+// The attention output in the same kernel too: the LayerNorms folded, heads of 32, and so few rows that their way from CTA to CTA is
+// shorter than another kernel's link (us apart / in one: 1 x 32 102.6 / 94.5, 2 x 32 107 / 98.8, 1 x 64 106.7 / 100.5 and 107.1 / 104.8, half
+// and all of the positions valid; 1 x 128 113.9 / 112.9 and 126 / 135, 3 x 64 114.8 / 119).
+constexpr int kMaxOutTokens = 64, kMaxOutBins = 2;
+bool uses_attention_out(const rlx_encoder_config_t& c, int B, int S) {
+    return uses_qkv_attention(c, B, S) && uses_fold_ln(c, B, S) && c.hidden / c.num_heads == 32 && c.num_heads <= rlx::tcqa::kMaxOutHeads &&
+           B * S <= kMaxOutTokens && max_bins(B, S) <= kMaxOutBins;
+}
+
 struct GraphEntry {
     int B, S;
     const void *ids, *mask, *out, *ws;
@@ -1272,7 +1305,7 @@ rlx_status_t enqueue_forward(const rlx_encoder* e, const int32_t* ids, const int
         }
     }
     Packing pk;
-    const bool fuse_qa = pack && uses_qkv_attention(c, B, S);
+    const bool fuse_qa = pack && uses_qkv_attention(c, B, S), fuse_out = fuse_qa && uses_attention_out(c, B, S);
     const bool fuse_pe = fuse_qa && uses_pack_embed(c, B, S);
     if (pack) {
         int32_t* seq_len = reinterpret_cast<int32_t*>(ws + a.seq_len);
@@ -1399,8 +1432,10 @@ rlx_status_t enqueue_forward(const rlx_encoder* e, const int32_t* ids, const int
                 lo.stats_in = stats_z; lo.stats_in_p = P; lo.gamma = pw.ln2_g; lo.beta = pw.ln2_b;
             }
             if (fuse_qa) {
+                const AttOut ao{(const bf16*)lw.wo, l == 0 ? x : z, lw.bo, y, lo};
                 RLX_TRY(launch_qkv_attention(l == 0 ? x : z, l == 0 ? (const bf16*)lw.wqkv : (const bf16*)(fb + a.f_wqkv), lw.bqkv,
-                                             l == 0 ? RLX_EPI_BIAS : 3, B, S, H, h, ctx, status, st, pk, fuse_pe && l == 0, l == 0 ? nullptr : &lf));
+                                             l == 0 ? RLX_EPI_BIAS : 3, B, S, H, h, ctx, status, st, pk, fuse_pe && l == 0, l == 0 ? nullptr : &lf,
+                                             fuse_out ? &ao : nullptr));
             } else if (l == 0) {
                 RLX_TRY(launch_gemm(x, (const bf16*)lw.wqkv, lw.bqkv, nullptr, RLX_EPI_BIAS, T, 3 * H, H, qkv, false, status, st, rows));
             } else {
@@ -1411,7 +1446,7 @@ rlx_status_t enqueue_forward(const rlx_encoder* e, const int32_t* ids, const int
                 RLX_TRY(launch_attention_fwd(qkv, T, pk.seq_start, pk.seq_len, B, S, h, d, 1, false, 0, nullptr, nullptr, ctx, status, st));
             else
                 RLX_TRY(launch_attention_bf16(qkv, mask, pk.seq_start, pk.seq_len, B, S, h, d, ctx, st));
-            RLX_TRY(launch_gemm(ctx, (const bf16*)lw.wo, lw.bo, l == 0 ? x : z, l == 0 ? 5 : 6, T, H, H, y, false, status, st, rows, 0, &lo));
+            if (!fuse_out) RLX_TRY(launch_gemm(ctx, (const bf16*)lw.wo, lw.bo, l == 0 ? x : z, l == 0 ? 5 : 6, T, H, H, y, false, status, st, rows, 0, &lo));
             // g = gelu(LN1(y) W1^T + b1) on the raw y with the folded weights
             if (l == 0 && fold_on_side) RLX_CUDA_TRY(cudaStreamWaitEvent(st, e->fold_event, 0));
             lf = LnFold();
@@ -1705,7 +1740,8 @@ int32_t rlx_encoder_kernels_per_forward(const rlx_encoder_t* e, int32_t batch, i
 int32_t rlx_encoder_launches_per_forward(const rlx_encoder_t* e, int32_t batch, int32_t seq) {
     if (!e || batch <= 0 || seq <= 0) return 0;
     return kernels_in_forward(e->cfg, batch, seq) -
-           (uses_qkv_attention(e->cfg, batch, seq) ? e->cfg.num_layers : 0) - (int)uses_pack_embed(e->cfg, batch, seq);
+           e->cfg.num_layers * ((int)uses_qkv_attention(e->cfg, batch, seq) + (int)uses_attention_out(e->cfg, batch, seq)) -
+           (int)uses_pack_embed(e->cfg, batch, seq);
 }
 
 rlx_status_t rlx_encoder_forward(rlx_encoder_t* e, const int32_t* ids, const int32_t* mask, int32_t B, int32_t S,

@@ -295,6 +295,19 @@ def test_projection_and_attention_in_one_kernel_give_the_bits_of_two(rlx, name, 
     assert hstatus == 0 and np.array_equal(host, one)
 
 
+@pytest.mark.parametrize("B,S,lengths", [(1, 64, [64]), (1, 64, [0]), (2, 32, [1, 32]), (2, 32, [0, 31]), (4, 16, [16, 3, 0, 16]), (1, 33, [33]),
+                                         (1, 16, [11]), (1, 65, [65]), (3, 22, [22, 1, 9])])
+def test_attention_output_of_tiny_calls_gives_the_bits_of_its_own_kernel(rlx, B, S, lengths):
+    """Up to 64 positions a cluster of the heads goes on to the attention output; the instrumented forward keeps every step apart."""
+    inp = make_inputs(CONFIGS["c1"], batch=B, seq=S, num_layers=3, lengths=lengths, ln_affine_random=True)
+    w = rlx.upload_weights(inp.params, inp.layers)
+    one, status = run_gpu(rlx, inp, weights=w)
+    apart, astatus = run_gpu(rlx, inp, weights=w, flags=4)
+    eager, estatus = run_gpu(rlx, inp, weights=w, flags=1)
+    assert status == 0 and astatus == 0 and estatus == 0
+    assert np.array_equal(one, apart) and np.array_equal(one, eager)
+
+
 @pytest.mark.parametrize("heads", [2, 4])
 @pytest.mark.parametrize("flags", [0, 0x200, 0x400])   # the host's choice, folded LayerNorm, none folded
 def test_a_short_last_chunk_takes_the_kernels_of_the_whole_call(rlx, heads, flags):
