@@ -1147,6 +1147,10 @@ bool uses_fold_ln(const rlx_encoder_config_t& c, int B, int S) {
     return !g_no_auto_fold && !(c.flags & RLX_FLAG_NO_AUTO_FOLD) && !other_fusion && call_tokens(B, S) <= kAutoFoldMaxTokens;
 }
 
+// The folded weights of the first two layers come from a launch of their own, which the chain reaches before those of all are done
+// (6 x 384: 1 x 32 94.5 -> 92.3 us, 1 x 128 114.3 -> 111.6, 16 x 128 153.4 -> 149.9, 16 x 64 138.1 -> 139.4, 32 x 128 the same).  At hidden 768
+// the 200 MB of the fold keep the memory busy far beyond that and the split gains nothing (7 x 120 404.6 / 406.2).
+constexpr size_t kFoldSplitLayerBytes = (size_t)4 << 20;
 int kernels_in_forward(const rlx_encoder_config_t& c, int B, int S) {
     const bool pack = !(c.flags & RLX_FLAG_NO_PACK) && !(c.flags & RLX_FLAG_GEMM_SIMT);
     const bool fused = uses_fold_ln(c, B, S) || uses_fused_ln(c, B, S) || uses_cluster_ln(c);
@@ -1222,7 +1226,7 @@ struct rlx_encoder {
     std::vector<cudaEvent_t> events;        // RLX_FLAG_KERNEL_EVENTS: one before the first kernel, one after each
     cudaStream_t side_stream = nullptr;     // side branch of the captured graph (weight prefetch)
     cudaStream_t body_stream = nullptr;     // the two bodies of a captured forward's IF / ELSE node are recorded here
-    cudaEvent_t fork_event = nullptr, join_event = nullptr, fold_event = nullptr;
+    cudaEvent_t fork_event = nullptr, join_event = nullptr, fold_event[2] = {};   // folded weights: of the first layers, of the rest
     cudaStream_t capture_stream = nullptr;  // graphs are recorded here (the caller's stream may be the
                                             // legacy default stream, which cannot be captured)
 };
@@ -1383,6 +1387,7 @@ rlx_status_t enqueue_forward(const rlx_encoder* e, const int32_t* ids, const int
             RLX_CUDA_TRY(cudaStreamWaitEvent(e->side_stream, e->fork_event, 0));
             forked = true;
         }
+        const int first_folds = std::min(a.fold_layer <= kFoldSplitLayerBytes ? 2 : c.num_layers, c.num_layers);
         auto flush_jobs = [&]() -> rlx_status_t {
             if (fl.n == 0) return RLX_OK;
             const int total_rows = fl.first_row[fl.n];
@@ -1401,10 +1406,15 @@ rlx_status_t enqueue_forward(const rlx_encoder* e, const int32_t* ids, const int
             }
             add_job(lw.w1, lw.ln1_g, lw.ln1_b, lw.b1, a.f_w1, a.f_c1, a.f_d1, l, F);
             if (fl.n == rlx::kFoldMaxJobs) { s = flush_jobs(); if (s != RLX_OK) return s; }
+            if (l + 1 == first_folds) {
+                s = flush_jobs();
+                if (s != RLX_OK) return s;
+                if (fold_on_side) RLX_CUDA_TRY(cudaEventRecord(e->fold_event[0], e->side_stream));
+            }
         }
         s = flush_jobs();
         if (s != RLX_OK) return s;
-        if (fold_on_side) RLX_CUDA_TRY(cudaEventRecord(e->fold_event, e->side_stream));
+        if (fold_on_side) RLX_CUDA_TRY(cudaEventRecord(e->fold_event[1], e->side_stream));
         if (forked) RLX_CUDA_TRY(cudaEventRecord(e->join_event, e->side_stream));
 
         float2* stats_y = reinterpret_cast<float2*>(ws + a.stats_y);
@@ -1419,6 +1429,7 @@ rlx_status_t enqueue_forward(const rlx_encoder* e, const int32_t* ids, const int
             unsigned char* fb = ws + a.fold + (size_t)l * a.fold_layer;
             LnFold lf;
             lf.eps = c.ln_eps;
+            if (l == first_folds && fold_on_side) RLX_CUDA_TRY(cudaStreamWaitEvent(st, e->fold_event[1], 0));
             if (l > 0) {
                 lf.cvec = (const float*)(fb + a.f_cqkv); lf.dvec = (const float*)(fb + a.f_dqkv);
                 lf.stats_in = stats_z; lf.stats_in_p = P;
@@ -1448,7 +1459,7 @@ rlx_status_t enqueue_forward(const rlx_encoder* e, const int32_t* ids, const int
                 RLX_TRY(launch_attention_bf16(qkv, mask, pk.seq_start, pk.seq_len, B, S, h, d, ctx, st));
             if (!fuse_out) RLX_TRY(launch_gemm(ctx, (const bf16*)lw.wo, lw.bo, l == 0 ? x : z, l == 0 ? 5 : 6, T, H, H, y, false, status, st, rows, 0, &lo));
             // g = gelu(LN1(y) W1^T + b1) on the raw y with the folded weights
-            if (l == 0 && fold_on_side) RLX_CUDA_TRY(cudaStreamWaitEvent(st, e->fold_event, 0));
+            if (l == 0 && fold_on_side) RLX_CUDA_TRY(cudaStreamWaitEvent(st, e->fold_event[0], 0));
             lf = LnFold();
             lf.eps = c.ln_eps;
             lf.cvec = (const float*)(fb + a.f_c1); lf.dvec = (const float*)(fb + a.f_d1);
@@ -1666,7 +1677,7 @@ rlx_status_t forward_device(rlx_encoder* e, const int32_t* ids, const int32_t* m
         RLX_CUDA_TRY(cudaStreamCreateWithFlags(&e->side_stream, cudaStreamNonBlocking));
         RLX_CUDA_TRY(cudaEventCreateWithFlags(&e->fork_event, cudaEventDisableTiming));
         RLX_CUDA_TRY(cudaEventCreateWithFlags(&e->join_event, cudaEventDisableTiming));
-        RLX_CUDA_TRY(cudaEventCreateWithFlags(&e->fold_event, cudaEventDisableTiming));
+        for (auto& evt : e->fold_event) RLX_CUDA_TRY(cudaEventCreateWithFlags(&evt, cudaEventDisableTiming));
     }
     RLX_CUDA_TRY(cudaStreamBeginCapture(e->capture_stream, cudaStreamCaptureModeThreadLocal));
     rlx_status_t s = enqueue_forward_any(e, ids, mask, B, S, &e->weights, out, ws, e->capture_stream, true);
@@ -1722,7 +1733,8 @@ void rlx_encoder_destroy(rlx_encoder_t* e) {
     if (e->body_stream) cudaStreamDestroy(e->body_stream);
     if (e->fork_event) cudaEventDestroy(e->fork_event);
     if (e->join_event) cudaEventDestroy(e->join_event);
-    if (e->fold_event) cudaEventDestroy(e->fold_event);
+    for (auto& evt : e->fold_event)
+        if (evt) cudaEventDestroy(evt);
     for (auto& evt : e->events) cudaEventDestroy(evt);
     delete e;
 }
