@@ -1,0 +1,191 @@
+// bf16 "Linear" GEMM of a CTA pair whose tile width is chosen on the device: out[M,N] = epilogue(A[M,K] W[N,K]^T + bias), K of at
+// least a few thousand, N a multiple of 192 and of 128 (the feed-forward down products).
+//
+// A packed batch has fewer rows than the host knows of (its padded count), and how wide a tile should be depends on them: as wide
+// as possible while all tiles run beside each other, narrower where that fills pairs that would idle.  61 sequences of
+// up to 203 at N = 384: 29 row blocks are 58 tiles of 192 columns, one round of 74 pairs, or 87 of 128, two; with every position
+// valid 49 are 98 or 147, two rounds each, and the narrow ones are shorter.
+// So everything that depends on the width (boxes of W, stage size and count, instruction shape, columns per epilogue
+// warp) is a variable here; the rest is gemm_tcgen05.cuh's pair kernel with two k-blocks per stage.
+// The order along K does not depend on the width: the bits are the same with each.
+#pragma once
+#include "gemm_tcgen05.cuh"
+
+namespace rlx {
+namespace tcpw {
+
+using namespace rlx::tc;
+
+constexpr int kMaxBN = 192, kKps = 2, kMaxStages = 4;
+constexpr int kABytes = BLOCK_M * BLOCK_K * 2;
+constexpr int kEpiWarps = 12, kThreads = 64 + 32 * kEpiWarps;
+constexpr int kBarBytes = 8 * (2 * kMaxStages + 4) + 16;
+template <int EPI>
+struct Cfg {
+    static constexpr bool VEC = EPI >= 3;
+    static constexpr int VEC_BYTES = VEC ? kEpiWarps * 384 : 0;
+    static constexpr int SMEM_BYTES = 227 * 1024;
+    static constexpr int RING_BYTES = (SMEM_BYTES - 1024 - kEpiWarps * kStageBufBytes - VEC_BYTES - kBarBytes) / 1024 * 1024;
+    static constexpr int STG_OFF = RING_BYTES, VEC_OFF = STG_OFF + kEpiWarps * kStageBufBytes, BAR_OFF = VEC_OFF + VEC_BYTES;
+    static_assert(3 * kKps * (kABytes + kMaxBN / 2 * BLOCK_K * 2) <= RING_BYTES, "three stages of the widest tile");
+};
+struct WidthMaps {
+    CUtensorMap w[3];   // W as pairs of k-blocks, boxes of 32, 64 and 96 rows: a CTA's half of a tile of 64, 128 and 192 columns
+};
+
+// Columns of a tile, in units of 64, for `blocks` 256-row blocks: the least rounds times the clocks that a k-block takes (measured:
+// operands at 70 bytes a clock and SM, at N = 64 the round to the barriers).
+__device__ __forceinline__ int pick_width(int blocks, int N, int pairs) {
+    int best = 3, cost = 0x7fffffff;
+#pragma unroll
+    for (int w = 3; w >= 1; --w) {
+        const int rounds = (blocks * (N / (64 * w)) + pairs - 1) / pairs, c = rounds * (w == 3 ? 410 : w == 2 ? 351 : 310);
+        if (c < cost) { cost = c; best = w; }
+    }
+    return best;
+}
+
+template <int EPI>
+__global__ void __launch_bounds__(kThreads, 1)
+gemm_pair_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ WidthMaps wm,
+                         const __grid_constant__ CUtensorMap tmap_out, const Params p) {
+    using C = Cfg<EPI>;
+    extern __shared__ unsigned char smem_raw[];
+    const uint32_t raw = smem_u32(smem_raw);
+    const uint32_t base = (raw + 1023u) & ~1023u;
+    unsigned char* gbase = smem_raw + (base - raw);
+    const uint32_t full_bar = base + C::BAR_OFF, empty_bar = full_bar + 8 * kMaxStages;
+    const uint32_t tfull_bar = empty_bar + 8 * kMaxStages, tempty_bar = tfull_bar + 16;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + C::BAR_OFF + 8 * (2 * kMaxStages + 4));
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const uint32_t cta_rank = warp_uniform(cluster_ctarank());   // rank 0 leads the pair
+    pdl_launch_dependents();
+
+    int M = p.M;
+    if (p.m_ptr != nullptr) M = min(M, ld_early(p.m_ptr));
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < kMaxStages; ++i) { mbar_init(full_bar + 8 * i, 1); mbar_init(empty_bar + 8 * i, 1); }
+        for (int i = 0; i < 2; ++i) { mbar_init(tfull_bar + 8 * i, 1); mbar_init(tempty_bar + 8 * i, 2 * kEpiWarps); }
+        *abort_flag = 0;
+        fence_barrier_init();
+        prefetch_tmap(&tmap_a);
+        prefetch_tmap(&tmap_out);
+        for (int i = 0; i < 3; ++i) prefetch_tmap(&wm.w[i]);
+    }
+    if (warp == 1) {
+        tmem_alloc<2>(smem_u32(tmem_slot), 512);
+        tmem_relinquish<2>();
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();
+    tc_fence_after();
+    const uint32_t tmem = warp_uniform(*tmem_slot);
+
+    const int pairs = gridDim.x / 2, m_tiles = (M + 255) / 256, num_kb = p.K / BLOCK_K;
+    const int width = (int)warp_uniform((uint32_t)pick_width(m_tiles, p.N, pairs)), bn = 64 * width;
+    const int n_tiles = p.N / bn, num_tiles = n_tiles * m_tiles;
+    const int b_bytes = 32 * width * BLOCK_K * 2, stage_bytes = kKps * (kABytes + b_bytes), stages = min(kMaxStages, C::RING_BYTES / stage_bytes);
+
+    if (warp == 0) {
+        // ------------------------------------------------------------ TMA producer (whole warp, one lane issues)
+        pdl_wait();
+        const CUtensorMap* map_w = &wm.w[width - 1];
+        int stage = 0;
+        uint32_t phase = 1;
+        bool ok = true;
+        for (int tile = blockIdx.x / 2; tile < num_tiles && ok; tile += pairs) {
+            const int arow = (tile / n_tiles) * 256 + (int)cta_rank * BLOCK_M, brow = (tile % n_tiles) * bn + (int)cta_rank * 32 * width;
+            for (int kb = 0; kb < num_kb; kb += kKps) {
+                if (!(ok = mbar_wait_warp(empty_bar + 8 * stage, phase, abort_flag))) break;
+                if (elect_one()) {
+                    const uint32_t st = base + stage * stage_bytes, lead_full = map_to_cta(full_bar + 8 * stage, 0);
+                    if (cta_rank == 0) mbar_expect_tx(full_bar + 8 * stage, 2 * stage_bytes);
+                    tma_load_3d_cg2(st, &tmap_a, 0, arow, kb, lead_full);
+                    tma_load_3d_cg2(st + kKps * kABytes, map_w, 0, brow, kb, lead_full);
+                }
+                __syncwarp();
+                if (++stage == stages) { stage = 0; phase ^= 1; }
+            }
+        }
+    } else if (warp == 1) {
+        // ------------------------------------------------------------ MMA issuer (leader CTA, whole warp, one lane issues)
+        if (cta_rank == 0) {
+            const uint32_t idesc = make_idesc(256, bn), b_kb = b_bytes >> 4;
+            const uint64_t ad0 = make_smem_desc(base), bd0 = make_smem_desc(base + kKps * kABytes);
+            int stage = 0, it = 0;
+            uint32_t phase = 0;
+            bool ok = true;
+            for (int tile = blockIdx.x / 2; tile < num_tiles && ok; tile += pairs, ++it) {
+                const int as = it & 1;
+                if (!(ok = mbar_wait_warp(tempty_bar + 8 * as, ((it >> 1) & 1) ^ 1, abort_flag))) break;
+                tc_fence_after();
+                const uint32_t acc = tmem + as * kMaxBN;
+                for (int kb = 0; kb < num_kb; kb += kKps) {
+                    if (!(ok = mbar_wait_warp(full_bar + 8 * stage, phase, abort_flag))) break;
+                    tc_fence_after();
+                    if (elect_one()) {
+                        const uint64_t ad = ad0 + (stage * stage_bytes >> 4), bd = bd0 + (stage * stage_bytes >> 4);
+#pragma unroll
+                        for (int i = 0; i < kKps; ++i)
+#pragma unroll
+                            for (int k = 0; k < BLOCK_K / UMMA_K; ++k)
+                                umma_bf16<2>(acc, ad + (i * (kABytes >> 4) + 2 * k), bd + (i * b_kb + 2 * k), idesc, (kb | i | k) != 0 ? 1u : 0u);
+                        umma_commit<2>(empty_bar + 8 * stage);
+                        if (kb + kKps >= num_kb) umma_commit<2>(tfull_bar + 8 * as);
+                    }
+                    __syncwarp();
+                    if (++stage == stages) { stage = 0; phase ^= 1; }
+                }
+            }
+        }
+    } else {
+        // ------------------------------------------------------------ epilogue warps: 32 rows x 64 columns, as many groups as the tile has
+        const int ew = warp - 2, quad = warp & 3, half = ew >> 2;
+        const uint32_t stg = base + C::STG_OFF + ew * kStageBufBytes;
+        using ET = EpilogueTile<EPI, 2, C::VEC>;
+        if ((int)blockIdx.x / 2 < num_tiles && half < width) ET::prefetch_bias(p, ((int)blockIdx.x / 2) % n_tiles * bn + half * 64);
+        pdl_wait();
+        int it = 0;
+        bool ok = true;
+        for (int tile = blockIdx.x / 2; tile < num_tiles && ok; tile += pairs, ++it) {
+            const int as = it & 1;
+            const uint32_t ph = (it >> 1) & 1;
+            if (half >= width) {                     // columns that this width does not have
+                if (!(ok = mbar_wait_warp(tfull_bar + 8 * as, ph, abort_flag))) break;
+                if (lane == 0) mbar_arrive_cluster_relaxed(map_to_cta(tempty_bar + 8 * as, 0));
+                continue;
+            }
+            const int m_row0 = (tile / n_tiles) * 256 + (int)cta_rank * BLOCK_M + quad * 32, n0 = (tile % n_tiles) * bn + half * 64;
+            const int next = tile + pairs;
+            if (next < num_tiles) ET::prefetch_bias(p, (next % n_tiles) * bn + half * 64);
+            ET et;
+            et.load_vectors(p, n0, base + C::VEC_OFF + ew * 384);
+            et.prefetch(p, M, m_row0 + lane, n0);
+            if (!(ok = mbar_wait_warp(tfull_bar + 8 * as, ph, abort_flag))) break;
+            tc_fence_after();
+            et.template drain<2>(p, &tmap_out, M, m_row0, n0, tmem + ((uint32_t)(quad * 32) << 16) + as * kMaxBN + half * 64, stg, lane,
+                                 tempty_bar + 8 * as, cta_rank);
+        }
+        ET::finish(lane);
+    }
+    // ---------------------------------------------------------------- teardown
+    __syncwarp();
+    if (*abort_flag) {
+        if (threadIdx.x == 0 && p.status) atomicOr(p.status, RLX_DEVSTAT_TIMEOUT_BIT);
+        const uint64_t t0 = global_timer_ns();
+        while (global_timer_ns() - t0 < 200000ull) __nanosleep(1000);
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();      // neither CTA leaves while the pair still uses its memory
+    if (warp == 1) {
+        __syncwarp();
+        tc_fence_after();
+        tmem_dealloc<2>(tmem, 512);
+    }
+}
+
+}  // namespace tcpw
+}  // namespace rlx

@@ -21,6 +21,7 @@
 #include "gemm_ares_tcgen05.cuh"
 #include "gemm_ln_tcgen05.cuh"
 #include "gemm_cln_tcgen05.cuh"
+#include "gemm_pair_tcgen05.cuh"
 #include "gemm_splitk_tcgen05.cuh"
 #include "rowwise.cuh"
 #include "qkv_attention_tcgen05.cuh"
@@ -269,6 +270,12 @@ cudaError_t init_kernels_for_current_device() {
                                   rlx::tcmx::MxCfg<128>::SMEM_BYTES)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(rlx::tcmx::gemm_mx_tcgen05_kernel<192>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   rlx::tcmx::MxCfg<192>::SMEM_BYTES)) != cudaSuccess) return e;
+#define RLX_PAIR_ATTR(EPI)                                                                                     \
+    if ((e = cudaFuncSetAttribute(rlx::tcpw::gemm_pair_tcgen05_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                                  rlx::tcpw::Cfg<EPI>::SMEM_BYTES)) != cudaSuccess)                            \
+        return e;
+    RLX_PAIR_ATTR(0) RLX_PAIR_ATTR(1) RLX_PAIR_ATTR(2) RLX_PAIR_ATTR(6)
+#undef RLX_PAIR_ATTR
 #define RLX_QA_ATTR(D, HPC, EPI, OUT)                                                                          \
     if ((e = cudaFuncSetAttribute(rlx::tcqa::qkv_attention_kernel<D, HPC, EPI, OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
                                   rlx::tcqa::Cfg<D, HPC, OUT>::SMEM_BYTES)) != cudaSuccess ||                   \
@@ -675,6 +682,41 @@ rlx_status_t launch_gemm_tc_bn(const CUtensorMap& ta, const CUtensorMap& tb, con
     return RLX_OK;
 }
 
+// CTA pairs whose tile width the kernel chooses from the rows that exist (gemm_pair_tcgen05.cuh): long contractions, columns that
+// every width divides, more tiles of 128 columns than pairs, so that the width decides on the rounds, and few enough rounds that one more
+// or less counts.  Whole forwards, us fixed / chosen: 6 x 384 61 x 203 435 / 422 and 587 / 589 (half and all of the positions valid),
+// 100 x 128 405 / 391, 60 x 256 459 / 443; 12 x 768 32 x 128 712 / 713 and 1068 / 1039, 64 x 128 1106 / 1070.  With fewer tiles the
+// fixed width's smaller code wins (32 x 128 181 / 185).
+bool pair_width_pays(int M, int N, int K, int epi, const TileChoice& tc) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const int pairs = (dev >= 0 && dev < 64) ? g_max_pairs[dev] : 0;
+    return tc.cg == 2 && tc.bn <= rlx::tcpw::kMaxBN && (epi <= 2 || epi == 6) && K >= 1536 && K % rlx::tc::BLOCK_K == 0 && N % 384 == 0 &&
+           (M + 255) / 256 * (N / 128) > pairs && (M + 255) / 256 * (N / 192) < 4 * pairs;
+}
+rlx_status_t launch_gemm_pair(const bf16* A, const bf16* W, const CUtensorMap& to, const rlx::tc::Params& p, int epi, cudaStream_t st) {
+    CUtensorMap ta;
+    rlx::tcpw::WidthMaps wm;
+    if (!make_tmap_kblocks(&ta, A, p.M, p.K, rlx::tc::BLOCK_M, rlx::tcpw::kKps)) return RLX_ERR_CUDA;
+    for (int i = 0; i < 3; ++i)
+        if (!make_tmap_kblocks(wm.w + i, W, p.N, p.K, 32 * (i + 1), rlx::tcpw::kKps)) return RLX_ERR_CUDA;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const int grid = 2 * std::min((p.M + 255) / 256 * (p.N / 64), g_max_pairs[dev]);
+    struct ClusterScope {
+        explicit ClusterScope(int x) { g_cluster_x = x; }
+        ~ClusterScope() { g_cluster_x = 1; }
+    } scope(2);
+    switch (epi) {
+#define RLX_CASE(E) case E: RLX_CUDA_TRY(launch_ex(rlx::tcpw::gemm_pair_tcgen05_kernel<E>, grid, rlx::tcpw::kThreads, rlx::tcpw::Cfg<E>::SMEM_BYTES, st, ta, wm, to, p)); break;
+        RLX_CASE(0) RLX_CASE(1) RLX_CASE(2) RLX_CASE(6)
+#undef RLX_CASE
+        default: return RLX_ERR_INVALID_ARG;
+    }
+    RLX_CUDA_TRY(cudaGetLastError());
+    return RLX_OK;
+}
+
 // A-resident CTA-pair GEMM (short contractions): grid = 2 x min(work units, resident pairs).
 template <int BN>
 rlx_status_t launch_gemm_resident_bn(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& to,
@@ -836,6 +878,7 @@ rlx_status_t launch_gemm(const bf16* A, const bf16* W, const float* bias, const 
     const TileChoice tc = pick_tile(M, N, K, want_cg);
     const int bn = tc.bn;
     if (bn == 0) return RLX_ERR_UNSUPPORTED;
+    if (want_cg == 0 && pair_width_pays(M, N, K, epi, tc)) return launch_gemm_pair(A, W, to, p, epi, st);
     int kps = 1;
     switch (bn * 10 + tc.cg) {
         case 641: kps = rlx::tc::Cfg<64, 1>::KPS; break;

@@ -308,6 +308,19 @@ def test_attention_output_of_tiny_calls_gives_the_bits_of_its_own_kernel(rlx, B,
     assert np.array_equal(one, apart) and np.array_equal(one, eager)
 
 
+@pytest.mark.parametrize("B,S,lo", [(61, 203, 40), (61, 203, 203), (40, 150, 20)])
+def test_packed_rows_choose_the_tile_width_and_not_the_result(rlx, B, S, lo):
+    """The packed and the padded layout (RLX_FLAG_NO_PACK) hand the feed-forward down product other row counts: other widths."""
+    lengths = np.linspace(lo, S, B).astype(int)
+    inp = make_inputs(CONFIGS["c1"], batch=B, seq=S, num_layers=2, lengths=lengths)
+    w = rlx.upload_weights(inp.params, inp.layers)
+    packed, status = run_gpu(rlx, inp, weights=w)
+    padded, pstatus = run_gpu(rlx, inp, weights=w, flags=8)
+    assert status == 0 and pstatus == 0 and np.array_equal(packed, padded)
+    pick = [0, B - 1]
+    check(packed[pick], oracle.encoder_forward(inp.cfg, inp.ids[pick], inp.mask[pick], inp.params, inp.layers), inp.lengths[pick])
+
+
 @pytest.mark.parametrize("heads", [2, 4])
 @pytest.mark.parametrize("flags", [0, 0x200, 0x400])   # the host's choice, folded LayerNorm, none folded
 def test_a_short_last_chunk_takes_the_kernels_of_the_whole_call(rlx, heads, flags):
