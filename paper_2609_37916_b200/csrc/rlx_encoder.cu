@@ -482,7 +482,13 @@ rlx_status_t launch_attention_fwd(const bf16* qkv, int rows, const int32_t* seq_
                                   int h, int d, int kv_group, bool positional, int window, const float* rope_cos,
                                   const float* rope_sin, bf16* ctx, int32_t* status, cudaStream_t st) {
     namespace tcat = rlx::tcat;
-    const bool pair = d <= 64 && kv_group == 1 && h % 2 == 0;
+    // Rotated heads of 64 that see many keys go by two row tiles of one head instead of one of two heads: a K block is loaded and
+    // rotated once for both, where a pair of heads has it rotated for every 128 rows.  The tiles' first and last blocks are
+    // one's only, which costs more than that under a short window (us pair / rows, 16 x 1000..4000, 8 heads: causal 271 / 237, window 768
+    // 149 / 137, 512 121 / 115, 384 110 / 105, 256 96.0 / 95.5; 23 x 100..1500, 16 heads: 512 102.4 / 101.1, 128 71.7 / 78.0; causal 64 x
+    // 30..300 49.6 / 53.4, 100..400 43.2 / 43.2, 32 x 200..600 42.5 / 40.6; heads of 32 the same either way).
+    const bool by_rows = rope_cos != nullptr && d == 64 && positional && std::min(window, max_len) >= 3 * tcat::kTile;
+    const bool pair = d <= 64 && kv_group == 1 && h % 2 == 0 && !by_rows;
     const bool rows_mode = !pair && kv_group % 2 != 0;
     tcat::Params p = {};
     p.seq_start = seq_start; p.seq_len = seq_len; p.ctx = ctx; p.rope_cos = rope_cos; p.rope_sin = rope_sin; p.status = status;

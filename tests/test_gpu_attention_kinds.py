@@ -333,3 +333,21 @@ def test_kernel_choice_at_its_edges(rlx, d, hq, hkv, n, length, kind, window):
     inside = rlx.attention_kind_bf16(bf16_dev(qkv), *args, kind, window, rope, num_kv_heads=hkv)
     turned = rlx.binding.qk_rope_bf16(bf16_dev(qkv), *args, rope, num_kv_heads=hkv)
     assert torch.equal(inside, rlx.attention_kind_bf16(turned, *args, kind, window, num_kv_heads=hkv))
+
+
+@pytest.mark.parametrize("lengths", [[383, 130, 1], [384, 257, 256, 255], [1000, 1, 129, 640, 383]])
+@pytest.mark.parametrize("kind,window", [(CAUSAL, 0), (SLIDING, 383), (SLIDING, 384), (SLIDING, 385), (SLIDING, 900)])
+def test_rotated_heads_of_64_by_row_tiles_or_by_pairs_of_heads(rlx, lengths, kind, window):
+    """Rotated inside, heads of 64 go by two row tiles of a head where a row sees 384 keys or more; rotated in front, by two heads.  Both
+    sides of that line, second tiles that are empty, partial and full, rows of NaN behind the last sequence: the same bits."""
+    h, d, total = 4, 64, sum(lengths)
+    rng = np.random.default_rng(total + window)
+    qkv = rand_bf16(rng, (total + 3, 3 * h * d))
+    qkv[total:] = np.float32("nan")
+    start = (np.cumsum(lengths) - lengths).astype(np.int32)
+    args = (i32_dev(start), i32_dev(np.array(lengths, np.int32)), max(lengths), h)
+    rope = rlx.rope_tables(max(lengths), d)
+    inside = rlx.attention_kind_bf16(bf16_dev(qkv), *args, kind, window, rope)
+    turned = rlx.binding.qk_rope_bf16(bf16_dev(qkv), *args, rope)
+    in_front = rlx.attention_kind_bf16(turned, *args, kind, window)
+    assert torch.isfinite(inside.float()).all() and torch.equal(inside, in_front)
