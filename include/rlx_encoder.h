@@ -75,8 +75,9 @@ typedef enum {
                                    not a multiple of 32 or max_seq exceeds 512; takes precedence over
                                    RLX_FLAG_FUSED_LN / RLX_FLAG_CLUSTER_LN.  Pays for small batches (launch-bound
                                    forwards); for large ones the separate LayerNorm kernels are faster.  Chosen
-                                   AUTOMATICALLY for calls with batch*seq <= 4096 unless one of the other two
-                                   fusion flags or RLX_FLAG_NO_AUTO_FOLD is set */
+                                   AUTOMATICALLY for calls with batch*seq <= 4096 (12544 at hidden <= 384) unless
+                                   one of the other two fusion flags or RLX_FLAG_NO_AUTO_FOLD is set; beyond 4096 a
+                                   workspace without room for the folded weights keeps the LayerNorm kernels */
 #define RLX_FLAG_NO_AUTO_FOLD 0x400u /* keep the 7-kernel layer (separate LayerNorm kernels) at every batch size */
 #define RLX_FLAG_FUSED_FFN 0x1000u /* everything of a layer behind the attention in ONE kernel (rlx_layer_tail_bf16:
                                       out-projection + residual + LayerNorm, FFN-up, GELU, FFN-down + residual +
@@ -291,9 +292,10 @@ rlx_status_t rlx_encoder_forward_static(rlx_encoder_t *encoder, const int32_t *t
 rlx_status_t rlx_encoder_last_device_status(rlx_encoder_t *encoder, void *workspace, void *cuda_stream);
 
 /* Number of kernels of one forward of (batch, seq), the steps of its layers counted apart: the entries of
- * rlx_encoder_kernel_times.  A forward of at most 4096 positions in sequences of at most 128 runs a layer's QKV GEMM and
- * attention as one kernel unless RLX_FLAG_KERNEL_EVENTS, _NO_PACK or _ATTN_TCGEN05 is set (bit for bit the same result);
- * rlx_encoder_launches_per_forward counts those as one. */
+ * rlx_encoder_kernel_times.  A forward of at most 4096 positions (6144 at hidden <= 384) in sequences of at
+ * most 128 runs a layer's QKV GEMM and attention as one kernel, the smallest ones more than that, unless
+ * RLX_FLAG_KERNEL_EVENTS, _NO_PACK or _ATTN_TCGEN05 is set (bit for bit the same result);
+ * rlx_encoder_launches_per_forward counts the kernels that it launches. */
 int32_t rlx_encoder_kernels_per_forward(const rlx_encoder_t *encoder, int32_t batch, int32_t seq);
 int32_t rlx_encoder_launches_per_forward(const rlx_encoder_t *encoder, int32_t batch, int32_t seq);
 

@@ -1182,9 +1182,11 @@ bool uses_cluster_ln(const rlx_encoder_config_t& c) {
 //              96 x 128 372 / 376 and 526 / 527, 61 x 203 396 / 402 and 595 / 591, 255 x 128 749 / 736 and 1364 / 1286
 //   12 x 768   1 x 128 387 / 450 and 406 / 459, 7 x 120 457 / 502 and 572 / 559, 32 x 128 740 / 732 and 1094 / 1042,
 //              64 x 128 1224 / 1134 and 2065 / 1833
-// One line for both widths: it costs the wider model up to 5 % between 2000 and 4096 tokens, and the narrower one would gain
-// up to 5 % from 4096 to 12000.
-constexpr int kAutoFoldMaxTokens = 4096;
+// With the width of the long contraction's tiles chosen on the device, and projection and attention in one kernel:
+//   6 x 384    64 x 128 288 / 302 and 389 / 397, 22 x 256 275 / 289, 16 x 512 336 / 345, 90 x 128 358 / 364, 61 x 203 415 / 424 and 599 / 597
+//   12 x 768   16 x 128 513 / 513, 32 x 128 717 / 714
+// The wider model's weights are four times as many to fold.  The narrower one's line lies in front of 12800 tokens.
+constexpr int kAutoFoldMaxTokens = 4096, kAutoFoldMaxTokensNarrow = 12544, kNarrowHidden = 384;
 // Set for the duration of a call that runs out of the built-in arena: the folded form needs room for a
 // gamma-scaled copy of every Linear weight (12 MB at H = 384), which that arena does not have.
 thread_local bool g_no_auto_fold = false;
@@ -1193,7 +1195,7 @@ bool uses_fold_ln(const rlx_encoder_config_t& c, int B, int S) {
     if (!can) return false;
     if (c.flags & RLX_FLAG_FOLD_LN) return true;
     const bool other_fusion = (c.flags & (RLX_FLAG_FUSED_LN | RLX_FLAG_CLUSTER_LN)) != 0;
-    return !g_no_auto_fold && !(c.flags & RLX_FLAG_NO_AUTO_FOLD) && !other_fusion && call_tokens(B, S) <= kAutoFoldMaxTokens;
+    return !g_no_auto_fold && !(c.flags & RLX_FLAG_NO_AUTO_FOLD) && !other_fusion && call_tokens(B, S) <= (c.hidden <= kNarrowHidden ? kAutoFoldMaxTokensNarrow : kAutoFoldMaxTokens);
 }
 
 // The folded weights of the first two layers come from a launch of their own, which the chain reaches before those of all are done
@@ -1231,11 +1233,13 @@ bool uses_attention_fwd(const rlx_encoder_config_t& c, int B, int S) {
 //   6 x 384    1 x 32 128 / 107, 1 x 128 142 / 119 and 150 / 126 (half and all of the positions valid), 4 x 128 160 / 125,
 //              16 x 64 155 / 145, 32 x 128 212 / 186 and 262 / 267, 256 x 16 276 / 227, 64 x 128 297 / 283, 128 x 64 296 / 304,
 //              96 x 128 374 / 387, 200 x 128 625 / 673
-//   12 x 768   1 x 128 386 / 349, 7 x 120 458 / 408 and 572 / 493, 32 x 128 745 / 706 and 1085 / 1073, 64 x 128 1107 / 1147
-constexpr long long kQkvAttentionMaxTokens = 4096;
+//   12 x 768   1 x 128 386 / 349, 7 x 120 458 / 408 and 572 / 493, 32 x 128 745 / 706 and 1085 / 1073, 48 x 128 889 / 924
+// With the LayerNorms folded, 6 x 384: 34 x 128 212 / 188 and 267 / 265, 48 x 128 257 / 247 and 305 / 311, 96 x 64 258 / 254, but 64 x 128 287 / 273
+// and 389 / 399, 128 x 64 289 / 294.
+constexpr long long kQkvAttentionMaxTokens = 4096, kQkvAttentionMaxTokensNarrow = 6144;
 bool uses_qkv_attention(const rlx_encoder_config_t& c, int B, int S) {
     if (c.flags & (RLX_FLAG_GEMM_SIMT | RLX_FLAG_KERNEL_EVENTS | RLX_FLAG_NO_PACK | RLX_FLAG_ATTN_TCGEN05)) return false;
-    return S <= rlx::kBinRows && B <= rlx::kPackEmbedMaxSeqs && call_tokens(B, S) <= kQkvAttentionMaxTokens && !uses_fused_ffn(c, B, S) && !uses_attention_fwd(c, B, S);
+    return S <= rlx::kBinRows && B <= rlx::kPackEmbedMaxSeqs && call_tokens(B, S) <= (c.hidden <= kNarrowHidden ? kQkvAttentionMaxTokensNarrow : kQkvAttentionMaxTokens) && !uses_fused_ffn(c, B, S) && !uses_attention_fwd(c, B, S);
 }
 
 // Packing and embedding in one kernel, in front of the above (us apart / in one: 6 x 384 1 x 32 106.5 / 102.6, 1 x 128 118.6 / 113.9,
@@ -1258,6 +1262,7 @@ bool uses_attention_out(const rlx_encoder_config_t& c, int B, int S) {
 
 struct GraphEntry {
     int B, S;
+    bool fold;
     const void *ids, *mask, *out, *ws;
     cudaGraphExec_t exec;
 };
@@ -1660,6 +1665,20 @@ rlx_status_t enqueue_forward_tp(const rlx_encoder* e, const int32_t* ids, const 
     return RLX_OK;
 }
 
+// Between kAutoFoldMaxTokens and the narrow models' line a workspace without room for the folded weights is as good: the call then
+// keeps the LayerNorm kernels.
+struct FoldIfItFits {
+    bool set = false;
+    FoldIfItFits(const rlx_encoder* e, int B, int S, size_t ws_bytes) {
+        if (!e || B <= 0 || S <= 0 || B > e->cfg.max_batch || S > e->cfg.max_seq || (long long)B * S <= kAutoFoldMaxTokens ||
+            (e->cfg.flags & RLX_FLAG_FOLD_LN) || g_no_auto_fold || !uses_fold_ln(e->cfg, B, S))
+            return;
+        set = ws_bytes < plan_arena(B, S, e->cfg.hidden, e->cfg.ffn, e->cfg.num_layers, true).total;
+        if (set) g_no_auto_fold = true;
+    }
+    ~FoldIfItFits() { if (set) g_no_auto_fold = false; }
+};
+
 rlx_status_t check_forward_args(const rlx_encoder* e, const void* ids, const void* mask, int B, int S,
                                 const rlx_encoder_weights_t* w, const void* out, const void* ws, size_t ws_bytes,
                                 bool host_io) {
@@ -1713,8 +1732,9 @@ rlx_status_t forward_device(rlx_encoder* e, const int32_t* ids, const int32_t* m
         e->weights.layers = e->layers.data();
         e->have_weights = true;
     }
+    const bool fold = uses_fold_ln(e->cfg, B, S);
     for (const auto& g : e->graphs)
-        if (g.B == B && g.S == S && g.ids == ids && g.mask == mask && g.out == out && g.ws == ws) {
+        if (g.B == B && g.S == S && g.fold == fold && g.ids == ids && g.mask == mask && g.out == out && g.ws == ws) {
             RLX_CUDA_TRY(cudaGraphLaunch(g.exec, st));
             return RLX_OK;
         }
@@ -1744,7 +1764,7 @@ rlx_status_t forward_device(rlx_encoder* e, const int32_t* ids, const int32_t* m
         cudaGraphExecDestroy(e->graphs.front().exec);
         e->graphs.erase(e->graphs.begin());
     }
-    e->graphs.push_back(GraphEntry{B, S, ids, mask, out, ws, exec});
+    e->graphs.push_back(GraphEntry{B, S, fold, ids, mask, out, ws, exec});
     RLX_CUDA_TRY(cudaGraphLaunch(exec, st));
     return RLX_OK;
 }
@@ -1807,6 +1827,7 @@ int32_t rlx_encoder_launches_per_forward(const rlx_encoder_t* e, int32_t batch, 
 
 rlx_status_t rlx_encoder_forward(rlx_encoder_t* e, const int32_t* ids, const int32_t* mask, int32_t B, int32_t S,
                                  const rlx_encoder_weights_t* w, float* out, void* ws, size_t ws_bytes, void* stream) {
+    FoldIfItFits fits(e, B, S, ws_bytes);
     rlx_status_t s = check_forward_args(e, ids, mask, B, S, w, out, ws, ws_bytes, false);
     if (s != RLX_OK) return s;
     return forward_device(e, ids, mask, B, S, w, out, static_cast<unsigned char*>(ws), static_cast<cudaStream_t>(stream));
@@ -1816,6 +1837,7 @@ rlx_status_t rlx_encoder_forward_tp(rlx_encoder_t* e, const int32_t* ids, const 
                                     const rlx_encoder_weights_t* w_shard, int32_t tp_rank, int32_t tp_size,
                                     rlx_allreduce_bf16_fn allreduce, void* allreduce_user, float* out, void* ws,
                                     size_t ws_bytes, void* stream) {
+    FoldIfItFits fits(e, B, S, ws_bytes);
     rlx_status_t s = check_forward_args(e, ids, mask, B, S, w_shard, out, ws, ws_bytes, false);
     if (s != RLX_OK) return s;
     if (!allreduce || tp_size < 1 || tp_rank < 0 || tp_rank >= tp_size) return RLX_ERR_INVALID_ARG;
@@ -1835,6 +1857,7 @@ rlx_status_t rlx_encoder_forward_tp(rlx_encoder_t* e, const int32_t* ids, const 
 rlx_status_t rlx_encoder_forward_host(rlx_encoder_t* e, const int32_t* ids_h, const int32_t* mask_h, int32_t B,
                                       int32_t S, const rlx_encoder_weights_t* w, float* out_h, void* ws,
                                       size_t ws_bytes, void* stream) {
+    FoldIfItFits fits(e, B, S, ws_bytes);
     rlx_status_t s = check_forward_args(e, ids_h, mask_h, B, S, w, out_h, ws, ws_bytes, true);
     if (s != RLX_OK) return s;
     cudaStream_t st = static_cast<cudaStream_t>(stream);

@@ -272,7 +272,8 @@ def test_folded_forward_splits_its_long_contraction(rlx, name, B, S, full):
     ("c1", 1, 1, "full"), ("c1", 1, 128, "full"), ("c1", 1, 16, "ragged"), ("c1", 5, 33, "ragged"),
     ("c1", 12, 128, "full"), ("c1", 13, 128, "ragged"),                    # one head per CTA, two
     ("c1", 40, 3, "ragged"), ("c1", 200, 17, "one"),                       # bins that are full by their number of sequences
-    ("c1", 32, 128, "ragged"), ("c1", 32, 128, "full"), ("c1", 31, 130, "ragged"), ("c1", 33, 125, "ragged"),   # the last sizes that take it, the first that do not
+    ("c1", 32, 128, "ragged"), ("c1", 33, 125, "ragged"), ("c1", 48, 128, "ragged"), ("c1", 48, 128, "full"), ("c1", 31, 130, "ragged"),
+    ("c1", 49, 126, "ragged"),                                             # the last sizes that take it, the first that do not
     ("c4", 1, 128, "full"), ("c4", 7, 120, "ragged"), ("c4", 9, 64, "holes"), ("c4", 64, 31, "ragged"), ("c4", 32, 128, "ragged")])
 @pytest.mark.parametrize("flags", [0, 0x400])   # LayerNorm folded into the product, and a kernel of its own
 def test_projection_and_attention_in_one_kernel_give_the_bits_of_two(rlx, name, B, S, lengths, flags):
@@ -319,6 +320,33 @@ def test_packed_rows_choose_the_tile_width_and_not_the_result(rlx, B, S, lo):
     assert status == 0 and pstatus == 0 and np.array_equal(packed, padded)
     pick = [0, B - 1]
     check(packed[pick], oracle.encoder_forward(inp.cfg, inp.ids[pick], inp.mask[pick], inp.params, inp.layers), inp.lengths[pick])
+
+
+@pytest.mark.parametrize("B,S,folds", [(64, 128, True), (61, 203, True), (98, 128, True), (99, 128, False), (33, 125, True)])
+def test_folding_line_of_the_narrow_models_and_workspaces_without_room_for_it(rlx, B, S, folds):
+    """Hidden 384 folds the LayerNorms up to 12544 positions; beyond 4096 a workspace sized for the separate LayerNorms still
+    does, and gives their bits, on an encoder that has replayed the folded form for the same buffers too."""
+    lengths = np.linspace(1, S, B).astype(int)
+    inp = make_inputs(CONFIGS["c1"], batch=B, seq=S, num_layers=2, lengths=lengths, ln_affine_random=True)
+    c = inp.cfg
+    w = rlx.upload_weights(inp.params, inp.layers)
+    enc = rlx.Encoder.from_config(c, max_batch=B, max_seq=S)
+    apart = rlx.Encoder.from_config(c, max_batch=B, max_seq=S, flags=0x400)
+    assert (enc.kernels_per_forward(B, S) == 3 + 5 * 2) == folds
+    n = apart.workspace_bytes(B, S)
+    assert (enc.workspace_bytes(B, S) > n) == folds
+    ids, mask, ws = i32_dev(inp.ids), i32_dev(inp.mask), enc.alloc_workspace(B, S)
+    out = torch.empty((B, c.hidden), dtype=torch.float32, device="cuda")
+    got = [to_np64(e.forward(ids, mask, w, out, space)) for e, space in ((enc, ws), (enc, ws[:n]), (apart, ws), (enc, ws))]
+    assert enc.last_device_status(ws) == 0
+    with pytest.raises(rlx.RlxError):
+        enc.forward(ids, mask, w, out, ws[:n - 256])
+    assert np.array_equal(got[1], got[2]) and np.array_equal(got[0], got[3])
+    pick = [0, B // 2, B - 1]
+    ref = oracle.encoder_forward(c, inp.ids[pick], inp.mask[pick], inp.params, inp.layers)
+    check(got[0][pick], ref, inp.lengths[pick])
+    check(got[1][pick], ref, inp.lengths[pick])
+    enc.close(); apart.close()
 
 
 @pytest.mark.parametrize("heads", [2, 4])
