@@ -1442,10 +1442,13 @@ rlx_status_t enqueue_forward(const rlx_encoder* e, const int32_t* ids, const int
             forked = true;
         }
         const int first_folds = std::min(a.fold_layer <= kFoldSplitLayerBytes ? 2 : c.num_layers, c.num_layers);
+        int fold_launches = 0;
         auto flush_jobs = [&]() -> rlx_status_t {
             if (fl.n == 0) return RLX_OK;
             const int total_rows = fl.first_row[fl.n];
-            rlx::ln_fold_weights_kernel<<<(total_rows + rlx::kFoldWarps - 1) / rlx::kFoldWarps, rlx::kFoldWarps * 32, 0, fold_st>>>(fl);
+            const int per_block = (fold_launches == 0 ? 2 : 4) * rlx::kFoldWarps, blocks = (total_rows + per_block - 1) / per_block;
+            if (fold_launches++ == 0) rlx::ln_fold_weights_kernel<2><<<blocks, rlx::kFoldWarps * 32, 0, fold_st>>>(fl);
+            else rlx::ln_fold_weights_kernel<4><<<blocks, rlx::kFoldWarps * 32, 0, fold_st>>>(fl);
             RLX_CUDA_TRY(cudaGetLastError());
             fl.n = 0;
             fl.first_row[0] = 0;

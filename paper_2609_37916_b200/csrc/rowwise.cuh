@@ -578,7 +578,13 @@ pool_l2norm_kernel(const __nv_bfloat16* __restrict__ x, const int32_t* __restric
 // d_n = sum_k beta_k W_nk + b_n: the GEMM that consumes a LayerNorm output can run on the RAW
 // activation y with gamma-scaled weights and fix the result up per row in its epilogue.  This kernel
 // prepares W' = bf16(gamma o W) (c is summed over the ROUNDED W', so the identity holds exactly for the
-// weights the tensor cores see), c and d for a list of matrices in one launch: one warp per output row.
+// weights the tensor cores see), c and d for a list of matrices in one launch: R consecutive rows of one
+// matrix per warp (the row counts, 3 H and F, are multiples of 64).  Bound by memory latency beside the forward's first kernels:
+// with one row per warp gamma and beta (fp32, two bytes of them per byte of weight) were loaded again for every row and a
+// lane had one load of the weights in flight.  Whole forwards, us, one row / two: 12 x 768 with 7 x 120 404.2 / 395.8, 1 x 128 339.0 / 330.5,
+// 16 x 128 516.7 / 509.7; 6 x 384 with 32 x 128 181.0 / 178.8, 61 x 203 414.0 / 409.3, 1 x 32 93.1 / 93.7.
+// The launch that the chain waits for first takes two rows, one that follows it four: 1 x 32 92.4, 1 x 128 111.8 -> 111.3, 32 x 128 178.5
+// (one row and four: 92.6, 111.0, 179.5 and 61 x 203 411.8 in place of 408.6).
 constexpr int kFoldMaxJobs = 24;
 constexpr int kFoldWarps = 8;
 struct FoldList {
@@ -594,10 +600,11 @@ struct FoldList {
     int K;                              // row length (the LayerNorm width), K % 256 == 0 not required: K % 8 == 0
 };
 
+template <int R>
 __global__ void __launch_bounds__(kFoldWarps * 32)
 ln_fold_weights_kernel(const __grid_constant__ FoldList fl) {
     const int lane = threadIdx.x & 31;
-    const int row = blockIdx.x * kFoldWarps + (threadIdx.x >> 5);
+    const int row = R * (blockIdx.x * kFoldWarps + (threadIdx.x >> 5));
     if (row >= fl.first_row[fl.n]) return;
     int j = 0;
     while (row >= fl.first_row[j + 1]) ++j;
@@ -605,28 +612,36 @@ ln_fold_weights_kernel(const __grid_constant__ FoldList fl) {
     const int K = fl.K;
     const __nv_bfloat16* wr = fl.w[j] + (size_t)n * K;
     __nv_bfloat16* wo = fl.wf[j] + (size_t)n * K;
-    float cs = 0.f, ds = 0.f;
+    float cs[R] = {}, ds[R] = {};
     for (int k = lane * 8; k < K; k += 256) {
-        const uint4 q = __ldg(reinterpret_cast<const uint4*>(wr + k));
+        uint4 q[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) q[r] = __ldcs(reinterpret_cast<const uint4*>(wr + (size_t)r * K + k));
         const float4 g0 = __ldg(reinterpret_cast<const float4*>(fl.gamma[j] + k)), g1 = __ldg(reinterpret_cast<const float4*>(fl.gamma[j] + k) + 1);
         const float4 b0 = __ldg(reinterpret_cast<const float4*>(fl.beta[j] + k)), b1 = __ldg(reinterpret_cast<const float4*>(fl.beta[j] + k) + 1);
-        const float wv[8] = {bf16lo(q.x), bf16hi(q.x), bf16lo(q.y), bf16hi(q.y), bf16lo(q.z), bf16hi(q.z), bf16lo(q.w), bf16hi(q.w)};
         const float gv[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
         const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-        uint32_t o[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            o[i] = pack_bf16(wv[2 * i] * gv[2 * i], wv[2 * i + 1] * gv[2 * i + 1]);
-            cs += bf16lo(o[i]) + bf16hi(o[i]);
-            ds = fmaf(bv[2 * i], wv[2 * i], fmaf(bv[2 * i + 1], wv[2 * i + 1], ds));
+        for (int r = 0; r < R; ++r) {
+            const float wv[8] = {bf16lo(q[r].x), bf16hi(q[r].x), bf16lo(q[r].y), bf16hi(q[r].y), bf16lo(q[r].z), bf16hi(q[r].z), bf16lo(q[r].w), bf16hi(q[r].w)};
+            uint32_t o[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                o[i] = pack_bf16(wv[2 * i] * gv[2 * i], wv[2 * i + 1] * gv[2 * i + 1]);
+                cs[r] += bf16lo(o[i]) + bf16hi(o[i]);
+                ds[r] = fmaf(bv[2 * i], wv[2 * i], fmaf(bv[2 * i + 1], wv[2 * i + 1], ds[r]));
+            }
+            *reinterpret_cast<uint4*>(wo + (size_t)r * K + k) = make_uint4(o[0], o[1], o[2], o[3]);
         }
-        *reinterpret_cast<uint4*>(wo + k) = make_uint4(o[0], o[1], o[2], o[3]);
     }
-    cs = warp_sum(cs);
-    ds = warp_sum(ds);
-    if (lane == 0) {
-        fl.c[j][n] = cs;
-        fl.d[j][n] = ds + __ldg(fl.bias[j] + n);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        cs[r] = warp_sum(cs[r]);
+        ds[r] = warp_sum(ds[r]);
+        if (lane == 0) {
+            fl.c[j][n + r] = cs[r];
+            fl.d[j][n + r] = ds[r] + __ldg(fl.bias[j] + n + r);
+        }
     }
 }
 

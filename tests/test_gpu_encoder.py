@@ -1,5 +1,6 @@
 """End-to-end parity of the CUDA encoder forward (through the C ABI) with the fp64 oracle on the
 five benchmark configurations, plus stress variants, edge cases and bitwise properties."""
+import dataclasses
 import os
 
 import numpy as np
@@ -266,6 +267,22 @@ def test_folded_forward_splits_its_long_contraction(rlx, name, B, S, full):
     check(got, ref, inp.lengths)
     again, _ = run_gpu(rlx, inp, weights=w)
     assert np.array_equal(got, again)
+
+
+@pytest.mark.parametrize("name,hidden,ffn,heads,layers", [("c1", 128, 64, 4, 3), ("c1", 384, 1536, 12, 4), ("c1", 640, 192, 10, 2), ("c4", 768, 3072, 12, 1),
+                                                          ("c1", 1024, 64, 16, 3), ("c1", 128, 64, 4, 16), ("c4", 768, 3072, 12, 13)])
+def test_folded_weights_by_launch(rlx, name, hidden, ffn, heads, layers):
+    """The folded weights of one launch and of two and three (the first two layers', 24 matrices at a time), where a row is less than one
+    pass of a warp, a pass and a part, and whole passes; on the side branch of the graph and in front of the eager launches."""
+    cfg = dataclasses.replace(CONFIGS[name], hidden=hidden, ffn=ffn, num_heads=heads, num_layers=layers)
+    inp = make_inputs(cfg, batch=3, seq=40, num_layers=layers, lengths=np.array([40, 1, 23]), ln_affine_random=True)
+    ref = oracle.encoder_forward(inp.cfg, inp.ids, inp.mask, inp.params, inp.layers)
+    w = rlx.upload_weights(inp.params, inp.layers)
+    got, status = run_gpu(rlx, inp, weights=w)
+    assert status == 0
+    check(got, ref, inp.lengths)
+    eager, _ = run_gpu(rlx, inp, weights=w, flags=1)
+    assert np.array_equal(got, eager)
 
 
 @pytest.mark.parametrize("name,B,S,lengths", [
