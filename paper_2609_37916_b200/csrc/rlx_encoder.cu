@@ -1200,7 +1200,7 @@ bool uses_fold_ln(const rlx_encoder_config_t& c, int B, int S) {
 
 // The folded weights of the first two layers come from a launch of their own, which the chain reaches before those of all are done
 // (6 x 384: 1 x 32 94.5 -> 92.3 us, 1 x 128 114.3 -> 111.6, 16 x 128 153.4 -> 149.9, 16 x 64 138.1 -> 139.4, 32 x 128 the same).  At hidden 768
-// the 200 MB of the fold keep the memory busy far beyond that and the split gains nothing (7 x 120 404.6 / 406.2).
+// the 200 MB of the fold keep the memory busy far beyond that and the split gains nothing (7 x 120 395.2 / 396.9, 1 x 128 330.2 / 329.5, 16 x 128 508.4 / 509.9).
 constexpr size_t kFoldSplitLayerBytes = (size_t)4 << 20;
 int kernels_in_forward(const rlx_encoder_config_t& c, int B, int S) {
     const bool pack = !(c.flags & RLX_FLAG_NO_PACK) && !(c.flags & RLX_FLAG_GEMM_SIMT);
