@@ -75,9 +75,8 @@ typedef enum {
                                    not a multiple of 32 or max_seq exceeds 512; takes precedence over
                                    RLX_FLAG_FUSED_LN / RLX_FLAG_CLUSTER_LN.  Pays for small batches (launch-bound
                                    forwards); for large ones the separate LayerNorm kernels are faster.  Chosen
-                                   AUTOMATICALLY for calls with batch*seq <= 4096 (12544 at hidden <= 384) unless
-                                   one of the other two fusion flags or RLX_FLAG_NO_AUTO_FOLD is set; beyond 4096 a
-                                   workspace without room for the folded weights keeps the LayerNorm kernels */
+                                   AUTOMATICALLY for calls with batch*seq <= 4096 unless one of the other two
+                                   fusion flags or RLX_FLAG_NO_AUTO_FOLD is set */
 #define RLX_FLAG_NO_AUTO_FOLD 0x400u /* keep the 7-kernel layer (separate LayerNorm kernels) at every batch size */
 #define RLX_FLAG_FUSED_FFN 0x1000u /* everything of a layer behind the attention in ONE kernel (rlx_layer_tail_bf16:
                                       out-projection + residual + LayerNorm, FFN-up, GELU, FFN-down + residual +

@@ -1182,11 +1182,10 @@ bool uses_cluster_ln(const rlx_encoder_config_t& c) {
 //              96 x 128 372 / 376 and 526 / 527, 61 x 203 396 / 402 and 595 / 591, 255 x 128 749 / 736 and 1364 / 1286
 //   12 x 768   1 x 128 387 / 450 and 406 / 459, 7 x 120 457 / 502 and 572 / 559, 32 x 128 740 / 732 and 1094 / 1042,
 //              64 x 128 1224 / 1134 and 2065 / 1833
-// With the width of the long contraction's tiles chosen on the device, and projection and attention in one kernel:
-//   6 x 384    64 x 128 288 / 302 and 389 / 397, 22 x 256 275 / 289, 16 x 512 336 / 345, 90 x 128 358 / 364, 61 x 203 415 / 424 and 599 / 597
-//   12 x 768   16 x 128 513 / 513, 32 x 128 717 / 714
-// The wider model's weights are four times as many to fold.  The narrower one's line lies in front of 12800 tokens.
-constexpr int kAutoFoldMaxTokens = 4096, kAutoFoldMaxTokensNarrow = 12544, kNarrowHidden = 384;
+// One line for both widths.  Between 4096 and 12383 tokens the narrower one would gain up to 5 % (64 x 128 288 / 302 and 389 / 397, 61 x 203
+// 415 / 424 and 599 / 597, but 97 x 128 with every position valid 541 / 518), and pays for it: gamma W is rounded to bf16 where W is used
+// as it is, the workspace grows, and RLX_FLAG_FUSED_FFN / _DEVICE_CHOICE, which promise their forms there, would lose them.
+constexpr int kAutoFoldMaxTokens = 4096;
 // Set for the duration of a call that runs out of the built-in arena: the folded form needs room for a
 // gamma-scaled copy of every Linear weight (12 MB at H = 384), which that arena does not have.
 thread_local bool g_no_auto_fold = false;
@@ -1195,7 +1194,7 @@ bool uses_fold_ln(const rlx_encoder_config_t& c, int B, int S) {
     if (!can) return false;
     if (c.flags & RLX_FLAG_FOLD_LN) return true;
     const bool other_fusion = (c.flags & (RLX_FLAG_FUSED_LN | RLX_FLAG_CLUSTER_LN)) != 0;
-    return !g_no_auto_fold && !(c.flags & RLX_FLAG_NO_AUTO_FOLD) && !other_fusion && call_tokens(B, S) <= (c.hidden <= kNarrowHidden ? kAutoFoldMaxTokensNarrow : kAutoFoldMaxTokens);
+    return !g_no_auto_fold && !(c.flags & RLX_FLAG_NO_AUTO_FOLD) && !other_fusion && call_tokens(B, S) <= kAutoFoldMaxTokens;
 }
 
 // The folded weights of the first two layers come from a launch of their own, which the chain reaches before those of all are done
@@ -1237,6 +1236,7 @@ bool uses_attention_fwd(const rlx_encoder_config_t& c, int B, int S) {
 // With the LayerNorms folded, 6 x 384: 34 x 128 212 / 188 and 267 / 265, 48 x 128 257 / 247 and 305 / 311, 96 x 64 258 / 254, but 64 x 128 287 / 273
 // and 389 / 399, 128 x 64 289 / 294.
 constexpr long long kQkvAttentionMaxTokens = 4096, kQkvAttentionMaxTokensNarrow = 6144;
+constexpr int kNarrowHidden = 384;
 bool uses_qkv_attention(const rlx_encoder_config_t& c, int B, int S) {
     if (c.flags & (RLX_FLAG_GEMM_SIMT | RLX_FLAG_KERNEL_EVENTS | RLX_FLAG_NO_PACK | RLX_FLAG_ATTN_TCGEN05)) return false;
     return S <= rlx::kBinRows && B <= rlx::kPackEmbedMaxSeqs && call_tokens(B, S) <= (c.hidden <= kNarrowHidden ? kQkvAttentionMaxTokensNarrow : kQkvAttentionMaxTokens) && !uses_fused_ffn(c, B, S) && !uses_attention_fwd(c, B, S);
@@ -1262,7 +1262,6 @@ bool uses_attention_out(const rlx_encoder_config_t& c, int B, int S) {
 
 struct GraphEntry {
     int B, S;
-    bool fold;
     const void *ids, *mask, *out, *ws;
     cudaGraphExec_t exec;
 };
@@ -1668,20 +1667,6 @@ rlx_status_t enqueue_forward_tp(const rlx_encoder* e, const int32_t* ids, const 
     return RLX_OK;
 }
 
-// Between kAutoFoldMaxTokens and the narrow models' line a workspace without room for the folded weights is as good: the call then
-// keeps the LayerNorm kernels.
-struct FoldIfItFits {
-    bool set = false;
-    FoldIfItFits(const rlx_encoder* e, int B, int S, size_t ws_bytes) {
-        if (!e || B <= 0 || S <= 0 || B > e->cfg.max_batch || S > e->cfg.max_seq || (long long)B * S <= kAutoFoldMaxTokens ||
-            (e->cfg.flags & RLX_FLAG_FOLD_LN) || g_no_auto_fold || !uses_fold_ln(e->cfg, B, S))
-            return;
-        set = ws_bytes < plan_arena(B, S, e->cfg.hidden, e->cfg.ffn, e->cfg.num_layers, true).total;
-        if (set) g_no_auto_fold = true;
-    }
-    ~FoldIfItFits() { if (set) g_no_auto_fold = false; }
-};
-
 rlx_status_t check_forward_args(const rlx_encoder* e, const void* ids, const void* mask, int B, int S,
                                 const rlx_encoder_weights_t* w, const void* out, const void* ws, size_t ws_bytes,
                                 bool host_io) {
@@ -1735,9 +1720,8 @@ rlx_status_t forward_device(rlx_encoder* e, const int32_t* ids, const int32_t* m
         e->weights.layers = e->layers.data();
         e->have_weights = true;
     }
-    const bool fold = uses_fold_ln(e->cfg, B, S);
     for (const auto& g : e->graphs)
-        if (g.B == B && g.S == S && g.fold == fold && g.ids == ids && g.mask == mask && g.out == out && g.ws == ws) {
+        if (g.B == B && g.S == S && g.ids == ids && g.mask == mask && g.out == out && g.ws == ws) {
             RLX_CUDA_TRY(cudaGraphLaunch(g.exec, st));
             return RLX_OK;
         }
@@ -1767,7 +1751,7 @@ rlx_status_t forward_device(rlx_encoder* e, const int32_t* ids, const int32_t* m
         cudaGraphExecDestroy(e->graphs.front().exec);
         e->graphs.erase(e->graphs.begin());
     }
-    e->graphs.push_back(GraphEntry{B, S, fold, ids, mask, out, ws, exec});
+    e->graphs.push_back(GraphEntry{B, S, ids, mask, out, ws, exec});
     RLX_CUDA_TRY(cudaGraphLaunch(exec, st));
     return RLX_OK;
 }
@@ -1830,7 +1814,6 @@ int32_t rlx_encoder_launches_per_forward(const rlx_encoder_t* e, int32_t batch, 
 
 rlx_status_t rlx_encoder_forward(rlx_encoder_t* e, const int32_t* ids, const int32_t* mask, int32_t B, int32_t S,
                                  const rlx_encoder_weights_t* w, float* out, void* ws, size_t ws_bytes, void* stream) {
-    FoldIfItFits fits(e, B, S, ws_bytes);
     rlx_status_t s = check_forward_args(e, ids, mask, B, S, w, out, ws, ws_bytes, false);
     if (s != RLX_OK) return s;
     return forward_device(e, ids, mask, B, S, w, out, static_cast<unsigned char*>(ws), static_cast<cudaStream_t>(stream));
@@ -1840,7 +1823,6 @@ rlx_status_t rlx_encoder_forward_tp(rlx_encoder_t* e, const int32_t* ids, const 
                                     const rlx_encoder_weights_t* w_shard, int32_t tp_rank, int32_t tp_size,
                                     rlx_allreduce_bf16_fn allreduce, void* allreduce_user, float* out, void* ws,
                                     size_t ws_bytes, void* stream) {
-    FoldIfItFits fits(e, B, S, ws_bytes);
     rlx_status_t s = check_forward_args(e, ids, mask, B, S, w_shard, out, ws, ws_bytes, false);
     if (s != RLX_OK) return s;
     if (!allreduce || tp_size < 1 || tp_rank < 0 || tp_rank >= tp_size) return RLX_ERR_INVALID_ARG;
@@ -1860,7 +1842,6 @@ rlx_status_t rlx_encoder_forward_tp(rlx_encoder_t* e, const int32_t* ids, const 
 rlx_status_t rlx_encoder_forward_host(rlx_encoder_t* e, const int32_t* ids_h, const int32_t* mask_h, int32_t B,
                                       int32_t S, const rlx_encoder_weights_t* w, float* out_h, void* ws,
                                       size_t ws_bytes, void* stream) {
-    FoldIfItFits fits(e, B, S, ws_bytes);
     rlx_status_t s = check_forward_args(e, ids_h, mask_h, B, S, w, out_h, ws, ws_bytes, true);
     if (s != RLX_OK) return s;
     cudaStream_t st = static_cast<cudaStream_t>(stream);

@@ -86,6 +86,20 @@ def test_kernel_count_follows_the_layernorm_fusion_flags(lib):
     big.close()
 
 
+@pytest.mark.parametrize("hidden,heads", [(128, 4), (256, 8), (384, 12), (768, 12)])
+def test_folding_line_is_one_for_all_widths(lib, hidden, heads):
+    """At most 4096 positions by itself; beyond, the layer and the workspace of the separate LayerNorms, or the layer tail asked for."""
+    shape = dict(hidden=hidden, num_heads=heads, ffn=4 * hidden, max_batch=256, max_seq=256)
+    enc, apart, tail = (binding.Encoder(**_cfg(**shape, flags=f)) for f in (0, binding.FLAG_NO_AUTO_FOLD, binding.FLAG_FUSED_FFN))
+    assert enc.kernels_per_forward(32, 128) == 3 + 5 * 6 and enc.workspace_bytes(32, 128) > apart.workspace_bytes(32, 128)
+    for batch, seq in ((33, 125), (48, 128), (61, 203), (96, 128), (98, 128)):
+        assert enc.kernels_per_forward(batch, seq) == 3 + 7 * 6
+        assert enc.workspace_bytes(batch, seq) == apart.workspace_bytes(batch, seq)
+        assert tail.kernels_per_forward(batch, seq) == 3 + (3 if hidden in (256, 384) else 7) * 6
+    for e in (enc, apart, tail):
+        e.close()
+
+
 def test_create_rejects_wrong_struct_size_and_null(lib):
     cfg = binding._Config(4, 6, 384, 12, 1536, 30522, 512, 2, 1e-12, 32, 128, 0, 0)
     h = C.c_void_p()

@@ -339,31 +339,27 @@ def test_packed_rows_choose_the_tile_width_and_not_the_result(rlx, B, S, lo):
     check(packed[pick], oracle.encoder_forward(inp.cfg, inp.ids[pick], inp.mask[pick], inp.params, inp.layers), inp.lengths[pick])
 
 
-@pytest.mark.parametrize("B,S,folds", [(64, 128, True), (61, 203, True), (98, 128, True), (99, 128, False), (33, 125, True)])
-def test_folding_line_of_the_narrow_models_and_workspaces_without_room_for_it(rlx, B, S, folds):
-    """Hidden 384 folds the LayerNorms up to 12544 positions; beyond 4096 a workspace sized for the separate LayerNorms still
-    does, and gives their bits, on an encoder that has replayed the folded form for the same buffers too."""
-    lengths = np.linspace(1, S, B).astype(int)
-    inp = make_inputs(CONFIGS["c1"], batch=B, seq=S, num_layers=2, lengths=lengths, ln_affine_random=True)
+@pytest.mark.parametrize("B,S", [(33, 125), (61, 203), (96, 128), (98, 128)])
+def test_calls_beyond_the_folding_line_keep_what_was_promised_for_them(rlx, B, S):
+    """Beyond 4096 positions: the bits of the separate LayerNorms, in a workspace sized for them, timed by kernel in the count that
+    is announced; the layer tail where RLX_FLAG_FUSED_FFN asks for it, and from 12288 positions on where the device chooses it."""
+    inp = make_inputs(CONFIGS["c1"], batch=B, seq=S, num_layers=2, lengths=np.full(B, S), ln_affine_random=True)
     c = inp.cfg
     w = rlx.upload_weights(inp.params, inp.layers)
-    enc = rlx.Encoder.from_config(c, max_batch=B, max_seq=S)
-    apart = rlx.Encoder.from_config(c, max_batch=B, max_seq=S, flags=0x400)
-    assert (enc.kernels_per_forward(B, S) == 3 + 5 * 2) == folds
-    n = apart.workspace_bytes(B, S)
-    assert (enc.workspace_bytes(B, S) > n) == folds
-    ids, mask, ws = i32_dev(inp.ids), i32_dev(inp.mask), enc.alloc_workspace(B, S)
+    apart, _ = run_gpu(rlx, inp, weights=w, flags=0x400)
+    got, status = run_gpu(rlx, inp, weights=w)
+    assert status == 0 and np.array_equal(got, apart)
+    with_tail, _ = run_gpu(rlx, inp, weights=w, flags=0x1400)
+    asked, _ = run_gpu(rlx, inp, weights=w, flags=0x1000)
+    assert np.array_equal(asked, with_tail) and not np.array_equal(asked, got)
+    chosen, _ = run_gpu(rlx, inp, weights=w, flags=0x4000)
+    assert np.array_equal(chosen, with_tail if B * S >= 12288 else apart)
+    plain, timed = (rlx.Encoder.from_config(c, max_batch=B, max_seq=S, flags=f) for f in (0x400, 4))
+    ids, mask, ws = i32_dev(inp.ids), i32_dev(inp.mask), plain.alloc_workspace(B, S)
     out = torch.empty((B, c.hidden), dtype=torch.float32, device="cuda")
-    got = [to_np64(e.forward(ids, mask, w, out, space)) for e, space in ((enc, ws), (enc, ws[:n]), (apart, ws), (enc, ws))]
-    assert enc.last_device_status(ws) == 0
-    with pytest.raises(rlx.RlxError):
-        enc.forward(ids, mask, w, out, ws[:n - 256])
-    assert np.array_equal(got[1], got[2]) and np.array_equal(got[0], got[3])
-    pick = [0, B // 2, B - 1]
-    ref = oracle.encoder_forward(c, inp.ids[pick], inp.mask[pick], inp.params, inp.layers)
-    check(got[0][pick], ref, inp.lengths[pick])
-    check(got[1][pick], ref, inp.lengths[pick])
-    enc.close(); apart.close()
+    assert np.array_equal(to_np64(timed.forward(ids, mask, w, out, ws)), got)
+    assert len(timed.kernel_times(B, S)) == 3 + 7 * 2
+    plain.close(); timed.close()
 
 
 @pytest.mark.parametrize("heads", [2, 4])
