@@ -143,6 +143,7 @@ cudaError_t set_gemm_attr_all() {
 int g_max_pairs[64] = {};
 int g_max_pairs_resident[64] = {};   // the same for the A-resident kernel (its own shared-memory footprint)
 int g_max_split2[64] = {}, g_max_split4[64] = {};   // clusters of two and four of the split-K kernel
+int g_max_out_heads[64] = {};   // heads that go on to the attention output as one cluster (a CTA each); 0: none
 
 // Multiprocessor count of the current device (grids of the persistent kernels are sized from it).
 constexpr int kNominalSMs = 148;   // B200; used only when no device can be queried (host-only callers)
@@ -285,6 +286,29 @@ cudaError_t init_kernels_for_current_device() {
     RLX_QA_ATTR(32, 1, 0, false) RLX_QA_ATTR(32, 1, 3, false) RLX_QA_ATTR(32, 2, 0, false) RLX_QA_ATTR(32, 2, 3, false)
     RLX_QA_ATTR(64, 1, 0, false) RLX_QA_ATTR(64, 1, 3, false) RLX_QA_ATTR(32, 1, 0, true) RLX_QA_ATTR(32, 1, 3, true)
 #undef RLX_QA_ATTR
+    // clusters of 4, 8 and 12 heads (hidden 128, 256 and 384): a partition of the device may not have an SM group of that size
+    for (int heads = 4; heads <= rlx::tcqa::kMaxOutHeads; heads += 4) {
+        using C = rlx::tcqa::Cfg<32, 1, true>;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(heads);
+        cfg.blockDim = dim3(C::THREADS);
+        cfg.dynamicSmemBytes = C::SMEM_BYTES;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = heads;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int n[2] = {0, 0};
+        if (cudaOccupancyMaxActiveClusters(&n[0], rlx::tcqa::qkv_attention_kernel<32, 1, 0, true>, &cfg) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&n[1], rlx::tcqa::qkv_attention_kernel<32, 1, 3, true>, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            break;
+        }
+        if (n[0] < 1 || n[1] < 1) break;
+        if (dev < 64) g_max_out_heads[dev] = heads;
+    }
 #define RLX_ATT_FWD_ATTR(D, PAIR)                                                                              \
     if ((e = cudaFuncSetAttribute(rlx::tcat::attention_fwd_kernel<D, PAIR, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
                                   rlx::tcat::Cfg<D, PAIR>::SMEM_BYTES)) != cudaSuccess ||                       \
@@ -1256,8 +1280,9 @@ bool uses_pack_embed(const rlx_encoder_config_t& c, int B, int S) {
 // and all of the positions valid; 1 x 128 113.9 / 112.9 and 126 / 135, 3 x 64 114.8 / 119).
 constexpr int kMaxOutTokens = 64, kMaxOutBins = 2;
 bool uses_attention_out(const rlx_encoder_config_t& c, int B, int S) {
-    return uses_qkv_attention(c, B, S) && uses_fold_ln(c, B, S) && c.hidden / c.num_heads == 32 && c.num_heads <= rlx::tcqa::kMaxOutHeads &&
-           B * S <= kMaxOutTokens && max_bins(B, S) <= kMaxOutBins;
+    const int max_heads = c.device < 64 ? g_max_out_heads[c.device] : 0;   // that a cluster can have on this device
+    return uses_qkv_attention(c, B, S) && uses_fold_ln(c, B, S) && c.hidden / c.num_heads == 32 && c.num_heads <= max_heads &&
+           (long long)B * S <= kMaxOutTokens && max_bins(B, S) <= kMaxOutBins;
 }
 
 struct GraphEntry {
@@ -1807,6 +1832,8 @@ int32_t rlx_encoder_kernels_per_forward(const rlx_encoder_t* e, int32_t batch, i
 
 int32_t rlx_encoder_launches_per_forward(const rlx_encoder_t* e, int32_t batch, int32_t seq) {
     if (!e || batch <= 0 || seq <= 0) return 0;
+    int dev = -1;   // what its clusters can hold decides on the smallest calls
+    if (cudaGetDevice(&dev) != cudaSuccess || (dev == e->cfg.device && init_kernels_for_current_device() != cudaSuccess)) (void)cudaGetLastError();
     return kernels_in_forward(e->cfg, batch, seq) -
            e->cfg.num_layers * ((int)uses_qkv_attention(e->cfg, batch, seq) + (int)uses_attention_out(e->cfg, batch, seq)) -
            (int)uses_pack_embed(e->cfg, batch, seq);

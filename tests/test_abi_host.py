@@ -100,6 +100,15 @@ def test_folding_line_is_one_for_all_widths(lib, hidden, heads):
         e.close()
 
 
+@pytest.mark.skipif(torch.cuda.is_available(), reason="the device at hand can hold clusters of twelve")
+@pytest.mark.parametrize("hidden", [128, 256, 384])
+def test_heads_go_on_to_the_attention_output_only_where_a_cluster_of_them_fits(lib, hidden):
+    """No device that says that it can hold the cluster, no cluster: a tiny call counts the kernels of a short one."""
+    enc = binding.Encoder(**_cfg(hidden=hidden, num_heads=hidden // 32, ffn=4 * hidden))
+    assert enc.launches_per_forward(1, 32) == enc.launches_per_forward(1, 128) < enc.kernels_per_forward(1, 128)
+    enc.close()
+
+
 def test_create_rejects_wrong_struct_size_and_null(lib):
     cfg = binding._Config(4, 6, 384, 12, 1536, 30522, 512, 2, 1e-12, 32, 128, 0, 0)
     h = C.c_void_p()

@@ -319,11 +319,14 @@ def test_attention_output_of_tiny_calls_gives_the_bits_of_its_own_kernel(rlx, B,
     """Up to 64 positions a cluster of the heads goes on to the attention output; the instrumented forward keeps every step apart."""
     inp = make_inputs(CONFIGS["c1"], batch=B, seq=S, num_layers=3, lengths=lengths, ln_affine_random=True)
     w = rlx.upload_weights(inp.params, inp.layers)
-    one, status = run_gpu(rlx, inp, weights=w)
+    enc = rlx.Encoder.from_config(inp.cfg, max_batch=B, max_seq=S)
+    assert enc.launches_per_forward(B, S) == enc.launches_per_forward(1, 1) + (3 if B * S > 64 else 0)   # a kernel less per layer, asked before any forward
+    one, status = run_gpu(rlx, inp, weights=w, enc=enc)
     apart, astatus = run_gpu(rlx, inp, weights=w, flags=4)
     eager, estatus = run_gpu(rlx, inp, weights=w, flags=1)
     assert status == 0 and astatus == 0 and estatus == 0
     assert np.array_equal(one, apart) and np.array_equal(one, eager)
+    enc.close()
 
 
 @pytest.mark.parametrize("B,S,lo", [(61, 203, 40), (61, 203, 203), (40, 150, 20)])
