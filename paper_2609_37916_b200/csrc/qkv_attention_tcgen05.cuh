@@ -363,8 +363,9 @@ qkv_attention_kernel(const __grid_constant__ RowMaps tmap_a, const __grid_consta
             ok = mbar_wait_warp(acc_bar, 0, abort_flag);   // the ring is free
         }
         if constexpr (OUT) {
-            // this CTA's ring is free: its peers may send context rows
-            if (ok && rows > 0 && e == 0 && lane < (int)gridDim.x) mbar_arrive_cluster_release_cta(map_to_cta(free_bar, lane));
+            // this CTA's ring is free: its peers may send context rows.  They write where this CTA's products have read, so the
+            // release reaches them: cluster scope.  The warp has no store to global memory outstanding that it would wait for.
+            if (ok && rows > 0 && e == 0 && lane < (int)gridDim.x) mbar_arrive_cluster(map_to_cta(free_bar, lane));
             __syncwarp();
         }
         asm volatile("bar.sync 1, %0;" ::"n"(32 * C::WARPS) : "memory");

@@ -329,6 +329,28 @@ def test_attention_output_of_tiny_calls_gives_the_bits_of_its_own_kernel(rlx, B,
     enc.close()
 
 
+def test_tiny_calls_one_behind_the_other_hand_their_context_over_each_time(rlx):
+    """The heads' CTAs write into each other's operand ring once its owner has read it: hundreds of calls back to back on changing
+    inputs, sequences of one row to four groups of 16, every result that of the separate kernels."""
+    rng = np.random.default_rng(11)
+    base = make_inputs(CONFIGS["c1"], batch=2, seq=32, num_layers=3, lengths=[32, 32], ln_affine_random=True)
+    w = rlx.upload_weights(base.params, base.layers)
+    enc, apart = (rlx.Encoder.from_config(base.cfg, max_batch=2, max_seq=32, flags=f) for f in (0, 4))
+    ws, ws_apart = enc.alloc_workspace(2, 32), apart.alloc_workspace(2, 32)
+    ids, mask = torch.empty(2, 32, dtype=torch.int32, device="cuda"), torch.empty(2, 32, dtype=torch.int32, device="cuda")
+    out = torch.empty((2, base.cfg.hidden), dtype=torch.float32, device="cuda")
+    inputs = [(i32_dev(rng.integers(0, base.cfg.vocab, size=(2, 32))),
+               i32_dev(np.arange(32)[None, :] < np.array([[1 + i % 32], [(7 * i) % 33]]))) for i in range(40)]
+    want = [apart.forward(a, m, w, torch.empty_like(out), ws_apart) for a, m in inputs]
+    got = []
+    for i in range(400):
+        ids.copy_(inputs[i % 40][0]); mask.copy_(inputs[i % 40][1])
+        got.append(enc.forward(ids, mask, w, out, ws).clone())
+    assert enc.last_device_status(ws) == 0 and apart.last_device_status(ws_apart) == 0
+    assert all(torch.equal(g, want[i % 40]) for i, g in enumerate(got))
+    enc.close(); apart.close()
+
+
 @pytest.mark.parametrize("B,S,lo", [(61, 203, 40), (61, 203, 203), (40, 150, 20)])
 def test_packed_rows_choose_the_tile_width_and_not_the_result(rlx, B, S, lo):
     """The packed and the padded layout (RLX_FLAG_NO_PACK) hand the feed-forward down product other row counts: other widths."""
