@@ -1230,6 +1230,21 @@ int kernels_in_forward(const rlx_encoder_config_t& c, int B, int S) {
     const bool fused = uses_fold_ln(c, B, S) || uses_fused_ln(c, B, S) || uses_cluster_ln(c);
     return 2 + ((fused ? 5 : 7) - (uses_fused_ffn(c, B, S) ? 4 : 0)) * c.num_layers + (pack ? 1 : 0);
 }
+// Launches of ln_fold_weights_kernel: the matrices of the first layers, kFoldMaxJobs at a time, then those of the rest.
+int first_folded_layers(const rlx_encoder_config_t& c, size_t fold_layer_bytes) {
+    return std::min(fold_layer_bytes <= kFoldSplitLayerBytes ? 2 : c.num_layers, c.num_layers);
+}
+int fold_launches_in_forward(const rlx_encoder_config_t& c) {
+    const int first = first_folded_layers(c, plan_arena(1, 1, c.hidden, c.ffn, c.num_layers, true).fold_layer), per = rlx::kFoldMaxJobs;
+    const int jobs = 2 * c.num_layers - 1, first_jobs = 2 * first - 1;   // W1 of every layer, Wqkv of all but the first
+    return (first_jobs + per - 1) / per + (jobs - first_jobs + per - 1) / per;
+}
+// Captured forwards bring the Linear weights into L2 on a side branch when they all fit; a fold pass reads them anyway.
+size_t linear_layer_bytes(const rlx_encoder_config_t& c) { return ((size_t)4 * c.hidden * c.hidden + (size_t)2 * c.hidden * c.ffn) * sizeof(bf16); }
+bool prefetches_weights(const rlx_encoder_config_t& c, bool fold) {
+    return !(c.flags & (RLX_FLAG_NO_PREFETCH | RLX_FLAG_NO_GRAPH)) && !fold && linear_layer_bytes(c) * c.num_layers <= ((size_t)48 << 20) &&
+           4 * c.num_layers <= rlx::kMaxPrefetch;
+}
 bool uses_chunks(const rlx_encoder_config_t& c, int B, int S);
 int chunk_batch(int B, int S);
 
@@ -1362,29 +1377,26 @@ rlx_status_t enqueue_forward(const rlx_encoder* e, const int32_t* ids, const int
     PdlScope pdl_scope(!(c.flags & RLX_FLAG_NO_PDL) && !timing);
     // side branch (captured graphs only): prefetch the Linear weights into L2 when they all fit
     bool forked = false;
-    if (capturing && !body_only && e->side_stream && !(c.flags & RLX_FLAG_NO_PREFETCH) && !fold) {   // the fold pass reads the weights anyway
-        const size_t per_layer = ((size_t)3 * H * H + (size_t)H * H + (size_t)2 * H * F) * sizeof(bf16);
-        if (per_layer * c.num_layers <= ((size_t)48 << 20) && 4 * c.num_layers <= rlx::kMaxPrefetch) {
-            rlx::PrefetchList pf = {};
-            for (int l = 0; l < c.num_layers; ++l) {
-                const rlx_layer_weights_t& lw = w->layers[l];
-                const void* ptrs[4] = {lw.wqkv, lw.wo, lw.w1, lw.w2};
-                const size_t bytes[4] = {(size_t)3 * H * H * 2, (size_t)H * H * 2, (size_t)F * H * 2, (size_t)H * F * 2};
-                for (int i = 0; i < 4; ++i) {
-                    pf.ptr[pf.n] = ptrs[i];
-                    pf.bytes[pf.n] = (uint32_t)bytes[i];
-                    pf.first_piece[pf.n] = pf.total_pieces;
-                    pf.total_pieces += (uint32_t)((bytes[i] + rlx::kPrefetchPiece - 1) / rlx::kPrefetchPiece);
-                    ++pf.n;
-                }
+    if (capturing && !body_only && e->side_stream && prefetches_weights(c, fold)) {
+        rlx::PrefetchList pf = {};
+        for (int l = 0; l < c.num_layers; ++l) {
+            const rlx_layer_weights_t& lw = w->layers[l];
+            const void* ptrs[4] = {lw.wqkv, lw.wo, lw.w1, lw.w2};
+            const size_t bytes[4] = {(size_t)3 * H * H * 2, (size_t)H * H * 2, (size_t)F * H * 2, (size_t)H * F * 2};
+            for (int i = 0; i < 4; ++i) {
+                pf.ptr[pf.n] = ptrs[i];
+                pf.bytes[pf.n] = (uint32_t)bytes[i];
+                pf.first_piece[pf.n] = pf.total_pieces;
+                pf.total_pieces += (uint32_t)((bytes[i] + rlx::kPrefetchPiece - 1) / rlx::kPrefetchPiece);
+                ++pf.n;
             }
-            RLX_CUDA_TRY(cudaEventRecord(e->fork_event, st));
-            RLX_CUDA_TRY(cudaStreamWaitEvent(e->side_stream, e->fork_event, 0));
-            rlx::prefetch_l2_kernel<<<sm_count(), 32, 0, e->side_stream>>>(pf);
-            RLX_CUDA_TRY(cudaGetLastError());
-            RLX_CUDA_TRY(cudaEventRecord(e->join_event, e->side_stream));
-            forked = true;
         }
+        RLX_CUDA_TRY(cudaEventRecord(e->fork_event, st));
+        RLX_CUDA_TRY(cudaStreamWaitEvent(e->side_stream, e->fork_event, 0));
+        rlx::prefetch_l2_kernel<<<sm_count(), 32, 0, e->side_stream>>>(pf);
+        RLX_CUDA_TRY(cudaGetLastError());
+        RLX_CUDA_TRY(cudaEventRecord(e->join_event, e->side_stream));
+        forked = true;
     }
     Packing pk;
     const bool fuse_qa = pack && uses_qkv_attention(c, B, S), fuse_out = fuse_qa && uses_attention_out(c, B, S);
@@ -1465,7 +1477,7 @@ rlx_status_t enqueue_forward(const rlx_encoder* e, const int32_t* ids, const int
             RLX_CUDA_TRY(cudaStreamWaitEvent(e->side_stream, e->fork_event, 0));
             forked = true;
         }
-        const int first_folds = std::min(a.fold_layer <= kFoldSplitLayerBytes ? 2 : c.num_layers, c.num_layers);
+        const int first_folds = first_folded_layers(c, a.fold_layer);
         int fold_launches = 0;
         auto flush_jobs = [&]() -> rlx_status_t {
             if (fl.n == 0) return RLX_OK;
@@ -1834,9 +1846,12 @@ int32_t rlx_encoder_launches_per_forward(const rlx_encoder_t* e, int32_t batch, 
     if (!e || batch <= 0 || seq <= 0) return 0;
     int dev = -1;   // what its clusters can hold decides on the smallest calls
     if (cudaGetDevice(&dev) != cudaSuccess || (dev == e->cfg.device && init_kernels_for_current_device() != cudaSuccess)) (void)cudaGetLastError();
-    return kernels_in_forward(e->cfg, batch, seq) -
-           e->cfg.num_layers * ((int)uses_qkv_attention(e->cfg, batch, seq) + (int)uses_attention_out(e->cfg, batch, seq)) -
-           (int)uses_pack_embed(e->cfg, batch, seq);
+    const rlx_encoder_config_t& c = e->cfg;
+    const bool fold = uses_fold_ln(c, batch, seq);
+    const int sub = uses_chunks(c, batch, seq) ? chunk_batch(batch, seq) : batch;   // sequences of a sub-batch
+    return (batch + sub - 1) / sub *
+           (kernels_in_forward(c, batch, seq) - c.num_layers * ((int)uses_qkv_attention(c, batch, seq) + (int)uses_attention_out(c, batch, seq)) -
+            (int)uses_pack_embed(c, batch, seq) + (fold ? fold_launches_in_forward(c) : 0) + (int)prefetches_weights(c, fold));
 }
 
 rlx_status_t rlx_encoder_forward(rlx_encoder_t* e, const int32_t* ids, const int32_t* mask, int32_t B, int32_t S,

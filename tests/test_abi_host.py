@@ -109,6 +109,29 @@ def test_heads_go_on_to_the_attention_output_only_where_a_cluster_of_them_fits(l
     enc.close()
 
 
+def test_launches_count_the_side_branch_and_every_sub_batch(lib):
+    """The folded weights (one launch per 24 matrices, those of the first two layers of a narrow model in one of their own), the weight
+    prefetch of a captured forward that folds nothing, the sub-batches of a chunked call."""
+    def launches(batch, seq, **kw):
+        enc = binding.Encoder(**_cfg(max_batch=256, max_seq=256, **kw))
+        n = enc.launches_per_forward(batch, seq)
+        enc.close()
+        return n
+    base = dict(hidden=768, num_heads=12, ffn=3072, num_layers=12)
+    assert launches(32, 128) == 2 + 4 * 6 + 2                       # packing + embedding in one, QKV + attention in one
+    assert launches(32, 128, num_layers=16) == 2 + 4 * 16 + 3       # 31 matrices: 3, 24 and 4
+    assert launches(32, 128, num_layers=1) == 2 + 4 + 1
+    assert launches(16, 128, **base) == 2 + 4 * 12 + 1              # 23 matrices in one
+    assert launches(16, 128, **dict(base, num_layers=13)) == 2 + 4 * 13 + 2
+    assert launches(16, 200) == 3 + 5 * 6 + 2
+    assert launches(16, 200, flags=binding.FLAG_KERNEL_EVENTS) == launches(16, 200)
+    assert launches(64, 256, flags=binding.FLAG_NO_FUSED_FFN) == 3 + 7 * 6 + 1          # weight prefetch
+    assert launches(64, 256, flags=binding.FLAG_NO_FUSED_FFN | binding.FLAG_NO_GRAPH) == 3 + 7 * 6
+    assert launches(64, 256, **base) == 3 + 7 * 12                  # too large for L2
+    assert launches(64, 256, num_layers=12) == launches(64, 256, num_layers=12, flags=binding.FLAG_NO_PREFETCH) + 1
+    assert launches(100, 256, flags=binding.FLAG_CHUNKED | binding.FLAG_NO_FUSED_FFN) == 2 * (3 + 7 * 6 + 1)
+
+
 def test_create_rejects_wrong_struct_size_and_null(lib):
     cfg = binding._Config(4, 6, 384, 12, 1536, 30522, 512, 2, 1e-12, 32, 128, 0, 0)
     h = C.c_void_p()

@@ -329,6 +329,33 @@ def test_attention_output_of_tiny_calls_gives_the_bits_of_its_own_kernel(rlx, B,
     enc.close()
 
 
+@pytest.mark.parametrize("name,B,S", [("c1", 1, 32), ("c1", 3, 22), ("c1", 7, 128), ("c1", 10, 200), ("c1", 50, 100), ("c1", 130, 256),
+                                      ("c4", 1, 128), ("c4", 9, 64)])
+def test_launches_per_forward_are_the_kernels_of_a_recorded_one(rlx, name, B, S):
+    """The kernel nodes of a forward that the caller records (RLX_FLAG_NO_GRAPH: kernel by kernel into the caller's graph)."""
+    from cuda.bindings import runtime as rt
+    cfg = dataclasses.replace(CONFIGS[name], num_layers=13 if name == "c4" else 3)
+    inp = make_inputs(cfg, batch=B, seq=S, lengths=np.full(B, S))
+    w = rlx.upload_weights(inp.params, inp.layers)
+    enc = rlx.Encoder.from_config(inp.cfg, max_batch=B, max_seq=S, flags=1)
+    ids, mask, ws = i32_dev(inp.ids), i32_dev(inp.mask), enc.alloc_workspace(B, S)
+    out = torch.empty((B, cfg.hidden), dtype=torch.float32, device="cuda")
+    enc.forward(ids, mask, w, out, ws)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        enc.forward(ids, mask, w, out, ws)
+    def ok(r):
+        assert int(r[0]) == 0, r[0]
+        return r[1:]
+    raw = rt.cudaGraph_t(graph.raw_cuda_graph())
+    n = ok(rt.cudaGraphGetNodes(raw))[1]
+    nodes = ok(rt.cudaGraphGetNodes(raw, n))[0]
+    kernels = sum(ok(rt.cudaGraphNodeGetType(x))[0] == rt.cudaGraphNodeType.cudaGraphNodeTypeKernel for x in nodes)
+    assert kernels == enc.launches_per_forward(B, S)
+    enc.close()
+
+
 def test_tiny_calls_one_behind_the_other_hand_their_context_over_each_time(rlx):
     """The heads' CTAs write into each other's operand ring once its owner has read it: hundreds of calls back to back on changing
     inputs, sequences of one row to four groups of 16, every result that of the separate kernels."""
