@@ -714,25 +714,37 @@ rlx_status_t launch_gemm_tc_bn(const CUtensorMap& ta, const CUtensorMap& tb, con
 
 // CTA pairs whose tile width the kernel chooses from the rows that exist (gemm_pair_tcgen05.cuh): long contractions, columns that
 // every width divides, more tiles of 128 columns than pairs, so that the width decides on the rounds, and few enough rounds that one more
-// or less counts.  Whole forwards, us fixed / chosen: 6 x 384 61 x 203 435 / 422 and 587 / 589 (half and all of the positions valid),
-// 100 x 128 405 / 391, 60 x 256 459 / 443; 12 x 768 32 x 128 712 / 713 and 1068 / 1039, 64 x 128 1106 / 1070.  With fewer tiles the
-// fixed width's smaller code wins (32 x 128 181 / 185).
+// or less counts.  Whole forwards, us fixed / chosen, with the share of the positions that are valid: where another width than the
+// fixed one wins (128 columns up to 73 row blocks at N = 384 and 36 at 768, 192 beyond)
+//   6 x 384    61 x 203 0.6 433 / 420, 64 x 128 0.8 378 / 365 and 1.0 409 / 395, 14 x 512 1.0 481 / 466, 100 x 128 0.6 417 / 405, 60 x 256 0.5 460 / 445,
+//              24 x 512 0.6 479 / 464, 140 x 128 0.5 448 / 434
+//   12 x 768   26 x 128 1.0 1026 / 961, 32 x 128 1.0 1098 / 1050, 48 x 128 0.5 944 / 906, 20 x 512 0.5 1421 / 1353
+// and where it does not, which the host cannot know
+//   6 x 384    64 x 128 0.5 288.6 / 290.9, 14 x 512 0.6 341.4 / 342.7, 24 x 400 0.6 385.9 / 389.2 and 1.0 566.9 / 570.3, 28 x 512 0.25 311.1 / 313.4,
+//              140 x 128 0.25 304.6 / 307.6, 61 x 203 1.0 590 / 591
+//   12 x 768   26 x 128 0.5 681.5 / 683.9 and 0.75 785 / 794, 16 x 256 0.5 748 / 750
+// With fewer tiles the fixed width's smaller code wins (32 x 128 181 / 185).
 bool pair_width_pays(int M, int N, int K, int epi, const TileChoice& tc) {
     int dev = 0;
     cudaGetDevice(&dev);
     const int pairs = (dev >= 0 && dev < 64) ? g_max_pairs[dev] : 0;
-    return tc.cg == 2 && tc.bn <= rlx::tcpw::kMaxBN && (epi <= 2 || epi == 6) && K >= 1536 && K % rlx::tc::BLOCK_K == 0 && N % 384 == 0 &&
+    return pairs > 1 && tc.cg == 2 && tc.bn <= rlx::tcpw::kMaxBN && (epi <= 2 || epi == 6) && K >= 1536 && K % rlx::tc::BLOCK_K == 0 && N % 384 == 0 &&
            (M + 255) / 256 * (N / 128) > pairs && (M + 255) / 256 * (N / 192) < 4 * pairs;
 }
 rlx_status_t launch_gemm_pair(const bf16* A, const bf16* W, const CUtensorMap& to, const rlx::tc::Params& p, int epi, cudaStream_t st) {
     CUtensorMap ta;
-    rlx::tcpw::WidthMaps wm;
+    rlx::tcpw::Widths wm;
     if (!make_tmap_kblocks(&ta, A, p.M, p.K, rlx::tc::BLOCK_M, rlx::tcpw::kKps)) return RLX_ERR_CUDA;
     for (int i = 0; i < 3; ++i)
         if (!make_tmap_kblocks(wm.w + i, W, p.N, p.K, 32 * (i + 1), rlx::tcpw::kKps)) return RLX_ERR_CUDA;
     int dev = 0;
     cudaGetDevice(&dev);
     const int grid = 2 * std::min((p.M + 255) / 256 * (p.N / 64), g_max_pairs[dev]);
+    for (int i = 0; i < 3; ++i) {
+        wm.n_tiles[i] = p.N / (64 * (i + 1));
+        wm.inv[i] = rlx::tcpw::reciprocal((uint32_t)wm.n_tiles[i]);
+    }
+    wm.inv_pairs = rlx::tcpw::reciprocal((uint32_t)grid / 2);
     struct ClusterScope {
         explicit ClusterScope(int x) { g_cluster_x = x; }
         ~ClusterScope() { g_cluster_x = 1; }

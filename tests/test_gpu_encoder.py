@@ -378,14 +378,16 @@ def test_tiny_calls_one_behind_the_other_hand_their_context_over_each_time(rlx):
     enc.close(); apart.close()
 
 
-@pytest.mark.parametrize("B,S,lo", [(61, 203, 40), (61, 203, 203), (40, 150, 20)])
-def test_packed_rows_choose_the_tile_width_and_not_the_result(rlx, B, S, lo):
-    """The packed and the padded layout (RLX_FLAG_NO_PACK) hand the feed-forward down product other row counts: other widths."""
-    lengths = np.linspace(lo, S, B).astype(int)
+@pytest.mark.parametrize("B,S,lo,hi", [(61, 203, 40, 203), (64, 128, 1, 90), (52, 128, 8, 128), (70, 128, 1, 70)])   # 192, 64, 128 and 64 columns
+@pytest.mark.parametrize("flags", [0, 0x200])   # the residual in the epilogue, and normalised there
+def test_packed_rows_choose_the_tile_width_and_not_the_result(rlx, B, S, lo, hi, flags):
+    """The packed and the padded layout (RLX_FLAG_NO_PACK: 128 columns, 192 from the second on) hand the feed-forward down product other row counts: other
+    widths, the same bits."""
+    lengths = np.linspace(lo, hi, B).astype(int)
     inp = make_inputs(CONFIGS["c1"], batch=B, seq=S, num_layers=2, lengths=lengths)
     w = rlx.upload_weights(inp.params, inp.layers)
-    packed, status = run_gpu(rlx, inp, weights=w)
-    padded, pstatus = run_gpu(rlx, inp, weights=w, flags=8)
+    packed, status = run_gpu(rlx, inp, weights=w, flags=flags)
+    padded, pstatus = run_gpu(rlx, inp, weights=w, flags=flags | 8)
     assert status == 0 and pstatus == 0 and np.array_equal(packed, padded)
     pick = [0, B - 1]
     check(packed[pick], oracle.encoder_forward(inp.cfg, inp.ids[pick], inp.mask[pick], inp.params, inp.layers), inp.lengths[pick])
