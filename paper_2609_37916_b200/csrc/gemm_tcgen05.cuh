@@ -718,21 +718,10 @@ struct EpilogueTile {
     }
 };
 
-// Maps of A with boxes of 32, 64 and 96 rows: the 32-row groups that a tile does not have are not loaded.  A row block of
-// A is what a small product waits for behind the previous kernel (W is there by then), 98 KB of it at K = 384.  Only the narrowest
-// tiles have them.
-template <bool SMALL>
-struct RowMaps {};
-template <>
-struct RowMaps<true> {
-    CUtensorMap m[3];
-};
-
 template <int BLOCK_N, int EPI, int CG>
 __global__ void __launch_bounds__((Cfg<BLOCK_N, CG, (EPI >= 3)>::THREADS), 1)
 gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
-                    const __grid_constant__ CUtensorMap tmap_out, const __grid_constant__ RowMaps<Cfg<BLOCK_N, CG>::SMALL> row_maps,
-                    const Params p) {
+                    const __grid_constant__ CUtensorMap tmap_out, const Params p) {
     using C = Cfg<BLOCK_N, CG, (EPI >= 3)>;
     constexpr int TILE_M = BLOCK_M * CG;   // rows of one output tile (per CTA pair when CG = 2)
     extern __shared__ unsigned char smem_raw[];
@@ -790,8 +779,6 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
     const int num_tiles = n_tiles * m_tiles;
     const int num_kb = (p.K + BLOCK_K - 1) / BLOCK_K;
     const int tile0 = blockIdx.x / CG, tile_step = gridDim.x / CG;   // both CTAs of a pair walk the same tiles
-    // 32-row groups of a tile that exist, and so the bytes of its k-blocks of A
-    auto row_groups = [&](int m_blk) { return C::SMALL ? min(4, (M - m_blk * BLOCK_M + 31) / 32) : 4; };
 
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer (whole warp, one lane issues)
@@ -806,20 +793,17 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
                 // 3-D maps: one load per operand brings all KPS k-blocks (a k-block past the end of K arrives as zeros and
                 // still counts its bytes)
                 const bool k3 = p.kblock_maps != 0;
-                const int groups = row_groups(m_blk), a_kb = groups * (C::A_BYTES / 4);
-                const int nbytes = (k3 ? C::KPS : cnt) * (a_kb + C::B_BYTES);
-                [[maybe_unused]] const CUtensorMap* map_a = &tmap_a;
-                if constexpr (C::SMALL) map_a = groups < 4 ? &row_maps.m[groups - 1] : &tmap_a;
+                const int nbytes = k3 ? C::KPS * C::KB_BYTES : cnt * C::KB_BYTES;
                 if (RLX_DBG(p, kDbgNoLoad)) {
                     if (W && cta_rank == 0) mbar_arrive(full_bar + 8 * stage);
                 } else if constexpr (CG == 1) {
                     if (W) mbar_expect_tx(full_bar + 8 * stage, nbytes);
                     if (k3) {
-                        if (A) tma_load_3d(st0, map_a, 0, m_blk * BLOCK_M, kb, full_bar + 8 * stage);
+                        if (A) tma_load_3d(st0, &tmap_a, 0, m_blk * BLOCK_M, kb, full_bar + 8 * stage);
                         if (W) tma_load_3d(sb0, &tmap_b, 0, n_blk * BLOCK_N, kb, full_bar + 8 * stage);
                     } else {
                         for (int i = 0; i < cnt; ++i) {
-                            if (A) tma_load_2d(st0 + i * a_kb, map_a, (kb + i) * BLOCK_K, m_blk * BLOCK_M, full_bar + 8 * stage);
+                            if (A) tma_load_2d(st0 + i * C::A_BYTES, &tmap_a, (kb + i) * BLOCK_K, m_blk * BLOCK_M, full_bar + 8 * stage);
                             if (W) tma_load_2d(sb0 + i * C::B_BYTES, &tmap_b, (kb + i) * BLOCK_K, n_blk * BLOCK_N, full_bar + 8 * stage);
                         }
                     }
@@ -845,7 +829,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
             if constexpr (C::SMALL) {
                 if (tile0 < num_tiles && !p.w_fresh)
                     for (; early < C::STAGES && early * C::KPS < num_kb; ++early) {
-                        if (elect_one()) load(std::integral_constant<int, kPartW>(), tile0 / n_tiles, tile0 % n_tiles, early * C::KPS, early);
+                        if (elect_one()) load(std::integral_constant<int, kPartW>(), 0, tile0 % n_tiles, early * C::KPS, early);
                         __syncwarp();
                     }
             }
@@ -894,7 +878,6 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
                 if (!got_acc) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t tmem_d = tmem_base + as * BLOCK_N;
-                const uint32_t a_kb = C::SMALL ? (uint32_t)row_groups(tile / n_tiles) * (C::A_BYTES / 4 >> 4) : C::A_BYTES >> 4;
                 for (int kb = 0; kb < num_kb; kb += C::KPS) {
                     const int cnt = min(C::KPS, num_kb - kb);
                     bool got_ops;
@@ -919,7 +902,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
 #pragma unroll
                                     for (int k = 0; k < BLOCK_K / UMMA_K; ++k) {
                                         // advancing 16 bf16 = 32 bytes along K inside the swizzle row: +2 in 16-byte units
-                                        umma_bf16<CG>(tmem_d, ad0 + (i * a_kb + 2 * k), bd0 + (i * (C::B_BYTES >> 4) + 2 * k),
+                                        umma_bf16<CG>(tmem_d, ad0 + (i * (C::A_BYTES >> 4) + 2 * k), bd0 + (i * (C::B_BYTES >> 4) + 2 * k),
                                                       idesc, (kb | i | k) != 0 ? 1u : 0u);
                                     }
                                 }

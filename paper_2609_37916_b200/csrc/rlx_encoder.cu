@@ -678,14 +678,8 @@ TileChoice pick_tile(int M, int N, int K, int want_cg = 0) {
 }
 
 template <int BN, int CG>
-rlx_status_t launch_gemm_tc_bn(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& to, const bf16* A,
+rlx_status_t launch_gemm_tc_bn(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& to,
                                const rlx::tc::Params& p, int epi, cudaStream_t st) {
-    rlx::tc::RowMaps<rlx::tc::Cfg<BN, CG>::SMALL> rm;
-    if constexpr (rlx::tc::Cfg<BN, CG>::SMALL)
-        for (int i = 0; i < 3; ++i)
-            if (!(p.kblock_maps ? make_tmap_kblocks(rm.m + i, A, p.M, p.K, 32 * (i + 1), rlx::tc::Cfg<BN, CG>::KPS)
-                                : make_tmap(rm.m + i, A, p.M, p.K, 32 * (i + 1))))
-                return RLX_ERR_CUDA;
     const int tile_m = rlx::tc::BLOCK_M * CG;
     const int tiles = ((p.M + tile_m - 1) / tile_m) * (p.N / BN);
     int dev = 0;
@@ -699,13 +693,13 @@ rlx_status_t launch_gemm_tc_bn(const CUtensorMap& ta, const CUtensorMap& tb, con
         ~ClusterScope() { g_cluster_x = 1; }
     } scope(CG);
     switch (epi) {
-        case 0: RLX_CUDA_TRY(launch_ex(rlx::tc::gemm_tcgen05_kernel<BN, 0, CG>, grid, rlx::tc::Cfg<BN, CG>::THREADS, smem, st, ta, tb, to, rm, p)); break;
-        case 1: RLX_CUDA_TRY(launch_ex(rlx::tc::gemm_tcgen05_kernel<BN, 1, CG>, grid, rlx::tc::Cfg<BN, CG>::THREADS, smem, st, ta, tb, to, rm, p)); break;
-        case 2: RLX_CUDA_TRY(launch_ex(rlx::tc::gemm_tcgen05_kernel<BN, 2, CG>, grid, rlx::tc::Cfg<BN, CG>::THREADS, smem, st, ta, tb, to, rm, p)); break;
-        case 3: RLX_CUDA_TRY(launch_ex(rlx::tc::gemm_tcgen05_kernel<BN, 3, CG>, grid, rlx::tc::Cfg<BN, CG>::THREADS, smem, st, ta, tb, to, rm, p)); break;
-        case 4: RLX_CUDA_TRY(launch_ex(rlx::tc::gemm_tcgen05_kernel<BN, 4, CG>, grid, rlx::tc::Cfg<BN, CG>::THREADS, smem, st, ta, tb, to, rm, p)); break;
-        case 5: RLX_CUDA_TRY(launch_ex(rlx::tc::gemm_tcgen05_kernel<BN, 5, CG>, grid, rlx::tc::Cfg<BN, CG>::THREADS, smem, st, ta, tb, to, rm, p)); break;
-        case 6: RLX_CUDA_TRY(launch_ex(rlx::tc::gemm_tcgen05_kernel<BN, 6, CG>, grid, rlx::tc::Cfg<BN, CG>::THREADS, smem, st, ta, tb, to, rm, p)); break;
+        case 0: RLX_CUDA_TRY(launch_ex(rlx::tc::gemm_tcgen05_kernel<BN, 0, CG>, grid, rlx::tc::Cfg<BN, CG>::THREADS, smem, st, ta, tb, to, p)); break;
+        case 1: RLX_CUDA_TRY(launch_ex(rlx::tc::gemm_tcgen05_kernel<BN, 1, CG>, grid, rlx::tc::Cfg<BN, CG>::THREADS, smem, st, ta, tb, to, p)); break;
+        case 2: RLX_CUDA_TRY(launch_ex(rlx::tc::gemm_tcgen05_kernel<BN, 2, CG>, grid, rlx::tc::Cfg<BN, CG>::THREADS, smem, st, ta, tb, to, p)); break;
+        case 3: RLX_CUDA_TRY(launch_ex(rlx::tc::gemm_tcgen05_kernel<BN, 3, CG>, grid, rlx::tc::Cfg<BN, CG>::THREADS, smem, st, ta, tb, to, p)); break;
+        case 4: RLX_CUDA_TRY(launch_ex(rlx::tc::gemm_tcgen05_kernel<BN, 4, CG>, grid, rlx::tc::Cfg<BN, CG>::THREADS, smem, st, ta, tb, to, p)); break;
+        case 5: RLX_CUDA_TRY(launch_ex(rlx::tc::gemm_tcgen05_kernel<BN, 5, CG>, grid, rlx::tc::Cfg<BN, CG>::THREADS, smem, st, ta, tb, to, p)); break;
+        case 6: RLX_CUDA_TRY(launch_ex(rlx::tc::gemm_tcgen05_kernel<BN, 6, CG>, grid, rlx::tc::Cfg<BN, CG>::THREADS, smem, st, ta, tb, to, p)); break;
         default: return RLX_ERR_INVALID_ARG;
     }
     RLX_CUDA_TRY(cudaGetLastError());
@@ -936,17 +930,17 @@ rlx_status_t launch_gemm(const bf16* A, const bf16* W, const float* bias, const 
     if (p.kblock_maps < 0) return RLX_ERR_CUDA;
     if (tc.cg == 2) {
         switch (bn) {
-            case 128: return launch_gemm_tc_bn<128, 2>(ta, tb, to, A, p, epi, st);
-            case 192: return launch_gemm_tc_bn<192, 2>(ta, tb, to, A, p, epi, st);
-            case 256: return launch_gemm_tc_bn<256, 2>(ta, tb, to, A, p, epi, st);
+            case 128: return launch_gemm_tc_bn<128, 2>(ta, tb, to, p, epi, st);
+            case 192: return launch_gemm_tc_bn<192, 2>(ta, tb, to, p, epi, st);
+            case 256: return launch_gemm_tc_bn<256, 2>(ta, tb, to, p, epi, st);
         }
         return RLX_ERR_UNSUPPORTED;
     }
     switch (bn) {
-        case 64: return launch_gemm_tc_bn<64, 1>(ta, tb, to, A, p, epi, st);
-        case 128: return launch_gemm_tc_bn<128, 1>(ta, tb, to, A, p, epi, st);
-        case 192: return launch_gemm_tc_bn<192, 1>(ta, tb, to, A, p, epi, st);
-        case 256: return launch_gemm_tc_bn<256, 1>(ta, tb, to, A, p, epi, st);
+        case 64: return launch_gemm_tc_bn<64, 1>(ta, tb, to, p, epi, st);
+        case 128: return launch_gemm_tc_bn<128, 1>(ta, tb, to, p, epi, st);
+        case 192: return launch_gemm_tc_bn<192, 1>(ta, tb, to, p, epi, st);
+        case 256: return launch_gemm_tc_bn<256, 1>(ta, tb, to, p, epi, st);
     }
     return RLX_ERR_UNSUPPORTED;
 }

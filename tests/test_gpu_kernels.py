@@ -185,8 +185,8 @@ def test_gemm_matches_oracle_linear(rlx, shape, epi, impl):
 
 @pytest.mark.parametrize("M", [1, 31, 32, 33, 64, 65, 96, 97, 129, 160, 225])
 @pytest.mark.parametrize("N,K", [(64, 64), (192, 384), (128, 200), (64, 1600)])   # k-blocks in pairs, an odd number of them, part of one
-def test_narrow_tiles_load_the_row_groups_that_exist(rlx, M, N, K):
-    """One to four 32-row groups in the last row block; small integers, so that a row or a k-block out of place is a wrong integer."""
+def test_narrow_tiles_at_the_edges_of_their_row_blocks(rlx, M, N, K):
+    """One row to a whole row block in the last one; small integers, so that a row or a k-block out of place is a wrong integer."""
     rng = np.random.default_rng(M + N + K)
     a, w = rng.integers(-1, 2, size=(M, K)).astype(np.float32), rng.integers(-1, 2, size=(N, K)).astype(np.float32)
     bias = rng.integers(-8, 9, size=N).astype(np.float32)
