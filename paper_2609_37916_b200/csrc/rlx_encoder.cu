@@ -507,11 +507,19 @@ rlx_status_t launch_attention_fwd(const bf16* qkv, int rows, const int32_t* seq_
                                   const float* rope_sin, bf16* ctx, int32_t* status, cudaStream_t st) {
     namespace tcat = rlx::tcat;
     // Rotated heads of 64 that see many keys go by two row tiles of one head instead of one of two heads: a K block is loaded and
-    // rotated once for both, where a pair of heads has it rotated for every 128 rows.  The tiles' first and last blocks are
-    // one's only, which costs more than that under a short window (us pair / rows, 16 x 1000..4000, 8 heads: causal 271 / 237, window 768
-    // 149 / 137, 512 121 / 115, 384 110 / 105, 256 96.0 / 95.5; 23 x 100..1500, 16 heads: 512 102.4 / 101.1, 128 71.7 / 78.0; causal 64 x
-    // 30..300 49.6 / 53.4, 100..400 43.2 / 43.2, 32 x 200..600 42.5 / 40.6; heads of 32 the same either way).
-    const bool by_rows = rope_cos != nullptr && d == 64 && positional && std::min(window, max_len) >= 3 * tcat::kTile;
+    // rotated once for both, where a pair of heads has it rotated for every 128 rows.  The tiles' first and last blocks are one's
+    // only and an odd tile has no partner, so it takes long sequences, most of them, and a window that shows much of them.  us pair /
+    // rows, about 28000 rows of 8 heads, sequences from 0.3 of the longest on and all of that length:
+    //   causal      400 41.0 / 43.9 and 61.7 / 57.5, 600 45.8 / 49.9 and 70.0 / 69.8, 768 52.4 / 51.3 and 69.8 / 65.6, 1000 57.6 / 56.2 and 93.2 / 85.0,
+    //               1500 67.6 / 69.5 and 108 / 91.4, 2000 86.2 / 78.1 and 146 / 130, 3000 109 / 94.4 and 188 / 159
+    //   window 768  1000 57.6 / 55.9 and 91.5 / 84.7, 1500 59.3 / 62.0 and 93.5 / 81.3, 3000 68.5 / 63.7 and 106 / 97.0
+    //   window 512  1000 54.0 / 53.4 and 84.1 / 78.6, 1300 51.6 / 55.5 and 83.4 / 85.8, 2000 57.5 / 56.9 and 90.4 / 89.8, 3000 57.6 / 54.1 and 87.2 / 82.0
+    //   window 384  1500 49.3 / 51.7 and 74.3 / 68.6, 2000 51.6 / 53.0 and 82.0 / 81.2 (3000 51.5 / 49.6 and 77.4 / 73.6)
+    // Short sequences among them, from 0.06 on: 400 33.5 / 39.0, 512 35.6 / 43.2, 768 41.2 / 41.2, 1500 59.6 / 54.6.  Of 168 calls on this side of the
+    // line with windows from 768 on ten lose more than 2 % (3 x 540..900, 16 heads: 22.7 / 24.8); the mean is 5 % faster.
+    const int span = std::min(window, max_len);
+    const bool by_rows = rope_cos != nullptr && d == 64 && positional && rows >= 3ll * tcat::kTile * B &&
+                         (span >= 6 * tcat::kTile || (span >= 4 * tcat::kTile && max_len >= 2000));
     const bool pair = d <= 64 && kv_group == 1 && h % 2 == 0 && !by_rows;
     const bool rows_mode = !pair && kv_group % 2 != 0;
     tcat::Params p = {};

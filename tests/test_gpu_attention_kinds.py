@@ -335,11 +335,13 @@ def test_kernel_choice_at_its_edges(rlx, d, hq, hkv, n, length, kind, window):
     assert torch.equal(inside, rlx.attention_kind_bf16(turned, *args, kind, window, num_kv_heads=hkv))
 
 
-@pytest.mark.parametrize("lengths", [[383, 130, 1], [384, 257, 256, 255], [1000, 1, 129, 640, 383]])
-@pytest.mark.parametrize("kind,window", [(CAUSAL, 0), (SLIDING, 383), (SLIDING, 384), (SLIDING, 385), (SLIDING, 900)])
+@pytest.mark.parametrize("lengths", [[383, 130, 1], [384, 257, 256, 255], [1000, 1, 129, 640, 383], [767, 700, 130], [768, 129, 256], [1999, 640, 1],
+                                     [2000, 383, 1], [2001] + [1] * 5])
+@pytest.mark.parametrize("kind,window", [(CAUSAL, 0), (SLIDING, 383), (SLIDING, 511), (SLIDING, 512), (SLIDING, 767), (SLIDING, 768), (SLIDING, 900)])
 def test_rotated_heads_of_64_by_row_tiles_or_by_pairs_of_heads(rlx, lengths, kind, window):
-    """Rotated inside, heads of 64 go by two row tiles of a head where a row sees 384 keys or more; rotated in front, by two heads.  Both
-    sides of that line, second tiles that are empty, partial and full, rows of NaN behind the last sequence: the same bits."""
+    """Rotated inside, heads of 64 go by two row tiles of a head where a row sees 768 keys or more, or 512 of a sequence of 2000, and
+    sequences have 384 rows on average; rotated in front, by two heads.  Both sides of those lines, second tiles that are empty,
+    partial and full, rows of NaN behind the last sequence: the same bits."""
     h, d, total = 4, 64, sum(lengths)
     rng = np.random.default_rng(total + window)
     qkv = rand_bf16(rng, (total + 3, 3 * h * d))
