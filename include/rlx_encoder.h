@@ -291,9 +291,9 @@ rlx_status_t rlx_encoder_forward_static(rlx_encoder_t *encoder, const int32_t *t
 rlx_status_t rlx_encoder_last_device_status(rlx_encoder_t *encoder, void *workspace, void *cuda_stream);
 
 /* Number of kernels of one forward of (batch, seq), the steps of its layers counted apart: the entries of
- * rlx_encoder_kernel_times.  A forward of at most 4096 positions (6144 at hidden <= 384) in sequences of at
- * most 128 runs a layer's QKV GEMM and attention as one kernel, the smallest ones more than that, unless
- * RLX_FLAG_KERNEL_EVENTS, _NO_PACK or _ATTN_TCGEN05 is set (bit for bit the same result);
+ * rlx_encoder_kernel_times.  A forward of a few thousand positions in sequences of at most 128 runs a layer's QKV GEMM
+ * and attention as one kernel, the smallest ones more than that, unless RLX_FLAG_KERNEL_EVENTS, _NO_PACK or
+ * _ATTN_TCGEN05 is set (bit for bit the same result).
  * rlx_encoder_launches_per_forward counts the kernels that one rlx_encoder_forward launches, those of the side
  * branch among them (folded weights, weight prefetch); with RLX_FLAG_DEVICE_CHOICE, of the form that the host would
  * choose.  rlx_encoder_forward_host from pinned buffers of more than 256 positions launches one more where packing and
