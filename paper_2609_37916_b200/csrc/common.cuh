@@ -62,11 +62,12 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// The tables of pack_sequences_kernel (lengths, starts, row count) may be read BEFORE pdl_wait by every kernel of a forward
-// from the third on: the embedding kernel, the second, allows its dependents only behind its own wait, so by the time
-// any later kernel starts, the packing kernel has completed.  The same holds for everything in front of the embedding
-// kernel in stream order (weights, and in eager forwards the folded weights; a captured forward joins the
-// folded weights with a full dependency).  An L2 round trip per kernel leaves the chain of dependent launches.
+// The tables of the packing (lengths, starts, row count, bins) may be read BEFORE pdl_wait by every kernel of a forward but the one
+// right behind it.  Packing and embedding apart: the embedding kernel, the second, allows its dependents only behind its own
+// wait, so by the time any later kernel starts, the packing kernel has completed.  Both in one (pack_embed_ln_kernel): the QKV +
+// attention kernel behind it does the same (AttParams::first).  The same holds for everything in front of that kernel in stream
+// order (weights, and in eager forwards the folded weights; a captured forward joins the folded weights with a full
+// dependency).  An L2 round trip per kernel leaves the chain of dependent launches.
 // Read past L1: a line of the previous forward's table could still sit there.
 __device__ __forceinline__ int ld_early(const int32_t* p) {
     int v;

@@ -193,7 +193,9 @@ gemm_mx_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
         uint32_t ph = 0, tcount = 0, ss = 0, sph = 0;
         // A group of four k-blocks' scale words goes to tensor memory at once, and a group ahead of its products where the words are
         // there: copies and products run in the order they are issued, and a product right behind the copy that it needs waits for
-        // all of that copy's latency (product alone, 36736 x 384 x 1536 23.0 -> 21.4 us, 20000 rows 18.8 -> 16.8).
+        // all of that copy's latency (product alone, 36736 x 384 x 1536 23.0 -> 21.4 us, 20000 rows 18.8 -> 16.8).  That order is also
+        // all that keeps a copy into a slot behind the products of the group before last, which read it: `sempty` frees the words
+        // in shared memory, once they are copied.
         auto copy_group = [&](uint32_t slot) {
 #pragma unroll
             for (int u = 0; u < ST; ++u)
