@@ -1282,25 +1282,43 @@ bool uses_attention_fwd(const rlx_encoder_config_t& c, int B, int S) {
 // QKV projection and attention in one kernel: no sequence longer than a bin, and few enough bins that they run beside each other (a
 // CTA does not overlap one bin's attention with the next one's products, as the separate kernels do): a round is 24 bins of two heads
 // of 32 or 12 of a head of 64.  A sequence of more than 64 positions has a bin for itself once the others are as long; how many
-// positions are valid only the device knows.  Whole forwards, us separate / in one, sequences from a quarter, a half and three quarters of the
-// longest on, and all that long:
-//   6 x 384    12 x 128 186 / 142, 193 / 147, 202 / 156 and 202 / 158, 24 x 128 199 / 168, 212 / 179, 229 / 196 and 237 / 202, 30 x 128 223 / 204, 230 / 226, 254 / 245 and
-//              256 / 250, 40 x 72 185 / 166, 199 / 177, 213 / 207 and 223 / 229, 40 x 96 214 / 211, 222 / 221, 243 / 243 and 248 / 250, 40 x 128 (a half, all) 276 / 276 and
-//              298 / 295; 44 x 128 281 / 281 and 303 / 304, 48 x 128 (all) 310 / 316, 50 x 72 196 / 186, 217 / 221, 238 / 239 and 253 / 272
-//              72 x 64 (a half, all) 268 / 262 and 279 / 269, 96 x 48 268 / 262 and 285 / 283; 104 x 48 279 / 270 and 304 / 307, 96 x 64 (all) 316 / 322
-//              144 x 32 279 / 261 and 290 / 274, 192 x 32 307 / 297 and 332 / 323
-//   12 x 768   12 x 128 500 / 457, 553 / 477, 603 / 530 and 616 / 544, 14 x 128 565 / 509, 571 / 594, 667 / 657 and 694 / 677, 16 x 128 568 / 588, 579 / 609, 702 / 684 and
-//              707 / 686, 20 x 128 645 / 644, 671 / 693, 716 / 698 and 774 / 752, 22 x 128 658 / 670, 699 / 699, 773 / 758 and 800 / 790 (from a sixteenth on
-//              14 x 128 558 / 498, 18 x 128 588 / 523, 20 x 128 613 / 602); 24 x 128 666 / 682, 714 / 709, 798 / 790 and 829 / 829, 32 x 128 (a half, all) 823 / 856 and
-//              1030 / 1048
-//              40 x 64 640 / 635, 666 / 671, 710 / 685 and 767 / 737, 60 x 48 689 / 671, 731 / 702, 794 / 783 and 832 / 844; 70 x 48 732 / 709, 751 / 747, 795 / 829 and
-//              970 / 980, 64 x 64 (a half, all) 785 / 846 and 1027 / 1050
-//              64 x 32 596 / 541, 606 / 595, 730 / 663 and 736 / 669, 128 x 32 (a half, all) 860 / 825 and 1103 / 1045
+// positions are valid only the device knows.  Whole forwards, us separate / in one, by the shortest sequence as a share of the longest:
+//                          1/4          1/2          3/4          1
+//   6 x 384   12 x 128   186 / 142    193 / 147    202 / 156    202 / 158
+//             24 x 128   199 / 168    212 / 179    229 / 196    237 / 202
+//             30 x 128   223 / 204    230 / 226    254 / 245    256 / 250
+//             40 x 72    185 / 166    199 / 177    213 / 207    223 / 229
+//             40 x 96    214 / 211    222 / 221    243 / 243    248 / 250
+//             33 x 125   248 / 247    263 / 262    276 / 272    281 / 278     LayerNorms apart from here on
+//             36 x 128   254 / 254    271 / 270    278 / 279    282 / 281
+//             72 x 64                 268 / 262                 279 / 269
+//             96 x 48                 268 / 262                 285 / 283
+//             192 x 32   299 / 283    308 / 299                 332 / 324
+//   not       37 x 115   246 / 254    262 / 273    275 / 282    282 / 289
+//             39 x 110   247 / 247    263 / 265    271 / 276    279 / 283
+//             48 x 128                                          310 / 316
+//             50 x 72    196 / 186    217 / 221    238 / 239    253 / 272     (3600 positions, folded)
+//             104 x 48                279 / 270                 304 / 307
+//             96 x 64                                           316 / 322
+//   12 x 768  12 x 128   500 / 457    553 / 477    603 / 530    616 / 544
+//             14 x 128   565 / 509    571 / 594    667 / 657    694 / 677
+//             16 x 128   568 / 588    579 / 609    702 / 684    707 / 686     from 1/16 on 562 / 511
+//             20 x 128   645 / 644    671 / 693    716 / 698    774 / 752     613 / 602
+//             22 x 128   658 / 670    699 / 699    773 / 758    800 / 790
+//             40 x 64    640 / 635    666 / 671    710 / 685    767 / 737
+//             60 x 48    689 / 671    731 / 702    794 / 783    832 / 844
+//             64 x 32    596 / 541    606 / 595    730 / 663    736 / 669
+//             128 x 32                860 / 825                 1103 / 1045
+//   not       24 x 128   666 / 682    714 / 709    798 / 790    829 / 829
+//             32 x 128                823 / 856                 1030 / 1048
+//             70 x 48    732 / 709    751 / 747    795 / 829    970 / 980
+//             64 x 64                 785 / 846                 1027 / 1050
 constexpr int kNarrowHidden = 384;
 bool qkv_attention_pays(const rlx_encoder_config_t& c, int B, int S) {
     const bool narrow = c.hidden <= kNarrowHidden;
-    if (S > rlx::kBinRows / 2) return call_tokens(B, S) <= (narrow ? 40ll : 22ll) * S;
-    return call_tokens(B, S) <= (S > rlx::kBinRows / 4 ? (narrow ? 4736 : 2880) : (narrow ? 6144 : 4096));
+    const long long tokens = call_tokens(B, S);
+    if (S > rlx::kBinRows / 2) return tokens <= (narrow ? (tokens <= kAutoFoldMaxTokens ? 40ll : 36ll) : 22ll) * S;
+    return tokens <= (S > rlx::kBinRows / 4 ? (narrow ? 4736 : 2880) : (narrow ? 6144 : 4096));
 }
 bool uses_qkv_attention(const rlx_encoder_config_t& c, int B, int S) {
     if (c.flags & (RLX_FLAG_GEMM_SIMT | RLX_FLAG_KERNEL_EVENTS | RLX_FLAG_NO_PACK | RLX_FLAG_ATTN_TCGEN05)) return false;

@@ -289,7 +289,7 @@ def test_folded_weights_by_launch(rlx, name, hidden, ffn, heads, layers):
     ("c1", 1, 1, "full"), ("c1", 1, 128, "full"), ("c1", 1, 16, "ragged"), ("c1", 5, 33, "ragged"),
     ("c1", 12, 128, "full"), ("c1", 13, 128, "ragged"),                    # one head per CTA, two
     ("c1", 40, 3, "ragged"), ("c1", 200, 17, "one"),                       # bins that are full by their number of sequences
-    ("c1", 32, 128, "ragged"), ("c1", 33, 125, "ragged"), ("c1", 40, 128, "ragged"), ("c1", 40, 128, "full"), ("c1", 192, 32, "ragged"), ("c1", 74, 64, "full"),
+    ("c1", 32, 128, "ragged"), ("c1", 33, 125, "ragged"), ("c1", 36, 128, "ragged"), ("c1", 36, 128, "full"), ("c1", 40, 102, "ragged"), ("c1", 192, 32, "ragged"), ("c1", 74, 64, "full"),
     ("c1", 31, 130, "ragged"), ("c1", 41, 65, "ragged"), ("c1", 193, 32, "ragged"), ("c1", 75, 64, "full"), ("c1", 48, 128, "full"),                                            # the last sizes that take it, the first that do not
     ("c4", 1, 128, "full"), ("c4", 7, 120, "ragged"), ("c4", 9, 64, "holes"), ("c4", 64, 31, "ragged"), ("c4", 22, 128, "ragged"),
     ("c4", 45, 64, "full"), ("c4", 128, 32, "ragged"), ("c4", 23, 65, "ragged"), ("c4", 32, 128, "ragged")])
