@@ -5,7 +5,8 @@
 // as possible while all tiles run beside each other, narrower where that fills pairs that would idle.  61 sequences of
 // up to 203 at N = 384: 29 row blocks are 58 tiles of 192 columns, one round of 74 pairs, or 87 of 128, two; with every position
 // valid 49 are 98 or 147, two rounds each, and the narrow ones are shorter.
-// So the width is a variable here; the rest is gemm_tcgen05.cuh's pair kernel with two k-blocks per stage.  The loops of
+// So the width is a variable here; the rest is gemm_tcgen05.cuh's pair kernel, with its stages of each width (192 columns in three
+// stages of two k-blocks instead of seven of one: 12 x 768, 20 x 512 with all positions valid 2477 us where the fixed kernel took 2424, now 2441).  The loops of
 // the producer and the issuer are compiled for each width, nothing is divided, and shared memory is left for the CTAs of the next
 // kernel: where the width comes out as the fixed kernel's, that much less is lost (us fixed / chosen, 6 x 384, before and now: 50 x 128 with
 // half of the positions valid 272.7 / 276.4 and 273.4 / 274.0, 64 x 128 288.1 / 292.4 and 288.6 / 290.9, 24 x 400 384.4 / 390.2 and 385.9 / 389.2).
@@ -18,7 +19,7 @@ namespace tcpw {
 
 using namespace rlx::tc;
 
-constexpr int kMaxBN = 192, kKps = 2, kMaxStages = 4;
+constexpr int kMaxBN = 192, kMaxStages = 7;
 constexpr int kABytes = BLOCK_M * BLOCK_K * 2;
 constexpr int kEpiWarps = 12, kThreads = 64 + 32 * kEpiWarps;
 constexpr int kBarBytes = 8 * (2 * kMaxStages + 4) + 16;
@@ -26,13 +27,13 @@ template <int EPI>
 struct Cfg {
     static constexpr bool VEC = EPI >= 3;
     static constexpr int VEC_BYTES = VEC ? kEpiWarps * 384 : 0;
-    static constexpr int RING_BYTES = kMaxStages * kKps * (kABytes + 64 * BLOCK_K * 2);   // four stages at 128 columns
+    static constexpr int RING_BYTES = kMaxStages * (kABytes + 96 * BLOCK_K * 2);   // seven k-blocks at 192 columns, four pairs of them at 128
     static constexpr int STG_OFF = RING_BYTES, VEC_OFF = STG_OFF + kEpiWarps * kStageBufBytes, BAR_OFF = VEC_OFF + VEC_BYTES, SMEM_BYTES = BAR_OFF + kBarBytes + 1024;
     static_assert(SMEM_BYTES <= 227 * 1024, "shared memory");
-    static_assert(3 * kKps * (kABytes + kMaxBN / 2 * BLOCK_K * 2) <= RING_BYTES, "three stages of the widest tile");
 };
 struct Widths {
-    CUtensorMap w[3];             // W as pairs of k-blocks, boxes of 32, 64 and 96 rows: a CTA's half of a tile of 64, 128 and 192 columns
+    CUtensorMap a1;               // A by single k-blocks
+    CUtensorMap w[3];             // W, boxes of 32, 64 and 96 rows: a CTA's half of a tile of 64, 128 (pairs of k-blocks) and 192 columns (single ones)
     int n_tiles[3];               // tiles of a row block at each width
     uint32_t inv[3], inv_pairs;   // reciprocals of those and of the number of pairs, see div_by
 };
@@ -53,12 +54,16 @@ __device__ __forceinline__ int pick_width(const Widths& wm, int blocks, int pair
     return best;
 }
 
+// k-blocks of a stage, as in gemm_tcgen05.cuh's Cfg: narrow tiles take two behind one barrier round, wide ones a deeper ring.
+constexpr int kps(int width) { return width == 3 ? 1 : 2; }
+
 // The loops of the producer and of the issuer, for each width: with stage size, box and instruction shape as variables a stage takes
 // the issuing thread longer than its products.
 template <int EPI, int WIDTH>
 struct Loop {
-    static constexpr int BN = 64 * WIDTH, B_ROWS = 32 * WIDTH, B_BYTES = B_ROWS * BLOCK_K * 2, STAGE_BYTES = kKps * (kABytes + B_BYTES);
+    static constexpr int KPS = kps(WIDTH), BN = 64 * WIDTH, B_ROWS = 32 * WIDTH, B_BYTES = B_ROWS * BLOCK_K * 2, STAGE_BYTES = KPS * (kABytes + B_BYTES);
     static constexpr int FIT = Cfg<EPI>::RING_BYTES / STAGE_BYTES, STAGES = FIT < kMaxStages ? FIT : kMaxStages;
+    static_assert(STAGES >= 4, "ring too shallow");
 
     static __device__ __forceinline__ void produce(const CUtensorMap* map_a, const CUtensorMap* map_w, uint32_t base, uint32_t full_bar,
                                                    uint32_t empty_bar, int n_tiles, uint32_t inv, int num_tiles, int num_kb, int pairs, uint32_t cta_rank,
@@ -68,13 +73,13 @@ struct Loop {
         for (int tile = blockIdx.x / 2; tile < num_tiles; tile += pairs) {
             const int m_blk = div_by(tile, inv);
             const int arow = m_blk * 256 + (int)cta_rank * BLOCK_M, brow = (tile - m_blk * n_tiles) * BN + (int)cta_rank * B_ROWS;
-            for (int kb = 0; kb < num_kb; kb += kKps) {
+            for (int kb = 0; kb < num_kb; kb += KPS) {
                 if (!mbar_wait_warp(empty_bar + 8 * stage, phase, abort_flag)) return;
                 if (elect_one()) {
                     const uint32_t st = base + stage * STAGE_BYTES, lead_full = map_to_cta(full_bar + 8 * stage, 0);
                     if (cta_rank == 0) mbar_expect_tx(full_bar + 8 * stage, 2 * STAGE_BYTES);
                     tma_load_3d_cg2(st, map_a, 0, arow, kb, lead_full);
-                    tma_load_3d_cg2(st + kKps * kABytes, map_w, 0, brow, kb, lead_full);
+                    tma_load_3d_cg2(st + KPS * kABytes, map_w, 0, brow, kb, lead_full);
                 }
                 __syncwarp();
                 if (++stage == STAGES) { stage = 0; phase ^= 1; }
@@ -85,7 +90,7 @@ struct Loop {
     static __device__ __forceinline__ void issue(uint32_t tmem, uint32_t base, uint32_t full_bar, uint32_t empty_bar, uint32_t tfull_bar,
                                                  uint32_t tempty_bar, int num_tiles, int num_kb, int pairs, volatile int* abort_flag) {
         constexpr uint32_t idesc = make_idesc(256, BN);
-        const uint64_t ad0 = make_smem_desc(base), bd0 = make_smem_desc(base + kKps * kABytes);
+        const uint64_t ad0 = make_smem_desc(base), bd0 = make_smem_desc(base + KPS * kABytes);
         uint32_t stage = 0, phase = 0;
         int it = 0;
         for (int tile = blockIdx.x / 2; tile < num_tiles; tile += pairs, ++it) {
@@ -93,13 +98,13 @@ struct Loop {
             if (!mbar_wait_warp(tempty_bar + 8 * as, ((it >> 1) & 1) ^ 1, abort_flag)) return;
             tc_fence_after();
             const uint32_t acc = tmem + as * kMaxBN;
-            for (int kb = 0; kb < num_kb; kb += kKps) {
+            for (int kb = 0; kb < num_kb; kb += KPS) {
                 if (!mbar_wait_warp(full_bar + 8 * stage, phase, abort_flag)) return;
                 tc_fence_after();
                 if (elect_one()) {
                     const uint64_t ad = ad0 + stage * (STAGE_BYTES >> 4), bd = bd0 + stage * (STAGE_BYTES >> 4);
 #pragma unroll
-                    for (int i = 0; i < kKps; ++i)
+                    for (int i = 0; i < KPS; ++i)
 #pragma unroll
                         for (int k = 0; k < BLOCK_K / UMMA_K; ++k)
                             umma_bf16<2>(acc, ad + (i * (kABytes >> 4) + 2 * k), bd + (i * (B_BYTES >> 4) + 2 * k), idesc, (kb | i | k) != 0 ? 1u : 0u);
@@ -139,6 +144,7 @@ gemm_pair_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gri
         *abort_flag = 0;
         fence_barrier_init();
         prefetch_tmap(&tmap_a);
+        prefetch_tmap(&wm.a1);
         prefetch_tmap(&tmap_out);
     }
     if (warp == 1) {
@@ -162,7 +168,7 @@ gemm_pair_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_a, const __gri
         if (lane == 0) prefetch_tmap(map_w);
         __syncwarp();
         pdl_wait();
-        if (width == 3) Loop<EPI, 3>::produce(&tmap_a, map_w, base, full_bar, empty_bar, n_tiles, inv, num_tiles, num_kb, pairs, cta_rank, abort_flag);
+        if (width == 3) Loop<EPI, 3>::produce(&wm.a1, map_w, base, full_bar, empty_bar, n_tiles, inv, num_tiles, num_kb, pairs, cta_rank, abort_flag);
         else if (width == 2) Loop<EPI, 2>::produce(&tmap_a, map_w, base, full_bar, empty_bar, n_tiles, inv, num_tiles, num_kb, pairs, cta_rank, abort_flag);
         else Loop<EPI, 1>::produce(&tmap_a, map_w, base, full_bar, empty_bar, n_tiles, inv, num_tiles, num_kb, pairs, cta_rank, abort_flag);
     } else if (warp == 1) {

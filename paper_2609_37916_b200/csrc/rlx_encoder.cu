@@ -718,13 +718,13 @@ rlx_status_t launch_gemm_tc_bn(const CUtensorMap& ta, const CUtensorMap& tb, con
 // every width divides, more tiles of 128 columns than pairs, so that the width decides on the rounds, and few enough rounds that one more
 // or less counts.  Whole forwards, us fixed / chosen, with the share of the positions that are valid: where another width than the
 // fixed one wins (128 columns up to 73 row blocks at N = 384 and 36 at 768, 192 beyond)
-//   6 x 384    61 x 203 0.6 433 / 420, 64 x 128 0.8 378 / 365 and 1.0 409 / 395, 14 x 512 1.0 481 / 466, 100 x 128 0.6 417 / 405, 60 x 256 0.5 460 / 445,
-//              24 x 512 0.6 479 / 464, 140 x 128 0.5 448 / 434
-//   12 x 768   26 x 128 1.0 1026 / 961, 32 x 128 1.0 1098 / 1050, 48 x 128 0.5 944 / 906, 20 x 512 0.5 1421 / 1353
+//   6 x 384    61 x 203 0.6 432 / 416, 64 x 128 0.8 378 / 364 and 1.0 407 / 392, 14 x 512 1.0 480 / 462, 100 x 128 0.6 416 / 402, 60 x 256 0.5 461 / 444,
+//              24 x 512 0.6 481 / 460, 140 x 128 0.5 445 / 432
+//   12 x 768   26 x 128 1.0 1021 / 943, 32 x 128 1.0 1108 / 1041, 48 x 128 0.5 949 / 892 and 0.75 1147 / 1096, 20 x 512 0.5 1487 / 1419, 90 x 128 0.5 1485 / 1413
 // and where it does not, which the host cannot know
-//   6 x 384    64 x 128 0.5 288.6 / 290.9, 14 x 512 0.6 341.4 / 342.7, 24 x 400 0.6 385.9 / 389.2 and 1.0 566.9 / 570.3, 28 x 512 0.25 311.1 / 313.4,
-//              140 x 128 0.25 304.6 / 307.6, 61 x 203 1.0 590 / 591
-//   12 x 768   26 x 128 0.5 681.5 / 683.9 and 0.75 785 / 794, 16 x 256 0.5 748 / 750
+//   6 x 384    64 x 128 0.5 287.8 / 290.5, 14 x 512 0.6 341.2 / 342.4, 24 x 400 0.6 385.0 / 388.7 and 1.0 564.7 / 568.6, 28 x 512 0.25 310.8 / 313.5,
+//              140 x 128 0.25 303.6 / 306.6
+//   12 x 768   26 x 128 0.5 682 / 682 and 0.75 784 / 791, 16 x 256 0.5 744 / 745, 20 x 512 0.75 1843 / 1844 and 1.0 2444 / 2441, 90 x 128 0.75 1947 / 1950 and 1.0 2495 / 2489
 // With fewer tiles the fixed width's smaller code wins (32 x 128 181 / 185).
 bool pair_width_pays(int M, int N, int K, int epi, const TileChoice& tc) {
     int dev = 0;
@@ -736,9 +736,11 @@ bool pair_width_pays(int M, int N, int K, int epi, const TileChoice& tc) {
 rlx_status_t launch_gemm_pair(const bf16* A, const bf16* W, const CUtensorMap& to, const rlx::tc::Params& p, int epi, cudaStream_t st) {
     CUtensorMap ta;
     rlx::tcpw::Widths wm;
-    if (!make_tmap_kblocks(&ta, A, p.M, p.K, rlx::tc::BLOCK_M, rlx::tcpw::kKps)) return RLX_ERR_CUDA;
+    if (!make_tmap_kblocks(&ta, A, p.M, p.K, rlx::tc::BLOCK_M, rlx::tcpw::kps(2)) ||
+        !make_tmap_kblocks(&wm.a1, A, p.M, p.K, rlx::tc::BLOCK_M, rlx::tcpw::kps(3)))
+        return RLX_ERR_CUDA;
     for (int i = 0; i < 3; ++i)
-        if (!make_tmap_kblocks(wm.w + i, W, p.N, p.K, 32 * (i + 1), rlx::tcpw::kKps)) return RLX_ERR_CUDA;
+        if (!make_tmap_kblocks(wm.w + i, W, p.N, p.K, 32 * (i + 1), rlx::tcpw::kps(i + 1))) return RLX_ERR_CUDA;
     int dev = 0;
     cudaGetDevice(&dev);
     const int grid = 2 * std::min((p.M + 255) / 256 * (p.N / 64), g_max_pairs[dev]);
