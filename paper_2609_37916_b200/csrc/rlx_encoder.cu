@@ -1292,7 +1292,7 @@ bool uses_attention_fwd(const rlx_encoder_config_t& c, int B, int S) {
 //             40 x 72    185 / 166    199 / 177    213 / 207    223 / 229
 //             40 x 96    214 / 211    222 / 221    243 / 243    248 / 250
 //             33 x 125   248 / 247    263 / 262    276 / 272    281 / 278     LayerNorms apart from here on
-//             36 x 128   254 / 254    271 / 270    278 / 279    282 / 281
+//             36 x 128   254 / 254    271 / 270    278 / 279    282 / 281     (6 heads of 64: 261 / 266 and 271 / 274)
 //             72 x 64                 268 / 262                 279 / 269
 //             96 x 48                 268 / 262                 285 / 283
 //             192 x 32   299 / 283    308 / 299                 332 / 324
@@ -1319,7 +1319,10 @@ constexpr int kNarrowHidden = 384;
 bool qkv_attention_pays(const rlx_encoder_config_t& c, int B, int S) {
     const bool narrow = c.hidden <= kNarrowHidden;
     const long long tokens = call_tokens(B, S);
-    if (S > rlx::kBinRows / 2) return tokens <= (narrow ? (tokens <= kAutoFoldMaxTokens ? 40ll : 36ll) : 22ll) * S;
+    if (S > rlx::kBinRows / 2) {
+        if (!narrow) return tokens <= 22ll * S;
+        return tokens <= kAutoFoldMaxTokens ? tokens <= 40ll * S : tokens <= 36ll * S && c.hidden / c.num_heads == 32;
+    }
     return tokens <= (S > rlx::kBinRows / 4 ? (narrow ? 4736 : 2880) : (narrow ? 6144 : 4096));
 }
 bool uses_qkv_attention(const rlx_encoder_config_t& c, int B, int S) {

@@ -112,7 +112,7 @@ def test_heads_go_on_to_the_attention_output_only_where_a_cluster_of_them_fits(l
 def test_projection_and_attention_are_one_kernel_up_to_the_line_of_the_width_and_of_the_length(lib):
     narrow = [(36, 128, 1), (37, 128, 0), (37, 111, 0), (40, 102, 1), (40, 65, 1), (41, 65, 0), (41, 128, 0), (74, 64, 1), (75, 64, 0), (143, 33, 1), (144, 33, 0), (192, 32, 1), (193, 32, 0), (1, 129, 0)]
     wide = [(22, 128, 1), (23, 65, 0), (45, 64, 1), (46, 64, 0), (87, 33, 1), (88, 33, 0), (128, 32, 1), (129, 32, 0)]
-    for hidden, heads, batch, seq, one in [(384, 12, *c) for c in narrow] + [(768, 12, *c) for c in wide]:
+    for hidden, heads, batch, seq, one in [(384, 12, *c) for c in narrow] + [(384, 6, 36, 128, 0), (384, 6, 40, 102, 1)] + [(768, 12, *c) for c in wide]:
         enc = binding.Encoder(**_cfg(hidden=hidden, num_heads=heads, ffn=4 * hidden, max_batch=256, max_seq=256, flags=binding.FLAG_NO_PREFETCH | binding.FLAG_NO_AUTO_FOLD))
         assert enc.launches_per_forward(batch, seq) == 3 + 7 * 6 - (6 + (batch * seq <= 4096) if one else 0), (hidden, batch, seq)
         enc.close()
